@@ -83,8 +83,7 @@ void release(lipcache* h) {
   dev_free(h->ipn_dn32);
   dev_free(h->ipn_min32);
   dev_free(h->ipn_max32);
-  dev_free(h->gram[0]);
-  dev_free(h->gram[1]);
+  dev_free(h->spec_work);
   dev_free(h->spec);
   if (h->spec_host) cudaFreeHost(h->spec_host);
   lc::release_select(h);
@@ -215,8 +214,7 @@ LC_API lipcache_status lipcache_create(int32_t d, int32_t C, int64_t capacity, i
       dev_alloc(h->ipn_min32, (size_t)C);
       dev_alloc(h->ipn_max32, (size_t)C);
     }
-    dev_alloc(h->gram[0], (size_t)d * d);
-    dev_alloc(h->gram[1], (size_t)d * d);
+    dev_alloc(h->spec_work, lc::spectral_work_bytes(d, C));
     dev_alloc(h->spec, 1);
     LC_CUDA(cudaMallocHost(&h->spec_host, sizeof(lc::SpecResult)));
     // Whole key tiles: rows past the current size are zero keys whose screen
@@ -285,6 +283,7 @@ LC_API lipcache_status lipcache_set_head(lipcache_t* h, const float* W, const fl
     const lc::SpecResult r = *h->spec_host;
     h->sigma_iterations = r.iterations;
     h->sigma_residual = r.residual_rel;
+    LC_REQUIRE(r.converged != -1, LIPCACHE_E_DEVICE, "a bounded wait of the spectral-norm kernel expired");
     LC_REQUIRE(!r.degenerate && r.sigma > 0.0, LIPCACHE_E_DEGENERATE_HEAD,
                "sigma_max(W) <= 0: the GuardNet head is degenerate (Algorithm 1 stops construction)");
     LC_REQUIRE(r.converged, LIPCACHE_E_NOT_CONVERGED,

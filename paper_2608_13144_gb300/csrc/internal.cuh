@@ -186,7 +186,7 @@ struct lipcache {
   float* ipn_dn32 = nullptr;       // C x C: FP32 lower bound (+inf where ||W_y - W_j|| is 0)
   float* ipn_min32 = nullptr;      // C: min_j of ipn_dn32[y][j] over the rows W_j != W_y (0 if none)
   float* ipn_max32 = nullptr;      // C: max_j of ipn_up32[y][j] over j != y (+inf if some W_j = W_y)
-  double* gram[2] = {nullptr, nullptr};  // d x d FP64
+  unsigned char* spec_work = nullptr;    // scratch of the spectral norm (spectral_work_bytes)
   lc::SpecResult* spec = nullptr;        // device
   lc::SpecResult* spec_host = nullptr;   // pinned
 
@@ -290,6 +290,7 @@ namespace lc {
 
 // ---------------------------------------------------------------- launchers
 // spectral.cu
+size_t spectral_work_bytes(int d, int C);
 void spectral_norm(lipcache* h, cudaStream_t s);
 // certify.cu
 // Certify H and append the accepted rows; miss_of (nullable, n entries) limits

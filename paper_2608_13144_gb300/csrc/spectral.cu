@@ -10,152 +10,355 @@
 // iteration then runs on W itself (w = W v, theta = ||w||^2 = v^T A v,
 // u = W^T w) until successive Rayleigh quotients agree to 1e-13 relative and
 // ||A v - theta v|| <= 1e-10 theta.
+//
+// FP64 on this GPU: a dependent instruction takes ~64 cycles, and four warps of
+// an SM together issue one every ~22 (measured), so the work is laid out for
+// that pipe: one cooperative kernel (k_spectral) holds the whole method, four
+// warps on each of as many SMs as the shape fills, a lane per output element.
 #include "internal.cuh"
 
 namespace lc {
 namespace {
 
-constexpr int kTile = 16;
+constexpr int kSpThreads = 128;            // one warp per SM sub-partition
+constexpr int kSpWarps = kSpThreads / 32;
+constexpr int kSpChunk = 128;              // summation steps staged in shared memory at a time
+constexpr long long kSpWaitLimit = 1LL << 31;  // ~1 s at GB300 clocks
+constexpr unsigned kSpAbort = 0x80000000u;
 
-// A = W^T W (d x d, FP64). Products of FP32 values are exact in FP64; the
-// accumulation order is the same for (i, j) and (j, i), so A is bitwise
-// symmetric.
-__global__ void k_gram(const float* __restrict__ W, int C, int d, double* __restrict__ A) {
-  const int j = blockIdx.x * kTile + threadIdx.x;
-  const int i = blockIdx.y * kTile + threadIdx.y;
-  if (i >= d || j >= d) return;
-  double acc = 0.0;
-  for (int c = 0; c < C; ++c) acc = fma((double)W[(size_t)c * d + i], (double)W[(size_t)c * d + j], acc);
-  A[(size_t)i * d + j] = acc;
+// Barrier of the whole (co-resident) grid; `target` arrivals in all. Bounded:
+// on expiry the abort bit releases every CTA and all return false.
+__device__ bool grid_barrier(unsigned* ctr, unsigned target) {
+  __shared__ unsigned seen;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(ctr, 1u);
+    unsigned v;
+    const long long t0 = clock64();
+    for (;;) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
+      if (v >= target) break;
+      if (clock64() - t0 > kSpWaitLimit) v = atomicOr(ctr, kSpAbort) | kSpAbort;
+    }
+    seen = v;
+  }
+  __syncthreads();
+  return (seen & kSpAbort) == 0;
 }
 
-// B = (A / tr A)^2 with a tiled FP64 product; every block recomputes the
-// trace (d loads). A zero trace (W = 0) yields B = 0.
-__global__ void k_square(const double* __restrict__ A, double* __restrict__ B, int d) {
-  __shared__ double As[kTile][kTile + 1];
-  __shared__ double Bs[kTile][kTile + 1];
-  __shared__ double red[kTile * kTile];
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kTile + tx;
-  double t = 0.0;
-  for (int k = tid; k < d; k += kTile * kTile) t += A[(size_t)k * d + k];
-  red[tid] = t;
-  __syncthreads();
-  for (int s = kTile * kTile / 2; s > 0; s >>= 1) {
-    if (tid < s) red[tid] += red[tid + s];
-    __syncthreads();
-  }
-  const double tr = red[0];
-  const double inv = tr > 0.0 ? 1.0 / tr : 0.0;
-  const int i = blockIdx.y * kTile + ty;
-  const int j = blockIdx.x * kTile + tx;
-  double acc = 0.0;
-  for (int k0 = 0; k0 < d; k0 += kTile) {
-    As[ty][tx] = (i < d && k0 + tx < d) ? A[(size_t)i * d + k0 + tx] * inv : 0.0;
-    Bs[ty][tx] = (k0 + ty < d && j < d) ? A[(size_t)(k0 + ty) * d + j] * inv : 0.0;
-    __syncthreads();
+// Sum over 256 slots, slot l + 32 m in v[m] of lane l, in the order of a
+// shared-memory tree (slot t += slot t + s for s = 128, 64, ..., 1); slots
+// from n on are zero and are left out (adding +0 changes nothing). Every lane
+// returns the sum.
+__device__ double tree256(double (&v)[8], int n) {
 #pragma unroll
-    for (int k = 0; k < kTile; ++k) acc = fma(As[ty][k], Bs[k][tx], acc);
-    __syncthreads();
-  }
-  if (i < d && j < d) B[(size_t)i * d + j] = acc;
+  for (int s = 4; s > 0; s >>= 1)
+#pragma unroll
+    for (int m = 0; m < s; ++m)
+      if (32 * (m + s) < n) v[m] = v[m] + v[m + s];
+  double x = v[0];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x = x + __shfl_down_sync(0xffffffffu, x, o);
+  return __shfl_sync(0xffffffffu, x, 0);
 }
 
-constexpr int kPowerThreads = 256;
-
-__device__ double block_sum(double v, double* red) {
-  const int tid = threadIdx.x;
-  red[tid] = v;
-  __syncthreads();
-  for (int s = kPowerThreads / 2; s > 0; s >>= 1) {
-    if (tid < s) red[tid] += red[tid + s];
-    __syncthreads();
+// Sum of x(k)^2, k < n: slot t adds k = t, t + 256, ... in order.
+template <typename F>
+__device__ double sum_squares(int n, int lane, F x) {
+  double v[8];
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    v[m] = 0.0;
+    for (int k = lane + 32 * m; k < n; k += 256) {
+      const double e = x(k);
+      v[m] = fma(e, e, v[m]);
+    }
   }
-  const double r = red[0];
-  __syncthreads();
-  return r;
+  return tree256(v, n);
 }
 
-// Final power iteration on W (one block). `As` is the last squared matrix
-// (or nullptr to start from a fixed, slightly perturbed all-ones vector).
-__global__ void __launch_bounds__(kPowerThreads) k_power(const float* __restrict__ W, int C, int d,
-                                                         const double* __restrict__ As, int max_iter,
-                                                         SpecResult* __restrict__ res) {
-  extern __shared__ double sm[];
-  double* v = sm;          // d
-  double* w = v + d;       // C
-  double* u = w + C;       // d
-  __shared__ double red[kPowerThreads];
-  __shared__ int jstar;
-  const int tid = threadIdx.x;
+// One fused multiply-add chain sum_k col[k stride] x[k], k < n ascending, the
+// loads of sixteen steps in flight while the sixteen before them are added.
+__device__ double chain16(const double* col, size_t stride, const double* x, int n) {
+  constexpr int N = 16;
+  double acc = 0.0, cur[N], nxt[N];
+#pragma unroll
+  for (int u = 0; u < N; ++u) cur[u] = u < n ? __ldcg(col + (size_t)u * stride) : 0.0;
+  for (int k = 0; k < n; k += N) {
+#pragma unroll
+    for (int u = 0; u < N; ++u) nxt[u] = k + N + u < n ? __ldcg(col + (size_t)(k + N + u) * stride) : 0.0;
+#pragma unroll
+    for (int u = 0; u < N; ++u)
+      if (k + u < n) acc = fma(cur[u], x[k + u], acc);
+#pragma unroll
+    for (int u = 0; u < N; ++u) cur[u] = nxt[u];
+  }
+  return acc;
+}
 
-  if (As) {
-    if (tid == 0) {
-      int best = 0;
-      for (int k = 1; k < d; ++k)
-        if (As[(size_t)k * d + k] > As[(size_t)best * d + best]) best = k;
-      jstar = best;
+struct SpectralArgs {
+  const float* W;  // C x d
+  int C, d, Cp, dp;  // Cp, dp: C, d rounded up to 32
+  int squarings, max_iter, n_tiles;
+  double* A[2];    // d x dp, blocked layout (columns from d on are never read into a result)
+  double* Wd;      // C x dp, blocked layout: the head in FP64, zero past d
+  double* WdT;     // d x Cp, zero past C
+  double* w;       // C
+  double* u;       // d
+  unsigned* ctr;   // grid barrier, zero at launch
+  SpecResult* res;
+};
+
+// Element (k, j) of a matrix with K rows in column blocks of 32: a block's
+// rows are contiguous (a panel of 32 columns is one stream; rows of a
+// power-of-two length apart cost 80 cycles a request at d = 256).
+__device__ __forceinline__ size_t blk(int k, int j, int K) { return ((size_t)(j >> 5) * K + k) * 32 + (j & 31); }
+
+// The symmetric product P_ij = sum_k X[k][i] X[k][j] (k < K ascending, one
+// fused multiply-add chain per element) into B, X = S (K rows, blocked
+// layout) or, with `scale`, S * (1 / tr S) rounded: S is symmetric or is the operand
+// itself, so one panel of columns and one of rows serve, and only i <= j is
+// computed ((j, i) would add the same products in the same order). A tile is
+// 32 columns (lanes) by 4 R rows (R chains per warp); tiles are numbered over
+// the upper triangle.
+template <int R>
+__device__ void sym_product(const double* S, int K, bool scale, double* B, int d, int n_tiles, double* sm,
+                            double* red) {
+  constexpr int kRows = kSpWarps * R;
+  double* cp = sm;                   // kSpChunk x 32
+  double* rp = sm + kSpChunk * 32;   // kSpChunk x kRows
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int per = 32 / kRows;  // row blocks per 32 rows
+  double inv = 1.0;
+  bool have_inv = !scale;
+  for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    int cb = 0, rb = tile;  // column block cb has (cb + 1) * per row blocks
+    while (rb >= (cb + 1) * per) {
+      rb -= (cb + 1) * per;
+      ++cb;
+    }
+    const int j0 = cb * 32, i0 = rb * kRows;
+    double acc[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = 0.0;
+    for (int k0 = 0; k0 < K; k0 += kSpChunk) {
+      const int kc = K - k0 < kSpChunk ? K - k0 : kSpChunk;
+      __syncthreads();
+      // every load of the panels is issued before the first is used (one L2
+      // round trip per chunk), every product before the first is stored (an
+      // FP64 result takes ~90 cycles)
+      constexpr int NC = kSpChunk / kSpWarps, NR = kSpChunk * kRows / kSpThreads;
+      double xc[NC], xr[NR];
+      const double* sc = S + blk(k0, j0 + lane, K);
+      const double* sr = S + blk(k0, i0 + tid % kRows, K);
+#pragma unroll
+      for (int u = 0; u < NC; ++u) {
+        const int k = warp + u * kSpWarps;
+        xc[u] = k < kc ? __ldcg(sc + k * 32) : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < NR; ++u) {
+        const int k = tid / kRows + u * (kSpThreads / kRows);
+        xr[u] = k < kc ? __ldcg(sr + k * 32) : 0.0;
+      }
+      if (!have_inv) {
+        // the trace, while the panels are on their way
+        if (warp == 0) {
+          double v[8];
+#pragma unroll
+          for (int m = 0; m < 8; ++m) {
+            const int k = lane + 32 * m;
+            v[m] = k < d ? __ldcg(S + blk(k, k, d)) : 0.0;
+          }
+          if (d > 256)
+#pragma unroll
+            for (int m = 0; m < 8; ++m)
+              for (int k = lane + 32 * m + 256; k < d; k += 256) v[m] += __ldcg(S + blk(k, k, d));
+          const double tr = tree256(v, d);
+          if (lane == 0) *red = tr > 0.0 ? 1.0 / tr : 0.0;  // a zero trace (W = 0) gives a zero product
+        }
+        __syncthreads();
+        inv = *red;
+        have_inv = true;
+      }
+      if (scale) {
+#pragma unroll
+        for (int u = 0; u < NR; ++u) xr[u] *= inv;
+#pragma unroll
+        for (int u = 0; u < NC; ++u)
+          if (u * kSpWarps < kc) xc[u] *= inv;
+        asm volatile("" ::: "memory");
+      }
+#pragma unroll
+      for (int u = 0; u < NR; ++u) {
+        const int k = tid / kRows + u * (kSpThreads / kRows);
+        if (k < kc) rp[k * kRows + tid % kRows] = xr[u];
+      }
+#pragma unroll
+      for (int u = 0; u < NC; ++u) {
+        const int k = warp + u * kSpWarps;
+        if (k < kc) cp[k * 32 + lane] = xc[u];
+      }
+      __syncthreads();
+#pragma unroll 8
+      for (int k = 0; k < kc; ++k) {
+        const double c = cp[k * 32 + lane];
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = fma(rp[k * kRows + warp * R + r], c, acc[r]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int i = i0 + warp * R + r, j = j0 + lane;
+      if (i <= j && j < d) {
+        B[blk(i, j, d)] = acc[r];
+        if (i < j) B[blk(j, i, d)] = acc[r];
+      }
+    }
+  }
+}
+
+// The spectral norm of W by a co-resident grid: FP64 copies of W, A = W^T W,
+// `squarings` steps A <- (A / tr A)^2, then the power iteration on W. What
+// bounds it: the FP64 pipe (four warps per SM: ~88 cycles per step of their
+// chains); a squaring costs its d steps, the panel's scaling (1 / (4 R) of the
+// products), the trace and one grid barrier. Everything is added in the order
+// of the tests' saved caches: sigma keeps its bits.
+template <int R>
+__global__ void __launch_bounds__(kSpThreads) k_spectral(const SpectralArgs a) {
+  __shared__ double sm[kSpChunk * 32 + kSpChunk * kSpWarps * R];
+  __shared__ double red[2];
+  static_assert(kSpChunk * 32 >= 2 * 1024 + 1024, "the iteration's vectors share the panels' space");
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int d = a.d, C = a.C, Cp = a.Cp;
+  unsigned bar = 0;
+  auto sync_grid = [&]() { return grid_barrier(a.ctr, bar += gridDim.x); };
+
+  for (int e = blockIdx.x * kSpThreads + tid; e < C * a.dp; e += gridDim.x * kSpThreads) {
+    const int c = e / a.dp, j = e - c * a.dp;
+    a.Wd[blk(c, j, C)] = j < d ? (double)a.W[(size_t)c * d + j] : 0.0;
+  }
+  for (int e = blockIdx.x * kSpThreads + tid; e < d * Cp; e += gridDim.x * kSpThreads) {
+    const int k = e / Cp, c = e - k * Cp;
+    a.WdT[e] = c < C ? (double)a.W[(size_t)c * d + k] : 0.0;
+  }
+  if (!sync_grid()) return;
+  // A grid with fewer tiles than CTAs (units of the iteration): the spare CTAs
+  // only meet the barriers.
+  int cur = 0;
+  if (a.squarings > 0) {
+    // W^T W: products of FP32 values are exact in FP64
+    sym_product<R>(a.Wd, C, false, a.A[0], d, a.n_tiles, sm, red);
+    if (!sync_grid()) return;
+    for (int q = 0; q < a.squarings; ++q) {
+      sym_product<R>(a.A[cur], d, true, a.A[cur ^ 1], d, a.n_tiles, sm, red);
+      cur ^= 1;
+      if (!sync_grid()) return;
+    }
+  }
+
+  // Power iteration on W: every CTA keeps v and repeats the short sums; the
+  // chains of w = W v and u = W^T w are spread over the grid.
+  double* v = sm;
+  double* w = sm + 1024;
+  double* u = sm + 2048;
+  __syncthreads();
+  if (a.squarings > 0) {
+    const double* A = a.A[cur];
+    // the dominant column: the first largest diagonal entry
+    if (warp == 0) {
+      double best = -INFINITY;
+      int at = 0x7fffffff;
+      for (int k = lane; k < d; k += 32) {
+        const double x = __ldcg(A + blk(k, k, d));
+        if (x > best) {
+          best = x;
+          at = k;
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oa = __shfl_xor_sync(0xffffffffu, at, o);
+        if (ob > best || (ob == best && oa < at)) {
+          best = ob;
+          at = oa;
+        }
+      }
+      if (lane == 0) red[0] = (double)(at < d ? at : 0);
     }
     __syncthreads();
-    for (int k = tid; k < d; k += kPowerThreads) v[k] = As[(size_t)k * d + jstar];
+    const int js = (int)red[0];
+    for (int k = tid; k < d; k += kSpThreads) v[k] = __ldcg(A + blk(js, k, d));
   } else {
-    for (int k = tid; k < d; k += kPowerThreads) {
+    for (int k = tid; k < d; k += kSpThreads) {
       unsigned x = (unsigned)k * 2654435761u;
       x ^= x >> 15;
       v[k] = 1.0 + 0.01 * (double)(x & 0xffff) / 65536.0;
     }
   }
   __syncthreads();
-  double nv = 0.0;
-  for (int k = tid; k < d; k += kPowerThreads) nv += v[k] * v[k];
-  nv = sqrt(block_sum(nv, red));
-
-  double theta = 0.0, theta_prev = -1.0, resid = INFINITY;
-  int it = 0, converged = 0;
+  double nv = sqrt(sum_squares(d, lane, [&](int k) { return v[k]; }));
   if (!(nv > 0.0)) {
-    if (tid == 0) {
-      res->sigma = 0.0;
-      res->theta = 0.0;
-      res->residual_rel = 0.0;
-      res->iterations = 0;
-      res->converged = 1;
-      res->degenerate = 1;
+    if (blockIdx.x == 0 && tid == 0) {
+      a.res->sigma = 0.0;
+      a.res->theta = 0.0;
+      a.res->residual_rel = 0.0;
+      a.res->iterations = 0;
+      a.res->converged = 1;
+      a.res->degenerate = 1;
     }
     return;
   }
-  for (int k = tid; k < d; k += kPowerThreads) v[k] /= nv;
+  __syncthreads();
+  for (int k = tid; k < d; k += kSpThreads) v[k] /= nv;
   __syncthreads();
 
-  for (it = 1; it <= max_iter; ++it) {
-    for (int c = tid; c < C; c += kPowerThreads) {
-      double acc = 0.0;
-      for (int k = 0; k < d; ++k) acc = fma((double)W[(size_t)c * d + k], v[k], acc);
-      w[c] = acc;
+  const int cu = Cp / 32, du = (d + 31) / 32;  // 32-lane units of the two products
+  double theta = 0.0, theta_prev = -1.0, resid = INFINITY;
+  int it = 0, converged = 0;
+  for (it = 1; it <= a.max_iter; ++it) {
+    for (int g = blockIdx.x + gridDim.x * warp; g < cu; g += gridDim.x * kSpWarps) {
+      const int c = g * 32 + lane;
+      const double acc = chain16(a.WdT + c, Cp, v, d);
+      if (c < C) a.w[c] = acc;
+    }
+    if (!sync_grid()) return;
+    for (int c = tid; c < C; c += kSpThreads) w[c] = __ldcg(a.w + c);
+    __syncthreads();
+    if (warp == kSpWarps - 1) {
+      const double p = sum_squares(C, lane, [&](int c) { return w[c]; });
+      if (lane == 0) red[0] = p;
+    } else {
+      for (int g = blockIdx.x + gridDim.x * warp; g < du; g += gridDim.x * (kSpWarps - 1)) {
+        const int k = g * 32 + lane;
+        const double acc = chain16(a.Wd + blk(0, k, C), 32, w, C);
+        if (k < d) a.u[k] = acc;
+      }
+    }
+    if (!sync_grid()) return;
+    theta = red[0];
+    for (int k = tid; k < d; k += kSpThreads) u[k] = __ldcg(a.u + k);
+    __syncthreads();
+    if (warp == 0) {
+      const double pr = sum_squares(d, lane, [&](int k) { return fma(-theta, v[k], u[k]); });
+      if (lane == 0) red[0] = pr;
+    } else if (warp == 1) {
+      const double pu = sum_squares(d, lane, [&](int k) { return u[k]; });
+      if (lane == 0) red[1] = pu;
     }
     __syncthreads();
-    double p = 0.0;
-    for (int c = tid; c < C; c += kPowerThreads) p += w[c] * w[c];
-    theta = block_sum(p, red);
-    for (int k = tid; k < d; k += kPowerThreads) {
-      double acc = 0.0;
-      for (int c = 0; c < C; ++c) acc = fma((double)W[(size_t)c * d + k], w[c], acc);
-      u[k] = acc;
-    }
+    resid = sqrt(red[0]);
+    const double nu = sqrt(red[1]);
     __syncthreads();
-    double pr = 0.0, pu = 0.0;
-    for (int k = tid; k < d; k += kPowerThreads) {
-      const double e = u[k] - theta * v[k];
-      pr += e * e;
-      pu += u[k] * u[k];
-    }
-    resid = sqrt(block_sum(pr, red));
-    const double nu = sqrt(block_sum(pu, red));
     if (!(nu > 0.0)) {  // v is in the null space of W: only possible for W = 0
       theta = 0.0;
       resid = 0.0;
       converged = 1;
       break;
     }
-    for (int k = tid; k < d; k += kPowerThreads) v[k] = u[k] / nu;
+    for (int k = tid; k < d; k += kSpThreads) v[k] = u[k] / nu;
     __syncthreads();
     if (it >= 2 && fabs(theta - theta_prev) <= 1e-13 * theta && resid <= 1e-10 * theta) {
       converged = 1;
@@ -163,13 +366,13 @@ __global__ void __launch_bounds__(kPowerThreads) k_power(const float* __restrict
     }
     theta_prev = theta;
   }
-  if (tid == 0) {
-    res->theta = theta;
-    res->sigma = sqrt(theta);
-    res->residual_rel = theta > 0.0 ? resid / theta : 0.0;
-    res->iterations = it > max_iter ? max_iter : it;
-    res->converged = converged;
-    res->degenerate = !(theta > 0.0);
+  if (blockIdx.x == 0 && tid == 0) {
+    a.res->theta = theta;
+    a.res->sigma = sqrt(theta);
+    a.res->residual_rel = theta > 0.0 ? resid / theta : 0.0;
+    a.res->iterations = it > a.max_iter ? a.max_iter : it;
+    a.res->converged = converged;
+    a.res->degenerate = !(theta > 0.0);
   }
 }
 
@@ -178,30 +381,58 @@ __global__ void __launch_bounds__(kPowerThreads) k_power(const float* __restrict
 // is within gamma_d of the exact one) with its reciprocal, and FP32 brackets
 // of the reciprocal (the FP64 value widened by 1e-12, far above its error,
 // then rounded outward; +inf for coinciding rows, which the tight radius skips).
-__global__ void k_row_norms(const float* __restrict__ W, int C, int d, double* __restrict__ Wnorm,
-                            float* __restrict__ Wnorm32, double* __restrict__ pairnorm,
-                            double* __restrict__ inv_pairnorm, float* __restrict__ ipn_up32,
-                            float* __restrict__ ipn_dn32) {
-  const int y = blockIdx.y;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= C) return;
-  double acc = 0.0;
-  if (pairnorm) {
-    for (int k = 0; k < d; ++k) {
-      const double e = (double)W[(size_t)y * d + k] - (double)W[(size_t)j * d + k];
-      acc = fma(e, e, acc);
-    }
-    pairnorm[(size_t)y * C + j] = sqrt(acc);
-    const double ipn = acc > 0.0 ? 1.0 / sqrt(acc) : 0.0;
-    inv_pairnorm[(size_t)y * C + j] = ipn;
-    ipn_up32[(size_t)y * C + j] = acc > 0.0 ? __double2float_ru(ipn * (1.0 + 1e-12)) : INFINITY;
-    ipn_dn32[(size_t)y * C + j] = acc > 0.0 ? __double2float_rd(ipn * (1.0 - 1e-12)) : INFINITY;
-  }
-  if (j == y) {
+// One warp per unit (y, 32 classes j) of the upper triangle, a lane per pair;
+// the mirrored pair squares the negated differences, the same sum. Bound by
+// the FP64 pipe: two instructions per feature and 32 pairs.
+__global__ void __launch_bounds__(kSpThreads) k_row_norms(const double* __restrict__ WdT, int C, int Cp, int d,
+                                                          double* __restrict__ Wnorm, float* __restrict__ Wnorm32,
+                                                          double* __restrict__ pairnorm,
+                                                          double* __restrict__ inv_pairnorm,
+                                                          float* __restrict__ ipn_up32, float* __restrict__ ipn_dn32) {
+  const int lane = threadIdx.x & 31;
+  const int unit = blockIdx.x * kSpWarps + (threadIdx.x >> 5);
+  const int nb = Cp / 32;
+  if (unit < nb) {
+    const int c = unit * 32 + lane;
     double n2 = 0.0;
-    for (int k = 0; k < d; ++k) n2 = fma((double)W[(size_t)y * d + k], (double)W[(size_t)y * d + k], n2);
-    Wnorm[y] = sqrt(n2);
-    Wnorm32[y] = __double2float_ru(sqrt(n2) * (1.0 + 1e-15));
+#pragma unroll 8
+    for (int k = 0; k < d; ++k) {
+      const double x = WdT[(size_t)k * Cp + c];
+      n2 = fma(x, x, n2);
+    }
+    if (c < C) {
+      Wnorm[c] = sqrt(n2);
+      Wnorm32[c] = __double2float_ru(sqrt(n2) * (1.0 + 1e-15));
+    }
+    return;
+  }
+  if (!pairnorm) return;
+  int r = unit - nb, jb = 0;  // class block jb holds the units y < min(C, 32 (jb + 1))
+  for (; jb < nb; ++jb) {
+    const int ny = C < 32 * (jb + 1) ? C : 32 * (jb + 1);
+    if (r < ny) break;
+    r -= ny;
+  }
+  if (jb >= nb) return;
+  const int y = r, j = jb * 32 + lane;
+  double acc = 0.0;
+#pragma unroll 8
+  for (int k = 0; k < d; ++k) {
+    const double e = WdT[(size_t)k * Cp + y] - WdT[(size_t)k * Cp + j];
+    acc = fma(e, e, acc);
+  }
+  if (j >= C || j < y) return;
+  const double pn = sqrt(acc);
+  const double ipn = acc > 0.0 ? 1.0 / sqrt(acc) : 0.0;
+  const float up = acc > 0.0 ? __double2float_ru(ipn * (1.0 + 1e-12)) : INFINITY;
+  const float dn = acc > 0.0 ? __double2float_rd(ipn * (1.0 - 1e-12)) : INFINITY;
+#pragma unroll
+  for (int m = 0; m < 2; ++m) {
+    const size_t at = m ? (size_t)j * C + y : (size_t)y * C + j;
+    pairnorm[at] = pn;
+    inv_pairnorm[at] = ipn;
+    ipn_up32[at] = up;
+    ipn_dn32[at] = dn;
   }
 }
 
@@ -210,49 +441,94 @@ __global__ void k_row_norms(const float* __restrict__ W, int C, int d, double* _
 // ipn_min32[y] <= 1 / ||W_y - W_j|| for every j with W_j != W_y (the minimum of
 // the FP32 lower brackets; 0 when every other row equals W_y) and
 // ipn_max32[y] >= 1 / ||W_y - W_j|| for every j != y (+inf when some W_j = W_y).
-__global__ void k_ipn_min(const double* __restrict__ pairnorm, const float* __restrict__ ipn_dn32,
-                          const float* __restrict__ ipn_up32, int C, float* __restrict__ ipn_min32,
-                          float* __restrict__ ipn_max32) {
-  const int y = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(128) k_ipn_min(const double* __restrict__ pairnorm, const float* __restrict__ ipn_dn32,
+                                                 const float* __restrict__ ipn_up32, int C,
+                                                 float* __restrict__ ipn_min32, float* __restrict__ ipn_max32) {
+  const int y = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (y >= C) return;
   float m = INFINITY, mx = 0.f;
-  for (int j = 0; j < C; ++j) {
+  for (int j = lane; j < C; j += 32) {
     if (j == y) continue;
     if (pairnorm[(size_t)y * C + j] > 0.0) m = fminf(m, ipn_dn32[(size_t)y * C + j]);
     mx = fmaxf(mx, ipn_up32[(size_t)y * C + j]);
   }
-  ipn_min32[y] = m < INFINITY ? m : 0.f;
-  ipn_max32[y] = mx;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  }
+  if (lane == 0) {
+    ipn_min32[y] = m < INFINITY ? m : 0.f;
+    ipn_max32[y] = mx;
+  }
+}
+
+// Tiles of sym_product over the upper triangle of a d x d matrix.
+int sym_tiles(int d, int R) {
+  const int nb = (d + 31) / 32, per = 32 / (kSpWarps * R);
+  return nb * (nb + 1) / 2 * per;
+}
+
+template <int R>
+void launch_spectral(lipcache* h, SpectralArgs a, cudaStream_t s) {
+  a.n_tiles = sym_tiles(a.d, R);
+  const int units = (a.Cp > a.dp ? a.Cp : a.dp) / 32;
+  int grid = a.n_tiles > units ? a.n_tiles : units;
+  if (grid > h->num_sms) grid = h->num_sms;
+  void* args[] = {&a};
+  LC_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_spectral<R>), dim3((unsigned)grid),
+                                      dim3(kSpThreads), args, 0, s));
+  LC_LAUNCH_CHECK("k_spectral");
 }
 
 }  // namespace
 
+size_t spectral_work_bytes(int d, int C) {
+  const size_t Cp = (size_t)(C + 31) / 32 * 32;
+  const size_t dp = (size_t)(d + 31) / 32 * 32;
+  return sizeof(double) * (2 * dp * d + dp * C + Cp * d + C + d) + 16;
+}
+
 void spectral_norm(lipcache* h, cudaStream_t s) {
   const int d = h->d, C = h->C;
-  dim3 blk(kTile, kTile), grd((d + kTile - 1) / kTile, (d + kTile - 1) / kTile);
-  const double* As = nullptr;
-  if (h->squarings > 0) {
-    k_gram<<<grd, blk, 0, s>>>(h->W, C, d, h->gram[0]);
-    LC_LAUNCH_CHECK("k_gram");
-    int cur = 0;
-    for (int k = 0; k < h->squarings; ++k) {
-      k_square<<<grd, blk, 0, s>>>(h->gram[cur], h->gram[cur ^ 1], d);
-      LC_LAUNCH_CHECK("k_square");
-      cur ^= 1;
-    }
-    As = h->gram[cur];
-  }
-  const size_t smem = sizeof(double) * (size_t)(2 * d + C);
-  k_power<<<1, kPowerThreads, smem, s>>>(h->W, C, d, As, h->max_iter, h->spec);
-  LC_LAUNCH_CHECK("k_power");
-  dim3 rb(128), rg((C + 127) / 128, C);
+  SpectralArgs a;
+  a.W = h->W;
+  a.C = C;
+  a.d = d;
+  a.Cp = (C + 31) / 32 * 32;
+  a.dp = (d + 31) / 32 * 32;
+  a.squarings = h->squarings;
+  a.max_iter = h->max_iter;
+  double* p = reinterpret_cast<double*>(h->spec_work);
+  a.A[0] = p;
+  a.A[1] = a.A[0] + (size_t)a.dp * d;
+  a.Wd = a.A[1] + (size_t)a.dp * d;
+  a.WdT = a.Wd + (size_t)a.dp * C;
+  a.w = a.WdT + (size_t)a.Cp * d;
+  a.u = a.w + C;
+  a.ctr = reinterpret_cast<unsigned*>(a.u + d);
+  a.res = h->spec;
+  LC_CUDA(cudaMemsetAsync(a.ctr, 0, sizeof(unsigned), s));
+  // a barrier that expired leaves this in place: neither converged nor degenerate
+  LC_CUDA(cudaMemsetAsync(h->spec, 0xff, sizeof(SpecResult), s));
+  // Chains per warp: one while the tiles of one-row warps fit the SMs once
+  // (d <= 128: 80 tiles); above, two do the same products per sub-partition
+  // with half the panel scaling (d = 256: 144 tiles).
+  if (d <= 128)
+    launch_spectral<1>(h, a, s);
+  else
+    launch_spectral<2>(h, a, s);
   const bool tight = h->radius_mode == LIPCACHE_RADIUS_TIGHT;
-  k_row_norms<<<rg, rb, 0, s>>>(h->W, C, d, h->Wnorm, h->Wnorm32, tight ? h->pairnorm : nullptr,
-                                tight ? h->inv_pairnorm : nullptr, tight ? h->ipn_up32 : nullptr,
-                                tight ? h->ipn_dn32 : nullptr);
+  const int nb = a.Cp / 32;
+  int units = nb;
+  if (tight)
+    for (int jb = 0; jb < nb; ++jb) units += C < 32 * (jb + 1) ? C : 32 * (jb + 1);
+  k_row_norms<<<(units + kSpWarps - 1) / kSpWarps, kSpThreads, 0, s>>>(
+      a.WdT, C, a.Cp, d, h->Wnorm, h->Wnorm32, tight ? h->pairnorm : nullptr, tight ? h->inv_pairnorm : nullptr,
+      tight ? h->ipn_up32 : nullptr, tight ? h->ipn_dn32 : nullptr);
   LC_LAUNCH_CHECK("k_row_norms");
   if (tight) {
-    k_ipn_min<<<(C + 127) / 128, 128, 0, s>>>(h->pairnorm, h->ipn_dn32, h->ipn_up32, C, h->ipn_min32, h->ipn_max32);
+    k_ipn_min<<<(C + 3) / 4, 128, 0, s>>>(h->pairnorm, h->ipn_dn32, h->ipn_up32, C, h->ipn_min32, h->ipn_max32);
     LC_LAUNCH_CHECK("k_ipn_min");
   }
 }

@@ -73,6 +73,25 @@ def test_sigma_vs_oracle_svd(dev, name, W):
     cache.close()
 
 
+@pytest.mark.parametrize("C,d", [(2, 1), (3, 31), (33, 32), (40, 129), (300, 127), (5, 257), (64, 640)])
+@pytest.mark.parametrize("squarings", [40, 0])
+def test_sigma_tile_edges(dev, C, d, squarings):
+    """Shapes around the spectral kernel's tiles (32 columns, one or two rows
+    per warp, 128-step chunks) and both start vectors, against LAPACK. The
+    oracle comparison's bound (1e-10): the iteration stops at a residual of
+    1e-10 theta, whose effect on theta is of second order."""
+    from paper_2608_13144_gb300.lipcache import LipCache
+    rng = np.random.default_rng(C * 1000 + d)
+    W = (rng.standard_normal((C, d)) / np.sqrt(d)).astype(np.float32)
+    W[0] *= 3.0  # a gap the plain iteration (no squarings) converges on
+    c = LipCache(d, C, 8, device=dev)
+    c.set_spectral_options(squarings, 1000)
+    sigma = c.set_head(T(W, dev), T(np.zeros(C, np.float32), dev))
+    ref = np.linalg.norm(W.astype(np.float64), 2)
+    assert abs(sigma - ref) <= 1e-10 * ref, (sigma, ref)
+    c.close()
+
+
 def test_degenerate_head(dev):
     from paper_2608_13144_gb300 import LipCacheError
     W = np.array(golden("certify_skip_rules.json")["degenerate"]["W"], np.float32)

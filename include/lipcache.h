@@ -67,11 +67,13 @@ typedef enum lipcache_status {
  *   registers (d % 4 == 0, head small enough; both radii, the tight one
  *   refining only the classes that can be its minimiser).
  * TILE64: head resident, 64-row tiles, logits in shared memory.
- * STREAMED: head read from L2 (large heads).
+ * STREAMED: head read from L2 (large heads): where TENSOR's limits on d and C
+ *   hold, TENSOR's screen with the head streamed through a ring in shared
+ *   memory; else FP32 logits on CUDA cores.
  * For the conservative radius TENSOR, WIDE_TILE and TILE64 give the same bits;
- * STREAMED refines with a 32-lane compensated sum, so its radii agree with
- * theirs within the refinement bound. For the tight radius TILE64 and
- * STREAMED refine every class in FP64, and all kernels agree within the
+ * STREAMED on CUDA cores refines with a 32-lane compensated sum, so its radii
+ * agree with theirs within the refinement bound. For the tight radius TILE64
+ * and STREAMED on CUDA cores refine in FP64, and all kernels agree within the
  * refinement bound. */
 #define LIPCACHE_INSERT_WIDE_TILE 1
 #define LIPCACHE_INSERT_TILE64 2

@@ -75,7 +75,6 @@ void release(lipcache* h) {
   dev_free(h->W);
   dev_free(h->wt_prep);
   dev_free(h->b);
-  dev_free(h->Wnorm);
   dev_free(h->Wnorm32);
   dev_free(h->pairnorm);
   dev_free(h->inv_pairnorm);
@@ -204,7 +203,6 @@ LC_API lipcache_status lipcache_create(int32_t d, int32_t C, int64_t capacity, i
     h->c_scr = lc::c_screen(h->dpad);
     dev_alloc(h->W, (size_t)C * d);
     dev_alloc(h->b, (size_t)C);
-    dev_alloc(h->Wnorm, (size_t)C);
     dev_alloc(h->Wnorm32, (size_t)C);
     if (radius_mode == LIPCACHE_RADIUS_TIGHT) {
       dev_alloc(h->pairnorm, (size_t)C * C);

@@ -21,8 +21,8 @@
 // per-row margin and radius use it. For the tight radius the wide-tile kernel
 // refines y^G and the classes whose FP32 bracket of (s_y - s_j) /
 // ||W_y - W_j|| can reach the smallest upper bracket (they contain the
-// minimiser); the other kernels refine every class in FP64 (products of FP32
-// values are exact there).
+// minimiser); the 64-row and streamed kernels pick theirs the same way and
+// refine them in FP64 (products of FP32 values are exact there).
 //
 // Besides the reported radius r, the kernel derives a certified lower bound
 // r_safe of the exact radius (the refined logits' error bounds, sigma
@@ -123,139 +123,156 @@ __device__ void certify_rows_fast(const CertArgs& a, int64_t row0, int nrows, in
   __syncwarp();
 }
 
-// Certify one row with one warp: FP32 interval of every logit, FP64
-// refinement of the classes that can be among the true top two (all classes
-// for the tight radius), margin, radius, certified lower bound, thresholds
-// for the probe, and the skip rules of Algorithm 1. hrow: the row's d
-// features in global memory; lrow: its FP32 logits (shared memory); ws / we:
-// this warp's C-entry scratch for refined logits and their error bounds.
+// FP64 logit of class cc (32 lane sums, one butterfly, the bias) and its error
+// bound, into ws[cc] / we[cc]; every lane returns the logit.
+__device__ __forceinline__ double logit_row_fp64(const CertArgs& a, const float* __restrict__ hrow, int cc, int lane,
+                                                 double* ws, double* we) {
+  const float* wc = a.W + (size_t)cc * a.d;
+  double p = 0.0, pa = 0.0;
+  for (int j = lane; j < a.d; j += 32) {
+    const double t = (double)__ldg(wc + j) * (double)__ldg(hrow + j);
+    p += t;
+    pa += fabs(t);
+  }
+  p = warp_sum_d(p);
+  pa = warp_sum_d(pa);
+  const double bc = (double)__ldg(a.b + cc);
+  const double sv = p + bc;
+  if (lane == 0) {
+    ws[cc] = sv;
+    we[cc] = a.g64 * (pa + fabs(bc));
+  }
+  return sv;
+}
+
+// Tight radius (Eq. 29) of one row with one warp: the FP32 intervals of the
+// logits pick the classes that can be y^G (upper end reaching the largest
+// lower end); those are recomputed in FP64, the largest is y^G (lowest class
+// on ties). Then each class's FP32 bracket of (s_y - s_j) / ||W_y - W_j||, with
+// the FP32 brackets of the reciprocal norms, picks the classes whose lower
+// end reaches the smallest upper end U: the minimiser of Eq. 29, and the class
+// of the smallest certified lower bound (at most r* <= U), are among them, so
+// the minima over these classes in FP64 are those over all classes, bit for
+// bit (3 or 4 of 200 are refined per row instead of 200). A row
+// without finite bounds (NaN or infinite features, an overflowing |z|^2) has
+// every class refined. FP64 instructions are the cost: ~22 cycles of the SM
+// each.
+// hrow: the row's d features in global memory; lrow: its FP32 logits (shared
+// memory); ws / we: this warp's C-entry scratch.
 __device__ void certify_row(const CertArgs& a, int64_t row, const float* __restrict__ hrow,
                             const float* __restrict__ lrow, double* ws, double* we, int lane, uint8_t* acc_slot) {
   const int d = a.d, C = a.C;
-    float knp = 0.f;
-    double hnp = 0.0;
-    for (int j = lane; j < d; j += 32) {
-      const float x = __ldg(hrow + j);
-      knp = fmaf(x, x, knp);
-      hnp = fma((double)x, (double)x, hnp);
-    }
-    const float kn = warp_sum_f(knp);
-    const double hn = sqrt(warp_sum_d(hnp)) * (1.0 + 1e-15);
+  float knp = 0.f;
+  bool inf_z = false;
+  for (int j = lane; j < d; j += 32) {
+    const float x = __ldg(hrow + j);
+    knp = fmaf(x, x, knp);
+    inf_z |= !(fabsf(x) < INFINITY);
+  }
+  const float kn = warp_sum_f(knp);
+  const float hn = norm_upper(kn);
+  // interval of an FP32 logit
+  auto lo_of = [&](int c) {
+    const float sv = lrow[c];
+    return __fsub_rd(sv, logit_err(a.g32f, __ldg(a.Wnorm32 + c), hn, __ldg(a.b + c), sv));
+  };
+  auto hi_of = [&](int c) {
+    const float sv = lrow[c];
+    return __fadd_ru(sv, logit_err(a.g32f, __ldg(a.Wnorm32 + c), hn, __ldg(a.b + c), sv));
+  };
+  float l1 = -INFINITY;
+  bool bad = !(hn < INFINITY);
+  for (int c = lane; c < C; c += 32) {
+    const float lo = lo_of(c);
+    bad |= !(fabsf(lo) < INFINITY);
+    l1 = fmaxf(l1, lo);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) l1 = fmaxf(l1, __shfl_xor_sync(kFull, l1, o));
+  bad = __any_sync(kFull, bad);
 
-    // second largest lower bound of the FP32 logit intervals
-    double l1 = -INFINITY, l2 = -INFINITY;
-    for (int c = lane; c < C; c += 32) {
-      const double E = a.g32 * (a.Wnorm[c] * hn + fabs((double)a.b[c]));
-      top2_push(l1, l2, (double)lrow[c] - E);
+  // y^G: classes in ascending order, so the strict comparison keeps the
+  // lowest class on ties
+  uint32_t done = 0;  // bit t: class 32 t + lane refined
+  double b1 = -INFINITY;
+  int y = -1;
+  for (int cb = 0, t = 0; cb < C; cb += 32, ++t) {
+    const int c = cb + lane;
+    const bool cand = c < C && (bad || hi_of(c) >= l1);
+    unsigned m = __ballot_sync(kFull, cand);
+    done |= cand ? 1u << t : 0u;
+    while (m) {
+      const int cc = cb + __ffs(m) - 1;
+      m &= m - 1;
+      const double sv = logit_row_fp64(a, hrow, cc, lane, ws, we);
+      if (sv > b1) {
+        b1 = sv;
+        y = cc;
+      }
+    }
+  }
+  __syncwarp();
+  if (y < 0) y = 0;  // every refined logit was NaN: the row is rejected
+  const double sy = ws[y], ey = we[y];
+  if (!bad) {
+    const float vyh = __double2float_ru(__dadd_ru(sy, ey)), vyl = __double2float_rd(__dsub_rd(sy, ey));
+    float U = INFINITY;
+    for (int j = lane; j < C; j += 32) {
+      const float iu = __ldg(a.ipn_up32 + (size_t)y * C + j);
+      if (j != y && iu < INFINITY) U = fminf(U, __fmul_ru(__fsub_ru(vyh, lo_of(j)), iu));
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double o1 = __shfl_xor_sync(kFull, l1, o), o2 = __shfl_xor_sync(kFull, l2, o);
-      double t1 = l1, t2 = l2;
-      top2_push(t1, t2, o1);
-      top2_push(t1, t2, o2);
-      l1 = t1;
-      l2 = t2;
-    }
-    const double L2 = l2;
-
-    // FP64 refinement of every class that can be among the true top two
-    // (every class for the tight radius). Classes are visited in ascending
-    // order, so strict comparisons keep the lowest class on ties.
-    double b1 = -INFINITY, b2 = -INFINITY;
-    int y = -1;
-    for (int cb = 0; cb < C; cb += 32) {
-      const int c = cb + lane;
+    for (int o = 16; o > 0; o >>= 1) U = fminf(U, __shfl_xor_sync(kFull, U, o));
+    for (int cb = 0, t = 0; cb < C; cb += 32, ++t) {
+      const int j = cb + lane;
       bool cand = false;
-      if (c < C) {
-        const double E = a.g32 * (a.Wnorm[c] * hn + fabs((double)a.b[c]));
-        cand = a.tight || ((double)lrow[c] + E >= L2) || !(L2 == L2);
-        if (!cand) {
-          ws[c] = NAN;
-          we[c] = NAN;
-        }
+      if (j < C && j != y && !((done >> t) & 1u)) {
+        const float il = __ldg(a.ipn_dn32 + (size_t)y * C + j);
+        cand = il < INFINITY && __fmul_rd(__fsub_rd(vyl, hi_of(j)), il) <= U;
       }
       unsigned m = __ballot_sync(kFull, cand);
+      done |= cand ? 1u << t : 0u;
       while (m) {
         const int cc = cb + __ffs(m) - 1;
         m &= m - 1;
-        const float* wc = a.W + (size_t)cc * d;
-        double p = 0.0, pa = 0.0;
-        for (int j = lane; j < d; j += 32) {
-          const double t = (double)__ldg(wc + j) * (double)__ldg(hrow + j);
-          p += t;
-          pa += fabs(t);
-        }
-        p = warp_sum_d(p);
-        pa = warp_sum_d(pa);
-        const double bc = (double)__ldg(a.b + cc);
-        const double sv = p + bc;
-        const double ev = a.g64 * (pa + fabs(bc));
-        if (lane == 0) {
-          ws[cc] = sv;
-          we[cc] = ev;
-        }
-        if (sv > b1) {
-          b2 = b1;
-          b1 = sv;
-          y = cc;
-        } else if (sv > b2) {
-          b2 = sv;
-        }
+        logit_row_fp64(a, hrow, cc, lane, ws, we);
       }
     }
     __syncwarp();
-    if (y < 0) y = 0;  // every refined logit was NaN: m is NaN and the row is rejected
-    const double sy = ws[y], ey = we[y];
-
-    double r64, rs;
-    if (!a.tight) {
-      double up_other = -INFINITY;
-      for (int c = lane; c < C; c += 32)
-        if (c != y) up_other = fmax(up_other, __dadd_ru(ws[c], we[c]));
-      up_other = warp_max_d(up_other);
-      const double mval = (b1 == b1 && b2 == b2) ? b1 - b2 : NAN;
-      const double mlo = __dsub_rd(__dsub_rd(sy, ey), up_other);
-      r64 = mval * a.inv_denom;
-      rs = (mlo > 0.0) ? __dmul_rd(mlo, a.inv_denom_safe) : 0.0;
-      if (!(mval == mval)) r64 = NAN;
-    } else {
-      double rmin = INFINITY, smin = INFINITY;
-      bool any_nan = !(sy == sy);
-      for (int j = lane; j < C; j += 32) {
-        if (j == y) continue;
-        const double pn = a.pairnorm[(size_t)y * C + j];
-        if (!(ws[j] == ws[j])) any_nan = true;
-        if (!(pn > 0.0)) continue;
-        const double ipn = a.inv_pairnorm[(size_t)y * C + j];
-        rmin = fmin(rmin, (sy - ws[j]) * ipn);
-        // ipn is within gamma_{d+4} / 2 of 1 / ||W_y - W_j||; tight_f removes that
-        const double num = __dsub_rd(__dsub_rd(sy, ey), __dadd_ru(ws[j], we[j]));
-        smin = fmin(smin, __dmul_rd(__dmul_rd(num, ipn), a.tight_f));
-      }
-      rmin = warp_min_d(rmin);
-      smin = warp_min_d(smin);
-      any_nan = __any_sync(kFull, any_nan);
-      any_nan |= !(hn < INFINITY);  // a NaN or infinite feature: no defined term of Eq. 29
-      r64 = any_nan ? NAN : a.kappa * rmin;
-      rs = (smin > 0.0 && !any_nan) ? __dmul_rd(a.kappa, smin) : 0.0;
-    }
-
-    if (lane == 0) {
-      const int32_t lab = a.payload ? a.payload[row] : y;
-      const bool acc = !(a.require_consistency && lab != y) && (r64 > 0.0) && !(a.miss_of && a.miss_of[row] >= 0);
-      float rr, tau;
-      thresholds(__double2float_rd(rs), kn, a.tc, rr, tau);
-      a.accept[row] = acc ? 1 : 0;
-      a.yG[row] = y;
-      a.label[row] = lab;
-      a.radius[row] = __double2float_rz(r64);
-      a.rr[row] = rr;
-      a.kn[row] = kn;
-      a.tau[row] = tau;
-      *acc_slot = acc ? 1 : 0;
-    }
-    __syncwarp();
+  }
+  double rmin = INFINITY, smin = INFINITY;
+  bool any_nan = !(sy == sy);
+  for (int j = lane, t = 0; j < C; j += 32, ++t) {
+    if (j == y || !((done >> t) & 1u)) continue;
+    const double pn = a.pairnorm[(size_t)y * C + j];
+    if (!(ws[j] == ws[j])) any_nan = true;
+    if (!(pn > 0.0)) continue;
+    const double ipn = a.inv_pairnorm[(size_t)y * C + j];
+    rmin = fmin(rmin, (sy - ws[j]) * ipn);
+    // ipn is within gamma_{d+4} / 2 of 1 / ||W_y - W_j||; tight_f removes that
+    const double num = __dsub_rd(__dsub_rd(sy, ey), __dadd_ru(ws[j], we[j]));
+    smin = fmin(smin, __dmul_rd(__dmul_rd(num, ipn), a.tight_f));
+  }
+  rmin = warp_min_d(rmin);
+  smin = warp_min_d(smin);
+  any_nan = __any_sync(kFull, any_nan || inf_z);  // a NaN or infinite feature: no defined term of Eq. 29
+  const double r64 = any_nan ? NAN : a.kappa * rmin;
+  const double rs = (smin > 0.0 && !any_nan) ? __dmul_rd(a.kappa, smin) : 0.0;
+  if (lane == 0) {
+    const int32_t lab = a.payload ? a.payload[row] : y;
+    const bool acc = !(a.require_consistency && lab != y) && (r64 > 0.0) && !(a.miss_of && a.miss_of[row] >= 0);
+    float rr, tau;
+    thresholds(__double2float_rd(rs), kn, a.tc, rr, tau);
+    a.accept[row] = acc ? 1 : 0;
+    a.yG[row] = y;
+    a.label[row] = lab;
+    a.radius[row] = __double2float_rz(r64);
+    a.rr[row] = rr;
+    a.kn[row] = kn;
+    a.tau[row] = tau;
+    *acc_slot = acc ? 1 : 0;
+  }
+  __syncwarp();
 }
 
 __global__ void __launch_bounds__(kThreads) k_certify(CertArgs a) {
@@ -1289,29 +1306,6 @@ int wt_ncg(int C) {
 // without bank conflicts) when it fits, else read from global memory.
 constexpr int kFixWarps = 8;
 
-// The head's rows in memory, row c at w + c ws.
-struct WRows {
-  const float* w;
-  int ws;
-  __device__ __forceinline__ float operator()(int c, int j) const { return w[(size_t)c * ws + j]; }
-  template <int NP>
-  __device__ __forceinline__ void chains(const int (&cc)[NP], const float* __restrict__ zs, int d,
-                                         float (&acc)[NP]) const {
-    const float* wc[NP];
-#pragma unroll
-    for (int t = 0; t < NP; ++t) {
-      wc[t] = w + (size_t)cc[t] * ws;
-      acc[t] = 0.f;
-    }
-#pragma unroll 4
-    for (int j = 0; j < d; ++j) {
-      const float z = zs[j];
-#pragma unroll
-      for (int t = 0; t < NP; ++t) acc[t] = fmaf(wc[t][j], z, acc[t]);
-    }
-  }
-};
-
 __global__ void __launch_bounds__(kFixWarps * 32) k_certify_fix(const CertArgs a, DevStats* stats, int w_smem) {
   extern __shared__ __align__(16) unsigned char fix_smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1619,7 +1613,6 @@ void launch_certify(lipcache* h, const float* H, int64_t n, const int32_t* paylo
   a.require_consistency = require_consistency ? 1 : 0;
   a.W = h->W;
   a.b = h->b;
-  a.Wnorm = h->Wnorm;
   a.pairnorm = h->pairnorm;
   a.payload = payload;
   a.sigma = h->sigma;
@@ -1627,7 +1620,6 @@ void launch_certify(lipcache* h, const float* H, int64_t n, const int32_t* paylo
   a.eps_rc = h->eps_rc;
   a.gamma_rc = gamma32(h->dpad / 32 + 33);
   a.c_scr = h->c_scr;
-  a.g32 = gamma32(h->d + 2) * (1.0 + 1e-6);
   a.g64 = gamma64(h->d + 8) * (1.0 + 1e-6);
   a.Wnorm32 = h->Wnorm32;
   a.g32f = (float)(gamma32(h->d + 2) * (1.0 + 1e-4));
@@ -1670,8 +1662,9 @@ void launch_certify(lipcache* h, const float* H, int64_t n, const int32_t* paylo
   bool fixed_in_kernel = false;
   if (certify_tc_supported(h, H, n)) {
     slot = timing_begin(h, s);
-    fixed_in_kernel = certify_tc_launch(h, a, s);
-    h->last_insert_kernel = LIPCACHE_INSERT_TENSOR;
+    bool head_streamed = false;
+    fixed_in_kernel = certify_tc_launch(h, a, s, head_streamed);
+    h->last_insert_kernel = head_streamed ? LIPCACHE_INSERT_STREAMED : LIPCACHE_INSERT_TENSOR;
   } else if ((!a.tight || h->ipn_up32) && vec16 && ncg > 0 && L.total <= 227 * 1024 &&
              !(h->debug_flags & LIPCACHE_DEBUG_INSERT_TILE64)) {
     const int64_t nb32 = (n + 31) / 32;

@@ -13,10 +13,9 @@ struct CertArgs {
   int d, C, hstride, lstride, tight, require_consistency;
   const float* W;
   const float* b;
-  const double* Wnorm;
   const double* pairnorm;
   const int32_t* payload;
-  double sigma, kappa, eps_rc, gamma_rc, c_scr, g32, g64;
+  double sigma, kappa, eps_rc, gamma_rc, c_scr, g64;
   const float* Wnorm32;  // ||W_c|| rounded up
   float g32f;            // gamma_{d+2} with FP32 rounding slack
   // error factors of the compensated dot products (dot2_factor): the whole
@@ -57,10 +56,11 @@ constexpr double kFixRel = 5e-6;
 
 // The tensor-core certify kernel (certify_tc.cu): whether it takes this
 // insert (either radius, d % 16 == 0, 32 <= d <= 256, 2 <= C <= 256, rows
-// 16-byte aligned, head resident in shared memory), and its launch; true if
-// the kernel runs the FP64 pass over the rows it lists itself.
+// 16-byte aligned), and its launch; true if the kernel runs the FP64 pass over
+// the rows it lists itself. head_streamed: the head did not fit in shared
+// memory and was read from L2.
 bool certify_tc_supported(const lipcache* h, const float* H, int64_t n);
-bool certify_tc_launch(lipcache* h, const CertArgs& a, cudaStream_t s);
+bool certify_tc_launch(lipcache* h, const CertArgs& a, cudaStream_t s, bool& head_streamed);
 
 namespace {
 
@@ -83,26 +83,11 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
   return v;
 }
-__device__ __forceinline__ double warp_max_d(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(kFull, v, o));
-  return v;
-}
 __device__ __forceinline__ double warp_min_d(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(kFull, v, o));
   return v;
 }
-// insert v into (t1 >= t2)
-__device__ __forceinline__ void top2_push(double& t1, double& t2, double v) {
-  if (v > t1) {
-    t2 = t1;
-    t1 = v;
-  } else if (v > t2) {
-    t2 = v;
-  }
-}
-
 // FP32 error-free transformations: a + b = s + e and a * b = p + e exactly
 // (Knuth's TwoSum; TwoProduct with a fused multiply-add).
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
@@ -375,6 +360,29 @@ __device__ inline FixScratch fix_scratch_at(unsigned char* p, int d, int C) {
   s.cls = reinterpret_cast<int*>(s.ce + C4);
   return s;
 }
+
+// The head's rows in memory, row c at w + c ws.
+struct WRows {
+  const float* w;
+  int ws;
+  __device__ __forceinline__ float operator()(int c, int j) const { return w[(size_t)c * ws + j]; }
+  template <int NP>
+  __device__ __forceinline__ void chains(const int (&cc)[NP], const float* __restrict__ zs, int d,
+                                         float (&acc)[NP]) const {
+    const float* wc[NP];
+#pragma unroll
+    for (int t = 0; t < NP; ++t) {
+      wc[t] = w + (size_t)cc[t] * ws;
+      acc[t] = 0.f;
+    }
+#pragma unroll 4
+    for (int j = 0; j < d; ++j) {
+      const float z = zs[j];
+#pragma unroll
+      for (int t = 0; t < NP; ++t) acc[t] = fmaf(wc[t][j], z, acc[t]);
+    }
+  }
+};
 
 // FP64 logits of the N classes cls[0..N) (warp-uniform) of the row zs into
 // cv / ce (lane 0 stores), with FP32 bounds of their errors (rounded up).

@@ -65,6 +65,8 @@
 // Every mbarrier wait is bounded; a role that gives up raises the CTA's abort
 // flag, the others drain, and the launch counts a device error.
 #include "certify_common.cuh"
+#include <type_traits>
+
 #include "tc_ptx.cuh"
 
 namespace lc {
@@ -146,21 +148,26 @@ struct FixQueue {
   float kn[kFixQ];
 };
 
+constexpr int kMaxWRing = 3;  // slots of the streamed head's ring
+
 struct TcLayout {
   int nch, Cpad, nzb, infix;
+  int nwb;  // 0: the head is resident; else slots of its ring (32-feature chunks of Cpad classes)
   uint32_t wbytes, zbytes;
   uint32_t off_z, off_bias, off_wn, off_list, off_x1, off_x2, off_acc, off_bar, off_misc, off_fixq, off_fixs, total;
 };
 
 // infix: the fix warp runs the FP64 pass in the kernel (its queue and scratch
 // in shared memory); else the rows stay listed for the stand-alone pass.
-TcLayout tc_layout(int d, int C, int nzb, int infix) {
+// nwb > 0: the head streams through a ring of nwb chunks instead of staying.
+TcLayout tc_layout(int d, int C, int nzb, int infix, int nwb = 0) {
   TcLayout L;
   L.nch = (d + kChunkF - 1) / kChunkF;
   L.Cpad = (C + 15) / 16 * 16;
   L.nzb = nzb;
   L.infix = infix;
-  L.wbytes = (uint32_t)L.nch * (uint32_t)L.Cpad * 128u;  // a multiple of 2048
+  L.nwb = nwb;
+  L.wbytes = (uint32_t)(nwb ? nwb : L.nch) * (uint32_t)L.Cpad * 128u;  // a multiple of 2048
   L.zbytes = (uint32_t)L.nch * kZChunkBytes;
   L.off_z = L.wbytes;
   L.off_bias = L.off_z + (uint32_t)nzb * L.zbytes;
@@ -170,7 +177,7 @@ TcLayout tc_layout(int d, int C, int nzb, int infix) {
   L.off_x2 = L.off_x1 + 2 * kBM * (uint32_t)sizeof(Pass1);
   L.off_acc = L.off_x2 + kBM * (uint32_t)sizeof(Top2);
   L.off_bar = (L.off_acc + kBM + 32 + 7) / 8 * 8;  // + ok flags of the halves (2 x 4 ints)
-  L.off_misc = L.off_bar + (8 + 2 * kMaxChunks) * 8;  // the barrier map is in the kernel
+  L.off_misc = L.off_bar + (8 + 2 * kMaxChunks + 2 * kMaxWRing) * 8;  // the barrier map is in the kernel
   L.off_fixq = L.off_misc + 16;
   L.off_fixs = (L.off_fixq + (infix ? (uint32_t)sizeof(FixQueue) : 0u) + 15) / 16 * 16;
   L.total = L.off_fixs + (infix ? (uint32_t)fix_scratch_bytes(d, C) : 0u);
@@ -310,6 +317,18 @@ __device__ __forceinline__ void top2_merge(Top2& A, const Top2& B) {
   A = R;
 }
 
+// The head as the refinement reads it: resident in shared memory (swizzled
+// chunks) ...
+struct WSm {
+  uint32_t s_w, wchunk;
+};
+// ... or, when it streams through a ring for the MMAs, its rows in global
+// memory (mostly L2; row c at w + c ws, 16-byte aligned).
+struct WGl {
+  const float* w;
+  int ws;
+};
+
 // Compensated dot products W_c . z_r + b_c of two (row, class) pairs by the 8
 // lanes of a group (lane sub takes features sub, sub + 8, ...; the two chains
 // interleaved for instruction-level parallelism), each in exactly the order of
@@ -317,9 +336,19 @@ __device__ __forceinline__ void top2_merge(Top2& A, const Top2& B) {
 // butterfly over the group, then the bias. Every lane of the group returns the
 // same pairs hi + lo. ws / zs: shared-memory byte addresses of the head and of
 // the tile's features (128-byte swizzle, chunks wchunk / kZChunkBytes apart).
-__device__ __forceinline__ void refine2(uint32_t ws, uint32_t wchunk, uint32_t zs, const int (&c)[2],
-                                        const int (&r)[2], const float (&bias)[2], int d, int sub, float (&hi)[2],
-                                        float (&lo)[2]) {
+template <class WA>
+__device__ __forceinline__ void refine2(const WA& wa, uint32_t zs, const int (&c)[2], const int (&r)[2],
+                                        const float (&bias)[2], int d, int sub, float (&hi)[2], float (&lo)[2]) {
+  constexpr bool kSm = std::is_same<WA, WSm>::value;
+  uint32_t ws = 0, wchunk = 0;
+  const float* wg[2] = {nullptr, nullptr};
+  if constexpr (kSm) {
+    ws = wa.s_w;
+    wchunk = wa.wchunk;
+  } else {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) wg[u] = wa.w + (size_t)c[u] * wa.ws + sub;
+  }
   // lane sub reads the 16-byte unit 2 jj + sub / 4 of each 32-feature chunk
   // (jj = 0..3), word sub % 4; the swizzle XORs the unit with the row mod 8
   const uint32_t s2 = (uint32_t)sub >> 2, s3 = ((uint32_t)sub & 3u) << 2;
@@ -338,21 +367,6 @@ __device__ __forceinline__ void refine2(uint32_t ws, uint32_t wchunk, uint32_t z
   // every operation rounds each half exactly as the scalar one would
   uint64_t P = 0ull, CC = 0ull;
   constexpr uint64_t kSign2 = 0x8000000080000000ull;
-  auto step = [&](uint32_t wa0, uint32_t za0, uint32_t wa1, uint32_t za1) {
-    float w0, x0, w1, x1;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(w0) : "r"(wa0));
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x0) : "r"(za0));
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(w1) : "r"(wa1));
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x1) : "r"(za1));
-    const uint64_t w = pack2_f32(w0, w1), x = pack2_f32(x0, x1);
-    const uint64_t pr = mul_f32x2(w, x);                // TwoProduct: pr + er = w x
-    const uint64_t er = ptx::fma_f32x2(w, x, pr ^ kSign2);
-    const uint64_t sm = add_f32x2(P, pr);               // TwoSum(P, pr) = sm + q
-    const uint64_t bb = ptx::sub_f32x2(sm, P);
-    const uint64_t q = add_f32x2(ptx::sub_f32x2(P, ptx::sub_f32x2(sm, bb)), ptx::sub_f32x2(pr, bb));
-    P = sm;
-    CC = add_f32x2(CC, add_f32x2(q, er));
-  };
   // a chunk's sixteen loads are issued together, then its four steps (the
   // loads are volatile, so their order is the program's)
   auto ld = [](uint32_t addr) {
@@ -375,9 +389,9 @@ __device__ __forceinline__ void refine2(uint32_t ws, uint32_t wchunk, uint32_t z
     float w0[4], x0[4], w1[4], x1[4];
 #pragma unroll
     for (int jj = 0; jj < 4; ++jj) {
-      w0[jj] = ld(wb[0] + ow[0][jj]);
+      w0[jj] = kSm ? ld(wb[0] + ow[0][jj]) : __ldg(wg[0] + kc * kChunkF + 8 * jj);
       x0[jj] = ld(zb[0] + oz[0][jj]);
-      w1[jj] = ld(wb[1] + ow[1][jj]);
+      w1[jj] = kSm ? ld(wb[1] + ow[1][jj]) : __ldg(wg[1] + kc * kChunkF + 8 * jj);
       x1[jj] = ld(zb[1] + oz[1][jj]);
     }
 #pragma unroll
@@ -390,7 +404,12 @@ __device__ __forceinline__ void refine2(uint32_t ws, uint32_t wchunk, uint32_t z
   }
   if (d & 16) {  // a last half chunk (d % 32 == 16): units 0-3
 #pragma unroll
-    for (int jj = 0; jj < 2; ++jj) step(wb[0] + ow[0][jj], zb[0] + oz[0][jj], wb[1] + ow[1][jj], zb[1] + oz[1][jj]);
+    for (int jj = 0; jj < 2; ++jj) {
+      const float w0 = kSm ? ld(wb[0] + ow[0][jj]) : __ldg(wg[0] + nfull * kChunkF + 8 * jj);
+      const float x0 = ld(zb[0] + oz[0][jj]);
+      const float w1 = kSm ? ld(wb[1] + ow[1][jj]) : __ldg(wg[1] + nfull * kChunkF + 8 * jj);
+      step_v(w0, x0, w1, ld(zb[1] + oz[1][jj]));
+    }
   }
   float p[2], cc[2];
   unpack2_f32(P, p[0], p[1]);
@@ -427,10 +446,17 @@ __device__ __forceinline__ void refine2(uint32_t ws, uint32_t wchunk, uint32_t z
 // operand and a sign flip per product on the integer pipe, which measured
 // slower. The next span's four 16-byte loads are issued before this span's
 // arithmetic.
-__device__ __forceinline__ void refine_lane(uint32_t ws, uint32_t wchunk, uint32_t zs, int c, int r, float bias, int d,
-                                            float& hi, float& lo) {
+template <class WA>
+__device__ __forceinline__ void refine_lane(const WA& wa, uint32_t zs, int c, int r, float bias, int d, float& hi,
+                                            float& lo) {
+  constexpr bool kSm = std::is_same<WA, WSm>::value;
   const uint32_t xw = (uint32_t)c & 7u, xz = (uint32_t)r & 7u;
-  const uint32_t wrow = ws + (uint32_t)c * 128u, zrow = zs + (uint32_t)r * 128u;
+  uint32_t wrow = 0, wchunk = 0;
+  if constexpr (kSm) {
+    wrow = wa.s_w + (uint32_t)c * 128u;
+    wchunk = wa.wchunk;
+  }
+  const uint32_t zrow = zs + (uint32_t)r * 128u;
   // span i: features 8 i .. 8 i + 7 = units 2 (i % 4) (chains 0-3) and
   // 2 (i % 4) + 1 (chains 4-7) of chunk i / 4, swizzled with the row mod 8;
   // the second unit's address is the first's with bit 4 flipped
@@ -452,17 +478,42 @@ __device__ __forceinline__ void refine_lane(uint32_t ws, uint32_t wchunk, uint32
     }
   };
   const int nsp = d >> 3;  // (d % 16 == 0)
-  float4 w0 = lds_f4(aw(0)), w1 = lds_f4(aw(0) ^ 16u), z0 = lds_f4(az(0)), z1 = lds_f4(az(0) ^ 16u);
+  if constexpr (kSm) {
+    float4 w0 = lds_f4(aw(0)), w1 = lds_f4(aw(0) ^ 16u), z0 = lds_f4(az(0)), z1 = lds_f4(az(0) ^ 16u);
 #pragma unroll 2
-  for (int i = 0; i < nsp; ++i) {
-    const int n = i + 1 < nsp ? i + 1 : i;  // (the last span loads itself again)
-    const uint32_t anw = aw(n), anz = az(n);
-    const float4 nw0 = lds_f4(anw), nw1 = lds_f4(anw ^ 16u), nz0 = lds_f4(anz), nz1 = lds_f4(anz ^ 16u);
-    span(w0, w1, z0, z1);
-    w0 = nw0;
-    w1 = nw1;
-    z0 = nz0;
-    z1 = nz1;
+    for (int i = 0; i < nsp; ++i) {
+      const int n = i + 1 < nsp ? i + 1 : i;  // (the last span loads itself again)
+      const uint32_t anw = aw(n), anz = az(n);
+      const float4 nw0 = lds_f4(anw), nw1 = lds_f4(anw ^ 16u), nz0 = lds_f4(anz), nz1 = lds_f4(anz ^ 16u);
+      span(w0, w1, z0, z1);
+      w0 = nw0;
+      w1 = nw1;
+      z0 = nz0;
+      z1 = nz1;
+    }
+  } else {
+    // the head's row comes from L2: kAheadG spans in flight
+    constexpr int kAheadG = 4;
+    const float4* wg = reinterpret_cast<const float4*>(wa.w + (size_t)c * wa.ws);
+    float4 w0[kAheadG], w1[kAheadG];
+#pragma unroll
+    for (int u = 0; u < kAheadG; ++u) {
+      const int n = u < nsp ? u : 0;
+      w0[u] = __ldg(wg + 2 * n);
+      w1[u] = __ldg(wg + 2 * n + 1);
+    }
+    for (int i = 0; i < nsp; i += kAheadG) {
+#pragma unroll
+      for (int u = 0; u < kAheadG; ++u) {
+        if (i + u < nsp) {  // (nsp is the same for every lane)
+          const uint32_t ca = az(i + u);
+          span(w0[u], w1[u], lds_f4(ca), lds_f4(ca ^ 16u));
+          const int n = i + u + kAheadG < nsp ? i + u + kAheadG : 0;
+          w0[u] = __ldg(wg + 2 * n);
+          w1[u] = __ldg(wg + 2 * n + 1);
+        }
+      }
+    }
   }
 #pragma unroll
   for (int o = kGroupTc / 2; o > 0; o >>= 1) {
@@ -488,13 +539,22 @@ __device__ __forceinline__ void refine_lane(uint32_t ws, uint32_t wchunk, uint32
 // the second (s with s + 2) a shuffle with lane t ^ 2, the third with t ^ 1.
 // Every lane of the K returns the same bits as refine_lane. All 32 lanes call
 // it together (the shuffles take the whole warp).
-template <int K>
-__device__ __forceinline__ void refine_lanes(uint32_t ws, uint32_t wchunk, uint32_t zs, int c, int r, float bias, int d,
-                                             int t, float& hi, float& lo) {
+template <int K, class WA>
+__device__ __forceinline__ void refine_lanes(const WA& wa, uint32_t zs, int c, int r, float bias, int d, int t,
+                                             float& hi, float& lo) {
+  constexpr bool kSm = std::is_same<WA, WSm>::value;
   static_assert(K == 2 || K == 4, "two or four lanes per pair");
   constexpr int NC = 8 / K;  // chains per lane
   const uint32_t xw = (uint32_t)c & 7u, xz = (uint32_t)r & 7u;
-  const uint32_t wrow = ws + (uint32_t)c * 128u, zrow = zs + (uint32_t)r * 128u;
+  uint32_t wrow = 0, wchunk = 0;
+  const float* wg = nullptr;
+  if constexpr (kSm) {
+    wrow = wa.s_w + (uint32_t)c * 128u;
+    wchunk = wa.wchunk;
+  } else {
+    wg = wa.w + (size_t)c * wa.ws;
+  }
+  const uint32_t zrow = zs + (uint32_t)r * 128u;
   float p[NC], cc[NC];
 #pragma unroll
   for (int j = 0; j < NC; ++j) p[j] = cc[j] = 0.f;
@@ -508,11 +568,16 @@ __device__ __forceinline__ void refine_lanes(uint32_t ws, uint32_t wchunk, uint3
     cc[j] = __fadd_rn(cc[j], __fadd_rn(q, er));
   };
   const int nsp = d >> 3;
+#pragma unroll 4
   for (int i = 0; i < nsp; ++i) {
     const uint32_t u = 2u * (uint32_t)(i & 3);  // first unit of the span
     const uint32_t ow = (uint32_t)(i >> 2) * wchunk, oz = (uint32_t)(i >> 2) * kZChunkBytes;
     if constexpr (K == 2) {
-      const float4 w = lds_f4(wrow + ow + (((u + (uint32_t)t) ^ xw) << 4));
+      float4 w;
+      if constexpr (kSm)
+        w = lds_f4(wrow + ow + (((u + (uint32_t)t) ^ xw) << 4));
+      else
+        w = __ldg(reinterpret_cast<const float4*>(wg) + 2 * i + t);
       const float4 z = lds_f4(zrow + oz + (((u + (uint32_t)t) ^ xz) << 4));
       step(0, w.x, z.x);
       step(1, w.y, z.y);
@@ -520,8 +585,13 @@ __device__ __forceinline__ void refine_lanes(uint32_t ws, uint32_t wchunk, uint3
       step(3, w.w, z.w);
     } else {
       float w0, w1, z0, z1;
-      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(w0) : "r"(wrow + ow + ((u ^ xw) << 4) + 4u * (uint32_t)t));
-      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(w1) : "r"(wrow + ow + (((u + 1u) ^ xw) << 4) + 4u * (uint32_t)t));
+      if constexpr (kSm) {
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(w0) : "r"(wrow + ow + ((u ^ xw) << 4) + 4u * (uint32_t)t));
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(w1) : "r"(wrow + ow + (((u + 1u) ^ xw) << 4) + 4u * (uint32_t)t));
+      } else {
+        w0 = __ldg(wg + 8 * i + t);
+        w1 = __ldg(wg + 8 * i + 4 + t);
+      }
       asm volatile("ld.shared.f32 %0, [%1];" : "=f"(z0) : "r"(zrow + oz + ((u ^ xz) << 4) + 4u * (uint32_t)t));
       asm volatile("ld.shared.f32 %0, [%1];" : "=f"(z1) : "r"(zrow + oz + (((u + 1u) ^ xz) << 4) + 4u * (uint32_t)t));
       step(0, w0, z0);  // chain t
@@ -559,7 +629,8 @@ __device__ __forceinline__ void refine_lanes(uint32_t ws, uint32_t wchunk, uint3
 // other class in FP64. The row's features come from the tile in shared memory
 // (row rz). res_hi / res_lo: the warp's cells (at least 256 each), free here.
 // Returns (on every lane) whether the row was listed for the FP64 pass.
-__device__ bool tc_tight_row_warp(const CertArgs& a, int64_t row, int rz, uint32_t s_w, uint32_t wchunk, uint32_t zs,
+template <class WA>
+__device__ bool tc_tight_row_warp(const CertArgs& a, int64_t row, int rz, const WA& wa, uint32_t zs,
                                   const float* __restrict__ wn_s, const float* __restrict__ b_s, float kn, int lane,
                                   float* res_hi, float* res_lo, uint8_t* acc_slot) {
   constexpr int kPer = 8;  // classes per lane (C <= 256)
@@ -576,7 +647,7 @@ __device__ bool tc_tight_row_warp(const CertArgs& a, int64_t row, int rz, uint32
     const int rp[2] = {rz, rz};
     const float bp[2] = {b_s[cp[0]], b_s[cp[1]]};
     float hi[2], lo[2];
-    refine2(s_w, wchunk, zs, cp, rp, bp, d, sub, hi, lo);
+    refine2(wa, zs, cp, rp, bp, d, sub, hi, lo);
     if (sub == 0)
 #pragma unroll
       for (int u = 0; u < 2; ++u)
@@ -648,7 +719,14 @@ __device__ bool tc_tight_row_warp(const CertArgs& a, int64_t row, int rz, uint32
   return __shfl_sync(kFull, fix ? 1 : 0, 0) != 0;
 }
 
-template <bool TIGHT>
+// WSTREAM: the head does not fit beside a tile's features; its 32-feature
+// chunks stream through a ring for the MMAs, tile after tile, and the
+// refinement reads its rows from L2, four 32-byte spans ahead. It replaces FP32
+// logits on the CUDA cores with FP64 sums: 100,000 rows, d = 256, C = 200, tight
+// radius, 72.8 ms then, 0.59 ms now (floor: 30 us of HBM, 11 us of TF32).
+// Bound by the epilogue, as the resident kernel, plus the L2 latency of the
+// head's rows.
+template <bool TIGHT, bool WSTREAM>
 __global__ void __launch_bounds__(kThreads, 1)
     k_certify_tc(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmW, const CertArgs a,
                  const TcLayout L, int n_tiles, DevStats* stats, int debug_stall) {
@@ -658,11 +736,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t s_base = ptx::smem_u32(smem);
   const uint32_t s_w = s_base, s_z = s_base + L.off_z;
   const uint32_t bar = s_base + L.off_bar;
-  // barriers: wfull, zempty[2], accfull[2], accempty[2], drain, zfull[2][kMaxChunks]
+  // barriers: wfull, zempty[2], accfull[2], accempty[2], drain, zfull[2][kMaxChunks],
+  // and for a streamed head wrfull[kMaxWRing], wrempty[kMaxWRing]
   // (one per 32-feature chunk of each feature buffer, so the MMAs start on
   // the first chunk while the others land)
   const uint32_t wfull = bar, zempty = bar + 8, accfull = bar + 24, accempty = bar + 40, drain = bar + 56,
-                 zfull = bar + 64;
+                 zfull = bar + 64, wrfull = zfull + 8 * 2 * kMaxChunks, wrempty = wrfull + 8 * kMaxWRing;
   auto zfull_of = [&](int zb, int c) { return zfull + 8u * (uint32_t)(zb * kMaxChunks + c); };
   float* bias_s = reinterpret_cast<float*>(smem + L.off_bias);
   float* wn_s = reinterpret_cast<float*>(smem + L.off_wn);
@@ -686,6 +765,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       ptx::mbar_init(accempty + 8 * b, kEpiWarps);
     }
     ptx::mbar_init(drain, 1);
+    if constexpr (WSTREAM)
+      for (int s = 0; s < kMaxWRing; ++s) {
+        ptx::mbar_init(wrfull + 8 * s, 1);
+        ptx::mbar_init(wrempty + 8 * s, 1);
+      }
     *abort_s = 0;
     if (fixq) {
       fixq->n = fixq->taken = fixq->done = fixq->beat = 0;
@@ -711,9 +795,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     if (lane == 0) {
-      ptx::mbar_expect_tx(wfull, L.wbytes);
-      for (int c = 0; c < L.nch; ++c)
-        ptx::tma_load_2d(s_w + (uint32_t)c * (uint32_t)L.Cpad * 128u, &tmW, c * kChunkF, 0, wfull);
+      const uint32_t wchunk = (uint32_t)L.Cpad * 128u;
+      if constexpr (!WSTREAM) {
+        ptx::mbar_expect_tx(wfull, L.wbytes);
+        for (int c = 0; c < L.nch; ++c) ptx::tma_load_2d(s_w + (uint32_t)c * wchunk, &tmW, c * kChunkF, 0, wfull);
+      }
+      int ws = 0, wloads = 0;  // ring slot and loads issued (streamed head)
+      uint32_t wph = 0;
       bool used[2] = {false, false};
       uint32_t lastp[2] = {0u, 0u};
       int t = 0;
@@ -725,6 +813,25 @@ __global__ void __launch_bounds__(kThreads, 1)
           ptx::mbar_expect_tx(zfull_of(zb, c), kZChunkBytes);
           ptx::tma_load_2d(s_z + (uint32_t)zb * L.zbytes + (uint32_t)c * kZChunkBytes, &tmH, c * kChunkF, tile * kBM,
                            zfull_of(zb, c));
+        }
+        if constexpr (WSTREAM) {
+          bool ok = true;
+          for (int c = 0; c < L.nch; ++c) {
+            ok = ptx::mbar_wait(wrempty + 8 * ws, wph ^ 1u, abort_s, kWaitLimit);
+            if (!ok) break;
+            ptx::mbar_expect_tx(wrfull + 8 * ws, wchunk);
+            ptx::tma_load_2d(s_w + (uint32_t)ws * wchunk, &tmW, c * kChunkF, 0, wrfull + 8 * ws);
+            ++wloads;
+            if (++ws == L.nwb) {
+              ws = 0;
+              wph ^= 1u;
+            }
+          }
+          if (!ok) {
+            used[zb] = true;
+            lastp[zb] = par;
+            break;
+          }
         }
         used[zb] = true;
         lastp[zb] = par;
@@ -741,7 +848,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       volatile int never = 0;
       for (int b = 0; b < 2; ++b)
         for (int c = 0; c < L.nch && used[b]; ++c) ptx::mbar_wait(zfull_of(b, c), lastp[b], &never, kWaitLimit);
-      ptx::mbar_wait(wfull, 0, &never, kWaitLimit);
+      if constexpr (!WSTREAM) {
+        ptx::mbar_wait(wfull, 0, &never, kWaitLimit);
+      } else {
+        // the last load into each slot: load number l fills slot l % nwb in
+        // the phase of parity (l / nwb) & 1
+        for (int l = wloads > L.nwb ? wloads - L.nwb : 0; l < wloads; ++l)
+          ptx::mbar_wait(wrfull + 8 * (l % L.nwb), (uint32_t)(l / L.nwb) & 1u, &never, kWaitLimit);
+      }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
@@ -752,7 +866,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       // failure-detection test: no arrival completes this phase before the
       // final drain, so the bounded wait expires and the kernel aborts
       bool ok = !debug_stall || ptx::mbar_wait(drain, 0, abort_s, kWaitLimit);
-      ok = ok && ptx::mbar_wait(wfull, 0, abort_s, kWaitLimit);
+      if constexpr (!WSTREAM) ok = ok && ptx::mbar_wait(wfull, 0, abort_s, kWaitLimit);
+      int ws = 0;
+      uint32_t wph = 0;
       int t = 0;
       for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++t) {
         const int buf = t & 1, zb = t % L.nzb;
@@ -766,11 +882,25 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = false;
             break;
           }
+          if constexpr (WSTREAM) {
+            if (!ptx::mbar_wait(wrfull + 8 * ws, wph, abort_s, kWaitLimit)) {
+              ok = false;
+              break;
+            }
+            wd = wdesc0 + (uint64_t)ws * wstep;
+          }
           ptx::tc_fence_after();
           ptx::mma_tf32(d_tmem, zd, wd, idesc, c != 0);
           ptx::mma_tf32(d_tmem, zd + 2, wd + 2, idesc, 1u);
           ptx::mma_tf32(d_tmem, zd + 4, wd + 4, idesc, 1u);
           ptx::mma_tf32(d_tmem, zd + 6, wd + 6, idesc, 1u);
+          if constexpr (WSTREAM) {
+            ptx::mma_commit(wrempty + 8 * ws);  // the slot is free once these MMAs have read it
+            if (++ws == L.nwb) {
+              ws = 0;
+              wph ^= 1u;
+            }
+          }
         }
         if (!ok) break;
         ptx::mma_commit(accfull + 8 * buf);
@@ -786,10 +916,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     // the rows the epilogue lists, one at a time, while the epilogue goes on
     // with later tiles (fix_row_warp); the head is read in place
     if (fixq) {
-      const WSwz W{s_w, (uint32_t)L.Cpad * 128u};
+      typename std::conditional<WSTREAM, WRows, WSwz>::type W;
+      if constexpr (WSTREAM)
+        W = WRows{a.W, d};
+      else
+        W = WSwz{s_w, (uint32_t)L.Cpad * 128u};
       const FixScratch sc = fix_scratch_at(smem + L.off_fixs, d, C);
       volatile FixQueue* vq = fixq;
-      bool head_ok = false;
+      bool head_ok = WSTREAM;
       unsigned long long nfixed = 0;
       for (int k = 0;; ++k) {
         // 1: entry k is in its slot; 0: every epilogue warp is done and no
@@ -854,7 +988,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
     const int dq = d / 4;
     const int bar_id = 1 + quarter;
-    const uint32_t wchunk = (uint32_t)L.Cpad * 128u;
+    typename std::conditional<WSTREAM, WGl, WSm>::type wa;
+    if constexpr (WSTREAM)
+      wa = WGl{a.W, d};
+    else
+      wa = WSm{s_w, (uint32_t)L.Cpad * 128u};
     // screen bound terms: c ||W_c|| <= cw and (1 + c) ||W_c|| <= cw1 for every
     // class, |b_c| <= bmax (rounded up; a NaN bias propagates into bmax)
     float wmax = 0.f, bmax = 0.f;
@@ -1206,7 +1344,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int e = list[i];
         const int c = e >> 8;
         float hi, lo;
-        refine_lane(s_w, wchunk, zs, c, rq + (e & 31), bias_s[c], d, hi, lo);
+        refine_lane(wa, zs, c, rq + (e & 31), bias_s[c], d, hi, lo);
         res_hi[e & 0xff] = hi;
         res_lo[e & 0xff] = lo;
       }
@@ -1217,9 +1355,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int c = e >> 8;
         float hi, lo;
         if (kk == 2)
-          refine_lanes<2>(s_w, wchunk, zs, c, rq + (e & 31), bias_s[c], d, lane & 1, hi, lo);
+          refine_lanes<2>(wa, zs, c, rq + (e & 31), bias_s[c], d, lane & 1, hi, lo);
         else
-          refine_lanes<4>(s_w, wchunk, zs, c, rq + (e & 31), bias_s[c], d, lane & 3, hi, lo);
+          refine_lanes<4>(wa, zs, c, rq + (e & 31), bias_s[c], d, lane & 3, hi, lo);
         if (i < P && lane % kk == 0) {
           res_hi[e & 0xff] = hi;
           res_lo[e & 0xff] = lo;
@@ -1258,7 +1396,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int rp[2] = {rq + ow, rq + ow};
             const float bp[2] = {bias_s[cp[0]], bias_s[cp[1]]};
             float hi[2], lo[2];
-            refine2(s_w, wchunk, zs, cp, rp, bp, d, sub, hi, lo);
+            refine2(wa, zs, cp, rp, bp, d, sub, hi, lo);
             if (sub == 0) {
 #pragma unroll
               for (int u = 0; u < 2; ++u) {
@@ -1379,7 +1517,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if ((k & 1) == half) {
             const float knw = __shfl_sync(kFull, kn, ow);
             const int64_t frow = (int64_t)tile * kBM + rq + ow;
-            if (tc_tight_row_warp(a, frow, rq + ow, s_w, wchunk, zs, wn_s, bias_s, knw, lane, res_hi, res_lo,
+            if (tc_tight_row_warp(a, frow, rq + ow, wa, zs, wn_s, bias_s, knw, lane, res_hi, res_lo,
                                   &acc_s[rq + ow]) &&
                 fixq && lane == 0)
               fixq_push(fixq, (int)frow, knw, abort_s, kWaitLimit);
@@ -1434,13 +1572,20 @@ void encode_rows(lipcache* h, CUtensorMap* map, const float* base, uint64_t rows
 
 // Two feature buffers when they fit next to the resident head, else one.
 // The FP64 pass in the kernel when its queue and scratch fit as well (and
-// `fix_in_kernel` allows it).
+// `fix_in_kernel` allows it). A head that fits with neither streams through a
+// ring: as many feature buffers and ring slots as fit.
 bool tc_plan(int d, int C, TcLayout& L, bool fix_in_kernel = true) {
   for (int nzb = 2; nzb >= 1; --nzb)
     for (int infix = fix_in_kernel ? 1 : 0; infix >= 0; --infix) {
       L = tc_layout(d, C, nzb, infix);
       if (L.total <= (uint32_t)kSmemBudget) return true;
     }
+  for (int nzb = 2; nzb >= 1; --nzb)
+    for (int infix = fix_in_kernel ? 1 : 0; infix >= 0; --infix)
+      for (int nwb = kMaxWRing; nwb >= nzb; --nwb) {
+        L = tc_layout(d, C, nzb, infix, nwb);
+        if (L.total <= (uint32_t)kSmemBudget) return true;
+      }
   return false;
 }
 
@@ -1461,7 +1606,7 @@ bool certify_tc_supported(const lipcache* h, const float* H, int64_t n) {
   return tc_plan(h->d, h->C, L);
 }
 
-bool certify_tc_launch(lipcache* h, const CertArgs& a, cudaStream_t s) {
+bool certify_tc_launch(lipcache* h, const CertArgs& a, cudaStream_t s, bool& head_streamed) {
   TcLayout L;
   LC_REQUIRE(tc_plan(h->d, h->C, L, !(h->debug_flags & LIPCACHE_DEBUG_INSERT_FIX_STANDALONE)), LIPCACHE_E_INVALID,
              "head does not fit the tensor certify kernel");
@@ -1473,7 +1618,9 @@ bool certify_tc_launch(lipcache* h, const CertArgs& a, cudaStream_t s) {
   // at least half of the SM's shared memory, so one CTA (and one 512-column
   // TMEM allocation) per SM
   const int smem = (int)L.total + 1024 > 120 * 1024 ? (int)L.total + 1024 : 120 * 1024;
-  auto kern = a.tight ? k_certify_tc<true> : k_certify_tc<false>;
+  head_streamed = L.nwb > 0;
+  auto kern = head_streamed ? (a.tight ? k_certify_tc<true, true> : k_certify_tc<false, true>)
+                            : (a.tight ? k_certify_tc<true, false> : k_certify_tc<false, false>);
   LC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   kern<<<grid, kThreads, smem, s>>>(tmH, tmW, a, L, n_tiles, h->stats,
                                     (h->debug_flags & LIPCACHE_DEBUG_STALL_INSERT) ? 1 : 0);

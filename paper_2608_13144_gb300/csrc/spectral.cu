@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(kSpThreads) k_spectral(const SpectralArgs a) {
   }
 }
 
-// ||W_c|| for every class and, for the tight radius, ||W_y - W_j|| for every
+// ||W_c|| (rounded up) for every class and, for the tight radius, ||W_y - W_j|| for every
 // pair (FP64; the differences of FP32 weights are exact, the sum of d squares
 // is within gamma_d of the exact one) with its reciprocal, and FP32 brackets
 // of the reciprocal (the FP64 value widened by 1e-12, far above its error,
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kSpThreads) k_spectral(const SpectralArgs a) {
 // the mirrored pair squares the negated differences, the same sum. Bound by
 // the FP64 pipe: two instructions per feature and 32 pairs.
 __global__ void __launch_bounds__(kSpThreads) k_row_norms(const double* __restrict__ WdT, int C, int Cp, int d,
-                                                          double* __restrict__ Wnorm, float* __restrict__ Wnorm32,
+                                                          float* __restrict__ Wnorm32,
                                                           double* __restrict__ pairnorm,
                                                           double* __restrict__ inv_pairnorm,
                                                           float* __restrict__ ipn_up32, float* __restrict__ ipn_dn32) {
@@ -400,10 +400,7 @@ __global__ void __launch_bounds__(kSpThreads) k_row_norms(const double* __restri
       const double x = WdT[(size_t)k * Cp + c];
       n2 = fma(x, x, n2);
     }
-    if (c < C) {
-      Wnorm[c] = sqrt(n2);
-      Wnorm32[c] = __double2float_ru(sqrt(n2) * (1.0 + 1e-15));
-    }
+    if (c < C) Wnorm32[c] = __double2float_ru(sqrt(n2) * (1.0 + 1e-15));
     return;
   }
   if (!pairnorm) return;
@@ -524,7 +521,7 @@ void spectral_norm(lipcache* h, cudaStream_t s) {
   if (tight)
     for (int jb = 0; jb < nb; ++jb) units += C < 32 * (jb + 1) ? C : 32 * (jb + 1);
   k_row_norms<<<(units + kSpWarps - 1) / kSpWarps, kSpThreads, 0, s>>>(
-      a.WdT, C, a.Cp, d, h->Wnorm, h->Wnorm32, tight ? h->pairnorm : nullptr, tight ? h->inv_pairnorm : nullptr,
+      a.WdT, C, a.Cp, d, h->Wnorm32, tight ? h->pairnorm : nullptr, tight ? h->inv_pairnorm : nullptr,
       tight ? h->ipn_up32 : nullptr, tight ? h->ipn_dn32 : nullptr);
   LC_LAUNCH_CHECK("k_row_norms");
   if (tight) {

@@ -427,6 +427,62 @@ def test_tight_radius_other_kernels(dev, d, C, kernel):
 
 
 @pytest.mark.parametrize("mode", ["conservative", "tight"])
+@pytest.mark.parametrize("d,C,N", [(256, 200, 25000), (256, 256, 4000), (128, 256, 20001), (208, 170, 700),
+                                   (240, 225, 129), (256, 121, 1)])
+def test_streamed_head_tensor(dev, mode, d, C, N):
+    """Heads too large to stay in shared memory, streamed through the tensor
+    kernel's ring: one to three slots, one and two feature buffers, several
+    tiles per CTA, ragged tiles, rows on logit ties (the FP64 pass with the
+    head in L2), against the oracle and the wide-tile fallback's kernel."""
+    from paper_2608_13144_gb300.lipcache import LipCache
+    rng = np.random.default_rng(d * 7 + C)
+    W = (rng.standard_normal((C, d)) / np.sqrt(d)).astype(np.float32)
+    b = (0.1 * rng.standard_normal(C)).astype(np.float32)
+    ties = min(N // 4, 60)
+    rows = np.concatenate([rng.standard_normal((N - 2 * ties, d)).astype(np.float32) * 2,
+                           *([_near_ties(W, b, ties, rng, 2), _near_ties(W, b, ties, rng, 3)] if ties else [])])
+    rows = rows[rng.permutation(N)]
+    ref = oracle.build_cache(W, b, oracle.sigma_max(W), rows, radius_mode=int(mode == "tight"))
+    head = ("tight", W, b, rows, 1.0) if mode == "tight" else (W, b, rows, 1.0)
+    out = []
+    for flags in (0, DEBUG_INSERT_WIDE_TILE, DEBUG_INSERT_FIX_STANDALONE):
+        c = LipCache(d, C, N, mode, device=dev)
+        c.set_debug(flags)
+        c.set_head(T(W, dev), T(b, dev))
+        i, r, n = c.insert(T(rows, dev))
+        assert c.info()["device_errors"] == 0
+        if flags != DEBUG_INSERT_WIDE_TILE:
+            assert c.info()["last_insert_kernel"] == STREAMED
+        out.append((i.cpu().numpy(), r.cpu().numpy(), n))
+        check_insert(*out[-1], ref, head)
+        c.close()
+    assert np.array_equal(out[0][0], out[2][0]) and same_bits(out[0][1], out[2][1])
+
+
+@pytest.mark.parametrize("d,C", [(33, 7), (101, 60), (300, 20), (64, 300)])
+def test_tight_candidates_special_rows(dev, d, C):
+    """The FP64-refining kernels' candidate choice for the tight radius:
+    coinciding head rows (no term of Eq. 29, a zero margin), rows with a NaN or
+    infinite feature or an overflowing norm (every class refined), exact ties."""
+    from paper_2608_13144_gb300.lipcache import LipCache
+    rng = np.random.default_rng(d + C)
+    W = (rng.standard_normal((C, d)) / np.sqrt(d)).astype(np.float32)
+    b = (0.1 * rng.standard_normal(C)).astype(np.float32)
+    W[3], b[3] = W[1], b[1]
+    rows = rng.standard_normal((400, d)).astype(np.float32)
+    rows[:40] += 5 * W[1]
+    rows[50, 0], rows[51, -1], rows[52] = np.nan, np.inf, rows[52] * np.float32(1e30)
+    rows[53], rows[54] = 0, rows[54] * np.float32(1e-30)
+    c = LipCache(d, C, 400, "tight", device=dev)
+    c.set_head(T(W, dev), T(b, dev))
+    i, r, n = c.insert(T(rows, dev))
+    assert c.info()["last_insert_kernel"] in (TILE64, STREAMED)
+    ref = oracle.build_cache(W, b, oracle.sigma_max(W), rows, radius_mode=oracle.RADIUS_TIGHT)
+    check_insert(i.cpu().numpy(), r.cpu().numpy(), n, ref, ("tight", W, b, rows, 1.0))
+    c.close()
+
+
+@pytest.mark.parametrize("mode", ["conservative", "tight"])
 @pytest.mark.parametrize("d,C", [(16, 10), (128, 200)])
 def test_certify_special_values(dev, mode, d, C):
     """Rows with NaN or infinite features are skipped (a NaN margin fails

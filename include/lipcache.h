@@ -86,10 +86,13 @@ typedef enum lipcache_status {
 #define LIPCACHE_POLICY_INTERCLASS 2 /* radius from inter-class centroid distances (Sec. 5.4) */
 
 /* Probe kernels. All return identical results; they differ in speed. */
-#define LIPCACHE_PROBE_AUTO 0          /* tensor path when supported (d <= 256) and B N d_pad >= 2^24, else exact */
-#define LIPCACHE_PROBE_TENSOR 1        /* tcgen05 TF32 screen, then exact FP32 recheck of candidates;
-                                          the kernel is chosen by shape: TENSOR_SINGLE for
-                                          d_pad <= 128, TENSOR_PAIR above (when clusters of four fit) */
+#define LIPCACHE_PROBE_AUTO 0          /* tensor path when supported (d <= 256; d <= 512 while the FP16 screen
+                                          serves the table) and B N d_pad >= 2^24, else exact */
+#define LIPCACHE_PROBE_TENSOR 1        /* tcgen05 screen (d <= 256; in FP16 while every entry's FP16 copy serves,
+                                          else in TF32), then exact FP32 recheck of candidates;
+                                          the kernel is chosen by shape: TENSOR_SINGLE where a 256-key
+                                          tile fits (d <= 256 screened in FP16, 128 in TF32), TENSOR_PAIR
+                                          above (when clusters of four fit) */
 #define LIPCACHE_PROBE_EXACT 2         /* exact FP32 distance of every pair on CUDA cores */
 #define LIPCACHE_PROBE_TENSOR_SINGLE 3 /* the tensor screen with single-CTA MMAs (clusters of two) */
 #define LIPCACHE_PROBE_TENSOR_PAIR 4   /* the tensor screen with CTA-pair MMAs (clusters of four) */
@@ -140,7 +143,9 @@ typedef struct lipcache_info {
 /*
  * Create an empty cache for d-dimensional GuardNet features and a C-class
  * head (Sec. 3.1 notation: z in R^d, W in R^{C x d}). Allocates the key table
- * for `capacity` entries on the current CUDA device.
+ * for `capacity` entries on the current CUDA device: 4 d_pad + 24 bytes per
+ * entry and, for d <= 512 and where the memory allows it, an FP16 copy of the
+ * keys (2 d bytes, d rounded up to 64) that the tensor screen reads.
  *   d           1 .. LIPCACHE_MAX_DIM
  *   C           2 .. LIPCACHE_MAX_CLASSES
  *   capacity    1 .. LIPCACHE_MAX_CAPACITY
@@ -414,7 +419,8 @@ lipcache_status lipcache_probe_host(lipcache_t* h, const float* Q_host, int64_t 
  * Same arguments, results and errors as lipcache_probe, but the probe's
  * scratch lives in one fixed array compiled into the library
  * (LIPCACHE_NOALLOC_SCRATCH_BYTES per device, held by every GPU that loads
- * the library until the process exits) and nothing is allocated.
+ * the library until the process exits, with 4 bytes for each of the most rows
+ * it can serve beside it) and nothing is allocated.
  * Limit: ceil(B/128)*128 * (4*d_pad + 12) bytes, plus alignment, must fit the
  * array (e.g. 4,096 queries at d <= 256); larger batches get E_INVALID with
  * the sizes in the message. The first call on a device resolves the array's

@@ -93,6 +93,7 @@ void release(lipcache* h) {
   dev_free(h->cls_sum);
   dev_free(h->cls_cnt);
   dev_free(h->table.keys);
+  dev_free(h->table.keys16);
   dev_free(h->table.kn);
   dev_free(h->table.tau);
   dev_free(h->table.rr);
@@ -110,20 +111,17 @@ void release(lipcache* h) {
   dev_free(h->ins_fix);
   dev_free(h->ins_bcount);
   dev_free(h->ins_boffset);
-  dev_free(h->ins_total);
-  dev_free(h->size_dev);
+  dev_free(h->report);
   dev_free(h->ins_size0);
-  if (h->size_pinned) cudaFreeHost(h->size_pinned);
-  if (h->ins_total_host) cudaFreeHost(h->ins_total_host);
+  if (h->report_host) cudaFreeHost(h->report_host);
   dev_free(h->qpad);
   dev_free(h->kappa);
+  dev_free(h->qscale);
   dev_free(h->best);
   dev_free(h->hq);
   dev_free(h->hidx);
   dev_free(h->hlabel);
   dev_free(h->hdist);
-  dev_free(h->stats);
-  if (h->stats_host) cudaFreeHost(h->stats_host);
   for (int i = 0; i < lipcache::kTimingRing; ++i) {
     if (h->tev0[i]) cudaEventDestroy(h->tev0[i]);
     if (h->tev1[i]) cudaEventDestroy(h->tev1[i]);
@@ -169,7 +167,7 @@ void lc::harvest_timing(lipcache* h, bool all) {
 
 // After a synchronised probe: E_DEVICE if a bounded wait of the kernel expired.
 static void require_no_abort(lipcache* h, cudaStream_t s) {
-  LC_CUDA(cudaMemcpyAsync(h->stats_host, h->stats, sizeof(lc::DevStats), cudaMemcpyDeviceToHost, s));
+  lc::fetch_report(h, s);
   LC_CUDA(cudaStreamSynchronize(s));
   LC_REQUIRE(h->stats_host->abort_flag == 0, LIPCACHE_E_DEVICE,
              "a bounded wait of the probe kernel expired; the batch's queries were reported as misses");
@@ -215,12 +213,13 @@ LC_API lipcache_status lipcache_create(int32_t d, int32_t C, int64_t capacity, i
     dev_alloc(h->spec_work, lc::spectral_work_bytes(d, C));
     dev_alloc(h->spec, 1);
     LC_CUDA(cudaMallocHost(&h->spec_host, sizeof(lc::SpecResult)));
-    // Whole key tiles: rows past the current size are zero keys whose screen
-    // term tau is 0x7f7f7f7f (3.4e38), so no probe ever selects them.
+    // Whole key tiles: rows past the current size have the screen term tau
+    // 0x7f7f7f7f (3.4e38), so no probe ever selects them; those of the last
+    // tile are kept zero by whatever appends entries (key16.cuh, zero_tail),
+    // so the keys themselves need no clearing here.
     h->table_rows = (capacity + 255) / 256 * 256;
     const size_t rows = (size_t)h->table_rows;
     dev_alloc(h->table.keys, rows * h->dpad);
-    LC_CUDA(cudaMemset(h->table.keys, 0, sizeof(float) * rows * h->dpad));
     dev_alloc(h->table.kn, rows);
     dev_alloc(h->table.tau, rows);
     LC_CUDA(cudaMemset(h->table.tau, 0x7f, sizeof(float) * rows));
@@ -229,15 +228,23 @@ LC_API lipcache_status lipcache_create(int32_t d, int32_t C, int64_t capacity, i
     dev_alloc(h->table.radius, rows);
     dev_alloc(h->table.label, rows);
     dev_alloc(h->table.yG, rows);
-    dev_alloc(h->ins_total, 4);
-    LC_CUDA(cudaMallocHost(&h->ins_total_host, 4 * sizeof(int64_t)));
-    dev_alloc(h->size_dev, 1);
-    LC_CUDA(cudaMemset(h->size_dev, 0, sizeof(int64_t)));
+    // The FP16 copy of the keys (d <= 512). A table whose copy does not fit
+    // the device's memory goes without and is screened in TF32.
+    if (d <= 512) {
+      h->table.d16 = (d + 63) / 64 * 64;
+      const size_t bytes = sizeof(__half) * rows * (size_t)h->table.d16;
+      if (cudaMalloc(&h->table.keys16, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        h->table.keys16 = nullptr;
+      }
+    }
+    dev_alloc(h->report, 1);
+    LC_CUDA(cudaMemset(h->report, 0, sizeof(lc::DevReport)));
+    LC_CUDA(cudaMallocHost(&h->report_host, sizeof(lc::DevReport)));
+    std::memset(h->report_host, 0, sizeof(lc::DevReport));
+    h->stats = &h->report->stats;
+    h->stats_host = &h->report_host->stats;
     dev_alloc(h->ins_size0, 1);
-    LC_CUDA(cudaMallocHost(&h->size_pinned, sizeof(int64_t)));
-    dev_alloc(h->stats, 1);
-    LC_CUDA(cudaMemset(h->stats, 0, sizeof(lc::DevStats)));
-    LC_CUDA(cudaMallocHost(&h->stats_host, sizeof(lc::DevStats)));
     for (int i = 0; i < lipcache::kTimingRing; ++i) {
       LC_CUDA(cudaEventCreate(&h->tev0[i]));
       LC_CUDA(cudaEventCreate(&h->tev1[i]));
@@ -319,15 +326,13 @@ LC_API lipcache_status lipcache_insert(lipcache_t* h, const float* H, int64_t n,
       h->pending_stream = s;
       return;
     }
-    LC_CUDA(cudaMemcpyAsync(h->ins_total_host, h->ins_total, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    LC_CUDA(cudaMemcpyAsync(h->size_pinned, h->size_dev, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    LC_CUDA(cudaMemcpyAsync(h->stats_host, h->stats, sizeof(lc::DevStats), cudaMemcpyDeviceToHost, s));
+    lc::fetch_report(h, s);
     LC_CUDA(cudaStreamSynchronize(s));
-    h->size = *h->size_pinned;  // includes earlier asynchronous inserts on this stream
+    h->size = h->report_host->size;  // includes earlier asynchronous inserts on this stream
     h->size_pending = false;
     h->pending_rows = 0;
     LC_REQUIRE(h->stats_host->abort_flag == 0, LIPCACHE_E_DEVICE, lc::kCertifyAbortMessage);
-    const int64_t acc = *h->ins_total_host;
+    const int64_t acc = h->report_host->total[0];
     const int64_t first = h->size - acc;
     if (n_accepted) *n_accepted = acc;
     if (h->policy != LIPCACHE_POLICY_CERTIFIED && acc > 0) {
@@ -393,6 +398,7 @@ LC_API lipcache_status lipcache_insert_select(lipcache_t* h, const float* H, int
             ? lc::select_kcenter(h, H, n, payload, require_consistency, budget_per_class, out_index, out_radius, s)
             : lc::select_insert(h, H, n, payload, require_consistency, budget_total, budget_per_class, out_index,
                                 out_radius, s);
+    lc::fetch_report(h, s);
     LC_CUDA(cudaStreamSynchronize(s));
     if (n_selected) *n_selected = kept;
   });
@@ -418,11 +424,10 @@ LC_API lipcache_status lipcache_probe_writeback(lipcache_t* h, const float* Q, i
     lc::probe(h, Q, B, out_index, out_label, out_dist, s);
     require_no_abort(h, s);  // an aborted probe reports misses: write nothing back
     lc::certify_insert(h, Q, B, payload, require_consistency, out_inserted, nullptr, s, out_index);
-    LC_CUDA(cudaMemcpyAsync(h->ins_total_host, h->ins_total, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    LC_CUDA(cudaMemcpyAsync(h->stats_host, h->stats, sizeof(lc::DevStats), cudaMemcpyDeviceToHost, s));
+    lc::fetch_report(h, s);
     LC_CUDA(cudaStreamSynchronize(s));
     LC_REQUIRE(h->stats_host->abort_flag == 0, LIPCACHE_E_DEVICE, lc::kCertifyAbortMessage);
-    const int64_t acc = *h->ins_total_host;
+    const int64_t acc = h->report_host->total[0];
     const int64_t first = h->size;
     h->size += acc;
     if (n_inserted) *n_inserted = acc;
@@ -450,13 +455,12 @@ LC_API lipcache_status lipcache_consistency(lipcache_t* h, const float* Q, int64
     use_device(h);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     lc::consistency_check(h, Q, B, hit_index, out_consistent, s);
-    LC_CUDA(cudaMemcpyAsync(h->ins_total_host + 1, h->ins_total + 1, 3 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    LC_CUDA(cudaMemcpyAsync(h->stats_host, h->stats, sizeof(lc::DevStats), cudaMemcpyDeviceToHost, s));
+    lc::fetch_report(h, s);
     LC_CUDA(cudaStreamSynchronize(s));
     LC_REQUIRE(h->stats_host->abort_flag == 0, LIPCACHE_E_DEVICE, lc::kCertifyAbortMessage);
-    if (n_hits) *n_hits = h->ins_total_host[1];
-    if (n_consistent) *n_consistent = h->ins_total_host[2];
-    LC_REQUIRE(h->ins_total_host[3] == 0, LIPCACHE_E_INVALID, "hit_index holds values outside [-1, size)");
+    if (n_hits) *n_hits = h->report_host->total[1];
+    if (n_consistent) *n_consistent = h->report_host->total[2];
+    LC_REQUIRE(h->report_host->total[3] == 0, LIPCACHE_E_INVALID, "hit_index holds values outside [-1, size)");
   });
 }
 

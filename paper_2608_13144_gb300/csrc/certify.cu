@@ -37,6 +37,7 @@
 // shared memory (k_certify_wres); for larger heads each CTA streams W from L2
 // (k_certify). Insertion order is kept by a block-count scan and a scatter.
 #include "certify_common.cuh"
+#include "key16.cuh"
 #include "tc_ptx.cuh"
 
 namespace lc {
@@ -1414,6 +1415,7 @@ struct ScatterArgs {
   const float* H;
   int64_t n;
   const int64_t* size0;  // device: the insert's base index
+  const int64_t* size;   // device: the table's size after it
   int d, dpad;
   const uint8_t* accept;
   const int32_t* yG;
@@ -1427,6 +1429,7 @@ struct ScatterArgs {
   Table t;
   int64_t* out_index;
   float* out_radius;
+  int64_t* unfit;      // device: entries whose FP16 copy does not serve
   const DevStats* st;  // abort_flag set: the certify kernel gave up, nothing is appended
 };
 
@@ -1439,10 +1442,15 @@ struct ScatterArgs {
 // mostly sit in L2), so they overlap the chain of dependent loads that
 // resolves the destinations; a rejected row is read for nothing.
 constexpr int kScatterRows = 8;
+constexpr int kTailBlocks = 8;  // blocks of the launch that clear the rows past the new end
 
 __global__ void __launch_bounds__(256) k_scatter(ScatterArgs a, int vec) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t row0 = ((int64_t)blockIdx.x * 8 + warp) * kScatterRows;
+  if (blockIdx.x < kTailBlocks) {
+    zero_tail(a.t, a.dpad, *a.size, (int)(blockIdx.x * 256 + threadIdx.x), kTailBlocks * 256);
+    return;
+  }
+  const int64_t row0 = ((int64_t)(blockIdx.x - kTailBlocks) * 8 + warp) * kScatterRows;
   if (row0 >= a.n) return;
   const int n4 = a.dpad / 4, d4 = a.d / 4;
   float4 v0[kScatterRows];
@@ -1471,32 +1479,84 @@ __global__ void __launch_bounds__(256) k_scatter(ScatterArgs a, int vec) {
   int64_t dst[kScatterRows];
 #pragma unroll
   for (int u = 0; u < kScatterRows; ++u) dst[u] = __shfl_sync(0xffffffffu, mydst, u);
+  // the FP16 copy beside the keys. Every four values passing the check on
+  // their own means every row passes; else the rows are checked whole, below.
+  const bool k16 = a.t.keys16 != nullptr;
+  const int h4 = k16 ? a.t.d16 / 4 : 0;
+  bool fits = true;
+  auto put16 = [&](int u, int j4, const float4& v) {
+    const __half2 lo = __floats2half2_rn(v.x, v.y), hi = __floats2half2_rn(v.z, v.w);
+    *reinterpret_cast<uint2*>(a.t.keys16 + (size_t)dst[u] * a.t.d16 + 4 * j4) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+    const float2 l = __half22float2(lo), h = __half22float2(hi);
+    Half16Check chk;
+    chk.add(v.x, l.x);
+    chk.add(v.y, l.y);
+    chk.add(v.z, h.x);
+    chk.add(v.w, h.y);
+    fits = fits && chk.fits();
+  };
   if (vec) {
     if (lane < n4) {
 #pragma unroll
       for (int u = 0; u < kScatterRows; ++u)
         if (dst[u] >= 0) reinterpret_cast<float4*>(a.t.keys + (size_t)dst[u] * a.dpad)[lane] = v0[u];
     }
-    for (int j4 = lane + 32; j4 < n4; j4 += 32) {
+    if (lane < h4) {
+#pragma unroll
+      for (int u = 0; u < kScatterRows; ++u)
+        if (dst[u] >= 0) put16(u, lane, v0[u]);
+    }
+    for (int j4 = lane + 32; j4 < n4 || j4 < h4; j4 += 32) {
       float4 v[kScatterRows];
 #pragma unroll
       for (int u = 0; u < kScatterRows; ++u)
         v[u] = (dst[u] >= 0 && j4 < d4) ? __ldg(reinterpret_cast<const float4*>(a.H + (size_t)(row0 + u) * a.d) + j4)
                                         : make_float4(0.f, 0.f, 0.f, 0.f);
+      if (j4 < n4) {
 #pragma unroll
-      for (int u = 0; u < kScatterRows; ++u)
-        if (dst[u] >= 0) reinterpret_cast<float4*>(a.t.keys + (size_t)dst[u] * a.dpad)[j4] = v[u];
+        for (int u = 0; u < kScatterRows; ++u)
+          if (dst[u] >= 0) reinterpret_cast<float4*>(a.t.keys + (size_t)dst[u] * a.dpad)[j4] = v[u];
+      }
+      if (j4 < h4) {
+#pragma unroll
+        for (int u = 0; u < kScatterRows; ++u)
+          if (dst[u] >= 0) put16(u, j4, v[u]);
+      }
     }
   } else {
-    for (int j = lane; j < a.dpad; j += 32) {
+    for (int j = lane; j < a.dpad || (k16 && j < a.t.d16); j += 32) {
       float v[kScatterRows];
 #pragma unroll
       for (int u = 0; u < kScatterRows; ++u)
         v[u] = (dst[u] >= 0 && j < a.d) ? __ldg(a.H + (size_t)(row0 + u) * a.d + j) : 0.f;
 #pragma unroll
-      for (int u = 0; u < kScatterRows; ++u)
-        if (dst[u] >= 0) a.t.keys[(size_t)dst[u] * a.dpad + j] = v[u];
+      for (int u = 0; u < kScatterRows; ++u) {
+        if (dst[u] < 0) continue;
+        if (j < a.dpad) a.t.keys[(size_t)dst[u] * a.dpad + j] = v[u];
+        if (k16 && j < a.t.d16) {
+          const __half x = __float2half_rn(v[u]);
+          a.t.keys16[(size_t)dst[u] * a.t.d16 + j] = x;
+          Half16Check chk;
+          chk.add(v[u], __half2float(x));
+          fits = fits && chk.fits();
+        }
+      }
     }
+  }
+  if (!__all_sync(0xffffffffu, fits)) {
+    int bad = 0;
+    for (int u = 0; u < kScatterRows; ++u) {
+      const int64_t to = __shfl_sync(0xffffffffu, mydst, u);
+      if (to < 0) continue;
+      Half16Check chk;
+      for (int j = lane; j < a.d; j += 32) {
+        const float x = __ldg(a.H + (size_t)(row0 + u) * a.d + j);
+        chk.add(x, __half2float(__float2half_rn(x)));
+      }
+      bad += chk.row_fits() ? 0 : 1;
+    }
+    if (lane == 0 && bad) atomicAdd(reinterpret_cast<unsigned long long*>(a.unfit), (unsigned long long)bad);
   }
 }
 
@@ -1729,13 +1789,14 @@ void certify_insert(lipcache* h, const float* H, int64_t n, const int32_t* paylo
                     int64_t* out_index, float* out_radius, cudaStream_t s, const int64_t* miss_of) {
   launch_certify(h, H, n, payload, require_consistency, miss_of, s);
   const int nb = (int)((n + kRows - 1) / kRows);
-  k_scan<<<1, 1024, 0, s>>>(h->ins_bcount, h->ins_boffset, nb, h->ins_total, h->stats, h->size_dev, h->ins_size0,
+  k_scan<<<1, 1024, 0, s>>>(h->ins_bcount, h->ins_boffset, nb, h->report->total, h->stats, &h->report->size, h->ins_size0,
                             h->ins_fix, h->ins_accept, h->ins_rank, n);
   LC_LAUNCH_CHECK("k_scan");
   ScatterArgs sa;
   sa.H = H;
   sa.n = n;
   sa.size0 = h->ins_size0;
+  sa.size = &h->report->size;
   sa.d = h->d;
   sa.dpad = h->dpad;
   sa.accept = h->ins_accept;
@@ -1750,29 +1811,34 @@ void certify_insert(lipcache* h, const float* H, int64_t n, const int32_t* paylo
   sa.t = h->table;
   sa.out_index = out_index;
   sa.out_radius = out_radius;
+  sa.unfit = &h->report->unfit;
   sa.st = h->stats;
   const int vec = (h->d % 4 == 0 && ((uintptr_t)H & 15) == 0) ? 1 : 0;
   const int64_t rows_per_block = 8 * kScatterRows;
-  k_scatter<<<(unsigned)((n + rows_per_block - 1) / rows_per_block), 256, 0, s>>>(sa, vec);
+  k_scatter<<<(unsigned)(kTailBlocks + (n + rows_per_block - 1) / rows_per_block), 256, 0, s>>>(sa, vec);
   LC_LAUNCH_CHECK("k_scatter");
 }
 
 void store_size_dev(lipcache* h, cudaStream_t s) {
-  k_set_i64<<<1, 1, 0, s>>>(h->size_dev, h->size);
+  k_set_i64<<<1, 1, 0, s>>>(&h->report->size, h->size);
   LC_LAUNCH_CHECK("k_set_i64");
 }
 
 void settle_size(lipcache* h) {
   if (!h->size_pending) return;
-  LC_CUDA(cudaMemcpyAsync(h->size_pinned, h->size_dev, sizeof(int64_t), cudaMemcpyDeviceToHost, h->pending_stream));
+  fetch_report(h, h->pending_stream);
   LC_CUDA(cudaStreamSynchronize(h->pending_stream));
-  h->size = *h->size_pinned;
+  h->size = h->report_host->size;
   h->size_pending = false;
   h->pending_rows = 0;
 }
 
+void fetch_report(lipcache* h, cudaStream_t s) {
+  LC_CUDA(cudaMemcpyAsync(h->report_host, h->report, sizeof(DevReport), cudaMemcpyDeviceToHost, s));
+}
+
 void require_certify_ok(lipcache* h, cudaStream_t s) {
-  LC_CUDA(cudaMemcpyAsync(h->stats_host, h->stats, sizeof(DevStats), cudaMemcpyDeviceToHost, s));
+  fetch_report(h, s);
   LC_CUDA(cudaStreamSynchronize(s));
   LC_REQUIRE(h->stats_host->abort_flag == 0, LIPCACHE_E_DEVICE, kCertifyAbortMessage);
 }
@@ -1785,9 +1851,9 @@ void certify_rows(lipcache* h, const float* H, int64_t n, const int32_t* payload
 void consistency_check(lipcache* h, const float* Q, int64_t B, const int64_t* hit_index, int8_t* out,
                        cudaStream_t s) {
   launch_certify(h, Q, B, nullptr, 0, nullptr, s);
-  LC_CUDA(cudaMemsetAsync(h->ins_total + 1, 0, 3 * sizeof(int64_t), s));
+  LC_CUDA(cudaMemsetAsync(h->report->total + 1, 0, 3 * sizeof(int64_t), s));
   k_consistency<<<(unsigned)((B + 255) / 256), 256, 0, s>>>(hit_index, h->ins_yG, h->table.yG, h->size, B, out,
-                                                           h->ins_total + 1);
+                                                           h->report->total + 1);
   LC_LAUNCH_CHECK("k_consistency");
 }
 

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -120,6 +121,14 @@ struct DevStats {
   unsigned long long ins_fp64_rows;  // rows re-certified by the FP64 pass
 };
 
+// What a call may have to report to the host, in one block: one copy.
+struct DevReport {
+  int64_t total[4];  // rows appended by the last insert; consistency counts
+  int64_t size;      // table size
+  int64_t unfit;     // entries whose FP16 copy does not serve the screen
+  DevStats stats;
+};
+
 // Scratch of the selection strategy (select.cu), grown on demand.
 struct SelectScratch {
   unsigned long long* keys = nullptr;
@@ -145,6 +154,8 @@ struct SelectScratch {
 // Per-entry table of the cache (structure of arrays, capacity entries).
 struct Table {
   float* keys = nullptr;     // capacity x dpad, zero padded
+  __half* keys16 = nullptr;  // capacity x d16, the FP16 copy the screen reads (key16.cuh); null: none
+  int d16 = 0;               // its row stride, d rounded up to 64
   float* kn = nullptr;       // FP32 ||k||^2
   float* tau = nullptr;      // screen threshold term
   float* rr = nullptr;       // acceptance threshold on the FP32 squared distance
@@ -204,15 +215,13 @@ struct lipcache {
   int32_t* ins_fix = nullptr;  // rows listed for the FP64 pass of the current certification
   int32_t* ins_bcount = nullptr;
   int32_t* ins_boffset = nullptr;
-  int64_t* ins_total = nullptr;       // device, 4: rows appended; consistency counts
-  int64_t* ins_total_host = nullptr;  // pinned, 4
+  lc::DevReport* report = nullptr;       // device
+  lc::DevReport* report_host = nullptr;  // pinned; report_host->unfit is settled with `size`
   // The table size also lives on the device: k_scan takes an insert's base
   // index from it and advances it, so inserts chain on their stream without
   // the host. An insert called without a host count does not wait; `size` is
   // then settled (synchronising pending_stream) by the next call that needs it.
-  int64_t* size_dev = nullptr;     // device, 1
   int64_t* ins_size0 = nullptr;    // device, 1: base index of the current insert
-  int64_t* size_pinned = nullptr;  // pinned, 1
   bool size_pending = false;       // an asynchronous insert is not yet in `size`
   int64_t pending_rows = 0;        // rows passed to those inserts (bounds their growth)
   cudaStream_t pending_stream = nullptr;
@@ -221,6 +230,7 @@ struct lipcache {
   int64_t q_cap = 0;  // rows (multiple of 128)
   float* qpad = nullptr;
   float* kappa = nullptr;
+  float* qscale = nullptr;  // power-of-two scale of each FP16 query
   unsigned long long* best = nullptr;
   // host-buffer probe staging
   int64_t hq_cap = 0;
@@ -229,8 +239,8 @@ struct lipcache {
   int32_t* hlabel = nullptr;
   float* hdist = nullptr;
 
-  lc::DevStats* stats = nullptr;
-  lc::DevStats* stats_host = nullptr;
+  lc::DevStats* stats = nullptr;       // in `report`
+  lc::DevStats* stats_host = nullptr;  // in `report_host`
 
   // main-kernel timing: a ring of event pairs harvested lazily
   static constexpr int kTimingRing = 64;
@@ -246,20 +256,20 @@ struct lipcache {
 
   double eps_rc = 0.0, c_scr = 0.0;
   lc::EncodeTiledFn encode = nullptr;
-  int pair_clusters = -1;  // resident clusters of the pair probe kernel (-1: not yet queried)
+  int pair_clusters[2] = {-1, -1};  // resident clusters of the pair probe kernel, TF32 / FP16 (-1: not yet queried)
   // Launch state of the tensor probe kernels kept across calls, so that a
   // probe's host side does not repeat the occupancy query, the shared-memory
   // attribute and the tensor-map encoding: [0] k_probe_tc with 256-key
-  // tiles, [1] with 128-key tiles, [2] k_probe_pair.
+  // tiles, [1] with 128-key tiles, [2] k_probe_pair, [3..5] the same in FP16.
   struct ProbeLaunch {
     int resident = 0;  // clusters that fit (0: not queried yet)
-    int smem = 0;      // dynamic shared memory the attribute was set for
+    bool smem[2] = {false, false};  // the kernels' dynamic shared memory attribute is set
     CUtensorMap tmK, tmQ;
     const void* k_base = nullptr;
     uint64_t k_rows = 0;
     const void* q_base = nullptr;
     uint64_t q_rows = 0;
-  } probe_launch[3];
+  } probe_launch[6];
   cudaEvent_t launch_event = nullptr;  // recorded right before the main probe kernel when set
   bool probe_carveout_set = false;     // the prologue / finalize kernels' carveout preference
   int debug_flags = 0;     // LIPCACHE_DEBUG_* test hooks
@@ -281,6 +291,8 @@ struct lipcache {
   int64_t* cls_cnt = nullptr;      // per-block class counts
   int64_t cls_blocks = 0;
 
+  // the FP16 screen serves every entry of the table (host view, settled with `size`)
+  bool f16_screen() const { return table.keys16 != nullptr && report_host->unfit == 0; }
   const float* probe_rr() const { return policy ? rr_emp : table.rr; }
   const float* probe_tau() const { return policy ? tau_emp : table.tau; }
 };
@@ -311,6 +323,8 @@ void require_certify_ok(lipcache* h, cudaStream_t s);
 // stream if one is pending), and write the host size to the device counter
 // after a path that grew the table from the host.
 void settle_size(lipcache* h);
+// Copy the report block to the host, asynchronously on `s`.
+void fetch_report(lipcache* h, cudaStream_t s);
 void store_size_dev(lipcache* h, cudaStream_t s);
 void certify_rows(lipcache* h, const float* H, int64_t n, const int32_t* payload, int require_consistency,
                   cudaStream_t s);
@@ -331,19 +345,28 @@ void consistency_check(lipcache* h, const float* Q, int64_t B, const int64_t* hi
 void probe(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* out_label, float* out_dist,
            cudaStream_t s);
 bool tensor_path_supported(int dpad);
+// The buffers of one probe. TF32: q is the padded FP32 batch (B rounded up to
+// 128 rows x dpad), which also serves the recheck; FP16: q is its scaled FP16
+// form (x d16), scale the rows' powers of two, and the recheck reads Q itself.
+struct ProbeBuffers {
+  const float* Q;   // the caller's queries, B x d
+  void* q;
+  float* kappa;
+  float* scale;
+  unsigned long long* best;
+};
 // probe_tc.cu: the tensor probe; `path` is LIPCACHE_PROBE_TENSOR (kernel
 // chosen by shape), _TENSOR_SINGLE or _TENSOR_PAIR. Returns the kernel that
 // ran (_TENSOR_SINGLE or _TENSOR_PAIR).
-int launch_probe_tc(lipcache* h, int64_t B, int path, cudaStream_t s);
+int launch_probe_tc(lipcache* h, int64_t B, int path, bool f16, const ProbeBuffers& b, cudaStream_t s);
+void encode_screen_map(lipcache* h, CUtensorMap* map, const void* base, uint64_t rows, uint32_t box_rows, bool f16);
 // probe_pair.cu
-int probe_pair_clusters(lipcache* h);
-void launch_probe_pair(lipcache* h, int64_t B, const float* qpad, const float* kappa, unsigned long long* best,
-                       cudaStream_t s);
+int probe_pair_clusters(lipcache* h, bool f16);
+void launch_probe_pair(lipcache* h, int64_t B, bool f16, const ProbeBuffers& b, cudaStream_t s);
 // probe.cu / probe_tc.cu: the probe on caller-provided scratch memory
 void probe_external_scratch(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* out_label,
-                            float* out_dist, float* qpad, float* kappa, unsigned long long* best, cudaStream_t s);
-int launch_probe_tc_external(lipcache* h, int64_t B, int path, const float* qpad, const float* kappa,
-                             unsigned long long* best, cudaStream_t s);
+                            float* out_dist, float* qpad, float* kappa, float* qscale, unsigned long long* best,
+                            cudaStream_t s);
 // api.cu: run fn(ctx) with the C ABI's error handling (status + message)
 lipcache_status run_guarded(void (*fn)(void*), void* ctx);
 // api.cu: harvest completed timing events (blocking on the oldest if `all`

@@ -23,24 +23,33 @@
 namespace {
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[LIPCACHE_NOALLOC_SCRATCH_BYTES];
+// the FP16 queries' scales, beside it: a row takes at least 4 * 32 + 12 bytes
+// of the array above
+constexpr int64_t kMaxRows = LIPCACHE_NOALLOC_SCRATCH_BYTES / (4 * 32 + 12);
+static __device__ float g_noalloc_scale[kMaxRows];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 void* g_scratch_addr[kMaxDevices] = {};
+void* g_scale_addr[kMaxDevices] = {};
 
 // Device address of g_noalloc_scratch on the current device. In host code the
 // symbol's name only stands for the variable; its device address comes from
 // cudaGetSymbolAddress, resolved once per device (on the first call of that
 // device) and cached.
-void* scratch_address(int device) {
+void* scratch_address(int device, void*& scale) {
   LC_REQUIRE(device >= 0 && device < kMaxDevices, LIPCACHE_E_INVALID, "device ordinal out of range");
   std::lock_guard<std::mutex> lock(g_mu);
   if (!g_scratch_addr[device]) {
     void* p = nullptr;
     LC_CUDA(cudaGetSymbolAddress(&p, g_noalloc_scratch));
     LC_REQUIRE(p != nullptr, LIPCACHE_E_CUDA, "cudaGetSymbolAddress returned NULL for the scratch array");
+    void* q = nullptr;
+    LC_CUDA(cudaGetSymbolAddress(&q, g_noalloc_scale));
+    g_scale_addr[device] = q;
     g_scratch_addr[device] = p;
   }
+  scale = g_scale_addr[device];
   return g_scratch_addr[device];
 }
 
@@ -99,9 +108,10 @@ LC_API lipcache_status lipcache_probe_noalloc(lipcache_t* h, const float* Q, int
                      "asynchronous inserts are pending: settle them (lipcache_size) before capturing a probe");
           lc::settle_size(c.h);
         }
-        unsigned char* base = static_cast<unsigned char*>(scratch_address(c.h->device));
+        void* scale = nullptr;
+        unsigned char* base = static_cast<unsigned char*>(scratch_address(c.h->device, scale));
         lc::probe_external_scratch(c.h, c.Q, c.B, c.oi, c.ol, c.od, reinterpret_cast<float*>(base + L.qpad),
-                                   reinterpret_cast<float*>(base + L.kappa),
+                                   reinterpret_cast<float*>(base + L.kappa), static_cast<float*>(scale),
                                    reinterpret_cast<unsigned long long*>(base + L.best),
                                    reinterpret_cast<cudaStream_t>(c.s));
       },

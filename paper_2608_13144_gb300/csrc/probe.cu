@@ -15,8 +15,8 @@
 // (bits(S~) << 32 | i) with atomicMin. S~ >= 0, so its IEEE bits order like
 // its value, and equal distances resolve to the lowest index.
 //
-// Kernels: k_prologue (pads the queries, per-query screen constant, clears
-// the reduction words), the main kernel (exact: every pair on CUDA cores;
+// Kernels: k_prologue / k_prologue16 (pads or rounds the queries, per-query
+// screen constant, clears the reduction words), the main kernel (exact: every pair on CUDA cores;
 // tensor: tcgen05 screen + recheck, probe_tc.cu), k_finalize (unpacks).
 #include "internal.cuh"
 #include "probe_common.cuh"
@@ -29,7 +29,7 @@ namespace {
 // 1,024 keys at d = 16 take 8.1 us exact against 11.7 us on tensor cores;
 // 256 x 50,000 at d = 64 take 80 against 14 us). Both return the same bits.
 int auto_path(const lipcache* h, int64_t B) {
-  if (!tensor_path_supported(h->dpad)) return LIPCACHE_PROBE_EXACT;
+  if (!tensor_path_supported(h->dpad) && !h->f16_screen()) return LIPCACHE_PROBE_EXACT;
   const double macs = (double)B * (double)h->size * (double)h->dpad;
   return macs < 16777216.0 ? LIPCACHE_PROBE_EXACT : LIPCACHE_PROBE_TENSOR;
 }
@@ -56,6 +56,54 @@ __global__ void __launch_bounds__(256) k_prologue(const float* __restrict__ Q, i
   for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(kFull, part, o);
   if (lane == 0) {
     kappa[row] = row < B ? __double2float_rd(one_minus_c * (double)part * 0.5) : INFINITY;
+    best[row] = ~0ull;
+  }
+}
+
+// Prologue of the FP16 screen: each query scaled by a power of two to a
+// largest magnitude in [1, 2) and rounded to FP16 (its error then at most
+// (2^-11 + 2^-20) ||q||, whatever the query's magnitude; NaN and infinities stay what
+// they are), the scale that undoes it, the screen constant, and the reduction
+// word. A warp per row, two features per lane and 64-feature chunk. The 1e-29
+// taken off kappa covers queries below 2^-100, whose scaled features can
+// underflow.
+__global__ void __launch_bounds__(256) k_prologue16(const float* __restrict__ Q, int64_t B, int d, int d16,
+                                                    int64_t Bpad, __half* __restrict__ q16, float* __restrict__ kappa,
+                                                    float* __restrict__ qscale, unsigned long long* __restrict__ best,
+                                                    double one_minus_c, DevStats* __restrict__ st) {
+  constexpr int kMaxChunk = 8;  // d <= 512
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (blockIdx.x == 0 && threadIdx.x == 0) st->abort_flag = 0;
+  const int64_t row = (int64_t)blockIdx.x * 8 + warp;
+  if (row >= Bpad) return;
+  const float* src = Q + (size_t)row * d;
+  float x[kMaxChunk][2];
+  float part = 0.f, m = 0.f;
+#pragma unroll
+  for (int i = 0; i < kMaxChunk; ++i)
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int j = 64 * i + 2 * lane + u;
+      x[i][u] = (row < B && j < d) ? __ldg(src + j) : 0.f;
+      part = fmaf(x[i][u], x[i][u], part);
+      m = fmaxf(m, fabsf(x[i][u]));
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    part += __shfl_xor_sync(kFull, part, o);
+    m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
+  }
+  int e = (int)((__float_as_uint(m) >> 23) & 0xffu) - 127;
+  e = m == 0.f ? 0 : max(-100, min(126, e));
+  const float down = __int_as_float((127 - e) << 23);
+#pragma unroll
+  for (int i = 0; i < kMaxChunk; ++i)
+    if (64 * i < d16)
+      *reinterpret_cast<__half2*>(q16 + (size_t)row * d16 + 64 * i + 2 * lane) =
+          __floats2half2_rn(x[i][0] * down, x[i][1] * down);
+  if (lane == 0) {
+    kappa[row] = row < B ? __fsub_rd(__double2float_rd(one_minus_c * (double)part * 0.5), 1e-29f) : INFINITY;
+    qscale[row] = __int_as_float((127 + e) << 23);
     best[row] = ~0ull;
   }
 }
@@ -162,13 +210,16 @@ void ensure_probe_scratch(lipcache* h, int64_t Bpad) {
   while (cap < Bpad) cap *= 2;
   if (h->qpad) cudaFree(h->qpad);
   if (h->kappa) cudaFree(h->kappa);
+  if (h->qscale) cudaFree(h->qscale);
   if (h->best) cudaFree(h->best);
   h->qpad = nullptr;
   h->kappa = nullptr;
+  h->qscale = nullptr;
   h->best = nullptr;
   h->q_cap = 0;
   LC_CUDA(cudaMalloc(&h->qpad, sizeof(float) * (size_t)cap * h->dpad));
   LC_CUDA(cudaMalloc(&h->kappa, sizeof(float) * (size_t)cap));
+  LC_CUDA(cudaMalloc(&h->qscale, sizeof(float) * (size_t)cap));
   LC_CUDA(cudaMalloc(&h->best, sizeof(unsigned long long) * (size_t)cap));
   h->q_cap = cap;
 }
@@ -188,25 +239,36 @@ void set_probe_carveout(lipcache* h) {
   if (h->probe_carveout_set) return;
   LC_CUDA(cudaFuncSetAttribute(k_prologue, cudaFuncAttributePreferredSharedMemoryCarveout,
                                (int)cudaSharedmemCarveoutMaxShared));
+  LC_CUDA(cudaFuncSetAttribute(k_prologue16, cudaFuncAttributePreferredSharedMemoryCarveout,
+                               (int)cudaSharedmemCarveoutMaxShared));
   LC_CUDA(cudaFuncSetAttribute(k_finalize, cudaFuncAttributePreferredSharedMemoryCarveout,
                                (int)cudaSharedmemCarveoutMaxShared));
   h->probe_carveout_set = true;
 }
 
-void probe(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* out_label, float* out_dist,
-           cudaStream_t s) {
+namespace {
+// The launch sequence of a probe on the given buffers.
+void probe_on(lipcache* h, int64_t B, const ProbeBuffers& b, int64_t* out_index, int32_t* out_label, float* out_dist,
+              bool timing, cudaStream_t s) {
   const int64_t Bpad = (B + 127) / 128 * 128;
-  ensure_probe_scratch(h, Bpad);
   set_probe_carveout(h);
-  k_prologue<<<(unsigned)((Bpad + 7) / 8), 256, 0, s>>>(Q, B, h->d, h->dpad, Bpad, h->qpad, h->kappa, h->best,
-                                                      1.0 - h->c_scr, h->stats);
-  LC_LAUNCH_CHECK("k_prologue");
   int path = h->probe_path;
   if (path == LIPCACHE_PROBE_AUTO) path = auto_path(h, B);
   h->last_probe_path = path;
+  const bool f16 = path != LIPCACHE_PROBE_EXACT && h->f16_screen();
+  const unsigned pgrid = (unsigned)((Bpad + 7) / 8);
+  if (f16) {
+    k_prologue16<<<pgrid, 256, 0, s>>>(b.Q, B, h->d, h->table.d16, Bpad, static_cast<__half*>(b.q), b.kappa, b.scale,
+                                       b.best, 1.0 - h->c_scr, h->stats);
+    LC_LAUNCH_CHECK("k_prologue16");
+  } else {
+    k_prologue<<<pgrid, 256, 0, s>>>(b.Q, B, h->d, h->dpad, Bpad, static_cast<float*>(b.q), b.kappa, b.best,
+                                     1.0 - h->c_scr, h->stats);
+    LC_LAUNCH_CHECK("k_prologue");
+  }
   if (h->size > 0) {
     int slot = -1;
-    if (h->timing) {
+    if (timing && h->timing) {
       if (h->t_issued - h->t_harvested >= lipcache::kTimingRing) harvest_timing(h, false);
       slot = (int)(h->t_issued % lipcache::kTimingRing);
       h->t_kind[slot] = 0;
@@ -215,14 +277,15 @@ void probe(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* 
       // the start event is recorded by the launcher, after its host-side
       // preparation, right before the kernel
       h->launch_event = slot >= 0 ? h->tev0[slot] : nullptr;
-      h->last_probe_path = launch_probe_tc(h, B, path, s);
+      h->last_probe_path = launch_probe_tc(h, B, path, f16, b, s);
       h->launch_event = nullptr;
     } else {
       if (slot >= 0) LC_CUDA(cudaEventRecord(h->tev0[slot], s));
       dim3 grid((unsigned)((h->size + kEK - 1) / kEK), (unsigned)((B + kEQ - 1) / kEQ));
       h->last_grid = (int)(grid.x * grid.y);
       h->last_cluster = 1;
-      k_probe_exact<<<grid, 256, 0, s>>>(h->qpad, B, h->table.keys, h->probe_rr(), h->size, h->dpad, h->best);
+      k_probe_exact<<<grid, 256, 0, s>>>(static_cast<float*>(b.q), B, h->table.keys, h->probe_rr(), h->size, h->dpad,
+                                         b.best);
       LC_LAUNCH_CHECK("k_probe_exact");
     }
     if (slot >= 0) {
@@ -230,36 +293,26 @@ void probe(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* 
       ++h->t_issued;
     }
   }
-  k_finalize<<<(unsigned)((B + 255) / 256), 256, 0, s>>>(h->best, B, h->table.label, out_index, out_label, out_dist,
-                                                       h->stats);
+  k_finalize<<<(unsigned)((B + 255) / 256), 256, 0, s>>>(b.best, B, h->table.label, out_index, out_label, out_dist,
+                                                         h->stats);
   LC_LAUNCH_CHECK("k_finalize");
+}
+}  // namespace
+
+void probe(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* out_label, float* out_dist,
+           cudaStream_t s) {
+  ensure_probe_scratch(h, (B + 127) / 128 * 128);
+  probe_on(h, B, ProbeBuffers{Q, h->qpad, h->kappa, h->qscale, h->best}, out_index, out_label, out_dist, true, s);
 }
 
 // The same launch sequence as probe(), on scratch memory the caller
-// provides (qpad: Bpad x d_pad floats, kappa: Bpad floats, best: Bpad words,
-// Bpad = B rounded up to 128). Allocates nothing.
+// provides (qpad: Bpad x d_pad floats, kappa and qscale: Bpad floats, best:
+// Bpad words, Bpad = B rounded up to 128; the FP16 form of the queries,
+// d16 <= 2 d_pad halves per row, takes qpad's place). Allocates nothing.
 void probe_external_scratch(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* out_label,
-                            float* out_dist, float* qpad, float* kappa, unsigned long long* best, cudaStream_t s) {
-  const int64_t Bpad = (B + 127) / 128 * 128;
-  set_probe_carveout(h);
-  k_prologue<<<(unsigned)((Bpad + 7) / 8), 256, 0, s>>>(Q, B, h->d, h->dpad, Bpad, qpad, kappa, best,
-                                                      1.0 - h->c_scr, h->stats);
-  LC_LAUNCH_CHECK("k_prologue");
-  int path = h->probe_path;
-  if (path == LIPCACHE_PROBE_AUTO) path = auto_path(h, B);
-  h->last_probe_path = path;
-  if (h->size > 0) {
-    if (path != LIPCACHE_PROBE_EXACT) {
-      h->last_probe_path = launch_probe_tc_external(h, B, path, qpad, kappa, best, s);
-    } else {
-      dim3 grid((unsigned)((h->size + kEK - 1) / kEK), (unsigned)((B + kEQ - 1) / kEQ));
-      k_probe_exact<<<grid, 256, 0, s>>>(qpad, B, h->table.keys, h->probe_rr(), h->size, h->dpad, best);
-      LC_LAUNCH_CHECK("k_probe_exact");
-    }
-  }
-  k_finalize<<<(unsigned)((B + 255) / 256), 256, 0, s>>>(best, B, h->table.label, out_index, out_label, out_dist,
-                                                       h->stats);
-  LC_LAUNCH_CHECK("k_finalize");
+                            float* out_dist, float* qpad, float* kappa, float* qscale, unsigned long long* best,
+                            cudaStream_t s) {
+  probe_on(h, B, ProbeBuffers{Q, qpad, kappa, qscale, best}, out_index, out_label, out_dist, false, s);
 }
 
 }  // namespace lc

@@ -1,8 +1,10 @@
 // Tensor-core probe on CTA pairs: the screen + recheck of probe_tc.cu with
 // 2-SM tcgen05 MMAs (Sec. 3.4, Algorithm 2, Eqs. 13-15; cost model Eq. 16).
 //
-// The screen, its bound and the recheck are those of probe_tc.cu; what
-// changes is the schedule. At the single-CTA MMA shape (M = 128 queries,
+// The screen, its operands (FP16 or TF32), its bound and the recheck are those
+// of probe_tc.cu; what changes is the schedule: it serves rows too long for
+// 256-key tiles of a single CTA (49,999 keys x 1,001 queries at d = 500, FP16:
+// 63 us, before on the CUDA cores 2,196 us). At the single-CTA MMA shape (M = 128 queries,
 // N = 256 keys) the operand reads plus the query-stage writes fill the SM's
 // shared-memory bandwidth, so the epilogue's reads come out of MMA
 // throughput. A pair MMA (tcgen05.mma.cta_group::2, M = 256, N = 256) reads
@@ -40,9 +42,8 @@ constexpr int kBM = 256;              // queries per pair tile (MMA M)
 constexpr int kHM = kBM / 2;          // queries per CTA
 constexpr int kBN = 256;              // keys per pair tile (MMA N)
 constexpr int kHN = kBN / 2;          // keys per CTA
-constexpr int kChunkF = 32;           // floats per K chunk (one 128-byte swizzle row)
 constexpr int kMaxStages = 8;
-constexpr int kMaxChunks = 8;         // d_pad <= 256
+constexpr int kMaxChunks = 8;         // d_pad <= 256 (TF32), d <= 512 (FP16)
 constexpr int kQStageBytes = kHM * 128;   // this CTA's 128 query rows of one chunk
 constexpr int kQQuarterBytes = kQStageBytes / 2;
 constexpr int kKChunkBytes = kHN * 128;   // this CTA's 128 keys of one chunk
@@ -56,8 +57,10 @@ constexpr long long kWaitLimit = 1LL << 31;  // ~1 s at GB300 clocks
 
 struct PairArgs {
   int nst;       // query ring stages
-  int nch;       // d_pad / 32
-  int dpad;
+  int nch;       // 128-byte chunks per row
+  int ksteps;    // MMAs of the last chunk that hold features (the others take four)
+  int dpad;      // row stride of keys (and of the padded queries)
+  int d, qvec;   // FP16: features of a query, its rows readable 16 bytes at a time
   int nq;        // query tiles of 256
   int64_t bpad;  // padded query rows (multiple of 128; rows past it are zero-filled by the TMA)
   int qpg;       // query tiles per unit
@@ -65,7 +68,8 @@ struct PairArgs {
   int n_units;   // key-tile quads x query groups
   int n_kt;      // key tiles of 256 holding cache entries
   const float* kappa;
-  const float* qpad;
+  const float* qscale;  // FP16: undoes the queries' scaling
+  const float* q;       // recheck: padded FP32 queries (TF32), the caller's own (FP16)
   const float* keys;
   const float* tau;
   const float* rr;
@@ -100,8 +104,11 @@ __device__ __forceinline__ void unit_range(const PairArgs& a, int u, uint32_t pa
   qt1 = min(a.nq, qt0 + a.qpg);
 }
 
+template <int KIND>
 __global__ void __launch_bounds__(kThreads, 1)
     k_probe_pair(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const PairArgs a) {
+  using Op = ScreenOp<KIND>;
+  constexpr int kChunkF = Op::kChunk;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -192,78 +199,60 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (pair leader)
-    if (pos == 0 && lane == 0) {
-      constexpr uint32_t idesc = ptx::idesc_tf32(kBM, kBN);
+    // the whole warp, converged, one elected lane issuing (probe_tc.cu)
+    if (pos == 0) {
+      constexpr uint32_t idesc = Op::idesc(kBM, kBN);
+      const bool lead = ptx::elect_one();
       const uint64_t qdesc0 = ptx::sw128_kmajor_desc(s_q);
       const uint64_t kdesc0 = ptx::sw128_kmajor_desc(s_k);
       constexpr uint64_t kQStride = kQStageBytes >> 4;
       constexpr uint64_t kKStride = kKChunkBytes >> 4;
-      const int nst = a.nst, nch = a.nch;
+      const int nst = a.nst, nch = a.nch, ksl = a.ksteps;
       int qs = 0;
       uint32_t qph = 0;
       int t = 0, i = 0;
       // failure-detection test: no arrival ever completes this phase, so the
       // bounded wait expires and the kernel takes its abort path
-      bool ok = !a.debug_stall || ptx::mbar_wait(drain, 0, abort_s, kWaitLimit);
+      bool ok = !a.debug_stall || ptx::mbar_wait_warp(drain, 0, abort_s, kWaitLimit);
       for (int u = cluster_id; u < a.n_units && ok; u += n_clusters, ++i) {
         int kt, qt0, qt1;
         unit_range(a, u, pair, kt, qt0, qt1);
         for (int qt = qt0; qt < qt1 && ok; ++qt, ++t) {
           const int buf = t & 1;
           // both CTAs' epilogues are done with this accumulator
-          ok = ptx::mbar_wait_cluster(acc_empty + 8 * buf, (uint32_t)((t >> 1) & 1) ^ 1u, abort_s, kWaitLimit);
+          ok = ptx::mbar_wait_warp<true>(acc_empty + 8 * buf, (uint32_t)((t >> 1) & 1) ^ 1u, abort_s, kWaitLimit);
           if (!ok) break;
-          ptx::tc_fence_after();
           const uint32_t d_tmem = tmem + (uint32_t)(buf * kBN);
           const bool first = qt == qt0, last = qt == qt1 - 1;
           uint64_t kd = kdesc0;
-          if (first || last) {
-            for (int c = 0; c < nch; ++c, kd += kKStride) {
-              if (first && !ptx::mbar_wait(full_k + 8 * c, (uint32_t)(i & 1), abort_s, kWaitLimit)) {
-                ok = false;
-                break;
-              }
-              if (!ptx::mbar_wait(full_q + 8 * qs, qph, abort_s, kWaitLimit)) {
-                ok = false;
-                break;
-              }
-              const uint64_t qd = qdesc0 + (uint64_t)qs * kQStride;
-              ptx::mma_tf32_pair(d_tmem, qd, kd, idesc, c != 0);
-              ptx::mma_tf32_pair(d_tmem, qd + 2, kd + 2, idesc, 1u);
-              ptx::mma_tf32_pair(d_tmem, qd + 4, kd + 4, idesc, 1u);
-              ptx::mma_tf32_pair(d_tmem, qd + 6, kd + 6, idesc, 1u);
+          for (int c = 0; c < nch; ++c, kd += kKStride) {
+            if ((first && !ptx::mbar_wait_warp(full_k + 8 * c, (uint32_t)(i & 1), abort_s, kWaitLimit)) ||
+                !ptx::mbar_wait_warp(full_q + 8 * qs, qph, abort_s, kWaitLimit)) {
+              ok = false;
+              break;
+            }
+            ptx::tc_fence_after();
+            const uint64_t qd = qdesc0 + (uint64_t)qs * kQStride;
+            const int steps = c == nch - 1 ? ksl : 4;
+            if (lead) {
+              Op::template chunk<true>(d_tmem, qd, kd, idesc, c != 0, steps);
               ptx::mma_commit_pair_multicast(empty_q + 8 * qs, (uint16_t)0xF);
               if (last) ptx::mma_commit_pair_multicast(empty_k + 8 * c, pair_mask);
-              if (++qs == nst) {
-                qs = 0;
-                qph ^= 1u;
-              }
+              if (c == nch - 1) ptx::mma_commit_pair_multicast(acc_full + 8 * buf, pair_mask);
             }
-          } else {
-            for (int c = 0; c < nch; ++c, kd += kKStride) {
-              if (!ptx::mbar_wait(full_q + 8 * qs, qph, abort_s, kWaitLimit)) {
-                ok = false;
-                break;
-              }
-              const uint64_t qd = qdesc0 + (uint64_t)qs * kQStride;
-              ptx::mma_tf32_pair(d_tmem, qd, kd, idesc, c != 0);
-              ptx::mma_tf32_pair(d_tmem, qd + 2, kd + 2, idesc, 1u);
-              ptx::mma_tf32_pair(d_tmem, qd + 4, kd + 4, idesc, 1u);
-              ptx::mma_tf32_pair(d_tmem, qd + 6, kd + 6, idesc, 1u);
-              ptx::mma_commit_pair_multicast(empty_q + 8 * qs, (uint16_t)0xF);
-              if (++qs == nst) {
-                qs = 0;
-                qph ^= 1u;
-              }
+            if (++qs == nst) {
+              qs = 0;
+              qph ^= 1u;
             }
           }
-          if (ok) ptx::mma_commit_pair_multicast(acc_full + 8 * buf, pair_mask);
         }
       }
       // all issued MMAs complete before the pair's TMEM can be released
-      volatile int never = 0;
-      ptx::mma_commit_pair_multicast(drain, (uint16_t)(1u << rank));
-      ptx::mbar_wait(drain, 0, &never, kWaitLimit);
+      if (lead) {
+        volatile int never = 0;
+        ptx::mma_commit_pair_multicast(drain, (uint16_t)(1u << rank));
+        ptx::mbar_wait(drain, 0, &never, kWaitLimit);
+      }
     }
     __syncwarp();
   } else {
@@ -300,54 +289,83 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int row_off = (int)pos * kHM + quarter * 32 + lane;
       int64_t row = (int64_t)qt0 * kBM + row_off;
       float kap = row < a.bpad ? __ldg(a.kappa + row) : INFINITY;
+      float scl = KIND == kF16 && row < a.bpad ? __ldg(a.qscale + row) : 1.f;
       for (int qt = qt0; qt < qt1; ++qt, ++t) {
         const int buf = t & 1;
         row = (int64_t)qt * kBM + row_off;
         const int64_t row_next = row + kBM;
         const float kap_next = (qt + 1 < qt1 && row_next < a.bpad) ? __ldg(a.kappa + row_next) : INFINITY;
+        const float scl_next = (KIND == kF16 && qt + 1 < qt1 && row_next < a.bpad) ? __ldg(a.qscale + row_next) : 1.f;
         ok = ptx::mbar_wait(acc_full + 8 * buf, (uint32_t)((t >> 1) & 1), abort_s, kWaitLimit);
         ok = __all_sync(0xffffffffu, ok);  // warp-uniform before the aligned TMEM loads
         if (!ok) break;
         ptx::tc_fence_after();
-        if (live) {
-          const uint32_t tbase = tmem + lane_base + (uint32_t)(buf * kBN + half * kColsPerWarp);
-          uint32_t r[2][32];
-          ptx::tmem_ld32(tbase, r[0]);
+        // Coarse test of each 32-key chunk: a_j - tau_j <= max_j a_j - min_j tau_j
+        // exactly, and rounding is monotone, so a chunk whose value for (max a,
+        // min tau) is below kappa holds no pair that passes. The TMEM load
+        // itself reduces the products (tcgen05.ld.red): no instruction per
+        // product, and an accumulator without a passing chunk is handed back
+        // at once.
+        const uint32_t tbase = tmem + lane_base + (uint32_t)(buf * kBN + half * kColsPerWarp);
+        uint32_t pass = 0;
+#pragma unroll
+        for (int ch = 0; ch < kChunks; ch += 2) {
+          uint32_t va[32], vb[32];
+          float amax[2];
+          ptx::tmem_ld32_max(tbase + (uint32_t)(ch * 32), va, amax[0]);
+          ptx::tmem_ld32_max(tbase + (uint32_t)(ch * 32 + 32), vb, amax[1]);
           ptx::tmem_wait_ld();
+          ptx::hold32(va);
+          ptx::hold32(vb);
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+            pass |= (uint32_t)(screen_value<KIND>(amax[u], scl, tmin[ch + u]) >= kap) << (ch + u);
+        }
+        if (!live) pass = 0;
+        const bool found = __any_sync(0xffffffffu, pass != 0);
+        uint32_t masks[kChunks];
+        if (found) {
 #pragma unroll
           for (int ch = 0; ch < kChunks; ++ch) {
-            if (ch + 1 < kChunks) ptx::tmem_ld32(tbase + (uint32_t)((ch + 1) * 32), r[(ch + 1) & 1]);
-            const uint32_t* v = r[ch & 1];
-            // coarse test of the chunk (probe_tc.cu): fl(max a - min tau)
-            float m0 = -INFINITY, m1 = -INFINITY;
+            masks[ch] = 0;
+            const bool mine = (pass >> ch) & 1u;
+            if (!__any_sync(0xffffffffu, mine)) continue;
+            uint32_t v[32];
+            ptx::tmem_ld32(tbase + (uint32_t)(ch * 32), v);
+            ptx::tmem_wait_ld();
+            uint32_t mask = 0;
 #pragma unroll
-            for (int j = 0; j < 16; j += 2) {
-              m0 = ptx::max3_f32(m0, __uint_as_float(v[j]), __uint_as_float(v[j + 1]));
-              m1 = ptx::max3_f32(m1, __uint_as_float(v[16 + j]), __uint_as_float(v[16 + j + 1]));
-            }
-            if (__fsub_rn(fmaxf(m0, m1), tmin[ch]) >= kap) {
-              uint32_t mask = 0;
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                mask |= (uint32_t)(__uint_as_float(v[j]) - my_tau[ch * 32 + j] >= kap) << j;
-              const float* qrow = a.qpad + (size_t)row * a.dpad;
-              while (mask) {
-                const int j = __ffs(mask) - 1;
-                mask &= mask - 1;
-                const int key = key0 + ch * 32 + j;
-                const float d2 = dist2_canonical(qrow, a.keys + (size_t)key * a.dpad, a.dpad);
-                ++ncand;
-                if (d2 < __ldg(a.rr + key)) atomicMin(a.best + row, pack_hit(d2, key));
-              }
-            }
-            __syncwarp();
-            if (ch + 1 < kChunks) ptx::tmem_wait_ld();
+            for (int j = 0; j < 32; ++j)
+              mask |= (uint32_t)(screen_value<KIND>(__uint_as_float(v[j]), scl, my_tau[ch * 32 + j]) >= kap) << j;
+            masks[ch] = mine ? mask : 0u;
           }
         }
         ptx::tc_fence_before();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive_cluster(lead_acc_empty + 8 * buf);
+        if (found) {
+#pragma unroll
+          for (int ch = 0; ch < kChunks; ++ch) {
+            uint32_t mask = masks[ch];
+            const float* qrow = a.q + (size_t)row * (KIND == kF16 ? a.d : a.dpad);
+            while (mask) {
+              const int j = __ffs(mask) - 1;
+              mask &= mask - 1;
+              const int key = key0 + ch * 32 + j;
+              const float* krow = a.keys + (size_t)key * a.dpad;
+              float d2;
+              if constexpr (KIND == kF16)
+                d2 = dist2_canonical_row(qrow, a.qvec != 0, krow, a.d);
+              else
+                d2 = dist2_canonical(qrow, krow, a.dpad);
+              ++ncand;
+              if (d2 < __ldg(a.rr + key)) atomicMin(a.best + row, pack_hit(d2, key));
+            }
+          }
+          __syncwarp();
+        }
         kap = kap_next;
+        scl = scl_next;
       }
     }
 #pragma unroll
@@ -373,18 +391,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-void encode_rows(lipcache* h, CUtensorMap* map, const float* base, uint64_t rows, uint32_t box_rows) {
-  LC_REQUIRE(h->encode != nullptr, LIPCACHE_E_CUDA, "cuTensorMapEncodeTiled is unavailable from the driver");
-  const cuuint64_t dims[2] = {(cuuint64_t)h->dpad, (cuuint64_t)rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)h->dpad * sizeof(float)};
-  const cuuint32_t box[2] = {(cuuint32_t)kChunkF, box_rows};
-  const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = h->encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box,
-                               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  LC_REQUIRE(r == CUDA_SUCCESS, LIPCACHE_E_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
-}
-
 cudaLaunchConfig_t pair_config(int smem, cudaStream_t s, cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kThreads);
@@ -402,15 +408,17 @@ cudaLaunchConfig_t pair_config(int smem, cudaStream_t s, cudaLaunchAttribute* at
 }  // namespace
 
 // Clusters of four that can be resident at once (0: use probe_tc.cu).
-int probe_pair_clusters(lipcache* h) {
-  if (h->pair_clusters >= 0) return h->pair_clusters;
-  h->pair_clusters = 0;
-  if (h->dpad > kMaxChunks * kChunkF) return 0;
-  const int nch = h->dpad / kChunkF;
+int probe_pair_clusters(lipcache* h, bool f16) {
+  int& known = h->pair_clusters[f16 ? 1 : 0];
+  if (known >= 0) return known;
+  known = 0;
+  const int nch = f16 ? h->table.d16 / 64 : h->dpad / 32;
+  if (nch > kMaxChunks) return 0;
+  auto kern = f16 ? k_probe_pair<kF16> : k_probe_pair<kTf32>;
   const int nst = PairLayout::stages_for(nch);
   if (nst < 2) return 0;
   const int smem = PairLayout{nch, nst}.total() + 1024;
-  if (cudaFuncSetAttribute(k_probe_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 1024) !=
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 1024) !=
       cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -419,32 +427,35 @@ int probe_pair_clusters(lipcache* h) {
   cudaLaunchConfig_t cfg = pair_config(smem, nullptr, attr);
   cfg.gridDim = dim3((unsigned)(h->num_sms / kCluster * kCluster));
   int resident = 0;
-  if (cudaOccupancyMaxActiveClusters(&resident, k_probe_pair, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&resident, kern, &cfg) != cudaSuccess) {
     cudaGetLastError();
     resident = 0;
   }
-  h->pair_clusters = resident;
+  known = resident;
   return resident;
 }
 
-void launch_probe_pair(lipcache* h, int64_t B, const float* qpad, const float* kappa, unsigned long long* best,
-                       cudaStream_t s) {
-  const int clusters_max = probe_pair_clusters(h);
+void launch_probe_pair(lipcache* h, int64_t B, bool f16, const ProbeBuffers& b, cudaStream_t s) {
+  const int clusters_max = probe_pair_clusters(h, f16);
   LC_REQUIRE(clusters_max >= 1, LIPCACHE_E_CUDA, "no cluster of the pair probe kernel fits on this device");
   const int64_t Bpad = (B + 127) / 128 * 128;  // rows of the padded query buffer
-  lipcache::ProbeLaunch& pl = h->probe_launch[2];
-  if (pl.q_base != qpad || pl.q_rows != (uint64_t)Bpad) {
-    encode_rows(h, &pl.tmQ, qpad, (uint64_t)Bpad, kHM / 2);  // a quarter of the pair's query tile per CTA
-    pl.q_base = qpad;
+  lipcache::ProbeLaunch& pl = h->probe_launch[f16 ? 5 : 2];
+  const void* kbase = f16 ? static_cast<const void*>(h->table.keys16) : h->table.keys;
+  if (pl.q_base != b.q || pl.q_rows != (uint64_t)Bpad) {
+    encode_screen_map(h, &pl.tmQ, b.q, (uint64_t)Bpad, kHM / 2, f16);  // a quarter of the pair's query tile per CTA
+    pl.q_base = b.q;
     pl.q_rows = (uint64_t)Bpad;
   }
-  if (pl.k_base != h->table.keys || pl.k_rows != (uint64_t)h->table_rows) {
-    encode_rows(h, &pl.tmK, h->table.keys, (uint64_t)h->table_rows, kHN);
-    pl.k_base = h->table.keys;
+  if (pl.k_base != kbase || pl.k_rows != (uint64_t)h->table_rows) {
+    encode_screen_map(h, &pl.tmK, kbase, (uint64_t)h->table_rows, kHN, f16);
+    pl.k_base = kbase;
     pl.k_rows = (uint64_t)h->table_rows;
   }
   PairArgs a;
-  a.nch = h->dpad / kChunkF;
+  a.nch = f16 ? h->table.d16 / 64 : h->dpad / 32;
+  a.ksteps = f16 ? (h->d - 64 * (a.nch - 1) + 15) / 16 : 4;
+  a.d = h->d;
+  a.qvec = h->d % 4 == 0 && ((uintptr_t)b.Q & 15) == 0;
   a.nst = PairLayout::stages_for(a.nch);
   a.dpad = h->dpad;
   a.bpad = Bpad;
@@ -474,19 +485,21 @@ void launch_probe_pair(lipcache* h, int64_t B, const float* qpad, const float* k
   LC_REQUIRE(n_units < (1LL << 31), LIPCACHE_E_INVALID, "too many work units");
   a.n_units = (int)n_units;
   a.n_kt = (int)n_kt;
-  a.kappa = kappa;
-  a.qpad = qpad;
+  a.kappa = b.kappa;
+  a.qscale = b.scale;
+  a.q = f16 ? b.Q : static_cast<const float*>(b.q);
   a.keys = h->table.keys;
   a.tau = h->probe_tau();
   a.rr = h->probe_rr();
-  a.best = best;
+  a.best = b.best;
   a.stats = h->stats;
   a.debug_stall = (h->debug_flags & LIPCACHE_DEBUG_STALL_PROBE) ? 1 : 0;
   const int smem = PairLayout{a.nch, a.nst}.total() + 1024;
-  if (pl.smem == 0) {
+  auto kern = f16 ? k_probe_pair<kF16> : k_probe_pair<kTf32>;
+  if (!pl.smem[0]) {
     // the attribute belongs to the kernel: the largest size any shape uses
-    LC_CUDA(cudaFuncSetAttribute(k_probe_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 1024));
-    pl.smem = kSmemBudget + 1024;
+    LC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 1024));
+    pl.smem[0] = true;
   }
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = pair_config(smem, s, attr);
@@ -496,7 +509,7 @@ void launch_probe_pair(lipcache* h, int64_t B, const float* qpad, const float* k
   h->last_grid = clusters * kCluster;
   h->last_cluster = kCluster;
   if (h->launch_event) LC_CUDA(cudaEventRecord(h->launch_event, s));
-  LC_CUDA(cudaLaunchKernelEx(&cfg, k_probe_pair, pl.tmQ, pl.tmK, a));
+  LC_CUDA(cudaLaunchKernelEx(&cfg, kern, pl.tmQ, pl.tmK, a));
   LC_LAUNCH_CHECK("k_probe_pair");
 }
 

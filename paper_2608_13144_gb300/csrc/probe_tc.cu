@@ -2,16 +2,29 @@
 // contraction, recheck the few candidates with the exact canonical FP32
 // distance (Sec. 3.4, Algorithm 2, Eqs. 13-15; cost model Eq. 16).
 //
+// Operands. The screen reads the table's FP16 copy and FP16 queries scaled per
+// row by a power of two (key16.cuh): the same 11-bit significand as TF32, at
+// half the bytes and twice the MMA rate. Its error against q.k in 64 bits is
+// that of cuBLAS' TF32 product (both 2.59e-5 |q| |k| root mean square, 1.5e-4
+// at most, d = 128; equal to three digits from d = 16 to 512). 4,096 queries x
+// 4M keys, d = 128: 4.26 ms in TF32, 2.25 ms in FP16 (1.87 PFLOP/s, against
+// 2.19 ms at the cuBLAS bf16 rate); bound by the tensor pipe and the ~100
+// issue cycles between accumulators. A table with an entry outside FP16's
+// range, or whose copy found no memory, is screened in TF32 from the FP32
+// keys. Either way the recheck below decides every pair in FP32, so the
+// results are the same bits.
+//
 // Screen. For a pair with exact squared distance S = |q|^2 + |k|^2 - 2 q.k,
 // the tensor cores return a = q.k up to |a - q.k| <= c |q| |k| <= c (|q|^2 +
-// |k|^2) / 2 (TF32 operands, FP32 accumulation; c = c_screen). Every pair the
+// |k|^2) / 2 (FP32 accumulation; c = c_screen). Every pair the
 // recheck can accept has S < R_k = rr_k / (1 - gamma_rc), hence
 //     a > (1 - c) |q|^2 / 2 + ((1 - c) |k|^2 - R_k) / 2 = kappa_q + tau_k,
 // with kappa_q (per query, k_prologue) rounded down and tau_k (per key,
 // stored at insertion) rounded down. The epilogue keeps a pair iff
 // fl(a - tau_k) >= kappa_q, which therefore never drops an acceptable pair.
-// It first tests each 32-key chunk with fl(max a - min tau) >= kappa_q (one
-// three-input max per two pairs), which no chunk holding a kept pair fails.
+// It first tests each 32-key chunk with fl(max a - min tau) >= kappa_q, which no
+// chunk holding a kept pair fails; the maximum comes with the TMEM load
+// (tcgen05.ld.red), and only a passing chunk's products are looked at.
 //
 // Schedule. Persistent CTAs, one per SM, launched as clusters of two. The two
 // CTAs of a cluster own two adjacent key tiles and stream the SAME sequence of
@@ -20,11 +33,11 @@
 // query byte once per pair of SMs (the query stream from L2 is what limits a
 // single CTA). Per CTA (320 threads):
 //   warp 0     TMA producer: the CTA's key tile (BN keys x d_pad, resident,
-//              one barrier pair per 32-float chunk so the next tile streams in
+//              one barrier pair per 128-byte chunk so the next tile streams in
 //              while the last query tile still runs) and its half of each
-//              query stage (128 queries x 32 floats per stage, multi-stage ring);
-//   warp 1     allocates TMEM, issues tcgen05.mma kind::tf32 (M=128 queries,
-//              N=BN keys, K=8) from one thread into one of two TMEM
+//              query stage (128 queries x 128 bytes per stage, multi-stage ring);
+//   warp 1     allocates TMEM, issues tcgen05.mma kind::f16 / kind::tf32 (M=128
+//              queries, N=BN keys, 32 bytes of K) into one of two TMEM
 //              accumulators; releases each query stage in BOTH CTAs;
 //   warps 2-9  epilogue: tcgen05.ld of the accumulator (warp w reads TMEM
 //              lane quarter w % 4, column half (w - 2) / 4), screen, recheck,
@@ -41,13 +54,11 @@
 #include "tc_ptx.cuh"
 
 namespace lc {
-int tc_key_tile(int dpad);
 namespace {
 
 constexpr int kBM = 128;              // queries per tile (MMA M)
-constexpr int kChunkF = 32;           // floats per K chunk (one 128-byte swizzle row)
 constexpr int kMaxStages = 8;         // query ring depth limit (runtime count fills shared memory)
-constexpr int kMaxChunks = 8;         // d_pad <= 256
+constexpr int kMaxChunks = 8;         // d_pad <= 256 (TF32), d <= 512 (FP16)
 constexpr int kQStageBytes = kBM * 128;
 constexpr int kQHalfBytes = kQStageBytes / 2;
 #ifndef LC_EPI_WARPS
@@ -65,13 +76,16 @@ struct TcArgs {
   int nst;       // query ring stages
   int qgroup;    // stages released together, 1 or 2 (the kernel instantiation; divides nst)
   int tau_staged;  // screen terms copied to shared memory per run (short runs), else read through L1
-  int nch;       // d_pad / 32
-  int dpad;
+  int nch;       // 128-byte chunks per row
+  int ksteps;    // MMAs of the last chunk that hold features (the others take four)
+  int dpad;      // row stride of keys (and of qpad)
+  int d, qvec;   // FP16: features of a query, its rows readable 16 bytes at a time
   int nq;        // query tiles
   int n_pairs;   // key-tile pairs
-  int n_kt;      // key tiles holding cache entries
+  int n_kt;      // key tiles (of BN) holding cache entries
   const float* kappa;
-  const float* qpad;
+  const float* qscale;  // FP16: undoes the queries' scaling
+  const float* q;       // recheck: padded FP32 queries (TF32), the caller's own (FP16)
   const float* keys;
   const float* tau;
   const float* rr;
@@ -85,19 +99,19 @@ struct Layout {
   static constexpr int kKChunkBytes = BN * 128;
   static constexpr int kTmemCols = 2 * BN;
   static constexpr int kTauStaged = 4 * BN * 4;  // one private slice of screen terms per epilogue warp
-  int nch, nst, tau_staged;  // tau_staged: the screen terms copied per run (else read through L1)
-  __device__ __host__ int kbytes() const { return nch * kKChunkBytes; }
+  int nk, nst, tau_staged;  // nk: resident key chunks; tau_staged: the screen terms copied per run (else through L1)
+  __device__ __host__ int kbytes() const { return nk * kKChunkBytes; }
   __device__ __host__ int qoff() const { return kbytes(); }
   __device__ __host__ int tauoff() const { return qoff() + nst * kQStageBytes; }
   __device__ __host__ int baroff() const { return tauoff() + (tau_staged ? kTauStaged : 0); }
-  // barriers: full_k[nch], empty_k[nch], full_q[nst], empty_q[nst], acc_full[2], acc_empty[2], drain
-  __device__ __host__ int nbar() const { return 2 * nch + 2 * nst + 5; }
+  // barriers: full_k[nk], empty_k[nk], full_q[nst], empty_q[nst], acc_full[2], acc_empty[2], drain
+  __device__ __host__ int nbar() const { return 2 * nk + 2 * nst + 5; }
   __device__ __host__ int miscoff() const { return baroff() + 8 * nbar(); }
   __device__ __host__ int total() const { return miscoff() + 16; }
   // deepest ring that fits the shared-memory budget
-  static __host__ int stages_for(int nch, int tau_staged) {
+  static __host__ int stages_for(int nk, int tau_staged) {
     for (int n = kMaxStages; n >= 2; --n) {
-      Layout<BN> L{nch, n, tau_staged};
+      Layout<BN> L{nk, n, tau_staged};
       if (L.total() <= kSmemBudget) return n;
     }
     return 0;
@@ -105,7 +119,8 @@ struct Layout {
 };
 
 // The runs of one cluster: its range [it, end) of items (pair, query tile),
-// pair-major; next() gives this CTA's key tile and the run's query tiles.
+// pair-major; next() gives this CTA's key tile (of NH times BN keys) and the
+// run's query tiles.
 struct RunCursor {
   long long it, end;
   __device__ RunCursor(const TcArgs& a, int cluster_id, int n_clusters) {
@@ -128,22 +143,29 @@ struct RunCursor {
 // MODE 0: short ranges (screen terms staged in shared memory, stages released
 // one at a time); 1: long ranges (screen terms through L1), single releases;
 // 2: long ranges, stages released in pairs.
-template <int BN, int MODE>
+// NH: key tiles of BN held side by side. With two (rows of at most two chunks,
+// long ranges), every query stage is multiplied by both before it is released,
+// half the stage writes, L2 reads and releases per MMA; the two accumulators
+// then belong to the two halves.
+template <int BN, int MODE, int KIND, int NH>
 __global__ void __launch_bounds__(kThreads, 1)
     k_probe_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const TcArgs a) {
   constexpr int QG = MODE == 2 ? 2 : 1;  // query stages released together
   constexpr bool kTauStaged = MODE == 0;
+  using Op = ScreenOp<KIND>;
+  constexpr int kChunkF = Op::kChunk;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // 1024-byte alignment of the swizzled tiles
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  const Layout<BN> L{a.nch, a.nst, a.tau_staged};
+  const int nk = NH * a.nch;
+  const Layout<BN> L{nk, a.nst, a.tau_staged};
   const uint32_t s_base = ptx::smem_u32(smem);
   const uint32_t s_k = s_base;
   const uint32_t s_q = s_base + L.qoff();
   const uint32_t s_bar = s_base + L.baroff();
-  const uint32_t full_k = s_bar, empty_k = s_bar + 8 * a.nch;
-  const uint32_t full_q = s_bar + 16 * a.nch, empty_q = full_q + 8 * a.nst;
+  const uint32_t full_k = s_bar, empty_k = s_bar + 8 * nk;
+  const uint32_t full_q = s_bar + 16 * nk, empty_q = full_q + 8 * a.nst;
   const uint32_t acc_full = empty_q + 8 * a.nst, acc_empty = acc_full + 16, drain = acc_empty + 16;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L.miscoff());
   volatile int* abort_s = reinterpret_cast<volatile int*>(smem + L.miscoff() + 4);
@@ -153,7 +175,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int cluster_id = blockIdx.x / kCluster, n_clusters = gridDim.x / kCluster;
 
   if (threadIdx.x == 0) {
-    for (int c = 0; c < a.nch; ++c) {
+    for (int c = 0; c < nk; ++c) {
       ptx::mbar_init(full_k + 8 * c, 1);
       ptx::mbar_init(empty_k + 8 * c, 1);
     }
@@ -200,15 +222,20 @@ __global__ void __launch_bounds__(kThreads, 1)
       int kt, qt0, qt1;
       for (; ok && rc.next(a, rank, kt, qt0, qt1); ++i) {
         for (int qt = qt0; qt < qt1 && ok; ++qt) {
+          // key chunk c of half h of this run, as soon as the previous run's
+          // last query tile has finished with it (past the table: zero fill)
+          auto load_key = [&](int h, int c) {
+            const int kc = h * a.nch + c;
+            if (!ptx::mbar_wait(empty_k + 8 * kc, (uint32_t)(i & 1) ^ 1u, abort_s, kWaitLimit)) return false;
+            ptx::mbar_expect_tx(full_k + 8 * kc, (uint32_t)Layout<BN>::kKChunkBytes);
+            ptx::tma_load_2d(s_k + kc * Layout<BN>::kKChunkBytes, &tmK, c * kChunkF, (kt * NH + h) * BN, full_k + 8 * kc);
+            last_k_par[kc] = i & 1;
+            return true;
+          };
           for (int c = 0; c < a.nch && ok; ++c) {
             if (qt == qt0) {
-              // key chunk c of this run, as soon as the previous run's last
-              // query tile has finished with it (past the table: zero fill)
-              ok = ptx::mbar_wait(empty_k + 8 * c, (uint32_t)(i & 1) ^ 1u, abort_s, kWaitLimit);
+              ok = load_key(0, c);
               if (!ok) break;
-              ptx::mbar_expect_tx(full_k + 8 * c, (uint32_t)Layout<BN>::kKChunkBytes);
-              ptx::tma_load_2d(s_k + c * Layout<BN>::kKChunkBytes, &tmK, c * kChunkF, kt * BN, full_k + 8 * c);
-              last_k_par[c] = i & 1;
             }
             // stage qs is free in both CTAs (its group was released); fetch
             // this CTA's half for both
@@ -226,6 +253,8 @@ __global__ void __launch_bounds__(kThreads, 1)
               qph ^= 1u;
             }
           }
+          if (NH == 2 && qt == qt0)
+            for (int c = 0; c < a.nch && ok; ++c) ok = load_key(1, c);
         }
       }
       // Let every copy into this CTA land before it can exit. (Bounded; a
@@ -233,123 +262,86 @@ __global__ void __launch_bounds__(kThreads, 1)
       volatile int never = 0;
       for (int s = 0; s < a.nst; ++s)
         if (q_used[s]) ptx::mbar_wait(full_q + 8 * s, last_q_par[s], &never, kWaitLimit);
-      for (int c = 0; c < a.nch; ++c)
+      for (int c = 0; c < nk; ++c)
         if (last_k_par[c] >= 0) ptx::mbar_wait(full_k + 8 * c, (uint32_t)last_k_par[c], &never, kWaitLimit);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    // The tensor pipe queues about one MMA ahead, so this loop keeps the work
-    // between MMA issues minimal: shared-memory descriptors are built once and
-    // advanced by adding encoded offsets (the start-address field holds
-    // address >> 4, so +32 bytes is +2 and never carries out of the field).
-    if (lane == 0) {
-      constexpr uint32_t idesc = ptx::idesc_tf32(kBM, BN);
+    // The tensor pipe queues about one MMA ahead, so the issuing path has to be
+    // short. The whole warp runs it converged (waits by vote, so the compiler
+    // keeps descriptors and loop state in uniform registers, which the MMA
+    // instruction reads) and one elected lane issues. Descriptors are advanced
+    // by adding encoded offsets (the start-address field holds address >> 4, so
+    // +32 bytes is +2 and never carries out of the field); the once-per-run key
+    // waits and releases run in a separate edge path.
+    {
+      constexpr uint32_t idesc = Op::idesc(kBM, BN);
+      const bool lead = ptx::elect_one();
       const uint64_t qdesc0 = ptx::sw128_kmajor_desc(s_q);
       const uint64_t kdesc0 = ptx::sw128_kmajor_desc(s_k);
       constexpr uint64_t kQStride = kQStageBytes >> 4;
       constexpr uint64_t kKStride = Layout<BN>::kKChunkBytes >> 4;
-      const int nst = a.nst, nch = a.nch;
+      const int nst = a.nst, nch = a.nch, ksl = a.ksteps;
       int qs = 0;
       uint32_t qph = 0;
       int t = 0, i = 0;
       // failure-detection test: no arrival ever completes this phase, so the
       // bounded wait expires and the kernel takes its abort path
-      bool ok = !a.debug_stall || ptx::mbar_wait(drain, 0, abort_s, kWaitLimit);
+      bool ok = !a.debug_stall || ptx::mbar_wait_warp(drain, 0, abort_s, kWaitLimit);
       RunCursor rc(a, cluster_id, n_clusters);
       int kt, qt0, qt1;
       for (; ok && rc.next(a, rank, kt, qt0, qt1); ++i) {
-        for (int qt = qt0; qt < qt1 && ok; ++qt, ++t) {
-          const int buf = t & 1;
-          ok = ptx::mbar_wait(acc_empty + 8 * buf, (uint32_t)((t >> 1) & 1) ^ 1u, abort_s, kWaitLimit);
-          if (!ok) break;
-          ptx::tc_fence_after();
-          const uint32_t d_tmem = tmem + (uint32_t)(buf * BN);
+        for (int qt = qt0; qt < qt1 && ok; ++qt) {
           const bool first = qt == qt0, last = qt == qt1 - 1;
-          uint64_t kd = kdesc0;
-          if (first || last) {
-            // Run edges: the key chunk arrives once per run (TMA completion on
-            // the mbarrier already orders the copies before the MMA's reads),
-            // and the last query tile hands each chunk back to the producer.
+          const int qb = qs;  // first stage of the query tile and its phase
+          const uint32_t qbph = qph;
+#pragma unroll
+          for (int h = 0; h < NH; ++h, ++t) {
+            if (NH == 2 && h == 1) {
+              qs = qb;
+              qph = qbph;
+            }
+            const int buf = NH == 2 ? h : t & 1;
+            if (!ptx::mbar_wait_warp(acc_empty + 8 * buf, (uint32_t)((t >> 1) & 1) ^ 1u, abort_s, kWaitLimit)) {
+              ok = false;
+              break;
+            }
+            const uint32_t d_tmem = tmem + (uint32_t)(buf * BN);
+            uint64_t kd = kdesc0 + (uint64_t)(h * nch) * kKStride;
             for (int c = 0; c < nch; ++c, kd += kKStride) {
-              if (first && !ptx::mbar_wait(full_k + 8 * c, (uint32_t)(i & 1), abort_s, kWaitLimit)) {
+              if (first && !ptx::mbar_wait_warp(full_k + 8 * (h * nch + c), (uint32_t)(i & 1), abort_s, kWaitLimit)) {
                 ok = false;
                 break;
               }
-              if (!ptx::mbar_wait(full_q + 8 * qs, qph, abort_s, kWaitLimit)) {
+              if (h == 0 && !ptx::mbar_wait_warp(full_q + 8 * qs, qph, abort_s, kWaitLimit)) {
                 ok = false;
                 break;
               }
+              ptx::tc_fence_after();
               const uint64_t qd = qdesc0 + (uint64_t)qs * kQStride;
-              ptx::mma_tf32(d_tmem, qd, kd, idesc, c != 0);
-              ptx::mma_tf32(d_tmem, qd + 2, kd + 2, idesc, 1u);
-              ptx::mma_tf32(d_tmem, qd + 4, kd + 4, idesc, 1u);
-              ptx::mma_tf32(d_tmem, qd + 6, kd + 6, idesc, 1u);
-              if (QG == 1 || (qs & 1)) ptx::mma_commit_multicast(empty_q + 8 * (qs >> (QG - 1)), kClusterMask);
-              if (last) ptx::mma_commit(empty_k + 8 * c);
+              const int steps = c == nch - 1 ? ksl : 4;
+              if (lead) {
+                Op::chunk(d_tmem, qd, kd, idesc, c != 0, steps);
+                if (h == NH - 1 && (QG == 1 || (qs & 1)))
+                  ptx::mma_commit_multicast(empty_q + 8 * (qs >> (QG - 1)), kClusterMask);
+                if (last) ptx::mma_commit(empty_k + 8 * (h * nch + c));
+                if (c == nch - 1) ptx::mma_commit(acc_full + 8 * buf);
+              }
               if (++qs == nst) {
                 qs = 0;
                 qph ^= 1u;
               }
             }
-          } else if (QG == 2) {
-            // Steady state, stages released in pairs (nch and nst even, so
-            // a tile starts on the first stage of a pair): the stage waits,
-            // eight MMAs and one release per two stages, no predicated
-            // tensor-pipe instructions.
-            for (int c = 0; c < nch && ok; c += 2, kd += 2 * kKStride) {
-              if (!ptx::mbar_wait(full_q + 8 * qs, qph, abort_s, kWaitLimit)) {
-                ok = false;
-                break;
-              }
-              uint64_t qd = qdesc0 + (uint64_t)qs * kQStride;
-              ptx::mma_tf32(d_tmem, qd, kd, idesc, c != 0);
-              ptx::mma_tf32(d_tmem, qd + 2, kd + 2, idesc, 1u);
-              ptx::mma_tf32(d_tmem, qd + 4, kd + 4, idesc, 1u);
-              ptx::mma_tf32(d_tmem, qd + 6, kd + 6, idesc, 1u);
-              ++qs;  // (even, below nst - 1: no wrap)
-              if (!ptx::mbar_wait(full_q + 8 * qs, qph, abort_s, kWaitLimit)) {
-                ok = false;
-                break;
-              }
-              qd = qdesc0 + (uint64_t)qs * kQStride;
-              const uint64_t kd1 = kd + kKStride;
-              ptx::mma_tf32(d_tmem, qd, kd1, idesc, 1u);
-              ptx::mma_tf32(d_tmem, qd + 2, kd1 + 2, idesc, 1u);
-              ptx::mma_tf32(d_tmem, qd + 4, kd1 + 4, idesc, 1u);
-              ptx::mma_tf32(d_tmem, qd + 6, kd1 + 6, idesc, 1u);
-              ptx::mma_commit_multicast(empty_q + 8 * (qs >> 1), kClusterMask);
-              if (++qs == nst) {
-                qs = 0;
-                qph ^= 1u;
-              }
-            }
-          } else {
-            // Steady state: nothing but the stage wait, four MMAs and the
-            // stage release (no predicated tensor-pipe instructions).
-            for (int c = 0; c < nch; ++c, kd += kKStride) {
-              if (!ptx::mbar_wait(full_q + 8 * qs, qph, abort_s, kWaitLimit)) {
-                ok = false;
-                break;
-              }
-              const uint64_t qd = qdesc0 + (uint64_t)qs * kQStride;
-              ptx::mma_tf32(d_tmem, qd, kd, idesc, c != 0);
-              ptx::mma_tf32(d_tmem, qd + 2, kd + 2, idesc, 1u);
-              ptx::mma_tf32(d_tmem, qd + 4, kd + 4, idesc, 1u);
-              ptx::mma_tf32(d_tmem, qd + 6, kd + 6, idesc, 1u);
-              ptx::mma_commit_multicast(empty_q + 8 * qs, kClusterMask);
-              if (++qs == nst) {
-                qs = 0;
-                qph ^= 1u;
-              }
-            }
+            if (!ok) break;
           }
-          if (ok) ptx::mma_commit(acc_full + 8 * buf);
         }
       }
       // all issued MMAs complete before TMEM can be released
-      volatile int never = 0;
-      ptx::mma_commit(drain);
-      ptx::mbar_wait(drain, 0, &never, kWaitLimit);
+      if (lead) {
+        volatile int never = 0;
+        ptx::mma_commit(drain);
+        ptx::mbar_wait(drain, 0, &never, kWaitLimit);
+      }
     }
     __syncwarp();
   } else {
@@ -368,8 +360,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     RunCursor rc(a, cluster_id, n_clusters);
     int kt, qt0, qt1;
     while (ok && rc.next(a, rank, kt, qt0, qt1)) {
-      const bool live = kt < a.n_kt;
-      const int key0 = kt * BN + half * kColsPerWarp;
+      const int key0 = kt * (NH * BN) + half * kColsPerWarp;  // + h BN for half h of the key tile
       // the minimum of this warp's screen terms over each 32-key chunk of
       // the run's key tile. The per-pair test, which few chunks reach, reads
       // the terms themselves from a copy in shared memory made here when the
@@ -377,77 +368,113 @@ __global__ void __launch_bounds__(kThreads, 1)
       // ring).
       if (kTauStaged) {
         __syncwarp();
-        if (live)
+        if (kt < a.n_kt)
           for (int v4 = lane; v4 < kColsPerWarp / 4; v4 += 32)
             reinterpret_cast<float4*>(my_tau)[v4] = __ldg(reinterpret_cast<const float4*>(a.tau + key0) + v4);
         __syncwarp();
       }
-      const float* __restrict__ tau_g = a.tau + key0;
-      float tmin[kChunks];
+      float tmin[NH][kChunks];
 #pragma unroll
-      for (int ch = 0; ch < kChunks; ++ch) {
-        float m = !live ? INFINITY : kTauStaged ? my_tau[ch * 32 + lane] : __ldg(tau_g + ch * 32 + lane);
+      for (int h = 0; h < NH; ++h)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        tmin[ch] = m;
-      }
+        for (int ch = 0; ch < kChunks; ++ch) {
+          float m = kt * NH + h >= a.n_kt ? INFINITY
+                    : kTauStaged          ? my_tau[ch * 32 + lane]
+                                          : __ldg(a.tau + key0 + h * BN + ch * 32 + lane);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+          tmin[h][ch] = m;
+        }
       float kap = __ldg(a.kappa + qt0 * kBM + quarter * 32 + lane);
-      for (int qt = qt0; qt < qt1; ++qt, ++t) {
-        const int buf = t & 1;
+      float scl = KIND == kF16 ? __ldg(a.qscale + qt0 * kBM + quarter * 32 + lane) : 1.f;
+      for (int qt = qt0; qt < qt1 && ok; ++qt) {
         const int row = qt * kBM + quarter * 32 + lane;
         // next tile's screen constant, fetched while this accumulator is produced
         const float kap_next = (qt + 1 < qt1) ? __ldg(a.kappa + row + kBM) : 0.f;
+        const float scl_next = (KIND == kF16 && qt + 1 < qt1) ? __ldg(a.qscale + row + kBM) : 1.f;
+#pragma unroll
+        for (int h = 0; h < NH; ++h, ++t) {
+        const int buf = t & 1;
+        const bool live = kt * NH + h < a.n_kt;
+        const float* __restrict__ tau_g = a.tau + key0 + h * BN;
         ok = ptx::mbar_wait(acc_full + 8 * buf, (uint32_t)((t >> 1) & 1), abort_s, kWaitLimit);
         ok = __all_sync(0xffffffffu, ok);  // warp-uniform before the aligned TMEM loads
         if (!ok) break;
         ptx::tc_fence_after();
-        if (live) {
-          const uint32_t tbase = tmem + lane_base + (uint32_t)(buf * BN + half * kColsPerWarp);
-          uint32_t r[2][32];
-          ptx::tmem_ld32(tbase, r[0]);
+        // Coarse test of each 32-key chunk: a_j - tau_j <= max_j a_j - min_j tau_j
+        // exactly, and rounding is monotone, so a chunk whose value for (max a,
+        // min tau) is below kappa holds no pair that passes. The TMEM load
+        // itself reduces the products (tcgen05.ld.red): no instruction per
+        // product, and an accumulator without a passing chunk is handed back
+        // at once.
+        const uint32_t tbase = tmem + lane_base + (uint32_t)(buf * BN + half * kColsPerWarp);
+        uint32_t pass = 0;
+#pragma unroll
+        for (int ch = 0; ch < kChunks; ch += 2) {
+          uint32_t va[32], vb[32];
+          float amax[2];
+          ptx::tmem_ld32_max(tbase + (uint32_t)(ch * 32), va, amax[0]);
+          ptx::tmem_ld32_max(tbase + (uint32_t)(ch * 32 + 32), vb, amax[1]);
           ptx::tmem_wait_ld();
+          ptx::hold32(va);
+          ptx::hold32(vb);
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+            pass |= (uint32_t)(screen_value<KIND>(amax[u], scl, tmin[h][ch + u]) >= kap) << (ch + u);
+        }
+        if (!live) pass = 0;
+        const bool found = __any_sync(0xffffffffu, pass != 0);
+        uint32_t masks[kChunks];
+        if (found) {
 #pragma unroll
           for (int ch = 0; ch < kChunks; ++ch) {
-            if (ch + 1 < kChunks) ptx::tmem_ld32(tbase + (uint32_t)((ch + 1) * 32), r[(ch + 1) & 1]);
-            const uint32_t* v = r[ch & 1];
-            // Coarse test of the chunk: a_j - tau_j <= max_j a_j - min_j tau_j
-            // exactly, and rounding is monotone, so a chunk whose
-            // fl(max a - min tau) is below kappa holds no pair that passes
-            // fl(a_j - tau_j) >= kappa. Two independent three-input max chains.
-            float m0 = -INFINITY, m1 = -INFINITY;
+            masks[ch] = 0;
+            const bool mine = (pass >> ch) & 1u;
+            if (!__any_sync(0xffffffffu, mine)) continue;
+            uint32_t v[32];
+            ptx::tmem_ld32(tbase + (uint32_t)(ch * 32), v);
+            ptx::tmem_wait_ld();
+            uint32_t mask = 0;
+            if (kTauStaged) {
 #pragma unroll
-            for (int j = 0; j < 16; j += 2) {
-              m0 = ptx::max3_f32(m0, __uint_as_float(v[j]), __uint_as_float(v[j + 1]));
-              m1 = ptx::max3_f32(m1, __uint_as_float(v[16 + j]), __uint_as_float(v[16 + j + 1]));
+              for (int j = 0; j < 32; ++j)
+                mask |= (uint32_t)(screen_value<KIND>(__uint_as_float(v[j]), scl, my_tau[ch * 32 + j]) >= kap) << j;
+            } else {
+#pragma unroll
+              for (int j = 0; j < 32; ++j)
+                mask |= (uint32_t)(screen_value<KIND>(__uint_as_float(v[j]), scl, __ldg(tau_g + ch * 32 + j)) >= kap)
+                        << j;
             }
-            if (__fsub_rn(fmaxf(m0, m1), tmin[ch]) >= kap) {
-              uint32_t mask = 0;
-              if (kTauStaged) {
-#pragma unroll
-                for (int j = 0; j < 32; ++j) mask |= (uint32_t)(__uint_as_float(v[j]) - my_tau[ch * 32 + j] >= kap) << j;
-              } else {
-#pragma unroll
-                for (int j = 0; j < 32; ++j)
-                  mask |= (uint32_t)(__uint_as_float(v[j]) - __ldg(tau_g + ch * 32 + j) >= kap) << j;
-              }
-              const float* qrow = a.qpad + (size_t)row * a.dpad;
-              while (mask) {
-                const int j = __ffs(mask) - 1;
-                mask &= mask - 1;
-                const int key = key0 + ch * 32 + j;
-                const float d2 = dist2_canonical(qrow, a.keys + (size_t)key * a.dpad, a.dpad);
-                ++ncand;
-                if (d2 < __ldg(a.rr + key)) atomicMin(a.best + row, pack_hit(d2, key));
-              }
-            }
-            __syncwarp();
-            if (ch + 1 < kChunks) ptx::tmem_wait_ld();
+            masks[ch] = mine ? mask : 0u;
           }
         }
         ptx::tc_fence_before();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(acc_empty + 8 * buf);
+        if (found) {
+#pragma unroll
+          for (int ch = 0; ch < kChunks; ++ch) {
+            uint32_t mask = masks[ch];
+            const float* qrow = a.q + (size_t)row * (KIND == kF16 ? a.d : a.dpad);
+            while (mask) {
+              const int j = __ffs(mask) - 1;
+              mask &= mask - 1;
+              const int key = key0 + h * BN + ch * 32 + j;
+              const float* krow = a.keys + (size_t)key * a.dpad;
+              float d2;
+              if constexpr (KIND == kF16)
+                d2 = dist2_canonical_row(qrow, a.qvec != 0, krow, a.d);
+              else
+                d2 = dist2_canonical(qrow, krow, a.dpad);
+              ++ncand;
+              if (d2 < __ldg(a.rr + key)) atomicMin(a.best + row, pack_hit(d2, key));
+            }
+          }
+          __syncwarp();
+        }
+        }
         kap = kap_next;
+        scl = scl_next;
       }
     }
     // candidate count: one atomic per warp
@@ -474,71 +501,69 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-void encode_2d(lipcache* h, CUtensorMap* map, const float* base, uint64_t rows, uint32_t box_rows) {
-  LC_REQUIRE(h->encode != nullptr, LIPCACHE_E_CUDA, "cuTensorMapEncodeTiled is unavailable from the driver");
-  const cuuint64_t dims[2] = {(cuuint64_t)h->dpad, (cuuint64_t)rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)h->dpad * sizeof(float)};
-  const cuuint32_t box[2] = {(cuuint32_t)kChunkF, box_rows};
-  const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = h->encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box,
-                               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  LC_REQUIRE(r == CUDA_SUCCESS, LIPCACHE_E_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
-}
-
-template <int BN>
-void launch(lipcache* h, int64_t B, const float* qpad, const float* kappa, unsigned long long* best, cudaStream_t s) {
+template <int BN, int KIND, int NH>
+void launch_nh(lipcache* h, int64_t B, const ProbeBuffers& b, bool long_ranges, cudaStream_t s) {
+  constexpr bool f16 = KIND == kF16;
   const int64_t Bpad = (B + kBM - 1) / kBM * kBM;
-  lipcache::ProbeLaunch& pl = h->probe_launch[BN == 256 ? 0 : 1];
-  if (pl.q_base != qpad || pl.q_rows != (uint64_t)Bpad) {
-    encode_2d(h, &pl.tmQ, qpad, (uint64_t)Bpad, kBM / 2);  // half a query tile per CTA of the pair
-    pl.q_base = qpad;
+  lipcache::ProbeLaunch& pl = h->probe_launch[(BN == 256 ? 0 : 1) + (f16 ? 3 : 0)];
+  const void* kbase = f16 ? static_cast<const void*>(h->table.keys16) : h->table.keys;
+  if (pl.q_base != b.q || pl.q_rows != (uint64_t)Bpad) {
+    encode_screen_map(h, &pl.tmQ, b.q, (uint64_t)Bpad, kBM / 2, f16);  // half a query tile per CTA of the pair
+    pl.q_base = b.q;
     pl.q_rows = (uint64_t)Bpad;
   }
-  if (pl.k_base != h->table.keys || pl.k_rows != (uint64_t)h->table_rows) {
-    encode_2d(h, &pl.tmK, h->table.keys, (uint64_t)h->table_rows, BN);
-    pl.k_base = h->table.keys;
+  if (pl.k_base != kbase || pl.k_rows != (uint64_t)h->table_rows) {
+    encode_screen_map(h, &pl.tmK, kbase, (uint64_t)h->table_rows, BN, f16);
+    pl.k_base = kbase;
     pl.k_rows = (uint64_t)h->table_rows;
   }
   TcArgs a;
-  a.nch = h->dpad / kChunkF;
+  a.nch = f16 ? h->table.d16 / 64 : h->dpad / 32;
+  a.ksteps = f16 ? (h->d - 64 * (a.nch - 1) + 15) / 16 : 4;
   // (the ring depth depends on whether the screen terms are staged: below)
   a.dpad = h->dpad;
+  a.d = h->d;
+  a.qvec = h->d % 4 == 0 && ((uintptr_t)b.Q & 15) == 0;
   a.nq = (int)(Bpad / kBM);
   const int64_t n_kt = (h->size + BN - 1) / BN;
-  const int64_t n_pairs = (n_kt + kCluster - 1) / kCluster;
+  const int64_t n_pairs = (n_kt + NH * kCluster - 1) / (NH * kCluster);
   const int max_clusters = h->num_sms / kCluster;
-  LC_REQUIRE(max_clusters >= 1, LIPCACHE_E_CUDA, "device has fewer than two SMs");
   // Long ranges (many items per cluster, the large caches): the screen terms
   // are read through L1, the shared memory goes to the query ring, and the
   // stages are released two at a time (one commit per pair) when a tile's
   // stages pair up and the ring holds whole pairs. Short ranges keep the
   // staged screen terms and single releases, which measure faster there.
-  const bool long_ranges = n_pairs * a.nq / max_clusters >= kPairedReleaseItems;
   a.tau_staged = long_ranges ? 0 : 1;
-  a.nst = Layout<BN>::stages_for(a.nch, a.tau_staged);
-  LC_REQUIRE(a.nst >= 2, LIPCACHE_E_INVALID, "key tile does not fit shared memory");
-  a.qgroup = (long_ranges && a.nst % 2 == 0 && a.nch % 2 == 0) ? 2 : 1;
+  a.nst = Layout<BN>::stages_for(NH * a.nch, a.tau_staged);
+  // (two halves hold a whole query tile of stages while the next one loads)
+  LC_REQUIRE(a.nst >= (NH == 2 ? a.nch + 2 : 2), LIPCACHE_E_INVALID, "key tile does not fit shared memory");
+  a.qgroup = (long_ranges && a.nst % 2 == 0 && a.nst >= 4 && a.nch % 2 == 0) ? 2 : 1;
   LC_REQUIRE(n_pairs * a.nq < (1LL << 40), LIPCACHE_E_INVALID, "too many work items");
   a.n_pairs = (int)n_pairs;
   a.n_kt = (int)n_kt;
-  a.kappa = kappa;
-  a.qpad = qpad;
+  a.kappa = b.kappa;
+  a.qscale = b.scale;
+  a.q = f16 ? b.Q : static_cast<const float*>(b.q);
   a.keys = h->table.keys;
   a.tau = h->probe_tau();
   a.rr = h->probe_rr();
-  a.best = best;
+  a.best = b.best;
   a.stats = h->stats;
   a.debug_stall = (h->debug_flags & LIPCACHE_DEBUG_STALL_PROBE) ? 1 : 0;
-  const Layout<BN> L{a.nch, a.nst, a.tau_staged};
+  const Layout<BN> L{NH * a.nch, a.nst, a.tau_staged};
   const int smem = L.total() + 1024;
-  if (pl.smem == 0) {
+  // (two halves only run the long modes)
+  constexpr int kM0 = NH == 2 ? 1 : 0;
+  if (!pl.smem[NH - 1]) {
     // the attribute belongs to the kernel, not to this cache: set it to the
     // largest size any shape uses, so other caches' launches stay valid
-    LC_CUDA(cudaFuncSetAttribute(k_probe_tc<BN, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 1024));
-    LC_CUDA(cudaFuncSetAttribute(k_probe_tc<BN, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 1024));
-    LC_CUDA(cudaFuncSetAttribute(k_probe_tc<BN, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 1024));
-    pl.smem = kSmemBudget + 1024;
+    LC_CUDA(cudaFuncSetAttribute(k_probe_tc<BN, kM0, KIND, NH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kSmemBudget + 1024));
+    LC_CUDA(cudaFuncSetAttribute(k_probe_tc<BN, 1, KIND, NH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kSmemBudget + 1024));
+    LC_CUDA(cudaFuncSetAttribute(k_probe_tc<BN, 2, KIND, NH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kSmemBudget + 1024));
+    pl.smem[NH - 1] = true;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(max_clusters * kCluster));
@@ -552,8 +577,13 @@ void launch(lipcache* h, int64_t B, const float* qpad, const float* kappa, unsig
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  // persistent grid: no more clusters than can be resident at once
-  if (pl.resident == 0) LC_CUDA(cudaOccupancyMaxActiveClusters(&pl.resident, k_probe_tc<BN, 0>, &cfg));
+  // persistent grid: no more clusters than can be resident at once (asked for
+  // with the most shared memory any launch uses)
+  if (pl.resident == 0) {
+    cfg.dynamicSmemBytes = (size_t)kSmemBudget + 1024;
+    LC_CUDA(cudaOccupancyMaxActiveClusters(&pl.resident, k_probe_tc<BN, 1, KIND, NH>, &cfg));
+    cfg.dynamicSmemBytes = (size_t)smem;
+  }
   const int resident = pl.resident;
   LC_REQUIRE(resident >= 1, LIPCACHE_E_CUDA, "no CTA pair of the probe kernel fits on this device");
   int clusters = max_clusters < resident ? max_clusters : resident;
@@ -563,36 +593,68 @@ void launch(lipcache* h, int64_t B, const float* qpad, const float* kappa, unsig
   h->last_cluster = kCluster;
   if (h->launch_event) LC_CUDA(cudaEventRecord(h->launch_event, s));
   void (*kern)(CUtensorMap, CUtensorMap, TcArgs) =
-      a.tau_staged ? k_probe_tc<BN, 0> : a.qgroup == 2 ? k_probe_tc<BN, 2> : k_probe_tc<BN, 1>;
+      a.tau_staged       ? k_probe_tc<BN, kM0, KIND, NH>
+      : a.qgroup == 2 ? k_probe_tc<BN, 2, KIND, NH>
+                      : k_probe_tc<BN, 1, KIND, NH>;
   LC_CUDA(cudaLaunchKernelEx(&cfg, kern, pl.tmQ, pl.tmK, a));
   LC_LAUNCH_CHECK("k_probe_tc");
 }
 
-}  // namespace
-
-int tc_key_tile(int dpad) { return dpad <= 128 ? 256 : 128; }
-
-int launch_probe_tc_external(lipcache* h, int64_t B, int path, const float* qpad, const float* kappa,
-                             unsigned long long* best, cudaStream_t s) {
-  LC_REQUIRE(tensor_path_supported(h->dpad), LIPCACHE_E_INVALID, "the tensor probe supports d <= 256");
-  // Pair MMAs read a third less shared memory per flop; that decides for
-  // d_pad > 128, where the single-CTA kernel has to use 128-key tiles. At
-  // d_pad <= 128 its 256-key tiles on all SMs (clusters of four leave some
-  // idle) are faster.
-  const bool pair = path == LIPCACHE_PROBE_TENSOR_PAIR || (path == LIPCACHE_PROBE_TENSOR && h->dpad > 128);
-  if (pair && probe_pair_clusters(h) >= 1) {
-    launch_probe_pair(h, B, qpad, kappa, best, s);
-    return LIPCACHE_PROBE_TENSOR_PAIR;
+template <int BN, int KIND>
+void launch(lipcache* h, int64_t B, const ProbeBuffers& b, cudaStream_t s) {
+  const int max_clusters = h->num_sms / kCluster;
+  LC_REQUIRE(max_clusters >= 1, LIPCACHE_E_CUDA, "device has fewer than two SMs");
+  const int64_t nq = (B + kBM - 1) / kBM, n_kt = (h->size + BN - 1) / BN;
+  const bool long_ranges = (n_kt + kCluster - 1) / kCluster * nq / max_clusters >= kPairedReleaseItems;
+  if constexpr (KIND == kF16 && BN == 256) {
+    // two key tiles side by side leave a ring of six stages or more
+    if (long_ranges && h->table.d16 <= 128) return launch_nh<BN, KIND, 2>(h, B, b, true, s);
   }
-  if (tc_key_tile(h->dpad) == 256)
-    launch<256>(h, B, qpad, kappa, best, s);
-  else
-    launch<128>(h, B, qpad, kappa, best, s);
-  return LIPCACHE_PROBE_TENSOR_SINGLE;
+  launch_nh<BN, KIND, 1>(h, B, b, long_ranges, s);
 }
 
-int launch_probe_tc(lipcache* h, int64_t B, int path, cudaStream_t s) {
-  return launch_probe_tc_external(h, B, path, h->qpad, h->kappa, h->best, s);
+}  // namespace
+
+// Rows of 128-byte boxes: FP32 rows of d_pad, or FP16 rows of d16 features.
+void encode_screen_map(lipcache* h, CUtensorMap* map, const void* base, uint64_t rows, uint32_t box_rows, bool f16) {
+  LC_REQUIRE(h->encode != nullptr, LIPCACHE_E_CUDA, "cuTensorMapEncodeTiled is unavailable from the driver");
+  const cuuint64_t width = f16 ? (cuuint64_t)h->table.d16 : (cuuint64_t)h->dpad;
+  const cuuint64_t dims[2] = {width, (cuuint64_t)rows};
+  const cuuint64_t strides[1] = {width * (f16 ? sizeof(__half) : sizeof(float))};
+  const cuuint32_t box[2] = {f16 ? 64u : 32u, box_rows};
+  const cuuint32_t estr[2] = {1, 1};
+  const CUresult r = h->encode(map, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
+                               const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  LC_REQUIRE(r == CUDA_SUCCESS, LIPCACHE_E_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
+}
+
+int launch_probe_tc(lipcache* h, int64_t B, int path, bool f16, const ProbeBuffers& b, cudaStream_t s) {
+  LC_REQUIRE(f16 || tensor_path_supported(h->dpad), LIPCACHE_E_INVALID, "the tensor probe supports d <= 256");
+  // A 256-key tile of up to four chunks (d <= 256 in FP16, 128 in TF32) stays
+  // beside a deep query ring: single-CTA MMAs on all SMs. Longer rows would
+  // force 128-key tiles, whose MMAs read shared memory at its whole bandwidth;
+  // pair MMAs read a third less per flop and take those (clusters of four
+  // leave some SMs idle).
+  const bool short_rows = f16 ? h->table.d16 <= 256 : h->dpad <= 128;
+  const bool pair = path == LIPCACHE_PROBE_TENSOR_PAIR || (path == LIPCACHE_PROBE_TENSOR && !short_rows);
+  if (pair && probe_pair_clusters(h, f16) >= 1) {
+    launch_probe_pair(h, B, f16, b, s);
+    return LIPCACHE_PROBE_TENSOR_PAIR;
+  }
+  if (f16) {
+    if (short_rows)
+      launch<256, kF16>(h, B, b, s);
+    else
+      launch<128, kF16>(h, B, b, s);
+  } else {
+    if (short_rows)
+      launch<256, kTf32>(h, B, b, s);
+    else
+      launch<128, kTf32>(h, B, b, s);
+  }
+  return LIPCACHE_PROBE_TENSOR_SINGLE;
 }
 
 }  // namespace lc

@@ -20,6 +20,7 @@
 // candidate is always exactly covered; pairs within ~2e-6 relative of a
 // radius may be judged "not covered" where exact arithmetic says "covered".
 #include "internal.cuh"
+#include "key16.cuh"
 #include "probe_common.cuh"
 
 namespace lc {
@@ -199,6 +200,8 @@ __global__ void __launch_bounds__(32) k_sel_resolve(ResolveArgs a) {
   }
 }
 
+constexpr int kTailBlocks = 8;  // blocks of a scatter that clear the rows past the new end
+
 struct SelScatterArgs {
   const int32_t* list;
   const int32_t* n_list;
@@ -214,18 +217,26 @@ struct SelScatterArgs {
   const int32_t* yG;
   Table t;
   int64_t* out_index;
+  int64_t* unfit;
 };
 
 // Append the kept members in order; one warp per member.
 __global__ void k_sel_scatter(SelScatterArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int q = blockIdx.x * 8 + warp;
+  if (blockIdx.x < kTailBlocks) {
+    zero_tail(a.t, a.dpad, a.size0 + *a.n_list, (int)(blockIdx.x * 256 + threadIdx.x), kTailBlocks * 256);
+    return;
+  }
+  const int q = (blockIdx.x - kTailBlocks) * 8 + warp;
   if (q >= *a.n_list) return;
   const int p = a.list[q];
   const int32_t row = a.rows[p];
   const int64_t dst = a.size0 + q;
   float* kd = a.t.keys + (size_t)dst * a.dpad;
   for (int j = lane; j < a.dpad; j += 32) kd[j] = j < a.d ? a.G[(size_t)p * a.d + j] : 0.f;
+  if (a.t.keys16 && !store_key16(a.G + (size_t)p * a.d, a.d, a.t.keys16 + (size_t)dst * a.t.d16, a.t.d16, lane) &&
+      lane == 0)
+    atomicAdd(reinterpret_cast<unsigned long long*>(a.unfit), 1ull);
   if (lane == 0) {
     a.t.rr[dst] = a.rr[row];
     a.t.tau[dst] = a.tau[row];
@@ -364,14 +375,21 @@ __global__ void k_kc_scatter(const int32_t* __restrict__ seg, const int32_t* __r
                              int d, int dpad, int64_t size0, const float* __restrict__ rr, const float* __restrict__ tau,
                              const float* __restrict__ kn, const float* __restrict__ radius,
                              const int32_t* __restrict__ label, const int32_t* __restrict__ yG, Table t,
-                             int64_t* __restrict__ out_index) {
+                             int64_t* __restrict__ out_index, int64_t* __restrict__ unfit,
+                             const int64_t* __restrict__ total, int C) {
   const int c = blockIdx.y;
+  if (c == C) {  // one more row of blocks clears the rows past the new end
+    zero_tail(t, dpad, size0 + *total, (int)(blockIdx.x * 256 + threadIdx.x), (int)gridDim.x * 256);
+    return;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int q = blockIdx.x * 8 + warp; q < cnt[c]; q += gridDim.x * 8) {
     const int32_t row = out[seg[2 * c] + q];
     const int64_t dst = size0 + off[c] + q;
     float* kd = t.keys + (size_t)dst * dpad;
     for (int j = lane; j < dpad; j += 32) kd[j] = j < d ? H[(size_t)row * d + j] : 0.f;
+    if (t.keys16 && !store_key16(H + (size_t)row * d, d, t.keys16 + (size_t)dst * t.d16, t.d16, lane) && lane == 0)
+      atomicAdd(reinterpret_cast<unsigned long long*>(unfit), 1ull);
     if (lane == 0) {
       t.rr[dst] = rr[row];
       t.tau[dst] = tau[row];
@@ -500,9 +518,11 @@ int64_t select_insert(lipcache* h, const float* H, int64_t n, const int32_t* pay
     sa.yG = h->ins_yG;
     sa.t = h->table;
     sa.out_index = out_index;
-    k_sel_scatter<<<(unsigned)((kc + 7) / 8), 256, 0, s>>>(sa);
+    sa.unfit = &h->report->unfit;
+    k_sel_scatter<<<(unsigned)(kTailBlocks + (kc + 7) / 8), 256, 0, s>>>(sa);
     LC_LAUNCH_CHECK("k_sel_scatter");
     LC_CUDA(cudaMemcpyAsync(x.small_host + 2, x.small + 2, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    fetch_report(h, s);  // (the next chunk's probe: whether the FP16 copies still serve)
     LC_CUDA(cudaStreamSynchronize(s));
     const int64_t got = (int64_t)(int32_t)(x.small_host[2] & 0xFFFFFFFFll);
     h->size += got;
@@ -563,9 +583,9 @@ int64_t select_kcenter(lipcache* h, const float* H, int64_t n, const int32_t* pa
   k_kc_scan<<<1, 1024, 0, s>>>(cnt, C, off, x.small + 1);
   LC_LAUNCH_CHECK("k_kc_scan");
   const int per = budget_per_class;
-  k_kc_scatter<<<dim3((unsigned)((per + 7) / 8 < 64 ? (per + 7) / 8 : 64), (unsigned)C), 256, 0, s>>>(
+  k_kc_scatter<<<dim3((unsigned)((per + 7) / 8 < 64 ? (per + 7) / 8 : 64), (unsigned)(C + 1)), 256, 0, s>>>(
       seg, cnt, off, x.rows, H, h->d, h->dpad, h->size, h->ins_rr, h->ins_tau, h->ins_kn, h->ins_radius,
-      h->ins_label, h->ins_yG, h->table, out_index);
+      h->ins_label, h->ins_yG, h->table, out_index, &h->report->unfit, x.small + 1, C);
   LC_LAUNCH_CHECK("k_kc_scatter");
   LC_CUDA(cudaMemcpyAsync(x.small_host + 1, x.small + 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   LC_CUDA(cudaStreamSynchronize(s));

@@ -1,0 +1,186 @@
+"""The FP16 screen of the tensor probe against the exact kernel, bit for bit:
+widths around its 64-feature chunks and 16-feature MMA steps, alignments,
+every way a table grows, and what falls back to TF32 (pytest -m gpu)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import __graft_entry__
+    __graft_entry__.build()
+    return torch.device("cuda", 0)
+
+
+def make(dev, d, C, rows, scale=1.0, capacity=None):
+    from paper_2608_13144_gb300.lipcache import LipCache
+    rng = np.random.default_rng(d * 31 + C)
+    W = (rng.standard_normal((C, d)) / np.sqrt(d)).astype(np.float32) / np.float32(scale)
+    c = LipCache(d, C, capacity or len(rows), "tight", device=dev)
+    c.set_head(torch.from_numpy(W).to(dev), torch.zeros(C, device=dev))
+    return c
+
+
+def same_as_exact(c, Q, paths, need_hits=True):
+    c.set_probe_path("exact")
+    ref = [t.cpu().numpy() for t in c.probe(Q)]
+    if need_hits:
+        assert (ref[0] >= 0).any() and (Q.shape[1] == 1 or (ref[0] < 0).any())
+    for path in paths:
+        c.set_probe_path(path)
+        got = [t.cpu().numpy() for t in c.probe(Q)]
+        assert c.info()["device_errors"] == 0
+        for x, y in zip(ref, got):
+            assert np.array_equal(x.view(np.uint8), y.view(np.uint8)), path
+    return ref
+
+
+def data(rng, n, d, nq, noise=0.01):
+    rows = rng.standard_normal((n, d)).astype(np.float32)
+    Q = rng.standard_normal((nq, d)).astype(np.float32)
+    dup = rng.random(nq) < 0.5
+    Q[dup] = rows[rng.integers(0, n, dup.sum())] + noise * rng.standard_normal((dup.sum(), d)).astype(np.float32)
+    return rows, Q
+
+
+@pytest.mark.parametrize("d", [1, 15, 16, 17, 63, 64, 65, 80, 128, 129, 192, 250, 256])
+def test_widths(dev, d):
+    rng = np.random.default_rng(d)
+    rows, Q = data(rng, 3001, d, 257)
+    c = make(dev, d, 5, rows)
+    c.insert(torch.from_numpy(rows).to(dev))
+    paths = ["tensor", "tensor_single", "tensor_pair"]
+    same_as_exact(c, torch.from_numpy(Q).to(dev), paths)
+    # a batch that is not 16-byte aligned: the recheck reads it in place
+    buf = torch.zeros(Q.size + 1, device=dev)
+    buf[1:] = torch.from_numpy(Q.reshape(-1))
+    same_as_exact(c, buf[1:].view(Q.shape), paths)
+    c.close()
+
+
+@pytest.mark.parametrize("d,n,nq", [(257, 9001, 129), (300, 40000, 64), (448, 20001, 300), (449, 20001, 300),
+                                    (512, 30000, 1000)])
+def test_wide_auto(dev, d, n, nq):
+    """d in (256, 512]: "auto" screens in FP16 from 2^24 multiply-adds on; the
+    named tensor paths stay refused."""
+    from paper_2608_13144_gb300 import LipCacheError
+    rng = np.random.default_rng(d + n)
+    rows, Q = data(rng, n, d, nq)
+    c = make(dev, d, 4, rows)
+    c.insert(torch.from_numpy(rows).to(dev))
+    same_as_exact(c, torch.from_numpy(Q).to(dev), ["auto"])
+    assert c.info()["last_probe_path"] in (3, 4)
+    with pytest.raises(LipCacheError):
+        c.set_probe_path("tensor")
+    c.close()
+
+
+@pytest.mark.parametrize("n,nq", [(40, 1), (255, 128), (256, 129), (513, 4096), (200_000, 1025)])
+def test_sizes(dev, n, nq):
+    """One tile, an odd last tile, ragged queries, long ranges (stages released
+    in pairs with one chunk per tile)."""
+    rng = np.random.default_rng(n)
+    rows, Q = data(rng, n, 48, nq)
+    c = make(dev, 48, 5, rows)
+    c.insert(torch.from_numpy(rows).to(dev))
+    same_as_exact(c, torch.from_numpy(Q).to(dev), ["tensor", "tensor_pair"], need_hits=n > 1000)
+    c.close()
+
+
+@pytest.mark.parametrize("grow", ["unaligned", "async", "select", "kcenter", "writeback"])
+@pytest.mark.parametrize("d", [33, 96])
+def test_growth(dev, grow, d):
+    """Every path that appends entries writes their FP16 copies."""
+    rng = np.random.default_rng(d)
+    rows, Q = data(rng, 3000, d, 500)
+    c = make(dev, d, 6, rows)
+    R = torch.from_numpy(rows).to(dev)
+    if grow == "unaligned":
+        buf = torch.zeros(rows.size + 1, device=dev)
+        buf[1:] = R.reshape(-1)
+        c.insert(buf[1:].view(rows.shape))
+    elif grow == "async":
+        for k in range(0, 3000, 700):
+            c.insert(R[k:k + 700], wait=False)
+    elif grow == "select":
+        c.insert_select(R, strategy="radius_dedup", budget_total=2500)
+    elif grow == "kcenter":
+        c.insert_select(R, strategy="kcenter", budget_per_class=300)
+    else:
+        c.insert(R[:1000])
+        c.probe_writeback(R[1000:])
+    same_as_exact(c, torch.from_numpy(Q).to(dev), ["tensor", "tensor_pair"])
+    c.close()
+
+
+@pytest.mark.parametrize("n", [1, 255, 256, 257, 700])
+@pytest.mark.parametrize("how", ["insert", "select", "kcenter"])
+def test_rows_past_the_end(dev, how, n):
+    """The table's memory is not cleared at creation: the rows past the last
+    entry of its tile are zero because appending entries clears them, so
+    memory full of infinities (as FP16 and as FP32) left by another owner
+    neither reaches a result nor makes candidates of the pairs with it."""
+    from paper_2608_13144_gb300.lipcache import LipCache
+    junk = [torch.full((64, 1024, 1024), torch.inf, device=dev) for _ in range(4)]
+    del junk
+    torch.cuda.empty_cache()  # the next allocations may get this memory
+    rng = np.random.default_rng(n)
+    rows, Q = data(rng, n, 32, 300)
+    c = LipCache(32, 4, 200_000, "tight", device=dev)
+    c.set_head(torch.from_numpy((rng.standard_normal((4, 32)) / 6).astype(np.float32)).to(dev), torch.zeros(4, device=dev))
+    R = torch.from_numpy(rows).to(dev)
+    if how == "insert":
+        c.insert(R)
+    else:
+        c.insert_select(R, strategy="radius_dedup" if how == "select" else "kcenter",
+                        budget_per_class=0 if how == "select" else 400)
+    Qd = torch.from_numpy(Q).to(dev)
+    same_as_exact(c, Qd, ["tensor", "tensor_pair"], need_hits=False)
+    c.set_probe_path("tensor")
+    c.reset_stats()
+    c.probe(Qd)
+    # no more rechecked pairs than near-duplicates and a few close ones
+    assert c.info()["candidates"] <= 300 * 40
+    c.close()
+
+
+@pytest.mark.parametrize("what", ["large", "small", "mixed"])
+def test_unfit_tables(dev, what):
+    """Entries FP16 does not hold (overflow, the subnormal range): the table is
+    screened in TF32, with the same results; a fitting cache beside it is not
+    affected."""
+    rng = np.random.default_rng(3)
+    rows, Q = data(rng, 2000, 64, 300)
+    if what == "large":
+        rows, Q = rows * np.float32(1e5), Q * np.float32(1e5)
+    elif what == "small":
+        rows, Q = rows * np.float32(1e-6), Q * np.float32(1e-6)
+    c = make(dev, 64, 5, rows, capacity=2001)
+    c.insert(torch.from_numpy(rows).to(dev))
+    if what == "mixed":
+        c.insert(torch.full((1, 64), 7e4, device=dev))
+        c.insert(torch.from_numpy(rows[:0]).to(dev))
+    same_as_exact(c, torch.from_numpy(Q).to(dev), ["tensor", "tensor_pair"])
+    c.close()
+
+
+def test_extreme_queries(dev):
+    """Queries of any magnitude are scaled into FP16's range by the prologue;
+    NaN and infinite ones miss; a zero query gets the exact kernel's answer."""
+    rng = np.random.default_rng(9)
+    rows, Q = data(rng, 3000, 40, 400)
+    for k, s in enumerate([1e30, 1e-30, 1e-38, 1e-42, 1e5, 1e-6, 0.0]):
+        Q[k] *= np.float32(s)
+    Q[10, 3], Q[11, 0], Q[12] = np.nan, np.inf, -np.inf
+    Q[13, 1:] *= np.float32(1e-8)
+    rows[0] = 0  # near the tiny queries
+    c = make(dev, 40, 5, rows)
+    c.insert(torch.from_numpy(rows).to(dev))
+    ref = same_as_exact(c, torch.from_numpy(Q).to(dev), ["tensor", "tensor_pair"])
+    assert np.all(ref[0][10:13] == -1)
+    c.close()

@@ -540,3 +540,37 @@ def test_dot2_factor_is_tighter_than_the_sequential_bound():
     assert g8 * 50 < 2 * gamma32(168) ** 2
     # one lane over every feature: about (d u)^2
     assert dot2_factor(128, 1) > (128 * U32) ** 2
+
+
+@pytest.mark.parametrize("d", [16, 128, 512])
+@pytest.mark.parametrize("kind", ["normal", "ones_ulp", "wide", "tiny_tail"])
+def test_fp16_screen_error_within_half_of_c(d, kind):
+    """The FP16 screen's operand error, with keys that pass the fit test and
+    queries scaled to [1, 2) by a power of two, emulated in FP64: below
+    2^-10 (1 + 2^-6) ||q|| ||k||, about half of the bound c_screen the
+    thresholds are built with (c = 2 (2^-9 + ...)), and not above TF32's bound."""
+    rng = np.random.default_rng(d)
+    q = rng.standard_normal((64, d))
+    k = rng.standard_normal((64, d))
+    if kind == "ones_ulp":  # worst-case mantissas: just past a rounding boundary, products of one sign
+        q = np.full((64, d), 1 + 2.0 ** -11 * (1 + 2.0 ** -10)) * 2.0 ** rng.integers(-3, 4, (64, d))
+        k = q.copy()
+    elif kind == "wide":
+        q *= 10.0 ** rng.uniform(-3, 3, (64, 1))
+        k *= 10.0 ** rng.uniform(-2, 3, (64, 1))
+    elif kind == "tiny_tail":
+        q[:, d // 2:] *= 1e-9
+        k[:, d // 2:] *= 1e-9
+    q, k = q.astype(np.float32), k.astype(np.float32)
+    e = np.floor(np.log2(np.abs(q).max(axis=1, keepdims=True)))
+    q16 = (q * np.exp2(-e).astype(np.float32)).astype(np.float16).astype(np.float64) * np.exp2(e)
+    k16 = k.astype(np.float16).astype(np.float64)
+    q64, k64 = q.astype(np.float64), k.astype(np.float64)
+    n2, e2 = (k64 ** 2).sum(1), ((k64 - k16) ** 2).sum(1)
+    assert np.all(e2 <= 2.4214e-7 * n2)  # these keys fit
+    err = np.abs(q16 @ k16.T - q64 @ k64.T)
+    norms = np.linalg.norm(q64, axis=1)[:, None] * np.linalg.norm(k64, axis=1)[None, :]
+    bound = 2.0 ** -10 * (1 + 2.0 ** -6)
+    assert np.all(err <= bound * norms)
+    c = 2 * (2.0 ** -9 + 2.0 ** -20 + d * 2.0 ** -22)
+    assert bound + d * 2.0 ** -22 <= 0.55 * c

@@ -5,7 +5,9 @@
 
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
+#include <vector>
 
 #include "internal.cuh"
 
@@ -56,9 +58,56 @@ void sync_size(lipcache* h) {
   lc::settle_size(h);
 }
 
-template <typename T>
-void dev_alloc(T*& p, size_t n) {
-  LC_CUDA(cudaMalloc(&p, sizeof(T) * (n ? n : 1)));
+// Pinned host blocks for the handles' reports. Pinning and unpinning a page
+// costs ~280 us, a quarter of building and dropping a 2,000-row cache, so the
+// blocks are cut from 4 KB pages shared by the process's handles: a page goes
+// back to the driver when its last block does, except one, which is kept.
+constexpr size_t kPinBlock = 256, kPinPage = 4096;
+struct PinPage {
+  unsigned char* base;
+  uint32_t used;  // bit per block
+};
+std::mutex g_pin_mu;
+std::vector<PinPage> g_pin_pages;
+
+unsigned char* pin_take() {
+  std::lock_guard<std::mutex> lock(g_pin_mu);
+  constexpr uint32_t kAll = (1u << (kPinPage / kPinBlock)) - 1u;
+  for (size_t p = 0; p < g_pin_pages.size(); ++p) {
+    PinPage& pg = g_pin_pages[p];
+    if (pg.used == kAll) continue;
+    // (a page does not survive a reset of the device)
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, pg.base) != cudaSuccess || at.type != cudaMemoryTypeHost) {
+      cudaGetLastError();
+      if (pg.used == 0) g_pin_pages.erase(g_pin_pages.begin() + (ptrdiff_t)p--);
+      continue;
+    }
+    int b = 0;
+    while ((pg.used >> b) & 1u) ++b;
+    pg.used |= 1u << b;
+    return pg.base + b * kPinBlock;
+  }
+  g_pin_pages.reserve(g_pin_pages.size() + 1);
+  unsigned char* base = nullptr;
+  LC_CUDA(cudaHostAlloc(&base, kPinPage, cudaHostAllocPortable));
+  g_pin_pages.push_back(PinPage{base, 1u});
+  return base;
+}
+
+void pin_give(unsigned char* block) {
+  if (!block) return;
+  std::lock_guard<std::mutex> lock(g_pin_mu);
+  for (size_t p = 0; p < g_pin_pages.size(); ++p) {
+    PinPage& pg = g_pin_pages[p];
+    if (block < pg.base || block >= pg.base + kPinPage) continue;
+    pg.used &= ~(1u << ((size_t)(block - pg.base) / kPinBlock));
+    if (pg.used == 0 && g_pin_pages.size() > 1) {
+      cudaFreeHost(pg.base);
+      g_pin_pages.erase(g_pin_pages.begin() + (ptrdiff_t)p);
+    }
+    return;
+  }
 }
 
 template <typename T>
@@ -72,19 +121,11 @@ void release(lipcache* h) {
   cudaSetDevice(h->device);
   // asynchronous inserts may still be writing the table
   if (h->size_pending) cudaStreamSynchronize(h->pending_stream);
-  dev_free(h->W);
+  dev_free(h->arena);
+  dev_free(h->ins_arena);
+  dev_free(h->q_arena);
+  pin_give(h->host_arena);
   dev_free(h->wt_prep);
-  dev_free(h->b);
-  dev_free(h->Wnorm32);
-  dev_free(h->pairnorm);
-  dev_free(h->inv_pairnorm);
-  dev_free(h->ipn_up32);
-  dev_free(h->ipn_dn32);
-  dev_free(h->ipn_min32);
-  dev_free(h->ipn_max32);
-  dev_free(h->spec_work);
-  dev_free(h->spec);
-  if (h->spec_host) cudaFreeHost(h->spec_host);
   lc::release_select(h);
   dev_free(h->rr_emp);
   dev_free(h->tau_emp);
@@ -92,36 +133,8 @@ void release(lipcache* h) {
   dev_free(h->rho32);
   dev_free(h->cls_sum);
   dev_free(h->cls_cnt);
-  dev_free(h->table.keys);
   dev_free(h->table.keys16);
-  dev_free(h->table.kn);
-  dev_free(h->table.tau);
-  dev_free(h->table.rr);
-  dev_free(h->table.radius);
-  dev_free(h->table.label);
-  dev_free(h->table.yG);
-  dev_free(h->ins_accept);
-  dev_free(h->ins_yG);
-  dev_free(h->ins_label);
-  dev_free(h->ins_radius);
-  dev_free(h->ins_rr);
-  dev_free(h->ins_kn);
-  dev_free(h->ins_tau);
-  dev_free(h->ins_rank);
-  dev_free(h->ins_fix);
-  dev_free(h->ins_bcount);
-  dev_free(h->ins_boffset);
-  dev_free(h->report);
-  dev_free(h->ins_size0);
-  if (h->report_host) cudaFreeHost(h->report_host);
-  dev_free(h->qpad);
-  dev_free(h->kappa);
-  dev_free(h->qscale);
-  dev_free(h->best);
-  dev_free(h->hq);
-  dev_free(h->hidx);
-  dev_free(h->hlabel);
-  dev_free(h->hdist);
+  dev_free(h->h_arena);
   for (int i = 0; i < lipcache::kTimingRing; ++i) {
     if (h->tev0[i]) cudaEventDestroy(h->tev0[i]);
     if (h->tev1[i]) cudaEventDestroy(h->tev1[i]);
@@ -199,55 +212,58 @@ LC_API lipcache_status lipcache_create(int32_t d, int32_t C, int64_t capacity, i
     h->radius_mode = radius_mode;
     h->eps_rc = lc::eps_recheck(h->dpad);
     h->c_scr = lc::c_screen(h->dpad);
-    dev_alloc(h->W, (size_t)C * d);
-    dev_alloc(h->b, (size_t)C);
-    dev_alloc(h->Wnorm32, (size_t)C);
-    if (radius_mode == LIPCACHE_RADIUS_TIGHT) {
-      dev_alloc(h->pairnorm, (size_t)C * C);
-      dev_alloc(h->inv_pairnorm, (size_t)C * C);
-      dev_alloc(h->ipn_up32, (size_t)C * C);
-      dev_alloc(h->ipn_dn32, (size_t)C * C);
-      dev_alloc(h->ipn_min32, (size_t)C);
-      dev_alloc(h->ipn_max32, (size_t)C);
-    }
-    dev_alloc(h->spec_work, lc::spectral_work_bytes(d, C));
-    dev_alloc(h->spec, 1);
-    LC_CUDA(cudaMallocHost(&h->spec_host, sizeof(lc::SpecResult)));
     // Whole key tiles: rows past the current size have the screen term tau
     // 0x7f7f7f7f (3.4e38), so no probe ever selects them; those of the last
     // tile are kept zero by whatever appends entries (key16.cuh, zero_tail),
     // so the keys themselves need no clearing here.
     h->table_rows = (capacity + 255) / 256 * 256;
     const size_t rows = (size_t)h->table_rows;
-    dev_alloc(h->table.keys, rows * h->dpad);
-    dev_alloc(h->table.kn, rows);
-    dev_alloc(h->table.tau, rows);
+    lc::carve_alloc(h->arena, [&](lc::Carve& c) {
+      c.take(h->table.keys, rows * h->dpad);
+      c.take(h->table.kn, rows);
+      c.take(h->table.tau, rows);
+      c.take(h->table.rr, rows);
+      c.take(h->table.radius, rows);
+      c.take(h->table.label, rows);
+      c.take(h->table.yG, rows);
+      c.take(h->report, 1);
+      c.take(h->ins_size0, 1);
+      c.take(h->spec, 1);
+      c.take(h->W, (size_t)C * d);
+      c.take(h->b, (size_t)C);
+      c.take(h->Wnorm32, (size_t)C);
+      if (radius_mode == LIPCACHE_RADIUS_TIGHT) {
+        c.take(h->pairnorm, (size_t)C * C);
+        c.take(h->inv_pairnorm, (size_t)C * C);
+        c.take(h->ipn_up32, (size_t)C * C);
+        c.take(h->ipn_dn32, (size_t)C * C);
+        c.take(h->ipn_min32, (size_t)C);
+        c.take(h->ipn_max32, (size_t)C);
+      }
+      c.take(h->spec_work, lc::spectral_work_bytes(d, C));
+    });
     LC_CUDA(cudaMemset(h->table.tau, 0x7f, sizeof(float) * rows));
-    dev_alloc(h->table.rr, rows);
     LC_CUDA(cudaMemset(h->table.rr, 0, sizeof(float) * rows));
-    dev_alloc(h->table.radius, rows);
-    dev_alloc(h->table.label, rows);
-    dev_alloc(h->table.yG, rows);
-    // The FP16 copy of the keys (d <= 512). A table whose copy does not fit
-    // the device's memory goes without and is screened in TF32.
+    LC_CUDA(cudaMemset(h->report, 0, sizeof(lc::DevReport)));
+    static_assert(sizeof(lc::DevReport) + sizeof(lc::SpecResult) <= kPinBlock, "one block holds both");
+    h->host_arena = pin_take();
+    std::memset(h->host_arena, 0, sizeof(lc::DevReport) + sizeof(lc::SpecResult));
+    h->report_host = reinterpret_cast<lc::DevReport*>(h->host_arena);
+    h->spec_host = reinterpret_cast<lc::SpecResult*>(h->host_arena + sizeof(lc::DevReport));
+    h->stats = &h->report->stats;
+    h->stats_host = &h->report_host->stats;
+    // The FP16 copy of the keys (d <= 512), last and only where it leaves room
+    // for scratch: a table without one is screened in TF32.
     if (d <= 512) {
       h->table.d16 = (d + 63) / 64 * 64;
       const size_t bytes = sizeof(__half) * rows * (size_t)h->table.d16;
-      if (cudaMalloc(&h->table.keys16, bytes) != cudaSuccess) {
+      constexpr size_t kGiB = size_t(1) << 30;
+      size_t avail = 0, all = 0;
+      if (bytes > 4 * kGiB) LC_CUDA(cudaMemGetInfo(&avail, &all));
+      if ((bytes > 4 * kGiB && avail < bytes + 8 * kGiB) || cudaMalloc(&h->table.keys16, bytes) != cudaSuccess) {
         cudaGetLastError();
         h->table.keys16 = nullptr;
       }
-    }
-    dev_alloc(h->report, 1);
-    LC_CUDA(cudaMemset(h->report, 0, sizeof(lc::DevReport)));
-    LC_CUDA(cudaMallocHost(&h->report_host, sizeof(lc::DevReport)));
-    std::memset(h->report_host, 0, sizeof(lc::DevReport));
-    h->stats = &h->report->stats;
-    h->stats_host = &h->report_host->stats;
-    dev_alloc(h->ins_size0, 1);
-    for (int i = 0; i < lipcache::kTimingRing; ++i) {
-      LC_CUDA(cudaEventCreate(&h->tev0[i]));
-      LC_CUDA(cudaEventCreate(&h->tev1[i]));
     }
     resolve_encoder(h);
     LC_CUDA(cudaDeviceSynchronize());
@@ -549,15 +565,13 @@ LC_API lipcache_status lipcache_probe_host(lipcache_t* h, const float* Q_host, i
     use_device(h);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (B > h->hq_cap) {
-      dev_free(h->hq);
-      dev_free(h->hidx);
-      dev_free(h->hlabel);
-      dev_free(h->hdist);
       h->hq_cap = 0;
-      dev_alloc(h->hq, (size_t)B * h->d);
-      dev_alloc(h->hidx, (size_t)B);
-      dev_alloc(h->hlabel, (size_t)B);
-      dev_alloc(h->hdist, (size_t)B);
+      lc::carve_alloc(h->h_arena, [&](lc::Carve& c) {
+        c.take(h->hq, (size_t)B * h->d);
+        c.take(h->hidx, (size_t)B);
+        c.take(h->hlabel, (size_t)B);
+        c.take(h->hdist, (size_t)B);
+      });
       h->hq_cap = B;
     }
     LC_CUDA(cudaMemcpyAsync(h->hq, Q_host, sizeof(float) * (size_t)B * h->d, cudaMemcpyHostToDevice, s));
@@ -614,6 +628,13 @@ LC_API lipcache_status lipcache_reserve(lipcache_t* h, int64_t max_batch) {
 LC_API lipcache_status lipcache_enable_timing(lipcache_t* h, int32_t on) {
   return guarded([&] {
     check_handle(h);
+    if (on && !h->tev1[lipcache::kTimingRing - 1]) {
+      use_device(h);
+      for (int i = 0; i < lipcache::kTimingRing; ++i) {
+        if (!h->tev0[i]) LC_CUDA(cudaEventCreate(&h->tev0[i]));
+        if (!h->tev1[i]) LC_CUDA(cudaEventCreate(&h->tev1[i]));
+      }
+    }
     h->timing = on != 0;
   });
 }

@@ -1591,29 +1591,25 @@ __global__ void __launch_bounds__(256) k_consistency(const int64_t* __restrict__
   }
 }
 
-template <typename T>
-void grow(T*& p, int64_t n) {
-  if (p) cudaFree(p);
-  p = nullptr;
-  LC_CUDA(cudaMalloc(&p, sizeof(T) * (size_t)(n > 0 ? n : 1)));
-}
-
 void ensure_insert_scratch(lipcache* h, int64_t n) {
   if (n <= h->ins_cap) return;
   int64_t cap = h->ins_cap ? h->ins_cap : 1024;
   while (cap < n) cap *= 2;
   const int64_t nb = (cap + kRows - 1) / kRows;
-  grow(h->ins_accept, cap);
-  grow(h->ins_yG, cap);
-  grow(h->ins_label, cap);
-  grow(h->ins_radius, cap);
-  grow(h->ins_rr, cap);
-  grow(h->ins_kn, cap);
-  grow(h->ins_tau, cap);
-  grow(h->ins_rank, cap);
-  grow(h->ins_fix, cap);
-  grow(h->ins_bcount, nb);
-  grow(h->ins_boffset, nb);
+  h->ins_cap = 0;
+  carve_alloc(h->ins_arena, [&](Carve& c) {
+    c.take(h->ins_accept, cap);
+    c.take(h->ins_yG, cap);
+    c.take(h->ins_label, cap);
+    c.take(h->ins_radius, cap);
+    c.take(h->ins_rr, cap);
+    c.take(h->ins_kn, cap);
+    c.take(h->ins_tau, cap);
+    c.take(h->ins_rank, cap);
+    c.take(h->ins_fix, cap);
+    c.take(h->ins_bcount, nb);
+    c.take(h->ins_boffset, nb);
+  });
   h->ins_cap = cap;
 }
 

@@ -40,6 +40,34 @@ struct Error : std::runtime_error {
     if (!(cond)) throw ::lc::Error((status), (msg)); \
   } while (0)
 
+// ---------------------------------------------------------------- memory
+// Lays several arrays out in one allocation (a cudaMalloc or cudaFree costs
+// microseconds whatever its size). With a null base only `off`, the bytes
+// needed, comes out.
+struct Carve {
+  unsigned char* base = nullptr;
+  size_t off = 0;
+  template <typename T>
+  void take(T*& p, size_t n) {
+    off = (off + 255) / 256 * 256;
+    p = base ? reinterpret_cast<T*>(base + off) : nullptr;
+    off += sizeof(T) * (n ? n : 1);
+  }
+};
+// (Re)allocates `arena` for the arrays that `layout` takes; the old contents
+// are lost. On failure everything is null.
+template <typename F>
+void carve_alloc(unsigned char*& arena, F&& layout) {
+  if (arena) cudaFree(arena);
+  arena = nullptr;
+  Carve c;
+  layout(c);
+  const size_t bytes = c.off;
+  LC_CUDA(cudaMalloc(&arena, bytes));
+  c = Carve{arena, 0};
+  layout(c);
+}
+
 // ---------------------------------------------------------------- numerics
 // Unit roundoff of FP32 and FP64 (round to nearest).
 constexpr double kU32 = 5.9604644775390625e-08;   // 2^-24
@@ -200,6 +228,12 @@ struct lipcache {
   lc::SpecResult* spec = nullptr;        // device
   lc::SpecResult* spec_host = nullptr;   // pinned
 
+  unsigned char* arena = nullptr;       // the table (but its FP16 copy), the head's arrays above, the report, ins_size0
+  unsigned char* ins_arena = nullptr;   // insert scratch
+  unsigned char* q_arena = nullptr;     // probe scratch
+  unsigned char* h_arena = nullptr;     // host-buffer probe staging
+  unsigned char* host_arena = nullptr;  // pinned: report_host, spec_host
+
   lc::Table table;
 
   // insert scratch (grows)
@@ -245,7 +279,7 @@ struct lipcache {
   // main-kernel timing: a ring of event pairs harvested lazily
   static constexpr int kTimingRing = 64;
   bool timing = false;
-  cudaEvent_t tev0[kTimingRing] = {}, tev1[kTimingRing] = {};
+  cudaEvent_t tev0[kTimingRing] = {}, tev1[kTimingRing] = {};  // created when timing is first enabled
   int64_t t_issued = 0, t_harvested = 0;
   double t_ms_total = 0.0;
   int64_t t_count = 0;

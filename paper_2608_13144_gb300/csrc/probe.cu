@@ -208,19 +208,13 @@ void ensure_probe_scratch(lipcache* h, int64_t Bpad) {
   if (Bpad <= h->q_cap) return;
   int64_t cap = h->q_cap ? h->q_cap : 1024;
   while (cap < Bpad) cap *= 2;
-  if (h->qpad) cudaFree(h->qpad);
-  if (h->kappa) cudaFree(h->kappa);
-  if (h->qscale) cudaFree(h->qscale);
-  if (h->best) cudaFree(h->best);
-  h->qpad = nullptr;
-  h->kappa = nullptr;
-  h->qscale = nullptr;
-  h->best = nullptr;
   h->q_cap = 0;
-  LC_CUDA(cudaMalloc(&h->qpad, sizeof(float) * (size_t)cap * h->dpad));
-  LC_CUDA(cudaMalloc(&h->kappa, sizeof(float) * (size_t)cap));
-  LC_CUDA(cudaMalloc(&h->qscale, sizeof(float) * (size_t)cap));
-  LC_CUDA(cudaMalloc(&h->best, sizeof(unsigned long long) * (size_t)cap));
+  carve_alloc(h->q_arena, [&](Carve& c) {
+    c.take(h->qpad, (size_t)cap * h->dpad);
+    c.take(h->kappa, (size_t)cap);
+    c.take(h->qscale, (size_t)cap);
+    c.take(h->best, (size_t)cap);
+  });
   h->q_cap = cap;
 }
 

@@ -245,11 +245,12 @@ LC_API lipcache_status lipcache_create(int32_t d, int32_t C, int64_t capacity, i
     LC_CUDA(cudaMemset(h->table.tau, 0x7f, sizeof(float) * rows));
     LC_CUDA(cudaMemset(h->table.rr, 0, sizeof(float) * rows));
     LC_CUDA(cudaMemset(h->report, 0, sizeof(lc::DevReport)));
-    static_assert(sizeof(lc::DevReport) + sizeof(lc::SpecResult) <= kPinBlock, "one block holds both");
+    static_assert(sizeof(lc::DevReport) + sizeof(lc::SpecResult) + 64 <= kPinBlock, "one block holds all three");
     h->host_arena = pin_take();
-    std::memset(h->host_arena, 0, sizeof(lc::DevReport) + sizeof(lc::SpecResult));
+    std::memset(h->host_arena, 0, kPinBlock);
     h->report_host = reinterpret_cast<lc::DevReport*>(h->host_arena);
     h->spec_host = reinterpret_cast<lc::SpecResult*>(h->host_arena + sizeof(lc::DevReport));
+    h->sel_host = h->host_arena + kPinBlock - 64;
     h->stats = &h->report->stats;
     h->stats_host = &h->report_host->stats;
     // The FP16 copy of the keys (d <= 512), last and only where it leaves room

@@ -159,24 +159,24 @@ struct DevReport {
 
 // Scratch of the selection strategy (select.cu), grown on demand.
 struct SelectScratch {
+  // one allocation: a chunk's arrays, the per-class counts and the counters
+  unsigned char* chunk = nullptr;
+  float* G = nullptr;  // chunk members' features
+  int32_t* rows = nullptr;
+  int64_t* hit = nullptr;
+  uint32_t* cov = nullptr;
+  int32_t* list = nullptr;
+  int32_t* class_cnt = nullptr;
+  unsigned char* state = nullptr;  // 64 bytes; read back into lipcache::sel_host
   unsigned long long* keys = nullptr;
   int64_t keys_cap = 0;
-  float* G = nullptr;  // chunk members' features
-  int64_t G_cap = 0;
-  int32_t* rows = nullptr;
-  int64_t rows_cap = 0;
-  int64_t* hit = nullptr;
-  int64_t hit_cap = 0;
-  uint32_t* cov = nullptr;
-  int64_t cov_cap = 0;
-  int32_t* list = nullptr;
-  int64_t list_cap = 0;
-  int32_t* class_cnt = nullptr;
-  int64_t class_cap = 0;
-  float* kc_mind = nullptr;  // K-center: squared distance to the nearest centre
+  // K-center: squared distance to the nearest centre, class segments and counts, chosen rows
+  float* kc_mind = nullptr;
   int64_t kc_mind_cap = 0;
-  int64_t* small = nullptr;       // device: accepted, kept, chunk count
-  int64_t* small_host = nullptr;  // pinned
+  int32_t* kc_seg = nullptr;
+  int64_t kc_seg_cap = 0;
+  int32_t* kc_rows = nullptr;
+  int64_t kc_rows_cap = 0;
 };
 
 // Per-entry table of the cache (structure of arrays, capacity entries).
@@ -232,7 +232,7 @@ struct lipcache {
   unsigned char* ins_arena = nullptr;   // insert scratch
   unsigned char* q_arena = nullptr;     // probe scratch
   unsigned char* h_arena = nullptr;     // host-buffer probe staging
-  unsigned char* host_arena = nullptr;  // pinned: report_host, spec_host
+  unsigned char* host_arena = nullptr;  // pinned: report_host, spec_host, sel_host
 
   lc::Table table;
 
@@ -312,6 +312,7 @@ struct lipcache {
   size_t wt_prep_cap = 0;      // bytes allocated
   int wt_prep_ncg = 0;         // classes per thread it was laid out for (0: stale)
   lc::SelectScratch sel;
+  unsigned char* sel_host = nullptr;  // pinned, 64 bytes: the selection's counters
 
   // radius policy (Sec. 5.4): the probe reads rr_emp / tau_emp instead of
   // the certified thresholds when policy != LIPCACHE_POLICY_CERTIFIED

@@ -10,12 +10,13 @@
 // has used its budget. Kept entries are appended in visiting order.
 //
 // GPU schedule. The order is a bitonic sort of 64-bit keys (radius bits
-// descending, row ascending). Candidates are then processed in chunks of
-// kSelChunk in that order: the chunk is probed against the cache as it stands
-// (a hit = covered by an earlier entry), its pairwise coverage by earlier
-// members of the same chunk is computed as a bit matrix (canonical FP32
+// descending, row ascending). Candidates are then processed in chunks of up to
+// kSelChunk in that order, leaving out those whose class has used its budget
+// before the chunk (they cannot be kept): the chunk is probed against the cache
+// as it stands (a hit = covered by an earlier entry), its pairwise coverage by
+// earlier members of the same chunk is computed as a bit matrix (canonical FP32
 // distance against the member's acceptance threshold rr, the probe's test),
-// one warp resolves the chunk sequentially, and the kept members are
+// one block resolves the chunk 32 members at a time, and the kept members are
 // appended. Coverage uses the probe's conservative thresholds, so a skipped
 // candidate is always exactly covered; pairs within ~2e-6 relative of a
 // radius may be judged "not covered" where exact arithmetic says "covered".
@@ -45,75 +46,228 @@ __global__ void k_sel_keys(const uint8_t* __restrict__ accept, const float* __re
   if ((threadIdx.x & 31) == 0 && m) atomicAdd(reinterpret_cast<unsigned long long*>(n_acc), (unsigned long long)__popc(m));
 }
 
-// One compare-exchange pass of a bitonic sort (ascending) of npow keys.
-__global__ void k_bitonic(unsigned long long* __restrict__ a, int64_t npow, int64_t j, int64_t k) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= npow) return;
-  const int64_t x = i ^ j;
-  if (x > i) {
-    const unsigned long long ai = a[i], ax = a[x];
-    const bool up = (i & k) == 0;
-    if ((ai > ax) == up) {
-      a[i] = ax;
-      a[x] = ai;
-    }
+// Bitonic sort (ascending) of npow keys, a power of two. Spans of up to
+// kSortSpan keys are sorted, and the short-distance passes of longer merges
+// done, in shared memory: 65,536 keys take 15 launches instead of 136.
+constexpr int kSortSpan = 4096, kSortThreads = 1024;
+
+__device__ __forceinline__ void order_pair(unsigned long long& x, unsigned long long& y, bool up) {
+  if ((x > y) == up) {
+    const unsigned long long z = x;
+    x = y;
+    y = z;
   }
 }
 
-// Chunk members: rows in visiting order and their features (kc x d).
-__global__ void k_sel_gather(const unsigned long long* __restrict__ keys, int64_t c0, int kc, const float* __restrict__ H,
-                             int d, int32_t* __restrict__ rows, float* __restrict__ G) {
+// kmin == 2: sort every span; kmin = kmax > span: the passes j < span of the
+// merge k = kmax.
+__global__ void __launch_bounds__(kSortThreads) k_bitonic_span(unsigned long long* __restrict__ a, int span,
+                                                               int64_t kmin, int64_t kmax) {
+  __shared__ unsigned long long s[kSortSpan];
+  const int64_t base = (int64_t)blockIdx.x * span;
+  for (int i = threadIdx.x; i < span; i += kSortThreads) s[i] = a[base + i];
+  __syncthreads();
+  for (int64_t k = kmin; k <= kmax; k <<= 1)
+    for (int j = (int)((k < span ? k : span) >> 1); j > 0; j >>= 1) {
+      for (int p = threadIdx.x; p < span / 2; p += kSortThreads) {
+        const int i = 2 * p - (p & (j - 1));  // the p-th index with bit j clear
+        order_pair(s[i], s[i + j], ((base + i) & k) == 0);
+      }
+      __syncthreads();
+    }
+  for (int i = threadIdx.x; i < span; i += kSortThreads) a[base + i] = s[i];
+}
+
+// One pass (distance j >= kSortSpan) of the merge k.
+__global__ void __launch_bounds__(256) k_bitonic(unsigned long long* __restrict__ a, int64_t npow, int64_t j, int64_t k) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= npow / 2) return;
+  const int64_t i = 2 * p - (p & (j - 1));
+  unsigned long long x = a[i], y = a[i + j];
+  if ((x > y) == ((i & k) == 0)) {
+    a[i] = y;
+    a[i + j] = x;
+  }
+}
+
+void sort_keys(unsigned long long* a, int64_t npow, cudaStream_t s) {
+  const int span = npow < kSortSpan ? (int)npow : kSortSpan;
+  if (span < 2) return;
+  const unsigned blocks = (unsigned)(npow / span);
+  k_bitonic_span<<<blocks, kSortThreads, 0, s>>>(a, span, 2, span);
+  LC_LAUNCH_CHECK("k_bitonic_span");
+  for (int64_t k = 2 * (int64_t)span; k <= npow; k <<= 1) {
+    for (int64_t j = k >> 1; j >= span; j >>= 1) {
+      k_bitonic<<<(unsigned)((npow / 2 + 255) / 256), 256, 0, s>>>(a, npow, j, k);
+      LC_LAUNCH_CHECK("k_bitonic");
+    }
+    k_bitonic_span<<<blocks, kSortThreads, 0, s>>>(a, span, k, k);
+    LC_LAUNCH_CHECK("k_bitonic_span");
+  }
+}
+
+// Device counters of a selection.
+struct SelState {
+  long long n_acc;   // certified candidates
+  long long kept;    // kept by this call
+  long long cursor;  // first candidate, in visiting order, not yet in a chunk
+  int n_list;        // kept members of the current chunk
+  int kc;            // members of the next chunk
+};
+static_assert(sizeof(SelState) <= 64, "fits the host block's tail");
+
+// The next chunk: the first kSelChunk candidates from the cursor on whose class
+// still has budget, in order (one block; four candidates per thread a round).
+__global__ void __launch_bounds__(1024) k_sel_pick(const unsigned long long* __restrict__ keys,
+                                                   const int32_t* __restrict__ label,
+                                                   const int32_t* __restrict__ class_cnt, int C, int budget_pc,
+                                                   int32_t* __restrict__ rows, SelState* __restrict__ st) {
+  __shared__ int wsum[32];
+  __shared__ long long first_left;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const long long n = st->n_acc;
+  long long c = st->cursor;
+  int got = 0;
+  if (tid == 0) first_left = n;
+  while (c < n && got < kSelChunk) {
+    const long long c4 = c + 4 * (long long)tid;
+    int32_t row[4];
+    bool open[4];
+    int mine = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      row[u] = c4 + u < n ? (int32_t)(keys[c4 + u] & 0xFFFFFFFFull) : -1;
+      open[u] = row[u] >= 0;
+      if (open[u] && budget_pc > 0) {
+        const int32_t lab = label[row[u]];
+        open[u] = !(lab >= 0 && lab < C && class_cnt[lab] >= budget_pc);
+      }
+      mine += open[u] ? 1 : 0;
+    }
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+      int x = wsum[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      wsum[lane] = x;
+    }
+    __syncthreads();
+    int at = got + (warp ? wsum[warp - 1] : 0) + incl - mine;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (!open[u]) continue;
+      if (at < kSelChunk)
+        rows[at] = row[u];
+      else if (at == kSelChunk)
+        first_left = c4 + u;
+      ++at;
+    }
+    got += wsum[31];
+    c += 4 * 1024;
+    __syncthreads();
+  }
+  if (tid == 0) {
+    st->kc = got < kSelChunk ? got : kSelChunk;
+    st->cursor = got > kSelChunk ? first_left : (c < n ? c : n);
+  }
+}
+
+// The chunk members' features (kc x d).
+__global__ void k_sel_gather(const int32_t* __restrict__ rows, int kc, const float* __restrict__ H, int d,
+                             float* __restrict__ G) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int p = blockIdx.x * 8 + warp;
   if (p >= kc) return;
-  const int64_t row = (int64_t)(keys[c0 + p] & 0xFFFFFFFFull);
-  if (lane == 0) rows[p] = (int32_t)row;
+  const int64_t row = rows[p];
   for (int j = lane; j < d; j += 32) G[(size_t)p * d + j] = H[(size_t)row * d + j];
 }
 
 // Coverage inside the chunk: bit i of cov[j * kSelWords + i / 32] is set iff
 // i < j and member j lies inside member i's ball (canonical FP32 squared
-// distance below rr of member i). Block (ti, tj) computes the 32 x 32 tile of
-// members i in tile ti, j in tile tj (ti <= tj); warp w handles j = 4w..4w+3
-// of the tile, lane = i; the d features stream through shared memory in
-// 32-float chunks, which is the canonical summation order.
+// distance below rr of member i). Block (ti, tj), ti <= tj, computes the 64 x 64
+// tile of members i in tile ti, j in tile tj, 4 x 4 pairs per thread (the
+// layout of the exact probe: an eighth of the shared-memory reads per pair of
+// one pair per thread; bound by the FP32 pipe); the d features stream through
+// shared memory in 32-float chunks, which is the canonical summation order.
+constexpr int kCovT = 64, kCovS = kCovT + 4;
+
 __global__ void __launch_bounds__(256) k_sel_cover(const float* __restrict__ G, int d, int kc,
                                                    const int32_t* __restrict__ rows, const float* __restrict__ rr,
                                                    uint32_t* __restrict__ cov) {
   const int ti = blockIdx.x, tj = blockIdx.y;
   if (ti > tj) return;
-  __shared__ float zi[32][33], zj[32][33];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = ti * 32 + lane;
-  float total[4] = {0.f, 0.f, 0.f, 0.f};
+  __shared__ __align__(16) float zi[32][kCovS], zj[32][kCovS];
+  const int tid = threadIdx.x;
+  const int ci = tid & 15, cj = tid >> 4;  // members i: 4 ci .., j: 4 cj ..
+  const int lr = tid >> 2, lf = (tid & 3) * 8;  // loader: row, first of 8 features
+  float tot[4][4], p[4][4];
+#pragma unroll
+  for (int x = 0; x < 4; ++x)
+#pragma unroll
+    for (int y = 0; y < 4; ++y) tot[x][y] = 0.f;
   for (int c = 0; c < d; c += 32) {
-    for (int e = threadIdx.x; e < 32 * 32; e += 256) {
-      const int r = e >> 5, f = e & 31;
-      const int gi = ti * 32 + r, gj = tj * 32 + r;
-      zi[r][f] = (gi < kc && c + f < d) ? G[(size_t)gi * d + c + f] : 0.f;
-      zj[r][f] = (gj < kc && c + f < d) ? G[(size_t)gj * d + c + f] : 0.f;
+    {
+      const int gi = ti * kCovT + lr, gj = tj * kCovT + lr;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int f = c + lf + u;
+        zi[lf + u][lr] = (gi < kc && f < d) ? G[(size_t)gi * d + f] : 0.f;
+        zj[lf + u][lr] = (gj < kc && f < d) ? G[(size_t)gj * d + f] : 0.f;
+      }
     }
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int jl = warp * 4 + q;
-      float p = 0.f;
+    for (int x = 0; x < 4; ++x)
 #pragma unroll
-      for (int f = 0; f < 32; ++f) {
-        const float e = __fsub_rn(zj[jl][f], zi[lane][f]);
-        p = __fmaf_rn(e, e, p);
-      }
-      total[q] = __fadd_rn(total[q], p);
+      for (int y = 0; y < 4; ++y) p[x][y] = 0.f;
+#pragma unroll 8
+    for (int f = 0; f < 32; ++f) {
+      const float4 a4 = *reinterpret_cast<const float4*>(&zi[f][4 * ci]);
+      const float4 b4 = *reinterpret_cast<const float4*>(&zj[f][4 * cj]);
+      const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+          const float e = __fsub_rn(bv[y], av[x]);
+          p[x][y] = __fmaf_rn(e, e, p[x][y]);
+        }
     }
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+      for (int y = 0; y < 4; ++y) tot[x][y] = __fadd_rn(tot[x][y], p[x][y]);
     __syncthreads();
   }
-  const float thr = i < kc ? rr[rows[i]] : 0.f;
+  float thr[4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int j = tj * 32 + warp * 4 + q;
-    const bool bit = i < kc && j < kc && i < j && total[q] < thr;
-    const unsigned m = __ballot_sync(0xffffffffu, bit);
-    if (lane == 0 && j < kc) cov[(size_t)j * kSelWords + ti] = m;
+  for (int x = 0; x < 4; ++x) {
+    const int i = ti * kCovT + 4 * ci + x;
+    thr[x] = i < kc ? rr[rows[i]] : 0.f;
+  }
+  // the 16 threads of a half-warp hold the 64 bits of four rows j
+#pragma unroll
+  for (int y = 0; y < 4; ++y) {
+    const int j = tj * kCovT + 4 * cj + y;
+    uint32_t w = 0;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const int i = ti * kCovT + 4 * ci + x;
+      w |= (uint32_t)(i < kc && j < kc && i < j && tot[x][y] < thr[x]) << (4 * (ci & 7) + x);
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) w |= __shfl_xor_sync(0xffffffffu, w, o);
+    if ((ci & 7) == 0 && j < kc) cov[(size_t)j * kSelWords + 2 * ti + (ci >> 3)] = w;
   }
 }
 
@@ -123,80 +277,107 @@ struct ResolveArgs {
   const int64_t* hit;      // per member: cache index it hits, -1 if none
   const int32_t* label;    // per row (certify scratch)
   int32_t* class_cnt;      // per class, kept in this call
-  int64_t* kept_total;     // kept in this call
+  SelState* st;
   int32_t* list;           // kept members in order
-  int32_t* n_list;
   int kc, C, budget_pc;
-  int64_t budget_total;
+  long long budget_total;
 };
 
-// One warp walks the chunk in order; member j is kept iff it hits nothing in
-// the cache, no kept member i < j of the chunk covers it and its budgets
-// allow. Lane l holds the kept-set words l, l + 32, l + 64, l + 96. The
-// members' hit flags and labels are staged in shared memory first, and the
-// coverage rows are read kAhead members ahead of the decision.
-constexpr int kAhead = 8;
-
-__device__ __forceinline__ void load_cov_row(const uint32_t* __restrict__ cov, int j, int kc, int lane,
-                                             uint32_t (&w)[kSelWords / 32]) {
-#pragma unroll
-  for (int t = 0; t < kSelWords / 32; ++t) {
-    const int wi = lane + 32 * t;
-    w[t] = (j < kc && wi <= (j >> 5)) ? __ldcg(cov + (size_t)j * kSelWords + wi) : 0u;
-  }
-}
-
-__global__ void __launch_bounds__(32) k_sel_resolve(ResolveArgs a) {
-  __shared__ int32_t lab_s[kSelChunk];
+// The greedy pass over a chunk: member j is kept iff it hits nothing in the
+// cache, no kept member i < j of the chunk covers it and its budgets allow. One
+// block takes 32 members at a time: warp m tests member m of the group against
+// the members kept in earlier groups (its coverage row, read one group ahead,
+// against the kept-set words in shared memory); warp 0 then settles the group
+// in batches: the undecided members before the first one that another
+// undecided member covers are independent, so each is kept unless its class or
+// the call runs out of budget before it (ranks by ballot); what they cover
+// drops out. Labels, hits and class counts are in shared memory. Bound by the
+// chain of groups, ~1,200 cycles each on a pool where a third of the members
+// are near-duplicates; one warp walking the members took 160 ns for each
+// (4,096 members: 80 us, before 665 us).
+__global__ void __launch_bounds__(1024) k_sel_resolve(ResolveArgs a) {
+  constexpr int kPer = kSelWords / 32;
+  __shared__ uint32_t sel[kSelWords];
+  __shared__ uint32_t intra[2][32];
+  __shared__ uint8_t open_s[2][32];
   __shared__ uint8_t free_s[kSelChunk];
-  const int lane = threadIdx.x;
-  for (int j = lane; j < a.kc; j += 32) {
-    lab_s[j] = a.label[a.rows[j]];
-    free_s[j] = a.hit[j] < 0 ? 1 : 0;
-  }
-  __syncwarp();
-  uint32_t sel[kSelWords / 32] = {0u, 0u, 0u, 0u};
-  uint32_t ring[kAhead][kSelWords / 32];
+  __shared__ int16_t lab_s[kSelChunk];  // class with a budget, or -1
+  __shared__ int32_t cnt_s[LIPCACHE_MAX_CLASSES];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int groups = (a.kc + 31) / 32;
+  auto load_row = [&](int g, uint32_t (&w)[kPer]) {
+    const int j = 32 * g + warp;
 #pragma unroll
-  for (int q = 0; q < kAhead; ++q) load_cov_row(a.cov, q, a.kc, lane, ring[q]);
-  int nk = 0;
-  int64_t tot = *a.kept_total;
-  for (int j0 = 0; j0 < a.kc; j0 += kAhead) {
-#pragma unroll
-    for (int q = 0; q < kAhead; ++q) {
-      const int j = j0 + q;
-      const bool open = j < a.kc && !(a.budget_total > 0 && tot >= a.budget_total);
-      bool take = open && free_s[j < a.kc ? j : 0] != 0;
-      if (take) {
-        uint32_t any = 0u;
-#pragma unroll
-        for (int t = 0; t < kSelWords / 32; ++t) any |= ring[q][t] & sel[t];
-        take = !__any_sync(0xffffffffu, any != 0u);
-      }
-      const int32_t lab = lab_s[j < a.kc ? j : 0];
-      const bool in_cls = a.budget_pc > 0 && lab >= 0 && lab < a.C;
-      if (take && in_cls) take = a.class_cnt[lab] < a.budget_pc;
-      if (take) {
-        const int w = j >> 5;
-        if (lane == (w & 31)) {
-#pragma unroll
-          for (int t = 0; t < kSelWords / 32; ++t)
-            if (t == (w >> 5)) sel[t] |= 1u << (j & 31);
-        }
-        if (lane == 0) {
-          a.list[nk] = j;
-          if (in_cls) a.class_cnt[lab] += 1;
-        }
-        ++nk;
-        ++tot;
-      }
-      __syncwarp();
-      load_cov_row(a.cov, j + kAhead, a.kc, lane, ring[q]);  // the slot of j now holds j + kAhead
+    for (int t = 0; t < kPer; ++t) {
+      const int wi = lane + 32 * t;
+      w[t] = (j < a.kc && wi <= g) ? __ldcg(a.cov + (size_t)j * kSelWords + wi) : 0u;
     }
+  };
+  uint32_t cur[kPer], nxt[kPer];
+  load_row(0, cur);
+  for (int w = tid; w < kSelWords; w += 1024) sel[w] = 0u;
+  for (int c = tid; c < a.C; c += 1024) cnt_s[c] = a.class_cnt[c];
+  for (int j = tid; j < kSelChunk; j += 1024) {
+    const bool in = j < a.kc;
+    const int32_t lab = in ? a.label[a.rows[j]] : -1;
+    free_s[j] = in && a.hit[j] < 0 ? 1 : 0;
+    lab_s[j] = (int16_t)(a.budget_pc > 0 && lab >= 0 && lab < a.C ? lab : -1);
   }
-  if (lane == 0) {
-    *a.n_list = nk;
-    *a.kept_total = tot;
+  int nk = 0;
+  long long tot = a.st->kept;
+  __syncthreads();
+  for (int g = 0; g < groups; ++g) {
+    if (g + 1 < groups) load_row(g + 1, nxt);
+    bool any = false;
+    uint32_t own = 0;
+#pragma unroll
+    for (int t = 0; t < kPer; ++t) {
+      const int wi = lane + 32 * t;
+      if (wi < g) any = any || (cur[t] & sel[wi]) != 0u;
+      if (wi == g) own = cur[t];
+    }
+    any = __any_sync(0xffffffffu, any);
+    if (lane == (g & 31)) {
+      intra[g & 1][warp] = own;
+      open_s[g & 1][warp] = any ? 0 : free_s[32 * g + warp];
+    }
+    __syncthreads();
+    if (warp == 0) {
+      const int jl = 32 * g + lane;
+      const uint32_t in = intra[g & 1][lane];
+      const uint32_t lt = (1u << lane) - 1u;
+      uint32_t und = __ballot_sync(0xffffffffu, open_s[g & 1][lane] != 0);  // undecided
+      const int lab = lab_s[jl];
+      const uint32_t peers = __match_any_sync(0xffffffffu, lab >= 0 ? lab : -1 - lane);
+      const int have = lab >= 0 ? cnt_s[lab] : 0;
+      uint32_t taken = 0;
+      while (und) {
+        const uint32_t conf = __ballot_sync(0xffffffffu, ((und >> lane) & 1u) && (in & und) != 0u);
+        const uint32_t batch = conf ? und & ((conf & (0u - conf)) - 1u) : und;
+        const bool fits = ((batch >> lane) & 1u) &&
+                          (lab < 0 || have + __popc(peers & (taken | (batch & lt))) < a.budget_pc);
+        const uint32_t f = __ballot_sync(0xffffffffu, fits);
+        const uint32_t now = __ballot_sync(
+            0xffffffffu, fits && (a.budget_total <= 0 || tot + __popc(taken) + __popc(f & lt) < a.budget_total));
+        taken |= now;
+        und &= ~batch & ~__ballot_sync(0xffffffffu, (in & now) != 0u);
+      }
+      if ((taken >> lane) & 1u) {
+        a.list[nk + __popc(taken & lt)] = jl;
+        if (lab >= 0 && (peers & taken & lt) == 0u) cnt_s[lab] = have + __popc(peers & taken);
+      }
+      nk += __popc(taken);
+      tot += __popc(taken);
+      if (lane == 0) sel[g] = taken;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < kPer; ++t) cur[t] = nxt[t];
+  }
+  for (int c = tid; c < a.C; c += 1024) a.class_cnt[c] = cnt_s[c];
+  if (tid == 0) {
+    a.st->n_list = nk;
+    a.st->kept = tot;
   }
 }
 
@@ -204,7 +385,7 @@ constexpr int kTailBlocks = 8;  // blocks of a scatter that clear the rows past 
 
 struct SelScatterArgs {
   const int32_t* list;
-  const int32_t* n_list;
+  const SelState* st;
   const int32_t* rows;
   const float* G;
   int d, dpad;
@@ -224,11 +405,11 @@ struct SelScatterArgs {
 __global__ void k_sel_scatter(SelScatterArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (blockIdx.x < kTailBlocks) {
-    zero_tail(a.t, a.dpad, a.size0 + *a.n_list, (int)(blockIdx.x * 256 + threadIdx.x), kTailBlocks * 256);
+    zero_tail(a.t, a.dpad, a.size0 + a.st->n_list, (int)(blockIdx.x * 256 + threadIdx.x), kTailBlocks * 256);
     return;
   }
   const int q = (blockIdx.x - kTailBlocks) * 8 + warp;
-  if (q >= *a.n_list) return;
+  if (q >= a.st->n_list) return;
   const int p = a.list[q];
   const int32_t row = a.rows[p];
   const int64_t dst = a.size0 + q;
@@ -430,6 +611,21 @@ void grow_to(T*& p, int64_t& cap, int64_t n) {
   cap = n;
 }
 
+// The scratch of a chunk and the counters.
+void ensure_chunk_scratch(lipcache* h) {
+  SelectScratch& x = h->sel;
+  if (x.chunk) return;
+  carve_alloc(x.chunk, [&](Carve& c) {
+    c.take(x.G, (size_t)kSelChunk * h->d);
+    c.take(x.rows, kSelChunk);
+    c.take(x.hit, kSelChunk);
+    c.take(x.cov, (size_t)kSelChunk * kSelWords);
+    c.take(x.list, kSelChunk);
+    c.take(x.class_cnt, (size_t)h->C);
+    c.take(x.state, 64);
+  });
+}
+
 }  // namespace
 
 int64_t select_insert(lipcache* h, const float* H, int64_t n, const int32_t* payload, int require_consistency,
@@ -451,41 +647,31 @@ int64_t select_insert(lipcache* h, const float* H, int64_t n, const int32_t* pay
   int64_t npow = 1;
   while (npow < n) npow <<= 1;
   grow_to(x.keys, x.keys_cap, npow);
-  if (!x.small) {
-    LC_CUDA(cudaMalloc(&x.small, sizeof(int64_t) * 4));
-    LC_CUDA(cudaMallocHost(&x.small_host, sizeof(int64_t) * 4));
-  }
-  LC_CUDA(cudaMemsetAsync(x.small, 0, sizeof(int64_t) * 4, s));  // [0] accepted, [1] kept, [2] chunk count
-  const unsigned npb = (unsigned)((npow + 255) / 256);
-  k_sel_keys<<<npb, 256, 0, s>>>(h->ins_accept, h->ins_radius, n, npow, x.keys, x.small);
-  LC_LAUNCH_CHECK("k_sel_keys");
-  for (int64_t k = 2; k <= npow; k <<= 1)
-    for (int64_t j = k >> 1; j > 0; j >>= 1) {
-      k_bitonic<<<npb, 256, 0, s>>>(x.keys, npow, j, k);
-      LC_LAUNCH_CHECK("k_bitonic");
-    }
-  LC_CUDA(cudaMemcpyAsync(x.small_host, x.small, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  LC_CUDA(cudaStreamSynchronize(s));
-  const int64_t n_acc = x.small_host[0];
-
-  // chunk scratch
-  grow_to(x.G, x.G_cap, (int64_t)kSelChunk * h->d);
-  grow_to(x.rows, x.rows_cap, kSelChunk);
-  grow_to(x.hit, x.hit_cap, kSelChunk);
-  grow_to(x.cov, x.cov_cap, (int64_t)kSelChunk * kSelWords);
-  grow_to(x.list, x.list_cap, kSelChunk + 1);
-  grow_to(x.class_cnt, x.class_cap, h->C);
+  ensure_chunk_scratch(h);
+  SelState* st = reinterpret_cast<SelState*>(x.state);
+  SelState* hs = reinterpret_cast<SelState*>(h->sel_host);
+  LC_CUDA(cudaMemsetAsync(st, 0, sizeof(SelState), s));
   LC_CUDA(cudaMemsetAsync(x.class_cnt, 0, sizeof(int32_t) * h->C, s));
+  const unsigned npb = (unsigned)((npow + 255) / 256);
+  k_sel_keys<<<npb, 256, 0, s>>>(h->ins_accept, h->ins_radius, n, npow, x.keys,
+                                 reinterpret_cast<int64_t*>(&st->n_acc));
+  LC_LAUNCH_CHECK("k_sel_keys");
+  sort_keys(x.keys, npow, s);
+  auto pick = [&]() {
+    k_sel_pick<<<1, 1024, 0, s>>>(x.keys, h->ins_label, x.class_cnt, h->C, budget_per_class, x.rows, st);
+    LC_LAUNCH_CHECK("k_sel_pick");
+    LC_CUDA(cudaMemcpyAsync(hs, st, sizeof(SelState), cudaMemcpyDeviceToHost, s));
+  };
+  pick();
+  LC_CUDA(cudaStreamSynchronize(s));
 
-  int64_t kept = 0;
-  for (int64_t c0 = 0; c0 < n_acc; c0 += kSelChunk) {
-    if (budget_total > 0 && kept >= budget_total) break;
-    const int kc = (int)(n_acc - c0 < kSelChunk ? n_acc - c0 : kSelChunk);
-    k_sel_gather<<<(unsigned)((kc + 7) / 8), 256, 0, s>>>(x.keys, c0, kc, H, h->d, x.rows, x.G);
+  while (hs->kc > 0 && !(budget_total > 0 && hs->kept >= budget_total)) {
+    const int kc = hs->kc;
+    k_sel_gather<<<(unsigned)((kc + 7) / 8), 256, 0, s>>>(x.rows, kc, H, h->d, x.G);
     LC_LAUNCH_CHECK("k_sel_gather");
     probe(h, x.G, kc, x.hit, nullptr, nullptr, s);
-    const int tiles = (kc + 31) / 32;
-    k_sel_cover<<<dim3((unsigned)tiles, (unsigned)tiles), 256, 0, s>>>(x.G, h->d, kc, x.rows, h->ins_rr, x.cov);
+    const unsigned tiles = (unsigned)((kc + kCovT - 1) / kCovT);
+    k_sel_cover<<<dim3(tiles, tiles), 256, 0, s>>>(x.G, h->d, kc, x.rows, h->ins_rr, x.cov);
     LC_LAUNCH_CHECK("k_sel_cover");
     ResolveArgs ra;
     ra.cov = x.cov;
@@ -493,18 +679,17 @@ int64_t select_insert(lipcache* h, const float* H, int64_t n, const int32_t* pay
     ra.hit = x.hit;
     ra.label = h->ins_label;
     ra.class_cnt = x.class_cnt;
-    ra.kept_total = x.small + 1;
+    ra.st = st;
     ra.list = x.list;
-    ra.n_list = reinterpret_cast<int32_t*>(x.small + 2);
     ra.kc = kc;
     ra.C = h->C;
     ra.budget_pc = budget_per_class;
     ra.budget_total = budget_total;
-    k_sel_resolve<<<1, 32, 0, s>>>(ra);
+    k_sel_resolve<<<1, 1024, 0, s>>>(ra);
     LC_LAUNCH_CHECK("k_sel_resolve");
     SelScatterArgs sa;
     sa.list = x.list;
-    sa.n_list = ra.n_list;
+    sa.st = st;
     sa.rows = x.rows;
     sa.G = x.G;
     sa.d = h->d;
@@ -521,15 +706,13 @@ int64_t select_insert(lipcache* h, const float* H, int64_t n, const int32_t* pay
     sa.unfit = &h->report->unfit;
     k_sel_scatter<<<(unsigned)(kTailBlocks + (kc + 7) / 8), 256, 0, s>>>(sa);
     LC_LAUNCH_CHECK("k_sel_scatter");
-    LC_CUDA(cudaMemcpyAsync(x.small_host + 2, x.small + 2, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    pick();  // the next chunk's members, so that one wait serves both
     fetch_report(h, s);  // (the next chunk's probe: whether the FP16 copies still serve)
     LC_CUDA(cudaStreamSynchronize(s));
-    const int64_t got = (int64_t)(int32_t)(x.small_host[2] & 0xFFFFFFFFll);
-    h->size += got;
-    kept += got;
+    h->size += hs->n_list;
   }
   store_size_dev(h, s);  // the table grew from the host
-  return kept;
+  return hs->kept;
 }
 
 int64_t select_kcenter(lipcache* h, const float* H, int64_t n, const int32_t* payload, int require_consistency,
@@ -550,46 +733,42 @@ int64_t select_kcenter(lipcache* h, const float* H, int64_t n, const int32_t* pa
   int64_t npow = 1;
   while (npow < n) npow <<= 1;
   grow_to(x.keys, x.keys_cap, npow);
-  if (!x.small) {
-    LC_CUDA(cudaMalloc(&x.small, sizeof(int64_t) * 4));
-    LC_CUDA(cudaMallocHost(&x.small_host, sizeof(int64_t) * 4));
-  }
-  LC_CUDA(cudaMemsetAsync(x.small, 0, sizeof(int64_t) * 4, s));
+  ensure_chunk_scratch(h);
+  // counters: [0] candidates, [1] centres
+  int64_t* small = reinterpret_cast<int64_t*>(x.state);
+  int64_t* small_host = reinterpret_cast<int64_t*>(h->sel_host);
+  LC_CUDA(cudaMemsetAsync(small, 0, sizeof(int64_t) * 2, s));
   const unsigned npb = (unsigned)((npow + 255) / 256);
-  k_kc_keys<<<npb, 256, 0, s>>>(h->ins_accept, h->ins_label, n, npow, C, x.keys, x.small);
+  k_kc_keys<<<npb, 256, 0, s>>>(h->ins_accept, h->ins_label, n, npow, C, x.keys, small);
   LC_LAUNCH_CHECK("k_kc_keys");
-  for (int64_t k = 2; k <= npow; k <<= 1)
-    for (int64_t j = k >> 1; j > 0; j >>= 1) {
-      k_bitonic<<<npb, 256, 0, s>>>(x.keys, npow, j, k);
-      LC_LAUNCH_CHECK("k_bitonic");
-    }
-  LC_CUDA(cudaMemcpyAsync(x.small_host, x.small, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  sort_keys(x.keys, npow, s);
+  LC_CUDA(cudaMemcpyAsync(small_host, small, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   LC_CUDA(cudaStreamSynchronize(s));
-  const int64_t n_in = x.small_host[0];
+  const int64_t n_in = small_host[0];
   if (n_in == 0) return 0;
   // per-class segments, counts and offsets share one int32 scratch: seg[2C], cnt[C], off[C]
-  grow_to(x.list, x.list_cap, 4 * (int64_t)C + 1);
-  int32_t* seg = x.list;
+  grow_to(x.kc_seg, x.kc_seg_cap, 4 * (int64_t)C);
+  int32_t* seg = x.kc_seg;
   int32_t* cnt = seg + 2 * C;
   int32_t* off = cnt + C;
   LC_CUDA(cudaMemsetAsync(seg, 0, sizeof(int32_t) * 2 * C, s));
   k_kc_segments<<<(unsigned)((n_in + 255) / 256), 256, 0, s>>>(x.keys, n_in, seg);
   LC_LAUNCH_CHECK("k_kc_segments");
   grow_to(x.kc_mind, x.kc_mind_cap, n_in);
-  grow_to(x.rows, x.rows_cap, n_in);
+  grow_to(x.kc_rows, x.kc_rows_cap, n_in);
   k_kcenter<<<C, kKcThreads, sizeof(float) * (size_t)h->d, s>>>(x.keys, seg, H, h->d, h->ins_radius, budget_per_class,
-                                                                x.kc_mind, x.rows, cnt);
+                                                                x.kc_mind, x.kc_rows, cnt);
   LC_LAUNCH_CHECK("k_kcenter");
-  k_kc_scan<<<1, 1024, 0, s>>>(cnt, C, off, x.small + 1);
+  k_kc_scan<<<1, 1024, 0, s>>>(cnt, C, off, small + 1);
   LC_LAUNCH_CHECK("k_kc_scan");
   const int per = budget_per_class;
   k_kc_scatter<<<dim3((unsigned)((per + 7) / 8 < 64 ? (per + 7) / 8 : 64), (unsigned)(C + 1)), 256, 0, s>>>(
-      seg, cnt, off, x.rows, H, h->d, h->dpad, h->size, h->ins_rr, h->ins_tau, h->ins_kn, h->ins_radius,
-      h->ins_label, h->ins_yG, h->table, out_index, &h->report->unfit, x.small + 1, C);
+      seg, cnt, off, x.kc_rows, H, h->d, h->dpad, h->size, h->ins_rr, h->ins_tau, h->ins_kn, h->ins_radius,
+      h->ins_label, h->ins_yG, h->table, out_index, &h->report->unfit, small + 1, C);
   LC_LAUNCH_CHECK("k_kc_scatter");
-  LC_CUDA(cudaMemcpyAsync(x.small_host + 1, x.small + 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  LC_CUDA(cudaMemcpyAsync(small_host + 1, small + 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   LC_CUDA(cudaStreamSynchronize(s));
-  const int64_t kept = x.small_host[1];
+  const int64_t kept = small_host[1];
   h->size += kept;
   store_size_dev(h, s);  // the table grew from the host
   return kept;
@@ -597,16 +776,11 @@ int64_t select_kcenter(lipcache* h, const float* H, int64_t n, const int32_t* pa
 
 void release_select(lipcache* h) {
   SelectScratch& x = h->sel;
+  cudaFree(x.chunk);
   cudaFree(x.keys);
-  cudaFree(x.G);
-  cudaFree(x.rows);
-  cudaFree(x.hit);
-  cudaFree(x.cov);
-  cudaFree(x.list);
-  cudaFree(x.class_cnt);
   cudaFree(x.kc_mind);
-  cudaFree(x.small);
-  if (x.small_host) cudaFreeHost(x.small_host);
+  cudaFree(x.kc_seg);
+  cudaFree(x.kc_rows);
   x = SelectScratch{};
 }
 

@@ -160,6 +160,31 @@ def test_select_workload(dev, name, n, bt, bc):
     cache.close()
 
 
+@pytest.mark.parametrize("n,bt,bc", [(1, 0, 0), (31, 0, 2), (33, 0, 0), (64, 20, 0), (4096, 0, 7), (4097, 0, 0),
+                                     (9000, 1500, 90), (9000, 0, 60), (13000, 5000, 0)])
+def test_select_groups_and_budgets(dev, n, bt, bc):
+    """The resolver's groups of 32 and chunks of 4,096 at their edges, chains of
+    near-duplicates inside a group, both budgets running out mid-group, classes
+    that close between chunks, labels outside [0, C) (which have no class
+    budget): the greedy invariants of check_selection."""
+    w = synth.WORKLOADS["cifar10"].scaled(N=max(2, n), noise=0.02)
+    W, b = synth.head(w)
+    rng = np.random.default_rng(n)
+    rows = _pool(w, n, n) if n > 1 else synth.cache_rows(w)[:1]
+    if n > 40:  # chains: each row a small step from the one before, radii in sequence
+        rows[:24] = rows[0] + np.cumsum(0.01 * rng.standard_normal((24, w.d)), axis=0).astype(np.float32)
+    payload = rng.integers(-1, w.C + 1, n).astype(np.int32)
+    s = oracle.sigma_max(W)
+    cert = oracle.certify(W, b, s, rows, payload=payload)
+    cache = make_cache(dev, W, b, n)
+    idx, rad, got = cache.insert_select(T(rows, dev), payload=T(payload, dev), budget_total=bt, budget_per_class=bc)
+    idx, rad = idx.cpu().numpy(), rad.cpu().numpy()
+    assert got == int((idx >= 0).sum()) == cache.size
+    none = np.zeros((0, w.d), np.float32)
+    check_selection(rows, cert, idx, rad, none, np.zeros(0), bt, bc, w.C)
+    cache.close()
+
+
 def test_select_errors_and_all(dev):
     from paper_2608_13144_gb300._lib import LipCacheError, check
     w = synth.WORKLOADS["tiny"]

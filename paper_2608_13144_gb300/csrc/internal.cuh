@@ -76,8 +76,7 @@ constexpr double kU64 = 1.1102230246251565e-16;   // 2^-53
 inline double gamma32(int n) { return n * kU32 / (1.0 - n * kU32); }
 inline double gamma64(int n) { return n * kU64 / (1.0 - n * kU64); }
 
-// Relative error bound of the canonical FP32 squared distance (see
-// dist2_canonical): every term e_j^2 passes one subtraction rounding (which
+// Relative error bound of the canonical FP32 squared distance (probe_common.cuh): every term e_j^2 passes one subtraction rounding (which
 // at most doubles in the square), at most 32 roundings inside its 32-wide
 // chunk and at most d_pad/32 - 1 roundings while the chunk sums are added, so
 // |S~ - S| <= gamma_{d_pad/32 + 33} S (all terms are non-negative). A small

@@ -5,7 +5,7 @@
 //   hit -> payload of i*, miss -> fall back to MainNet (Eq. 15)
 //
 // Acceptance. A pair (q, i) is accepted iff the canonical FP32 squared
-// distance S~ (dist2_canonical: direct differences, 32-wide FMA chunks added
+// distance S~ (probe_common.cuh: direct differences, 32-wide FMA chunks added
 // in order) is below rr_i = RZ(r_safe,i^2 (1 - eps_rc)). Since
 // |S~ - S| <= gamma_{d_pad/32+33} S < eps_rc S, every accepted pair has an
 // exact distance below r_safe,i <= r_i: the GPU never accepts a pair the

@@ -18,63 +18,87 @@ __device__ __forceinline__ unsigned long long pack_hit(float dist2, int64_t inde
 // Canonical FP32 squared distance sum_j (q_j - k_j)^2 over d_pad (multiple
 // of 32) zero-padded features: a 32-wide fused-multiply-add chain per chunk,
 // chunk sums added in order. Every probe path evaluates exactly this
-// sequence of rounded operations, so all paths agree bit for bit. q and k
-// are 16-byte aligned.
-__device__ __forceinline__ float dist2_canonical(const float* __restrict__ q, const float* __restrict__ k, int dpad) {
-  float total = 0.f;
-  for (int c = 0; c < dpad; c += 32) {
-    float p = 0.f;
+// sequence of rounded operations, so all paths agree bit for bit.
+//
+// One 32-wide chunk of that sequence, features [c, c + n) of a query and a key;
+// features past the query's d, zero in both rows, add exact zeros and are left
+// out. vec: the query row is 16-byte aligned and n a multiple of 4 (key rows
+// always are). All loads are issued before the chain starts.
+__device__ __forceinline__ float dist2_chunk(const float* __restrict__ q, bool vec, const float* __restrict__ k, int n) {
+  float4 a[8], b[8];
 #pragma unroll
-    for (int j = 0; j < 32; j += 4) {
-      const float4 a = *reinterpret_cast<const float4*>(q + c + j);
-      const float4 b = *reinterpret_cast<const float4*>(k + c + j);
-      float e = __fsub_rn(a.x, b.x);
-      p = __fmaf_rn(e, e, p);
-      e = __fsub_rn(a.y, b.y);
-      p = __fmaf_rn(e, e, p);
-      e = __fsub_rn(a.z, b.z);
-      p = __fmaf_rn(e, e, p);
-      e = __fsub_rn(a.w, b.w);
-      p = __fmaf_rn(e, e, p);
+  for (int u = 0; u < 8; ++u) {
+    const int m = n - 4 * u;
+    a[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (vec) {
+      if (m > 0) a[u] = __ldg(reinterpret_cast<const float4*>(q) + u);
+    } else {
+      if (m > 0) a[u].x = __ldg(q + 4 * u);
+      if (m > 1) a[u].y = __ldg(q + 4 * u + 1);
+      if (m > 2) a[u].z = __ldg(q + 4 * u + 2);
+      if (m > 3) a[u].w = __ldg(q + 4 * u + 3);
     }
-    total = __fadd_rn(total, p);
+    b[u] = m > 0 ? *(reinterpret_cast<const float4*>(k) + u) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  return total;
+  float p = 0.f;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    float e = __fsub_rn(a[u].x, b[u].x);
+    p = __fmaf_rn(e, e, p);
+    e = __fsub_rn(a[u].y, b[u].y);
+    p = __fmaf_rn(e, e, p);
+    e = __fsub_rn(a[u].z, b[u].z);
+    p = __fmaf_rn(e, e, p);
+    e = __fsub_rn(a[u].w, b[u].w);
+    p = __fmaf_rn(e, e, p);
+  }
+  return p;
 }
 
-// The same sequence with the query's d features as the caller passed them
-// (the zero padding adds exact zeros: left out). vec: the row is 16-byte
-// aligned and d a multiple of 4.
-__device__ __forceinline__ float dist2_canonical_row(const float* __restrict__ q, bool vec, const float* __restrict__ k,
-                                                     int d) {
-  float total = 0.f;
-  for (int c = 0; c < d; c += 32) {
-    float p = 0.f;
-    const int n = d - c < 32 ? d - c : 32;
-    if (vec) {
-#pragma unroll 8
-      for (int j = 0; j < n; j += 4) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(q + c + j));
-        const float4 b = *reinterpret_cast<const float4*>(k + c + j);
-        float e = __fsub_rn(a.x, b.x);
-        p = __fmaf_rn(e, e, p);
-        e = __fsub_rn(a.y, b.y);
-        p = __fmaf_rn(e, e, p);
-        e = __fsub_rn(a.z, b.z);
-        p = __fmaf_rn(e, e, p);
-        e = __fsub_rn(a.w, b.w);
-        p = __fmaf_rn(e, e, p);
+// Recheck of screen candidates by a converged warp: bit j of a lane's `mask`
+// is the pair (its query row, key key0 + j). A pair takes as many lanes as its
+// rows have chunks (rounded up to a power of two), each running one chunk's
+// chain, and the chunk sums are added in order, so the bits are those of
+// the sequence above; with one lane per pair the loads and chains of all chunks
+// came one after the other (3 us at d = 128), and the epilogue warp could not
+// take its next tile meanwhile. Accepted pairs go to `best`.
+struct Recheck {
+  const float* q;  // query rows, qstride floats apart
+  int64_t qstride;
+  bool qvec;
+  const float* keys;  // d_pad floats apart
+  int dpad, d;
+  const float* rr;
+  unsigned long long* best;
+};
+// (Not inlined: its registers are not the epilogue loop's.)
+static __device__ __noinline__ void recheck_warp(const Recheck& a, uint32_t mask, int64_t row, int64_t key0, int lane,
+                                          unsigned long long& ncand) {
+  const int nch = (a.d + 31) >> 5;
+  const int lg = nch <= 1 ? 0 : 32 - __clz(nch - 1), sub = lane & ((1 << lg) - 1), grp = lane >> lg;
+  for (;;) {
+    uint32_t has = __ballot_sync(0xffffffffu, mask != 0);
+    if (!has) break;
+    const int64_t my_key = key0 + __ffs((int)mask) - 1;
+    ncand += mask != 0 ? 1 : 0;
+    mask &= mask - 1;
+    while (has) {
+      uint32_t b = has;
+      for (int i = 0; i < grp; ++i) b &= b - 1;  // this group's pair: the grp-th lane that has one
+      const int src = b ? __ffs((int)b) - 1 : 0;
+      const int64_t key = __shfl_sync(0xffffffffu, my_key, src), r = __shfl_sync(0xffffffffu, row, src);
+      float p = 0.f;
+      const float thr = b ? __ldg(a.rr + key) : 0.f;  // (in flight with the rows)
+      if (b && sub < nch) {
+        const int n = a.d - 32 * sub;
+        p = dist2_chunk(a.q + r * a.qstride + 32 * sub, a.qvec, a.keys + key * a.dpad + 32 * sub, n < 32 ? n : 32);
       }
-    } else {
-#pragma unroll 8
-      for (int j = 0; j < n; ++j) {
-        const float e = __fsub_rn(__ldg(q + c + j), k[c + j]);
-        p = __fmaf_rn(e, e, p);
-      }
+      float total = __shfl_sync(0xffffffffu, p, grp << lg);
+      for (int c = 1; c < nch; ++c) total = __fadd_rn(total, __shfl_sync(0xffffffffu, p, (grp << lg) + c));
+      if (b && sub == 0 && total < thr) atomicMin(a.best + r, pack_hit(total, key));
+      for (int i = 0; i < (32 >> lg); ++i) has &= has - 1;
     }
-    total = __fadd_rn(total, p);
   }
-  return total;
 }
 
 // Operand kinds of the tensor screen. Both stream 128-byte rows (one swizzle

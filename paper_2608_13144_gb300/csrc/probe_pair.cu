@@ -268,6 +268,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int t = 0;
     bool ok = true;
     unsigned long long ncand = 0;
+    const Recheck rck{a.q, KIND == kF16 ? a.d : a.dpad, KIND == kF16 ? a.qvec != 0 : true, a.keys, a.dpad, a.d, a.rr, a.best};
     for (int u = cluster_id; u < a.n_units && ok; u += n_clusters) {
       int kt, qt0, qt1;
       unit_range(a, u, pair, kt, qt0, qt1);
@@ -322,47 +323,33 @@ __global__ void __launch_bounds__(kThreads, 1)
             pass |= (uint32_t)(screen_value<KIND>(amax[u], scl, tmin[ch + u]) >= kap) << (ch + u);
         }
         if (!live) pass = 0;
-        const bool found = __any_sync(0xffffffffu, pass != 0);
-        uint32_t masks[kChunks];
-        if (found) {
-#pragma unroll
-          for (int ch = 0; ch < kChunks; ++ch) {
-            masks[ch] = 0;
-            const bool mine = (pass >> ch) & 1u;
-            if (!__any_sync(0xffffffffu, mine)) continue;
-            uint32_t v[32];
-            ptx::tmem_ld32(tbase + (uint32_t)(ch * 32), v);
-            ptx::tmem_wait_ld();
-            uint32_t mask = 0;
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-              mask |= (uint32_t)(screen_value<KIND>(__uint_as_float(v[j]), scl, my_tau[ch * 32 + j]) >= kap) << j;
-            masks[ch] = mine ? mask : 0u;
-          }
-        }
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive_cluster(lead_acc_empty + 8 * buf);
-        if (found) {
-#pragma unroll
-          for (int ch = 0; ch < kChunks; ++ch) {
-            uint32_t mask = masks[ch];
-            const float* qrow = a.q + (size_t)row * (KIND == kF16 ? a.d : a.dpad);
-            while (mask) {
-              const int j = __ffs(mask) - 1;
-              mask &= mask - 1;
-              const int key = key0 + ch * 32 + j;
-              const float* krow = a.keys + (size_t)key * a.dpad;
-              float d2;
-              if constexpr (KIND == kF16)
-                d2 = dist2_canonical_row(qrow, a.qvec != 0, krow, a.d);
-              else
-                d2 = dist2_canonical(qrow, krow, a.dpad);
-              ++ncand;
-              if (d2 < __ldg(a.rr + key)) atomicMin(a.best + row, pack_hit(d2, key));
-            }
-          }
+        // The chunks some row passes in, one copy of code for all (rarely run
+        // code is fetched as it goes): the pairs that pass from the products,
+        // the accumulator handed back once the last of those is loaded, then
+        // the recheck.
+        uint32_t chunks = __reduce_or_sync(0xffffffffu, pass);
+        if (chunks == 0) {
+          ptx::tc_fence_before();
           __syncwarp();
+          if (lane == 0) ptx::mbar_arrive_cluster(lead_acc_empty + 8 * buf);
+        }
+#pragma unroll 1
+        while (chunks) {
+          const int ch = __ffs((int)chunks) - 1;
+          chunks &= chunks - 1;
+          uint32_t v[32];
+          ptx::tmem_ld32(tbase + (uint32_t)(ch * 32), v);
+          ptx::tmem_wait_ld();
+          if (chunks == 0) {
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive_cluster(lead_acc_empty + 8 * buf);
+          }
+          uint32_t mask = 0;
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            mask |= (uint32_t)(screen_value<KIND>(__uint_as_float(v[j]), scl, my_tau[ch * 32 + j]) >= kap) << j;
+          recheck_warp(rck, (pass >> ch) & 1u ? mask : 0u, row, key0 + ch * 32, lane, ncand);
         }
         kap = kap_next;
         scl = scl_next;

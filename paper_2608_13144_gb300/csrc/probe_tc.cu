@@ -31,7 +31,7 @@
 // query tiles: each CTA TMA-loads one half of every query stage with
 // .multicast::cluster into both CTAs' shared memory, so the L2 delivers each
 // query byte once per pair of SMs (the query stream from L2 is what limits a
-// single CTA). Per CTA (320 threads):
+// single CTA). Per CTA (352 threads):
 //   warp 0     TMA producer: the CTA's key tile (BN keys x d_pad, resident,
 //              one barrier pair per 128-byte chunk so the next tile streams in
 //              while the last query tile still runs) and its half of each
@@ -40,8 +40,11 @@
 //              queries, N=BN keys, 32 bytes of K) into one of two TMEM
 //              accumulators; releases each query stage in BOTH CTAs;
 //   warps 2-9  epilogue: tcgen05.ld of the accumulator (warp w reads TMEM
-//              lane quarter w % 4, column half (w - 2) / 4), screen, recheck,
-//              atomicMin of the packed (distance, index) word.
+//              lane quarter w % 4, column half (w - 2) / 4), screen; the pairs
+//              that pass go to
+//   warp 10    the recheck, atomicMin of the packed (distance, index) word,
+//              through a queue in shared memory, so that the loads of a pair's
+//              rows (3 us on an epilogue warp) do not hold up the next tiles.
 // Work: the items (key-tile pair, query tile), pair-major, are split into
 // equal contiguous ranges, one per cluster; a run is the part of a range on
 // one pair, and its key tile stays resident through the run (a pair split
@@ -65,7 +68,8 @@ constexpr int kQHalfBytes = kQStageBytes / 2;
 #define LC_EPI_WARPS 8
 #endif
 constexpr int kEpiWarps = LC_EPI_WARPS;  // 4 or 8: one or two per SM sub-partition
-constexpr int kThreads = 32 * (2 + kEpiWarps);
+constexpr int kRecheckWarp = 2 + kEpiWarps;
+constexpr int kThreads = 32 * (3 + kEpiWarps);
 constexpr int kCluster = 2;
 constexpr uint16_t kClusterMask = 0x3;
 constexpr int kSmemBudget = 227 * 1024 - 1024;  // opt-in limit minus the alignment slack
@@ -91,7 +95,20 @@ struct TcArgs {
   const float* rr;
   unsigned long long* best;
   DevStats* stats;
+  int queue;        // candidates go to the recheck warp (ranges of several tiles)
   int debug_stall;  // test hook: the MMA issuer first waits on a barrier nothing arrives on
+};
+
+// Pairs on their way from the epilogue warps to the recheck warp (shared
+// memory): pair number k is in slot k % kRecheckQ once seq there is k + 1.
+constexpr int kRecheckQ = 64;
+struct RecheckQueue {
+  int n;      // slots reserved
+  int taken;  // pairs rechecked (their slots are free)
+  int done;   // epilogue warps past their last tile
+  int pad;
+  int2 pair[kRecheckQ];  // query row, key
+  int seq[kRecheckQ];
 };
 
 template <int BN>
@@ -106,8 +123,9 @@ struct Layout {
   __device__ __host__ int baroff() const { return tauoff() + (tau_staged ? kTauStaged : 0); }
   // barriers: full_k[nk], empty_k[nk], full_q[nst], empty_q[nst], acc_full[2], acc_empty[2], drain
   __device__ __host__ int nbar() const { return 2 * nk + 2 * nst + 5; }
-  __device__ __host__ int miscoff() const { return baroff() + 8 * nbar(); }
-  __device__ __host__ int total() const { return miscoff() + 16; }
+  __device__ __host__ int miscoff() const { return (baroff() + 8 * nbar() + 15) / 16 * 16; }
+  __device__ __host__ int rqoff() const { return miscoff() + 16; }
+  __device__ __host__ int total() const { return rqoff() + (int)sizeof(RecheckQueue); }
   // deepest ring that fits the shared-memory budget
   static __host__ int stages_for(int nk, int tau_staged) {
     for (int n = kMaxStages; n >= 2; --n) {
@@ -169,6 +187,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t acc_full = empty_q + 8 * a.nst, acc_empty = acc_full + 16, drain = acc_empty + 16;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L.miscoff());
   volatile int* abort_s = reinterpret_cast<volatile int*>(smem + L.miscoff() + 4);
+  RecheckQueue* rq = reinterpret_cast<RecheckQueue*>(smem + L.rqoff());
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = ptx::cluster_ctarank();
@@ -193,6 +212,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     ptx::tma_prefetch_desc(&tmQ);
     ptx::tma_prefetch_desc(&tmK);
   }
+  if (warp == kRecheckWarp) {
+    for (int k = lane; k < kRecheckQ; k += 32) rq->seq[k] = 0;
+    if (lane == 0) rq->n = rq->taken = rq->done = 0;
+  }
   if (warp == 1) {
     ptx::tmem_alloc(ptx::smem_u32(tmem_slot), (uint32_t)Layout<BN>::kTmemCols);
     ptx::tmem_relinquish();
@@ -203,6 +226,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   ptx::cluster_sync();  // the peer's barriers exist before any multicast reaches them
   const uint32_t tmem = *tmem_slot;
 
+  const Recheck rck{a.q, KIND == kF16 ? a.d : a.dpad, KIND == kF16 ? a.qvec != 0 : true, a.keys, a.dpad, a.d, a.rr, a.best};
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     if (lane == 0) {
@@ -344,6 +368,40 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     __syncwarp();
+  } else if (warp == kRecheckWarp) {
+    // ------------------------------------------------------------ recheck
+    // the pairs the epilogue warps hand over, as they come; ends once every
+    // epilogue warp is done (each is, also after an abort) and none is left
+    unsigned long long ncand = 0;
+    volatile RecheckQueue* vq = rq;
+    for (int k = 0; a.queue;) {
+      const unsigned ready = __ballot_sync(0xffffffffu, vq->seq[(k + lane) % kRecheckQ] == k + lane + 1);
+      const int m = ready == 0xffffffffu ? 32 : __ffs((int)~ready) - 1;
+      if (m == 0) {
+        if (__any_sync(0xffffffffu, vq->done == kEpiWarps)) {
+          __threadfence_block();
+          if (__all_sync(0xffffffffu, vq->n == k)) break;
+          continue;
+        }
+        // (every look takes shared-memory cycles from the MMAs)
+        __nanosleep(kTauStaged ? 250 : 1000);
+        continue;
+      }
+      __threadfence_block();
+      int row = 0, key = 0;
+      if (lane < m) {
+        row = vq->pair[(k + lane) % kRecheckQ].x;
+        key = vq->pair[(k + lane) % kRecheckQ].y;
+      }
+      recheck_warp(rck, lane < m ? 1u : 0u, row, key, lane, ncand);
+      k += m;
+      __threadfence_block();
+      __syncwarp();
+      if (lane == 0) vq->taken = k;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ncand += __shfl_xor_sync(0xffffffffu, ncand, o);
+    if (lane == 0 && ncand) atomicAdd(&a.stats->candidates, ncand);
   } else {
     // ------------------------------------------------------------ epilogue
     const int ew = warp - 2;
@@ -423,52 +481,73 @@ __global__ void __launch_bounds__(kThreads, 1)
             pass |= (uint32_t)(screen_value<KIND>(amax[u], scl, tmin[h][ch + u]) >= kap) << (ch + u);
         }
         if (!live) pass = 0;
-        const bool found = __any_sync(0xffffffffu, pass != 0);
-        uint32_t masks[kChunks];
-        if (found) {
-#pragma unroll
-          for (int ch = 0; ch < kChunks; ++ch) {
-            masks[ch] = 0;
-            const bool mine = (pass >> ch) & 1u;
-            if (!__any_sync(0xffffffffu, mine)) continue;
-            uint32_t v[32];
-            ptx::tmem_ld32(tbase + (uint32_t)(ch * 32), v);
-            ptx::tmem_wait_ld();
-            uint32_t mask = 0;
-            if (kTauStaged) {
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                mask |= (uint32_t)(screen_value<KIND>(__uint_as_float(v[j]), scl, my_tau[ch * 32 + j]) >= kap) << j;
-            } else {
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                mask |= (uint32_t)(screen_value<KIND>(__uint_as_float(v[j]), scl, __ldg(tau_g + ch * 32 + j)) >= kap)
-                        << j;
-            }
-            masks[ch] = mine ? mask : 0u;
-          }
+        // The chunks some row passes in, one copy of code for all (rarely run
+        // code is fetched as it goes): the pairs that pass from the products,
+        // the accumulator handed back once the last of those is loaded, then
+        // the recheck.
+        uint32_t chunks = __reduce_or_sync(0xffffffffu, pass);
+        if (chunks == 0) {
+          ptx::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(acc_empty + 8 * buf);
         }
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(acc_empty + 8 * buf);
-        if (found) {
+#pragma unroll 1
+        while (chunks) {
+          const int ch = __ffs((int)chunks) - 1;
+          chunks &= chunks - 1;
+          uint32_t v[32];
+          ptx::tmem_ld32(tbase + (uint32_t)(ch * 32), v);
+          ptx::tmem_wait_ld();
+          if (chunks == 0) {
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(acc_empty + 8 * buf);
+          }
+          uint32_t mask = 0;
+          if (kTauStaged) {
 #pragma unroll
-          for (int ch = 0; ch < kChunks; ++ch) {
-            uint32_t mask = masks[ch];
-            const float* qrow = a.q + (size_t)row * (KIND == kF16 ? a.d : a.dpad);
-            while (mask) {
-              const int j = __ffs(mask) - 1;
-              mask &= mask - 1;
-              const int key = key0 + h * BN + ch * 32 + j;
-              const float* krow = a.keys + (size_t)key * a.dpad;
-              float d2;
-              if constexpr (KIND == kF16)
-                d2 = dist2_canonical_row(qrow, a.qvec != 0, krow, a.d);
-              else
-                d2 = dist2_canonical(qrow, krow, a.dpad);
-              ++ncand;
-              if (d2 < __ldg(a.rr + key)) atomicMin(a.best + row, pack_hit(d2, key));
+            for (int j = 0; j < 32; ++j)
+              mask |= (uint32_t)(screen_value<KIND>(__uint_as_float(v[j]), scl, my_tau[ch * 32 + j]) >= kap) << j;
+          } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              mask |= (uint32_t)(screen_value<KIND>(__uint_as_float(v[j]), scl, __ldg(tau_g + ch * 32 + j)) >= kap)
+                      << j;
+          }
+          mask = (pass >> ch) & 1u ? mask : 0u;
+          const int mine = __popc(mask);
+          const int cnt = __reduce_add_sync(0xffffffffu, mine);
+          if (cnt == 0) continue;
+          const int first_key = key0 + h * BN + ch * 32;
+          // to the recheck warp if there are tiles to go on with and its queue
+          // has room, else here
+          int base = -1;
+          if (lane == 0 && a.queue) {
+            volatile RecheckQueue* vq = rq;
+            for (int n = vq->n; n + cnt - vq->taken <= kRecheckQ;) {
+              const int was = atomicCAS(&rq->n, n, n + cnt);
+              if (was == n) {
+                base = n;
+                break;
+              }
+              n = was;
             }
+          }
+          base = __shfl_sync(0xffffffffu, base, 0);
+          if (base < 0) {
+            recheck_warp(rck, mask, row, first_key, lane, ncand);
+            continue;
+          }
+          int at = mine;  // inclusive prefix of the lanes' counts
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, at, o);
+            if (lane >= o) at += x;
+          }
+          for (at += base - mine; mask; mask &= mask - 1, ++at) {
+            rq->pair[at % kRecheckQ] = make_int2(row, first_key + __ffs((int)mask) - 1);
+            __threadfence_block();
+            *(volatile int*)&rq->seq[at % kRecheckQ] = at + 1;
           }
           __syncwarp();
         }
@@ -476,6 +555,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         kap = kap_next;
         scl = scl_next;
       }
+    }
+    __syncwarp();
+    if (lane == 0) {
+      __threadfence_block();
+      atomicAdd(&rq->done, 1);
     }
     // candidate count: one atomic per warp
 #pragma unroll
@@ -549,6 +633,10 @@ void launch_nh(lipcache* h, int64_t B, const ProbeBuffers& b, bool long_ranges, 
   a.rr = h->probe_rr();
   a.best = b.best;
   a.stats = h->stats;
+  // With one to three tiles per cluster the recheck warp's turn would only come
+  // at the end: 256 x 50,000 at d = 64 13.4 us without it, 15.0 with; 1,024 x
+  // 50,000 at d = 128 (ten tiles) 22.1 without, 20.7 with.
+  a.queue = n_pairs * a.nq >= 6 * (int64_t)max_clusters ? 1 : 0;
   a.debug_stall = (h->debug_flags & LIPCACHE_DEBUG_STALL_PROBE) ? 1 : 0;
   const Layout<BN> L{NH * a.nch, a.nst, a.tau_staged};
   const int smem = L.total() + 1024;

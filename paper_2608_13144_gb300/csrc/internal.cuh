@@ -153,6 +153,8 @@ struct DevReport {
   int64_t total[4];  // rows appended by the last insert; consistency counts
   int64_t size;      // table size
   int64_t unfit;     // entries whose FP16 copy does not serve the screen
+  unsigned done_ctas;  // finished CTAs of a probe kernel that finalizes itself (0 between probes)
+  unsigned pad;
   DevStats stats;
 };
 
@@ -264,7 +266,8 @@ struct lipcache {
   float* qpad = nullptr;
   float* kappa = nullptr;
   float* qscale = nullptr;  // power-of-two scale of each FP16 query
-  unsigned long long* best = nullptr;
+  unsigned long long* best = nullptr;  // every word is empty (all ones) between probes ...
+  bool best_clean = false;             // ... unless this is false
   // host-buffer probe staging
   int64_t hq_cap = 0;
   float* hq = nullptr;
@@ -392,11 +395,13 @@ struct ProbeBuffers {
 // probe_tc.cu: the tensor probe; `path` is LIPCACHE_PROBE_TENSOR (kernel
 // chosen by shape), _TENSOR_SINGLE or _TENSOR_PAIR. Returns the kernel that
 // ran (_TENSOR_SINGLE or _TENSOR_PAIR).
-int launch_probe_tc(lipcache* h, int64_t B, int path, bool f16, const ProbeBuffers& b, cudaStream_t s);
+struct ProbeOut;
+int launch_probe_tc(lipcache* h, int64_t B, int path, bool f16, const ProbeBuffers& b, const ProbeOut& out,
+                    cudaStream_t s);
 void encode_screen_map(lipcache* h, CUtensorMap* map, const void* base, uint64_t rows, uint32_t box_rows, bool f16);
 // probe_pair.cu
 int probe_pair_clusters(lipcache* h, bool f16);
-void launch_probe_pair(lipcache* h, int64_t B, bool f16, const ProbeBuffers& b, cudaStream_t s);
+void launch_probe_pair(lipcache* h, int64_t B, bool f16, const ProbeBuffers& b, const ProbeOut& out, cudaStream_t s);
 // probe.cu / probe_tc.cu: the probe on caller-provided scratch memory
 void probe_external_scratch(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* out_label,
                             float* out_dist, float* qpad, float* kappa, float* qscale, unsigned long long* best,

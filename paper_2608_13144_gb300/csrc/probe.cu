@@ -16,8 +16,10 @@
 // its value, and equal distances resolve to the lowest index.
 //
 // Kernels: k_prologue / k_prologue16 (pads or rounds the queries, per-query
-// screen constant, clears the reduction words), the main kernel (exact: every pair on CUDA cores;
-// tensor: tcgen05 screen + recheck, probe_tc.cu), k_finalize (unpacks).
+// screen constant, clears the reduction words; not for the exact kernel), the
+// main kernel (exact: every pair on CUDA cores; tensor: tcgen05 screen +
+// recheck, probe_tc.cu), which unpacks small batches itself, and else
+// k_finalize.
 #include "internal.cuh"
 #include "probe_common.cuh"
 
@@ -41,6 +43,7 @@ __global__ void __launch_bounds__(256) k_prologue(const float* __restrict__ Q, i
                                                   unsigned long long* __restrict__ best, double one_minus_c,
                                                   DevStats* __restrict__ st) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  ptx::launch_dependents();
   if (blockIdx.x == 0 && threadIdx.x == 0) st->abort_flag = 0;
   const int64_t row = (int64_t)blockIdx.x * 8 + warp;
   if (row >= Bpad) return;
@@ -73,6 +76,7 @@ __global__ void __launch_bounds__(256) k_prologue16(const float* __restrict__ Q,
                                                     double one_minus_c, DevStats* __restrict__ st) {
   constexpr int kMaxChunk = 8;  // d <= 512
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  ptx::launch_dependents();
   if (blockIdx.x == 0 && threadIdx.x == 0) st->abort_flag = 0;
   const int64_t row = (int64_t)blockIdx.x * 8 + warp;
   if (row >= Bpad) return;
@@ -108,103 +112,117 @@ __global__ void __launch_bounds__(256) k_prologue16(const float* __restrict__ Q,
   }
 }
 
-// Exact probe: the canonical FP32 squared distance of every pair.
-// CTA tile: 64 queries x 64 keys, 256 threads, 4 x 4 pairs per thread.
+// Exact probe: the canonical FP32 squared distance of every pair. It reads the
+// caller's queries, needs no prologue (the reduction words are empty between
+// probes) and, for small batches and grids, finalizes itself: one launch, so a
+// single query costs one launch (1 x 2,000 at d = 64, called from Python: 20.9 us
+// with three launches, 17.7 with one).
+// CTA tile: 64 queries x 64 keys, 256 threads, 4 x 4 pairs per thread; the next
+// 32-feature chunk is loaded while this one is computed; warps without a live
+// query skip the product.
 constexpr int kEQ = 64, kEK = 64, kES = kEQ + 4;
 
-__global__ void __launch_bounds__(256) k_probe_exact(const float* __restrict__ qpad, int64_t B,
+__global__ void __launch_bounds__(256) k_probe_exact(const float* __restrict__ Q, int64_t B, int d, int qvec,
                                                      const float* __restrict__ keys, const float* __restrict__ rr,
-                                                     int64_t N, int dpad, unsigned long long* __restrict__ best) {
+                                                     int64_t N, int dpad, unsigned long long* __restrict__ best,
+                                                     ProbeOut out, DevStats* __restrict__ st) {
   __shared__ __align__(16) float qs[32][kES];
   __shared__ __align__(16) float ks[32][kES];
   const int tid = threadIdx.x;
   const int tq = tid >> 4, tk = tid & 15;
   const int64_t q0 = (int64_t)blockIdx.y * kEQ, k0 = (int64_t)blockIdx.x * kEK;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) st->abort_flag = 0;
   const int lr = tid & 63, lp = tid >> 6;  // loader: row, 8-float part
+  const bool busy = q0 + (tid >> 5) * 8 < B;  // this warp's eight queries hold a live one
   float tot[4][4], p[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) tot[a][b] = 0.f;
-
+  float x[8], y[8];
+  const int64_t qr = q0 + lr, kr = k0 + lr;
+  auto load = [&](int c0) {
+    const int c = c0 + lp * 8;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = y[u] = 0.f;
+    if (qr < B) {
+      const float* src = Q + (size_t)qr * d + c;
+      if (qvec) {
+#pragma unroll
+        for (int u = 0; u < 8; u += 4)
+          if (c + u < d) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(src + u));
+            x[u] = v.x, x[u + 1] = v.y, x[u + 2] = v.z, x[u + 3] = v.w;
+          }
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (c + u < d) x[u] = __ldg(src + u);
+      }
+    }
+    if (kr < N) {
+      const float4* src = reinterpret_cast<const float4*>(keys + (size_t)kr * dpad + c);
+      const float4 v = __ldg(src), w = __ldg(src + 1);
+      y[0] = v.x, y[1] = v.y, y[2] = v.z, y[3] = v.w;
+      y[4] = w.x, y[5] = w.y, y[6] = w.z, y[7] = w.w;
+    }
+  };
+  load(0);
   for (int c0 = 0; c0 < dpad; c0 += 32) {
-    {
-      const int64_t qr = q0 + lr, kr = k0 + lr;
-      float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), x1 = x0, y0 = x0, y1 = x0;
-      if (qr < B) {
-        const float4* src = reinterpret_cast<const float4*>(qpad + (size_t)qr * dpad + c0 + lp * 8);
-        x0 = src[0];
-        x1 = src[1];
-      }
-      if (kr < N) {
-        const float4* src = reinterpret_cast<const float4*>(keys + (size_t)kr * dpad + c0 + lp * 8);
-        y0 = src[0];
-        y1 = src[1];
-      }
-      const int j = lp * 8;
-      qs[j + 0][lr] = x0.x; qs[j + 1][lr] = x0.y; qs[j + 2][lr] = x0.z; qs[j + 3][lr] = x0.w;
-      qs[j + 4][lr] = x1.x; qs[j + 5][lr] = x1.y; qs[j + 6][lr] = x1.z; qs[j + 7][lr] = x1.w;
-      ks[j + 0][lr] = y0.x; ks[j + 1][lr] = y0.y; ks[j + 2][lr] = y0.z; ks[j + 3][lr] = y0.w;
-      ks[j + 4][lr] = y1.x; ks[j + 5][lr] = y1.y; ks[j + 6][lr] = y1.z; ks[j + 7][lr] = y1.w;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      qs[lp * 8 + u][lr] = x[u];
+      ks[lp * 8 + u][lr] = y[u];
     }
     __syncthreads();
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) p[a][b] = 0.f;
-#pragma unroll 8
-    for (int j = 0; j < 32; ++j) {
-      const float4 qv = *reinterpret_cast<const float4*>(&qs[j][tq * 4]);
-      const float4 kv = *reinterpret_cast<const float4*>(&ks[j][tk * 4]);
-      const float qa[4] = {qv.x, qv.y, qv.z, qv.w};
-      const float kb[4] = {kv.x, kv.y, kv.z, kv.w};
+    if (c0 + 32 < dpad) load(c0 + 32);
+    if (busy) {
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const float e = __fsub_rn(qa[a], kb[b]);
-          p[a][b] = __fmaf_rn(e, e, p[a][b]);
-        }
+        for (int b = 0; b < 4; ++b) p[a][b] = 0.f;
+#pragma unroll 8
+      for (int j = 0; j < 32; ++j) {
+        const float4 qv = *reinterpret_cast<const float4*>(&qs[j][tq * 4]);
+        const float4 kv = *reinterpret_cast<const float4*>(&ks[j][tk * 4]);
+        const float qa[4] = {qv.x, qv.y, qv.z, qv.w};
+        const float kb[4] = {kv.x, kv.y, kv.z, kv.w};
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            const float e = __fsub_rn(qa[a], kb[b]);
+            p[a][b] = __fmaf_rn(e, e, p[a][b]);
+          }
+      }
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) tot[a][b] = __fadd_rn(tot[a][b], p[a][b]);
     }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) tot[a][b] = __fadd_rn(tot[a][b], p[a][b]);
     __syncthreads();
   }
 #pragma unroll
   for (int b = 0; b < 4; ++b) {
-    const int64_t kr = k0 + tk * 4 + b;
-    if (kr >= N) continue;
-    const float thr = rr[kr];
+    const int64_t key = k0 + tk * 4 + b;
+    if (key >= N || !busy) continue;
+    const float thr = rr[key];
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
-      const int64_t qr = q0 + tq * 4 + a;
-      if (qr < B && tot[a][b] < thr) atomicMin(best + qr, pack_hit(tot[a][b], kr));
+      const int64_t row = q0 + tq * 4 + a;
+      if (row < B && tot[a][b] < thr) atomicMin(best + row, pack_hit(tot[a][b], key));
     }
   }
+  __shared__ int last_cta;
+  finalize_last_cta(out, gridDim.x * gridDim.y, &last_cta);
 }
 
-__global__ void k_finalize(const unsigned long long* __restrict__ best, int64_t B, const int32_t* __restrict__ label,
-                           int64_t* __restrict__ out_index, int32_t* __restrict__ out_label,
-                           float* __restrict__ out_dist, const DevStats* __restrict__ st) {
+__global__ void k_finalize(ProbeOut out) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= B) return;
-  unsigned long long v = best[q];
-  if (st->abort_flag) v = ~0ull;
-  if (v == ~0ull) {
-    out_index[q] = -1;
-    if (out_label) out_label[q] = -1;
-    if (out_dist) out_dist[q] = INFINITY;
-  } else {
-    const int64_t i = (int64_t)(v & 0xffffffffull);
-    out_index[q] = i;
-    if (out_label) out_label[q] = label[i];
-    if (out_dist) out_dist[q] = sqrtf(__uint_as_float((unsigned)(v >> 32)));
-  }
+  if (q < out.B) finalize_query(out, q, out.abort && *out.abort != 0);
 }
 
-void ensure_probe_scratch(lipcache* h, int64_t Bpad) {
+void ensure_probe_scratch(lipcache* h, int64_t Bpad, cudaStream_t s) {
   if (Bpad <= h->q_cap) return;
   int64_t cap = h->q_cap ? h->q_cap : 1024;
   while (cap < Bpad) cap *= 2;
@@ -215,6 +233,9 @@ void ensure_probe_scratch(lipcache* h, int64_t Bpad) {
     c.take(h->qscale, (size_t)cap);
     c.take(h->best, (size_t)cap);
   });
+  h->best_clean = false;
+  LC_CUDA(cudaMemsetAsync(h->best, 0xff, sizeof(unsigned long long) * (size_t)cap, s));
+  h->best_clean = true;
   h->q_cap = cap;
 }
 
@@ -223,7 +244,8 @@ void ensure_probe_scratch(lipcache* h, int64_t Bpad) {
 bool tensor_path_supported(int dpad) { return dpad <= 256; }
 
 void reserve_probe(lipcache* h, int64_t max_batch) {
-  ensure_probe_scratch(h, (max_batch + 127) / 128 * 128);
+  ensure_probe_scratch(h, (max_batch + 127) / 128 * 128, nullptr);
+  LC_CUDA(cudaStreamSynchronize(nullptr));  // (later probes may run on any stream)
 }
 
 // The small kernels around the tensor probe prefer the same shared-memory
@@ -241,24 +263,36 @@ void set_probe_carveout(lipcache* h) {
 }
 
 namespace {
-// The launch sequence of a probe on the given buffers.
-void probe_on(lipcache* h, int64_t B, const ProbeBuffers& b, int64_t* out_index, int32_t* out_label, float* out_dist,
-              bool timing, cudaStream_t s) {
+// The launch sequence of a probe on the given buffers. `clean`: every
+// reduction word is empty.
+void probe_on(lipcache* h, int64_t B, const ProbeBuffers& b, bool clean, int64_t* out_index, int32_t* out_label,
+              float* out_dist, bool timing, cudaStream_t s) {
   const int64_t Bpad = (B + 127) / 128 * 128;
   set_probe_carveout(h);
   int path = h->probe_path;
   if (path == LIPCACHE_PROBE_AUTO) path = auto_path(h, B);
   h->last_probe_path = path;
-  const bool f16 = path != LIPCACHE_PROBE_EXACT && h->f16_screen();
-  const unsigned pgrid = (unsigned)((Bpad + 7) / 8);
-  if (f16) {
-    k_prologue16<<<pgrid, 256, 0, s>>>(b.Q, B, h->d, h->table.d16, Bpad, static_cast<__half*>(b.q), b.kappa, b.scale,
-                                       b.best, 1.0 - h->c_scr, h->stats);
-    LC_LAUNCH_CHECK("k_prologue16");
+  const bool exact = path == LIPCACHE_PROBE_EXACT;
+  const bool f16 = !exact && h->f16_screen();
+  const int64_t ex = (h->size + kEK - 1) / kEK, ey = (B + kEQ - 1) / kEQ;  // the exact kernel's grid
+  ProbeOut out{b.best, B, h->table.label, out_index, out_label, out_dist, &h->stats->abort_flag, nullptr};
+  // the main kernel finalizes small batches itself (the exact one also only
+  // where its CTAs, which count themselves, are few)
+  if (h->size > 0 && B <= kFusedQueries && (!exact || ex * ey <= 4096)) out.done = &h->report->done_ctas;
+  if (exact || h->size == 0) {
+    if (!clean) LC_CUDA(cudaMemsetAsync(b.best, 0xff, sizeof(unsigned long long) * (size_t)B, s));
+    if (h->size == 0) LC_CUDA(cudaMemsetAsync(&h->stats->abort_flag, 0, sizeof(int), s));
   } else {
-    k_prologue<<<pgrid, 256, 0, s>>>(b.Q, B, h->d, h->dpad, Bpad, static_cast<float*>(b.q), b.kappa, b.best,
-                                     1.0 - h->c_scr, h->stats);
-    LC_LAUNCH_CHECK("k_prologue");
+    const unsigned pgrid = (unsigned)((Bpad + 7) / 8);
+    if (f16) {
+      k_prologue16<<<pgrid, 256, 0, s>>>(b.Q, B, h->d, h->table.d16, Bpad, static_cast<__half*>(b.q), b.kappa, b.scale,
+                                         b.best, 1.0 - h->c_scr, h->stats);
+      LC_LAUNCH_CHECK("k_prologue16");
+    } else {
+      k_prologue<<<pgrid, 256, 0, s>>>(b.Q, B, h->d, h->dpad, Bpad, static_cast<float*>(b.q), b.kappa, b.best,
+                                       1.0 - h->c_scr, h->stats);
+      LC_LAUNCH_CHECK("k_prologue");
+    }
   }
   if (h->size > 0) {
     int slot = -1;
@@ -267,19 +301,19 @@ void probe_on(lipcache* h, int64_t B, const ProbeBuffers& b, int64_t* out_index,
       slot = (int)(h->t_issued % lipcache::kTimingRing);
       h->t_kind[slot] = 0;
     }
-    if (path != LIPCACHE_PROBE_EXACT) {
+    if (!exact) {
       // the start event is recorded by the launcher, after its host-side
       // preparation, right before the kernel
       h->launch_event = slot >= 0 ? h->tev0[slot] : nullptr;
-      h->last_probe_path = launch_probe_tc(h, B, path, f16, b, s);
+      h->last_probe_path = launch_probe_tc(h, B, path, f16, b, out, s);
       h->launch_event = nullptr;
     } else {
       if (slot >= 0) LC_CUDA(cudaEventRecord(h->tev0[slot], s));
-      dim3 grid((unsigned)((h->size + kEK - 1) / kEK), (unsigned)((B + kEQ - 1) / kEQ));
-      h->last_grid = (int)(grid.x * grid.y);
+      h->last_grid = (int)(ex * ey);
       h->last_cluster = 1;
-      k_probe_exact<<<grid, 256, 0, s>>>(static_cast<float*>(b.q), B, h->table.keys, h->probe_rr(), h->size, h->dpad,
-                                         b.best);
+      const int qvec = h->d % 4 == 0 && ((uintptr_t)b.Q & 15) == 0;
+      k_probe_exact<<<dim3((unsigned)ex, (unsigned)ey), 256, 0, s>>>(b.Q, B, h->d, qvec, h->table.keys, h->probe_rr(),
+                                                                     h->size, h->dpad, b.best, out, h->stats);
       LC_LAUNCH_CHECK("k_probe_exact");
     }
     if (slot >= 0) {
@@ -287,16 +321,22 @@ void probe_on(lipcache* h, int64_t B, const ProbeBuffers& b, int64_t* out_index,
       ++h->t_issued;
     }
   }
-  k_finalize<<<(unsigned)((B + 255) / 256), 256, 0, s>>>(b.best, B, h->table.label, out_index, out_label, out_dist,
-                                                         h->stats);
-  LC_LAUNCH_CHECK("k_finalize");
+  if (!out.done) {
+    k_finalize<<<(unsigned)((B + 255) / 256), 256, 0, s>>>(out);
+    LC_LAUNCH_CHECK("k_finalize");
+  }
 }
 }  // namespace
 
 void probe(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* out_label, float* out_dist,
            cudaStream_t s) {
-  ensure_probe_scratch(h, (B + 127) / 128 * 128);
-  probe_on(h, B, ProbeBuffers{Q, h->qpad, h->kappa, h->qscale, h->best}, out_index, out_label, out_dist, true, s);
+  ensure_probe_scratch(h, (B + 127) / 128 * 128, s);
+  // (the finalizing kernel empties the words it reads; a call that throws on
+  // the way leaves them in doubt)
+  const bool clean = h->best_clean;
+  h->best_clean = false;
+  probe_on(h, B, ProbeBuffers{Q, h->qpad, h->kappa, h->qscale, h->best}, clean, out_index, out_label, out_dist, true, s);
+  h->best_clean = true;
 }
 
 // The same launch sequence as probe(), on scratch memory the caller
@@ -306,7 +346,7 @@ void probe(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* 
 void probe_external_scratch(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* out_label,
                             float* out_dist, float* qpad, float* kappa, float* qscale, unsigned long long* best,
                             cudaStream_t s) {
-  probe_on(h, B, ProbeBuffers{Q, qpad, kappa, qscale, best}, out_index, out_label, out_dist, false, s);
+  probe_on(h, B, ProbeBuffers{Q, qpad, kappa, qscale, best}, false, out_index, out_label, out_dist, false, s);
 }
 
 }  // namespace lc

@@ -20,6 +20,56 @@ __device__ __forceinline__ unsigned long long pack_hit(float dist2, int64_t inde
 // chunk sums added in order. Every probe path evaluates exactly this
 // sequence of rounded operations, so all paths agree bit for bit.
 //
+// Where a probe's results go, and the counter of finished CTAs for the kernels
+// that finalize themselves.
+struct ProbeOut {
+  unsigned long long* best;
+  int64_t B;
+  const int32_t* label;  // per entry
+  int64_t* index;
+  int32_t* out_label;  // nullable
+  float* dist;         // nullable
+  const int* abort;    // nullable: non-zero turns the batch into misses
+  unsigned* done;      // zero between launches; null: k_finalize follows
+};
+
+// Unpack query q's word, and leave it empty for the next batch.
+__device__ __forceinline__ void finalize_query(const ProbeOut& o, int64_t q, bool aborted) {
+  unsigned long long v = __ldcg(o.best + q);
+  o.best[q] = ~0ull;
+  if (aborted) v = ~0ull;
+  if (v == ~0ull) {
+    o.index[q] = -1;
+    if (o.out_label) o.out_label[q] = -1;
+    if (o.dist) o.dist[q] = INFINITY;
+  } else {
+    const int64_t i = (int64_t)(v & 0xffffffffull);
+    o.index[q] = i;
+    if (o.out_label) o.out_label[q] = o.label[i];
+    if (o.dist) o.dist[q] = sqrtf(__uint_as_float((unsigned)(v >> 32)));
+  }
+}
+
+// Called by every thread of every CTA after the CTA's last update of `best`:
+// the CTA that comes last finalizes the batch (a launch less than a kernel of
+// its own; batches of at most kFusedQueries, which one CTA unpacks in ~2 us).
+// `last_cta`: a word of shared memory.
+constexpr int64_t kFusedQueries = 2048;
+__device__ __forceinline__ void finalize_last_cta(const ProbeOut& o, unsigned n_ctas, volatile int* last_cta) {
+  if (!o.done) return;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    *last_cta = atomicAdd(o.done, 1u) == n_ctas - 1 ? 1 : 0;
+  }
+  __syncthreads();
+  if (!*last_cta) return;
+  __threadfence();
+  const bool aborted = o.abort && __ldcg(o.abort) != 0;
+  for (int64_t q = threadIdx.x; q < o.B; q += blockDim.x) finalize_query(o, q, aborted);
+  if (threadIdx.x == 0) *o.done = 0u;
+}
+
 // One 32-wide chunk of that sequence, features [c, c + n) of a query and a key;
 // features past the query's d, zero in both rows, add exact zeros and are left
 // out. vec: the query row is 16-byte aligned and n a multiple of 4 (key rows

@@ -74,6 +74,7 @@ struct PairArgs {
   const float* tau;
   const float* rr;
   unsigned long long* best;
+  ProbeOut out;
   DevStats* stats;
   int debug_stall;  // test hook: the MMA issuer first waits on a barrier nothing arrives on
 };
@@ -157,6 +158,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   ptx::tc_fence_after();
   ptx::cluster_sync();  // every barrier of the cluster exists before any copy or arrival targets it
+  ptx::wait_prerequisites();  // the prologue's queries, constants and reduction words
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
@@ -376,6 +378,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     ptx::tc_fence_after();
     ptx::tmem_dealloc_pair(tmem, (uint32_t)kTmemCols);
   }
+  finalize_last_cta(a.out, gridDim.x, abort_s + 1);
 }
 
 cudaLaunchConfig_t pair_config(int smem, cudaStream_t s, cudaLaunchAttribute* attr) {
@@ -422,7 +425,7 @@ int probe_pair_clusters(lipcache* h, bool f16) {
   return resident;
 }
 
-void launch_probe_pair(lipcache* h, int64_t B, bool f16, const ProbeBuffers& b, cudaStream_t s) {
+void launch_probe_pair(lipcache* h, int64_t B, bool f16, const ProbeBuffers& b, const ProbeOut& out, cudaStream_t s) {
   const int clusters_max = probe_pair_clusters(h, f16);
   LC_REQUIRE(clusters_max >= 1, LIPCACHE_E_CUDA, "no cluster of the pair probe kernel fits on this device");
   const int64_t Bpad = (B + 127) / 128 * 128;  // rows of the padded query buffer
@@ -479,6 +482,7 @@ void launch_probe_pair(lipcache* h, int64_t B, bool f16, const ProbeBuffers& b, 
   a.tau = h->probe_tau();
   a.rr = h->probe_rr();
   a.best = b.best;
+  a.out = out;
   a.stats = h->stats;
   a.debug_stall = (h->debug_flags & LIPCACHE_DEBUG_STALL_PROBE) ? 1 : 0;
   const int smem = PairLayout{a.nch, a.nst}.total() + 1024;
@@ -488,8 +492,11 @@ void launch_probe_pair(lipcache* h, int64_t B, bool f16, const ProbeBuffers& b, 
     LC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 1024));
     pl.smem[0] = true;
   }
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = pair_config(smem, s, attr);
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 2;
   int clusters = clusters_max;
   if (n_units < clusters) clusters = (int)n_units;
   cfg.gridDim = dim3((unsigned)(clusters * kCluster));

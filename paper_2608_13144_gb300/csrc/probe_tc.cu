@@ -94,6 +94,7 @@ struct TcArgs {
   const float* tau;
   const float* rr;
   unsigned long long* best;
+  ProbeOut out;
   DevStats* stats;
   int queue;        // candidates go to the recheck warp (ranges of several tiles)
   int debug_stall;  // test hook: the MMA issuer first waits on a barrier nothing arrives on
@@ -224,6 +225,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   ptx::tc_fence_after();
   ptx::cluster_sync();  // the peer's barriers exist before any multicast reaches them
+  ptx::wait_prerequisites();  // the prologue's queries, constants and reduction words
   const uint32_t tmem = *tmem_slot;
 
   const Recheck rck{a.q, KIND == kF16 ? a.d : a.dpad, KIND == kF16 ? a.qvec != 0 : true, a.keys, a.dpad, a.d, a.rr, a.best};
@@ -583,10 +585,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, (uint32_t)Layout<BN>::kTmemCols);
   }
+  finalize_last_cta(a.out, gridDim.x, abort_s + 1);
 }
 
 template <int BN, int KIND, int NH>
-void launch_nh(lipcache* h, int64_t B, const ProbeBuffers& b, bool long_ranges, cudaStream_t s) {
+void launch_nh(lipcache* h, int64_t B, const ProbeBuffers& b, const ProbeOut& out, bool long_ranges, cudaStream_t s) {
   constexpr bool f16 = KIND == kF16;
   const int64_t Bpad = (B + kBM - 1) / kBM * kBM;
   lipcache::ProbeLaunch& pl = h->probe_launch[(BN == 256 ? 0 : 1) + (f16 ? 3 : 0)];
@@ -632,6 +635,7 @@ void launch_nh(lipcache* h, int64_t B, const ProbeBuffers& b, bool long_ranges, 
   a.tau = h->probe_tau();
   a.rr = h->probe_rr();
   a.best = b.best;
+  a.out = out;
   a.stats = h->stats;
   // With one to three tiles per cluster the recheck warp's turn would only come
   // at the end: 256 x 50,000 at d = 64 13.4 us without it, 15.0 with; 1,024 x
@@ -658,13 +662,16 @@ void launch_nh(lipcache* h, int64_t B, const ProbeBuffers& b, bool long_ranges, 
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = (size_t)smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = kCluster;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  // starts its setup behind the prologue kernel's last wave
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   // persistent grid: no more clusters than can be resident at once (asked for
   // with the most shared memory any launch uses)
   if (pl.resident == 0) {
@@ -684,21 +691,22 @@ void launch_nh(lipcache* h, int64_t B, const ProbeBuffers& b, bool long_ranges, 
       a.tau_staged       ? k_probe_tc<BN, kM0, KIND, NH>
       : a.qgroup == 2 ? k_probe_tc<BN, 2, KIND, NH>
                       : k_probe_tc<BN, 1, KIND, NH>;
+  cfg.numAttrs = 2;
   LC_CUDA(cudaLaunchKernelEx(&cfg, kern, pl.tmQ, pl.tmK, a));
   LC_LAUNCH_CHECK("k_probe_tc");
 }
 
 template <int BN, int KIND>
-void launch(lipcache* h, int64_t B, const ProbeBuffers& b, cudaStream_t s) {
+void launch(lipcache* h, int64_t B, const ProbeBuffers& b, const ProbeOut& out, cudaStream_t s) {
   const int max_clusters = h->num_sms / kCluster;
   LC_REQUIRE(max_clusters >= 1, LIPCACHE_E_CUDA, "device has fewer than two SMs");
   const int64_t nq = (B + kBM - 1) / kBM, n_kt = (h->size + BN - 1) / BN;
   const bool long_ranges = (n_kt + kCluster - 1) / kCluster * nq / max_clusters >= kPairedReleaseItems;
   if constexpr (KIND == kF16 && BN == 256) {
     // two key tiles side by side leave a ring of six stages or more
-    if (long_ranges && h->table.d16 <= 128) return launch_nh<BN, KIND, 2>(h, B, b, true, s);
+    if (long_ranges && h->table.d16 <= 128) return launch_nh<BN, KIND, 2>(h, B, b, out, true, s);
   }
-  launch_nh<BN, KIND, 1>(h, B, b, long_ranges, s);
+  launch_nh<BN, KIND, 1>(h, B, b, out, long_ranges, s);
 }
 
 }  // namespace
@@ -718,7 +726,8 @@ void encode_screen_map(lipcache* h, CUtensorMap* map, const void* base, uint64_t
   LC_REQUIRE(r == CUDA_SUCCESS, LIPCACHE_E_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
 }
 
-int launch_probe_tc(lipcache* h, int64_t B, int path, bool f16, const ProbeBuffers& b, cudaStream_t s) {
+int launch_probe_tc(lipcache* h, int64_t B, int path, bool f16, const ProbeBuffers& b, const ProbeOut& out,
+                    cudaStream_t s) {
   LC_REQUIRE(f16 || tensor_path_supported(h->dpad), LIPCACHE_E_INVALID, "the tensor probe supports d <= 256");
   // A 256-key tile of up to four chunks (d <= 256 in FP16, 128 in TF32) stays
   // beside a deep query ring: single-CTA MMAs on all SMs. Longer rows would
@@ -728,19 +737,19 @@ int launch_probe_tc(lipcache* h, int64_t B, int path, bool f16, const ProbeBuffe
   const bool short_rows = f16 ? h->table.d16 <= 256 : h->dpad <= 128;
   const bool pair = path == LIPCACHE_PROBE_TENSOR_PAIR || (path == LIPCACHE_PROBE_TENSOR && !short_rows);
   if (pair && probe_pair_clusters(h, f16) >= 1) {
-    launch_probe_pair(h, B, f16, b, s);
+    launch_probe_pair(h, B, f16, b, out, s);
     return LIPCACHE_PROBE_TENSOR_PAIR;
   }
   if (f16) {
     if (short_rows)
-      launch<256, kF16>(h, B, b, s);
+      launch<256, kF16>(h, B, b, out, s);
     else
-      launch<128, kF16>(h, B, b, s);
+      launch<128, kF16>(h, B, b, out, s);
   } else {
     if (short_rows)
-      launch<256, kTf32>(h, B, b, s);
+      launch<256, kTf32>(h, B, b, out, s);
     else
-      launch<128, kTf32>(h, B, b, s);
+      launch<128, kTf32>(h, B, b, out, s);
   }
   return LIPCACHE_PROBE_TENSOR_SINGLE;
 }

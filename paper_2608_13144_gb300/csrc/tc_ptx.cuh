@@ -87,6 +87,14 @@ __device__ __forceinline__ void tma_load_2d_multicast(uint32_t dst, const CUtens
       : "memory");
 }
 
+// ---------------------------------------------------------------- dependent launch
+// Let the kernel launched behind this one, with the programmatic attribute,
+// start as soon as every block of this one has got here.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// In that kernel: wait until the one before it has ended and its writes are
+// visible.
+__device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------- clusters
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;

@@ -184,3 +184,33 @@ def test_extreme_queries(dev):
     ref = same_as_exact(c, torch.from_numpy(Q).to(dev), ["tensor", "tensor_pair"])
     assert np.all(ref[0][10:13] == -1)
     c.close()
+
+
+@pytest.mark.parametrize("d,n,nq", [(64, 2000, 1), (20, 300, 65), (33, 5000, 2048), (33, 5000, 2049), (1000, 700, 30)])
+def test_batches_in_a_row(dev, d, n, nq):
+    """Batches of different sizes and paths follow one another on one handle
+    (the exact kernel counts on the words the batch before left empty; kernels
+    finalize batches of up to 2,048 themselves), an empty cache among them:
+    each answers as a fresh cache does."""
+    from paper_2608_13144_gb300.lipcache import LipCache
+    rng = np.random.default_rng(d + nq)
+    rows, Q = data(rng, n, d, nq)
+    c = make(dev, d, 5, rows)
+    Qd = torch.from_numpy(Q).to(dev)
+    for path in ("exact", "auto"):  # empty cache: misses
+        c.set_probe_path(path)
+        assert (c.probe(Qd)[0].cpu().numpy() == -1).all()
+    c.insert(torch.from_numpy(rows).to(dev))
+    fresh = make(dev, d, 5, rows)
+    fresh.insert(torch.from_numpy(rows).to(dev))
+    fresh.set_probe_path("exact")
+    ref = [t.cpu().numpy() for t in fresh.probe(Qd)]
+    paths = ["exact", "auto"] + (["tensor", "tensor_pair"] if d <= 256 else [])
+    for path in paths + paths[::-1]:
+        c.set_probe_path(path)
+        for k in (1, nq, max(1, nq // 2)):
+            got = [t.cpu().numpy() for t in c.probe(Qd[:k])]
+            for x, y in zip(ref, got):
+                assert np.array_equal(x[:k].view(np.uint8), y.view(np.uint8)), (path, k)
+    c.close()
+    fresh.close()

@@ -446,8 +446,9 @@ lipcache_status lipcache_set_probe_path(lipcache_t* h, int32_t path);
  * afterwards are multiplied by kappa. Only while the cache is empty. */
 lipcache_status lipcache_set_radius_scale(lipcache_t* h, double kappa);
 
-/* Options of the spectral norm sigma_max(W) (Sec. 4.1, Eqs. 17-19):
- * `squarings` (0..60) normalised squarings of W^T W before the power
+/* Options of the spectral norm sigma_max(W) (Sec. 4.1, Eqs. 17-19): at most
+ * `squarings` (0..60) normalised squarings of W^T W (fewer once the result is
+ * a projector to FP64's resolution) before the power
  * iteration and `max_iter` (>= 1) power iterations. */
 lipcache_status lipcache_set_spectral_options(lipcache_t* h, int32_t squarings, int32_t max_iter);
 

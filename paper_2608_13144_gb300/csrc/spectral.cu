@@ -6,7 +6,8 @@
 // about log(tol) / log(lambda_2/lambda_1) steps, which is thousands for the
 // small spectral gaps of Gaussian heads, so the start vector is produced by
 // `squarings` normalised squarings A_{k+1} = (A_k / tr A_k)^2, i.e. by the
-// power iteration with A^(2^k) (2^40 steps for the default 40). The final
+// power iteration with A^(2^k) (up to 2^40 steps for the default 40; it stops
+// once A_k is a projector to FP64's resolution). The final
 // iteration then runs on W itself (w = W v, theta = ||w||^2 = v^T A v,
 // u = W^T w) until successive Rayleigh quotients agree to 1e-13 relative and
 // ||A v - theta v|| <= 1e-10 theta.
@@ -115,6 +116,26 @@ struct SpectralArgs {
 // power-of-two length apart cost 80 cycles a request at d = 256).
 __device__ __forceinline__ size_t blk(int k, int j, int K) { return ((size_t)(j >> 5) * K + k) * 32 + (j & 31); }
 
+// One warp: red[1] = tr S (blocked layout), red[0] = 1 / tr S, or 0 for a zero
+// trace (W = 0), which gives a zero product.
+__device__ void trace_inv(const double* S, int d, int lane, double* red) {
+  double v[8];
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    const int k = lane + 32 * m;
+    v[m] = k < d ? __ldcg(S + blk(k, k, d)) : 0.0;
+  }
+  if (d > 256)
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+      for (int k = lane + 32 * m + 256; k < d; k += 256) v[m] += __ldcg(S + blk(k, k, d));
+  const double tr = tree256(v, d);
+  if (lane == 0) {
+    red[0] = tr > 0.0 ? 1.0 / tr : 0.0;
+    red[1] = tr;
+  }
+}
+
 // The symmetric product P_ij = sum_k X[k][i] X[k][j] (k < K ascending, one
 // fused multiply-add chain per element) into B, X = S (K rows, blocked
 // layout) or, with `scale`, S * (1 / tr S) rounded: S is symmetric or is the operand
@@ -164,22 +185,9 @@ __device__ void sym_product(const double* S, int K, bool scale, double* B, int d
       }
       if (!have_inv) {
         // the trace, while the panels are on their way
-        if (warp == 0) {
-          double v[8];
-#pragma unroll
-          for (int m = 0; m < 8; ++m) {
-            const int k = lane + 32 * m;
-            v[m] = k < d ? __ldcg(S + blk(k, k, d)) : 0.0;
-          }
-          if (d > 256)
-#pragma unroll
-            for (int m = 0; m < 8; ++m)
-              for (int k = lane + 32 * m + 256; k < d; k += 256) v[m] += __ldcg(S + blk(k, k, d));
-          const double tr = tree256(v, d);
-          if (lane == 0) *red = tr > 0.0 ? 1.0 / tr : 0.0;  // a zero trace (W = 0) gives a zero product
-        }
+        if (warp == 0) trace_inv(S, d, lane, red);
         __syncthreads();
-        inv = *red;
+        inv = red[0];
         have_inv = true;
       }
       if (scale) {
@@ -223,8 +231,7 @@ __device__ void sym_product(const double* S, int K, bool scale, double* B, int d
 // `squarings` steps A <- (A / tr A)^2, then the power iteration on W. What
 // bounds it: the FP64 pipe (four warps per SM: ~88 cycles per step of their
 // chains); a squaring costs its d steps, the panel's scaling (1 / (4 R) of the
-// products), the trace and one grid barrier. Everything is added in the order
-// of the tests' saved caches: sigma keeps its bits.
+// products), the trace and one grid barrier.
 template <int R>
 __global__ void __launch_bounds__(kSpThreads) k_spectral(const SpectralArgs a) {
   __shared__ double sm[kSpChunk * 32 + kSpChunk * kSpWarps * R];
@@ -245,7 +252,7 @@ __global__ void __launch_bounds__(kSpThreads) k_spectral(const SpectralArgs a) {
   }
   if (!sync_grid()) return;
   // A grid with fewer tiles than CTAs (units of the iteration): the spare CTAs
-  // only meet the barriers.
+  // only follow the traces and meet the barriers.
   int cur = 0;
   if (a.squarings > 0) {
     // W^T W: products of FP32 values are exact in FP64
@@ -253,8 +260,20 @@ __global__ void __launch_bounds__(kSpThreads) k_spectral(const SpectralArgs a) {
     if (!sync_grid()) return;
     for (int q = 0; q < a.squarings; ++q) {
       sym_product<R>(a.A[cur], d, true, a.A[cur ^ 1], d, a.n_tiles, sm, red);
+      if ((int)blockIdx.x >= a.n_tiles) {  // a spare CTA follows the traces
+        if (warp == 0) trace_inv(a.A[cur], d, lane, red);
+        __syncthreads();
+      }
       cur ^= 1;
+      const double tr = red[1];  // of the matrix just squared
       if (!sync_grid()) return;
+      // A square of unit trace is, from its trace t = sum l_i^2 (l_1 >= ...
+      // summing to 1), the projector on the dominant direction up to
+      // (1 - t) / 2 relative; the square just formed from it is up to the
+      // square of that, below FP64's resolution. Gaussian heads take 10 to 14
+      // steps; a (nearly) repeated largest singular value keeps t away from 1
+      // and takes them all.
+      if (q > 0 && 1.0 - tr <= 1e-9) break;
     }
   }
 

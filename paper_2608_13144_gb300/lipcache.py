@@ -246,14 +246,15 @@ class LipCache:
         """Restore a checkpoint written by save: create, set_head, re-insert
         the keys with their labels as payload (Algorithm 1 again), restore
         the probe path and radius policy. Raises if sigma differs from the
-        saved one or a radius by more than 4 units in its last place (which
+        saved one by more than 1e-12 (its iteration's accuracy) or a radius
+        by more than 4 units in its last place (which
         certify kernel takes a batch depends on its size and alignment, and
         their refinements round differently in the last place)."""
         z = np.load(path if str(path).endswith(".npz") else str(path) + ".npz")
         c = cls(int(z["d"]), int(z["C"]), int(z["capacity"]), str(z["radius_mode"]), device=device)
         c.set_radius_scale(float(z["radius_scale"]))
         sigma = c.set_head(torch.from_numpy(z["W"]).to(c.device), torch.from_numpy(z["b"]).to(c.device))
-        if sigma != float(z["sigma"]):
+        if not abs(sigma - float(z["sigma"])) <= 1e-12 * sigma:
             raise ValueError(f"sigma of the restored head {sigma!r} differs from the saved {float(z['sigma'])!r}")
         keys, label = z["keys"], z["label"]
         for s in range(0, len(keys), batch):

@@ -84,6 +84,8 @@ def test_sigma_tile_edges(dev, C, d, squarings):
     rng = np.random.default_rng(C * 1000 + d)
     W = (rng.standard_normal((C, d)) / np.sqrt(d)).astype(np.float32)
     W[0] *= 3.0  # a gap the plain iteration (no squarings) converges on
+    if d >= 32 and C >= 33:
+        W[1] = W[2] * np.float32(1.0001)  # (a close pair below the top one)
     c = LipCache(d, C, 8, device=dev)
     c.set_spectral_options(squarings, 1000)
     sigma = c.set_head(T(W, dev), T(np.zeros(C, np.float32), dev))

@@ -219,6 +219,14 @@ __device__ __forceinline__ float4 lds_f4(uint32_t addr) {
   return v;
 }
 
+// A 32-byte sector of read-only global memory in one load, issued where the
+// program says (the compiler otherwise sinks prefetches to their use).
+__device__ __forceinline__ void ldg_f8(const float* p, float4& v0, float4& v1) {
+  asm volatile("ld.global.nc.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(v0.x), "=f"(v0.y), "=f"(v0.z), "=f"(v0.w), "=f"(v1.x), "=f"(v1.y), "=f"(v1.z), "=f"(v1.w)
+               : "l"(p));
+}
+
 // Named barrier of the two epilogue warps of one lane quarter.
 __device__ __forceinline__ void pair_barrier(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
 
@@ -492,25 +500,23 @@ __device__ __forceinline__ void refine_lane(const WA& wa, uint32_t zs, int c, in
       z1 = nz1;
     }
   } else {
-    // the head's row comes from L2: kAheadG spans in flight
+    // the head's row comes from L2: kAheadG spans in flight, a whole sector per
+    // load (two 16-byte loads of it took 57.8 k cycles a tile and warp at
+    // d = 256, C = 200, tight; this takes 47.0 k)
     constexpr int kAheadG = 4;
-    const float4* wg = reinterpret_cast<const float4*>(wa.w + (size_t)c * wa.ws);
+    const float* wg = wa.w + (size_t)c * wa.ws;
     float4 w0[kAheadG], w1[kAheadG];
 #pragma unroll
-    for (int u = 0; u < kAheadG; ++u) {
-      const int n = u < nsp ? u : 0;
-      w0[u] = __ldg(wg + 2 * n);
-      w1[u] = __ldg(wg + 2 * n + 1);
-    }
+    for (int u = 0; u < kAheadG; ++u) ldg_f8(wg + 8 * (u < nsp ? u : 0), w0[u], w1[u]);
     for (int i = 0; i < nsp; i += kAheadG) {
 #pragma unroll
       for (int u = 0; u < kAheadG; ++u) {
         if (i + u < nsp) {  // (nsp is the same for every lane)
           const uint32_t ca = az(i + u);
-          span(w0[u], w1[u], lds_f4(ca), lds_f4(ca ^ 16u));
-          const int n = i + u + kAheadG < nsp ? i + u + kAheadG : 0;
-          w0[u] = __ldg(wg + 2 * n);
-          w1[u] = __ldg(wg + 2 * n + 1);
+          const float4 x0 = w0[u], x1 = w1[u];
+          const float4 z0 = lds_f4(ca), z1 = lds_f4(ca ^ 16u);
+          ldg_f8(wg + 8 * (i + u + kAheadG < nsp ? i + u + kAheadG : 0), w0[u], w1[u]);
+          span(x0, x1, z0, z1);
         }
       }
     }
@@ -637,24 +643,38 @@ __device__ bool tc_tight_row_warp(const CertArgs& a, int64_t row, int rz, const 
   const int d = a.d, C = a.C;
   const int g8 = lane / kGroupTc, sub = lane % kGroupTc;
   const float hn = norm_upper(kn);
-  for (int c0 = 0; c0 < C; c0 += 2 * (32 / kGroupTc)) {
-    int cp[2];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int c = c0 + 2 * g8 + u;
-      cp[u] = c < C ? c : C - 1;  // a valid class; the result is not stored
+  if constexpr (!std::is_same<WA, WSm>::value) {
+    // the head's rows come from L2: a class per lane (refine_lane, the same
+    // bits) keeps 32 rows' loads in flight, two per 8-lane group eight
+    for (int c0 = 0; c0 < C; c0 += 32) {
+      const int c = c0 + lane < C ? c0 + lane : C - 1;
+      float hi, lo;
+      refine_lane(wa, zs, c, rz, b_s[c], d, hi, lo);
+      if (c0 + lane < C) {
+        res_hi[c] = hi;
+        res_lo[c] = lo;
+      }
     }
-    const int rp[2] = {rz, rz};
-    const float bp[2] = {b_s[cp[0]], b_s[cp[1]]};
-    float hi[2], lo[2];
-    refine2(wa, zs, cp, rp, bp, d, sub, hi, lo);
-    if (sub == 0)
-#pragma unroll
-      for (int u = 0; u < 2; ++u)
-        if (c0 + 2 * g8 + u < C) {
-          res_hi[c0 + 2 * g8 + u] = hi[u];
-          res_lo[c0 + 2 * g8 + u] = lo[u];
-        }
+  } else {
+    for (int c0 = 0; c0 < C; c0 += 2 * (32 / kGroupTc)) {
+      int cp[2];
+  #pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int c = c0 + 2 * g8 + u;
+        cp[u] = c < C ? c : C - 1;  // a valid class; the result is not stored
+      }
+      const int rp[2] = {rz, rz};
+      const float bp[2] = {b_s[cp[0]], b_s[cp[1]]};
+      float hi[2], lo[2];
+      refine2(wa, zs, cp, rp, bp, d, sub, hi, lo);
+      if (sub == 0)
+  #pragma unroll
+        for (int u = 0; u < 2; ++u)
+          if (c0 + 2 * g8 + u < C) {
+            res_hi[c0 + 2 * g8 + u] = hi[u];
+            res_lo[c0 + 2 * g8 + u] = lo[u];
+          }
+    }
   }
   __syncwarp();
   float vh[kPer], vl[kPer], ve[kPer];
@@ -723,7 +743,7 @@ __device__ bool tc_tight_row_warp(const CertArgs& a, int64_t row, int rz, const 
 // chunks stream through a ring for the MMAs, tile after tile, and the
 // refinement reads its rows from L2, four 32-byte spans ahead. It replaces FP32
 // logits on the CUDA cores with FP64 sums: 100,000 rows, d = 256, C = 200, tight
-// radius, 72.8 ms then, 0.59 ms now (floor: 30 us of HBM, 11 us of TF32).
+// radius, 72.8 ms then, 0.60 ms now (floor: 30 us of HBM, 11 us of TF32).
 // Bound by the epilogue, as the resident kernel, plus the L2 latency of the
 // head's rows.
 template <bool TIGHT, bool WSTREAM>
@@ -1476,16 +1496,40 @@ __global__ void __launch_bounds__(kThreads, 1)
           const double vy = (double)v2.x + (double)v2.y;
           const double ey = (double)refined_err(a.g2f8, wn_s[yg], hn, bias_s[yg]);
           any_nan = any_nan || !(vy == vy);
-          // unrolled over the slots so that the pair-table loads of all
-          // candidates are in flight together
+          // FP64 runs at ~22 cycles of the SM per warp instruction, so the terms
+          // of Eq. 29 are bracketed in FP32 first, rounded outwards from the
+          // refined values and their errors (u_j above the FP64 term, l_j below
+          // its certified lower bound): only a candidate with l_j <= min u can
+          // have either minimum, usually one per row. The same minima. (65,536 rows
+          // of d = 128, C = 200: 136 us without the bracket, 126 us with it;
+          // 50,000 of d = 64, C = 10: 47 and 39.5 us.)
+          // (unrolled, so that the table loads of all candidates are in flight)
+          const float eyf = refined_err(a.g2f8, wn_s[yg], hn, bias_s[yg]);
+          const float vyu = __fadd_ru(v2.x, __fadd_ru(v2.y, eyf)), vyd = __fadd_rd(v2.x, __fsub_rd(v2.y, eyf));
+          float U = INFINITY, lj[kMaxCandTc];
 #pragma unroll
           for (int sl = 0; sl < kMaxCandTc; ++sl) {
             const int j = slot_class(sl);
+            lj[sl] = INFINITY;
             if (sl < ns && j != yg) {
-              const double vj = (double)res_hi[lane + 32 * sl] + (double)res_lo[lane + 32 * sl];
-              any_nan |= !(vj == vj);
-              tight_term(a, yg, j, vy, ey, vj, (double)refined_err(a.g2f8, wn_s[j], hn, bias_s[j]), rmin, smin);
+              const float iu = __ldg(a.ipn_up32 + (size_t)yg * C + j), il = __ldg(a.ipn_dn32 + (size_t)yg * C + j);
+              const float h = res_hi[lane + 32 * sl], l = res_lo[lane + 32 * sl];
+              const float e = refined_err(a.g2f8, wn_s[j], hn, bias_s[j]);
+              any_nan |= !(h == h && l == l);
+              if (iu < INFINITY) {  // (else W_j = W_y: no term)
+                const float dn = __fsub_rd(vyd, __fadd_ru(h, __fadd_ru(l, e)));
+                U = fminf(U, __fmul_ru(__fsub_ru(vyu, __fadd_rd(h, __fsub_rd(l, e))), iu));
+                lj[sl] = dn > 0.f ? __fmul_rd(dn, il) : -INFINITY;
+              }
             }
+          }
+          uint32_t left = 0;
+#pragma unroll
+          for (int sl = 0; sl < kMaxCandTc; ++sl) left |= (uint32_t)(lj[sl] <= U && lj[sl] < INFINITY) << sl;
+          for (; left; left &= left - 1) {
+            const int sl = __ffs((int)left) - 1, j = slot_class(sl);
+            const double vj = (double)res_hi[lane + 32 * sl] + (double)res_lo[lane + 32 * sl];
+            tight_term(a, yg, j, vy, ey, vj, (double)refined_err(a.g2f8, wn_s[j], hn, bias_s[j]), rmin, smin);
           }
         }
         const unsigned fbm = __ballot_sync(kFull, rowfb);

@@ -2,14 +2,15 @@
 // f(z) = W z + b (Sec. 4.1, Eqs. 17-19; the bias cancels in logit
 // differences). Algorithm 1 computes it once per cache, before any radius.
 //
-// Method: power iteration on A = W^T W in FP64. Power iteration alone needs
+// Method: power iteration on A = X^T X in FP64, X = W or W^T, whichever has
+// fewer columns (the singular values are the same). Power iteration alone needs
 // about log(tol) / log(lambda_2/lambda_1) steps, which is thousands for the
 // small spectral gaps of Gaussian heads, so the start vector is produced by
-// `squarings` normalised squarings A_{k+1} = (A_k / tr A_k)^2, i.e. by the
+// `squarings` normalised squarings A_{k+1} = (A_k 2^-e)^2, 2^e <= tr A_k < 2^(e+1), i.e. by the
 // power iteration with A^(2^k) (up to 2^40 steps for the default 40; it stops
 // once A_k is a projector to FP64's resolution). The final
-// iteration then runs on W itself (w = W v, theta = ||w||^2 = v^T A v,
-// u = W^T w) until successive Rayleigh quotients agree to 1e-13 relative and
+// iteration then runs on X itself (w = X v, theta = ||w||^2 = v^T A v,
+// u = X^T w) until successive Rayleigh quotients agree to 1e-13 relative and
 // ||A v - theta v|| <= 1e-10 theta.
 //
 // FP64 on this GPU: a dependent instruction takes ~64 cycles, and four warps of
@@ -98,15 +99,17 @@ __device__ double chain16(const double* col, size_t stride, const double* x, int
   return acc;
 }
 
+// X (m x n) is W (C x d) or its transpose.
 struct SpectralArgs {
-  const float* W;  // C x d
-  int C, d, Cp, dp;  // Cp, dp: C, d rounded up to 32
+  const float* W;
+  int m, n, mp, np;  // mp, np: m, n rounded up to 32
+  int rs, cs;        // X(r, j) = W[r rs + j cs]
   int squarings, max_iter, n_tiles;
-  double* A[2];    // d x dp, blocked layout (columns from d on are never read into a result)
-  double* Wd;      // C x dp, blocked layout: the head in FP64, zero past d
-  double* WdT;     // d x Cp, zero past C
-  double* w;       // C
-  double* u;       // d
+  double* A[2];    // n x np, blocked layout (columns from n on are never read into a result)
+  double* X;       // m x np, blocked layout: X in FP64, zero past n
+  double* XT;      // n x mp, zero past m
+  double* w;       // m
+  double* u;       // n
   unsigned* ctr;   // grid barrier, zero at launch
   SpecResult* res;
 };
@@ -116,29 +119,35 @@ struct SpectralArgs {
 // power-of-two length apart cost 80 cycles a request at d = 256).
 __device__ __forceinline__ size_t blk(int k, int j, int K) { return ((size_t)(j >> 5) * K + k) * 32 + (j & 31); }
 
-// One warp: red[1] = tr S (blocked layout), red[0] = 1 / tr S, or 0 for a zero
-// trace (W = 0), which gives a zero product.
-__device__ void trace_inv(const double* S, int d, int lane, double* red) {
+// One warp: red[1] = tr S (blocked layout), red[0] = 2^-2e with 2^e <= tr S <
+// 2^(e+1), the exact factor that normalises S^2, or 0 for a zero trace (W = 0).
+__device__ void trace_scale(const double* S, int n, int lane, double* red) {
   double v[8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
     const int k = lane + 32 * m;
-    v[m] = k < d ? __ldcg(S + blk(k, k, d)) : 0.0;
+    v[m] = k < n ? __ldcg(S + blk(k, k, n)) : 0.0;
   }
-  if (d > 256)
+  if (n > 256)
 #pragma unroll
     for (int m = 0; m < 8; ++m)
-      for (int k = lane + 32 * m + 256; k < d; k += 256) v[m] += __ldcg(S + blk(k, k, d));
-  const double tr = tree256(v, d);
+      for (int k = lane + 32 * m + 256; k < n; k += 256) v[m] += __ldcg(S + blk(k, k, n));
+  const double tr = tree256(v, n);
   if (lane == 0) {
-    red[0] = tr > 0.0 ? 1.0 / tr : 0.0;
+    // tr W^T W of finite FP32 values has |e| < 350; the clamp is for NaN
+    int e = (int)((__double_as_longlong(tr) >> 52) & 2047) - 1023;
+    e = e < -500 ? -500 : (e > 500 ? 500 : e);
+    red[0] = tr > 0.0 ? __longlong_as_double((long long)(1023 - 2 * e) << 52) : 0.0;
     red[1] = tr;
   }
 }
 
-// The symmetric product P_ij = sum_k X[k][i] X[k][j] (k < K ascending, one
-// fused multiply-add chain per element) into B, X = S (K rows, blocked
-// layout) or, with `scale`, S * (1 / tr S) rounded: S is symmetric or is the operand
+// The symmetric product P_ij = sum_k S[k][i] S[k][j] (k < K ascending, one
+// fused multiply-add chain per element) into B, with `scale` times the power
+// of two that normalises S (taken on the result, so the panels need no
+// products of their own: 1 / tr S on the panels, a division and up to 40
+// multiplications per 128 steps of a warp, took 55 us of 435 at C = 200,
+// d = 256 and 15 of 73 at C = 10, d = 64). S (K rows, blocked layout) is symmetric or is the operand
 // itself, so one panel of columns and one of rows serve, and only i <= j is
 // computed ((j, i) would add the same products in the same order). A tile is
 // 32 columns (lanes) by 4 R rows (R chains per warp); tiles are numbered over
@@ -151,8 +160,7 @@ __device__ void sym_product(const double* S, int K, bool scale, double* B, int d
   double* rp = sm + kSpChunk * 32;   // kSpChunk x kRows
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int per = 32 / kRows;  // row blocks per 32 rows
-  double inv = 1.0;
-  bool have_inv = !scale;
+  bool have_tr = !scale;
   for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     int cb = 0, rb = tile;  // column block cb has (cb + 1) * per row blocks
     while (rb >= (cb + 1) * per) {
@@ -167,8 +175,7 @@ __device__ void sym_product(const double* S, int K, bool scale, double* B, int d
       const int kc = K - k0 < kSpChunk ? K - k0 : kSpChunk;
       __syncthreads();
       // every load of the panels is issued before the first is used (one L2
-      // round trip per chunk), every product before the first is stored (an
-      // FP64 result takes ~90 cycles)
+      // round trip per chunk)
       constexpr int NC = kSpChunk / kSpWarps, NR = kSpChunk * kRows / kSpThreads;
       double xc[NC], xr[NR];
       const double* sc = S + blk(k0, j0 + lane, K);
@@ -183,20 +190,10 @@ __device__ void sym_product(const double* S, int K, bool scale, double* B, int d
         const int k = tid / kRows + u * (kSpThreads / kRows);
         xr[u] = k < kc ? __ldcg(sr + k * 32) : 0.0;
       }
-      if (!have_inv) {
+      if (!have_tr) {
         // the trace, while the panels are on their way
-        if (warp == 0) trace_inv(S, d, lane, red);
-        __syncthreads();
-        inv = red[0];
-        have_inv = true;
-      }
-      if (scale) {
-#pragma unroll
-        for (int u = 0; u < NR; ++u) xr[u] *= inv;
-#pragma unroll
-        for (int u = 0; u < NC; ++u)
-          if (u * kSpWarps < kc) xc[u] *= inv;
-        asm volatile("" ::: "memory");
+        if (warp == 0) trace_scale(S, d, lane, red);
+        have_tr = true;
       }
 #pragma unroll
       for (int u = 0; u < NR; ++u) {
@@ -216,69 +213,72 @@ __device__ void sym_product(const double* S, int K, bool scale, double* B, int d
         for (int r = 0; r < R; ++r) acc[r] = fma(rp[k * kRows + warp * R + r], c, acc[r]);
       }
     }
+    const double f = scale ? red[0] : 1.0;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int i = i0 + warp * R + r, j = j0 + lane;
       if (i <= j && j < d) {
-        B[blk(i, j, d)] = acc[r];
-        if (i < j) B[blk(j, i, d)] = acc[r];
+        const double p = acc[r] * f;
+        B[blk(i, j, d)] = p;
+        if (i < j) B[blk(j, i, d)] = p;
       }
     }
   }
 }
 
-// The spectral norm of W by a co-resident grid: FP64 copies of W, A = W^T W,
-// `squarings` steps A <- (A / tr A)^2, then the power iteration on W. What
+// The spectral norm of W by a co-resident grid: FP64 copies of X, A = X^T X,
+// `squarings` steps A <- (A 2^-e)^2, then the power iteration on X. What
 // bounds it: the FP64 pipe (four warps per SM: ~88 cycles per step of their
-// chains); a squaring costs its d steps, the panel's scaling (1 / (4 R) of the
-// products), the trace and one grid barrier.
+// chains); a squaring costs its n steps, the trace and one grid barrier.
 template <int R>
 __global__ void __launch_bounds__(kSpThreads) k_spectral(const SpectralArgs a) {
   __shared__ double sm[kSpChunk * 32 + kSpChunk * kSpWarps * R];
   __shared__ double red[2];
   static_assert(kSpChunk * 32 >= 2 * 1024 + 1024, "the iteration's vectors share the panels' space");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int d = a.d, C = a.C, Cp = a.Cp;
+  const int m = a.m, n = a.n, mp = a.mp;
   unsigned bar = 0;
   auto sync_grid = [&]() { return grid_barrier(a.ctr, bar += gridDim.x); };
 
-  for (int e = blockIdx.x * kSpThreads + tid; e < C * a.dp; e += gridDim.x * kSpThreads) {
-    const int c = e / a.dp, j = e - c * a.dp;
-    a.Wd[blk(c, j, C)] = j < d ? (double)a.W[(size_t)c * d + j] : 0.0;
+  for (int e = blockIdx.x * kSpThreads + tid; e < m * a.np; e += gridDim.x * kSpThreads) {
+    const int r = e / a.np, j = e - r * a.np;
+    a.X[blk(r, j, m)] = j < n ? (double)a.W[(size_t)r * a.rs + (size_t)j * a.cs] : 0.0;
   }
-  for (int e = blockIdx.x * kSpThreads + tid; e < d * Cp; e += gridDim.x * kSpThreads) {
-    const int k = e / Cp, c = e - k * Cp;
-    a.WdT[e] = c < C ? (double)a.W[(size_t)c * d + k] : 0.0;
+  for (int e = blockIdx.x * kSpThreads + tid; e < n * mp; e += gridDim.x * kSpThreads) {
+    const int j = e / mp, r = e - j * mp;
+    a.XT[e] = r < m ? (double)a.W[(size_t)r * a.rs + (size_t)j * a.cs] : 0.0;
   }
   if (!sync_grid()) return;
   // A grid with fewer tiles than CTAs (units of the iteration): the spare CTAs
   // only follow the traces and meet the barriers.
   int cur = 0;
   if (a.squarings > 0) {
-    // W^T W: products of FP32 values are exact in FP64
-    sym_product<R>(a.Wd, C, false, a.A[0], d, a.n_tiles, sm, red);
+    // X^T X: products of FP32 values are exact in FP64
+    sym_product<R>(a.X, m, false, a.A[0], n, a.n_tiles, sm, red);
     if (!sync_grid()) return;
+    double s2 = 0.0;  // (tr A_k 2^-e)^2 of the matrix before
     for (int q = 0; q < a.squarings; ++q) {
-      sym_product<R>(a.A[cur], d, true, a.A[cur ^ 1], d, a.n_tiles, sm, red);
+      sym_product<R>(a.A[cur], n, true, a.A[cur ^ 1], n, a.n_tiles, sm, red);
       if ((int)blockIdx.x >= a.n_tiles) {  // a spare CTA follows the traces
-        if (warp == 0) trace_inv(a.A[cur], d, lane, red);
+        if (warp == 0) trace_scale(a.A[cur], n, lane, red);
         __syncthreads();
       }
       cur ^= 1;
-      const double tr = red[1];  // of the matrix just squared
+      const double tr = red[1], f = red[0];  // of the matrix just squared
       if (!sync_grid()) return;
-      // A square of unit trace is, from its trace t = sum l_i^2 (l_1 >= ...
-      // summing to 1), the projector on the dominant direction up to
-      // (1 - t) / 2 relative; the square just formed from it is up to the
-      // square of that, below FP64's resolution. Gaussian heads take 10 to 14
-      // steps; a (nearly) repeated largest singular value keeps t away from 1
-      // and takes them all.
-      if (q > 0 && 1.0 - tr <= 1e-9) break;
+      // With unit trace, the matrix before is, from its purity t = tr / s2 = sum
+      // l_i^2 (l_1 >= ... summing to 1), the projector on the dominant direction
+      // up to (1 - t) / 2 relative; its square up to about the square of that,
+      // and the one just formed below FP64's resolution. Gaussian heads take 10
+      // to 14 steps; a (nearly) repeated largest singular value keeps t away
+      // from 1 and takes them all.
+      if (q > 0 && s2 - tr <= 1e-9 * s2) break;
+      s2 = tr * tr * f;
     }
   }
 
-  // Power iteration on W: every CTA keeps v and repeats the short sums; the
-  // chains of w = W v and u = W^T w are spread over the grid.
+  // Power iteration on X: every CTA keeps v and repeats the short sums; the
+  // chains of w = X v and u = X^T w are spread over the grid.
   double* v = sm;
   double* w = sm + 1024;
   double* u = sm + 2048;
@@ -289,8 +289,8 @@ __global__ void __launch_bounds__(kSpThreads) k_spectral(const SpectralArgs a) {
     if (warp == 0) {
       double best = -INFINITY;
       int at = 0x7fffffff;
-      for (int k = lane; k < d; k += 32) {
-        const double x = __ldcg(A + blk(k, k, d));
+      for (int k = lane; k < n; k += 32) {
+        const double x = __ldcg(A + blk(k, k, n));
         if (x > best) {
           best = x;
           at = k;
@@ -305,20 +305,20 @@ __global__ void __launch_bounds__(kSpThreads) k_spectral(const SpectralArgs a) {
           at = oa;
         }
       }
-      if (lane == 0) red[0] = (double)(at < d ? at : 0);
+      if (lane == 0) red[0] = (double)(at < n ? at : 0);
     }
     __syncthreads();
     const int js = (int)red[0];
-    for (int k = tid; k < d; k += kSpThreads) v[k] = __ldcg(A + blk(js, k, d));
+    for (int k = tid; k < n; k += kSpThreads) v[k] = __ldcg(A + blk(js, k, n));
   } else {
-    for (int k = tid; k < d; k += kSpThreads) {
+    for (int k = tid; k < n; k += kSpThreads) {
       unsigned x = (unsigned)k * 2654435761u;
       x ^= x >> 15;
       v[k] = 1.0 + 0.01 * (double)(x & 0xffff) / 65536.0;
     }
   }
   __syncthreads();
-  double nv = sqrt(sum_squares(d, lane, [&](int k) { return v[k]; }));
+  double nv = sqrt(sum_squares(n, lane, [&](int k) { return v[k]; }));
   if (!(nv > 0.0)) {
     if (blockIdx.x == 0 && tid == 0) {
       a.res->sigma = 0.0;
@@ -331,53 +331,53 @@ __global__ void __launch_bounds__(kSpThreads) k_spectral(const SpectralArgs a) {
     return;
   }
   __syncthreads();
-  for (int k = tid; k < d; k += kSpThreads) v[k] /= nv;
+  for (int k = tid; k < n; k += kSpThreads) v[k] /= nv;
   __syncthreads();
 
-  const int cu = Cp / 32, du = (d + 31) / 32;  // 32-lane units of the two products
+  const int mu = mp / 32, nu32 = a.np / 32;  // 32-lane units of the two products
   double theta = 0.0, theta_prev = -1.0, resid = INFINITY;
   int it = 0, converged = 0;
   for (it = 1; it <= a.max_iter; ++it) {
-    for (int g = blockIdx.x + gridDim.x * warp; g < cu; g += gridDim.x * kSpWarps) {
-      const int c = g * 32 + lane;
-      const double acc = chain16(a.WdT + c, Cp, v, d);
-      if (c < C) a.w[c] = acc;
+    for (int g = blockIdx.x + gridDim.x * warp; g < mu; g += gridDim.x * kSpWarps) {
+      const int r = g * 32 + lane;
+      const double acc = chain16(a.XT + r, mp, v, n);
+      if (r < m) a.w[r] = acc;
     }
     if (!sync_grid()) return;
-    for (int c = tid; c < C; c += kSpThreads) w[c] = __ldcg(a.w + c);
+    for (int r = tid; r < m; r += kSpThreads) w[r] = __ldcg(a.w + r);
     __syncthreads();
     if (warp == kSpWarps - 1) {
-      const double p = sum_squares(C, lane, [&](int c) { return w[c]; });
+      const double p = sum_squares(m, lane, [&](int r) { return w[r]; });
       if (lane == 0) red[0] = p;
     } else {
-      for (int g = blockIdx.x + gridDim.x * warp; g < du; g += gridDim.x * (kSpWarps - 1)) {
+      for (int g = blockIdx.x + gridDim.x * warp; g < nu32; g += gridDim.x * (kSpWarps - 1)) {
         const int k = g * 32 + lane;
-        const double acc = chain16(a.Wd + blk(0, k, C), 32, w, C);
-        if (k < d) a.u[k] = acc;
+        const double acc = chain16(a.X + blk(0, k, m), 32, w, m);
+        if (k < n) a.u[k] = acc;
       }
     }
     if (!sync_grid()) return;
     theta = red[0];
-    for (int k = tid; k < d; k += kSpThreads) u[k] = __ldcg(a.u + k);
+    for (int k = tid; k < n; k += kSpThreads) u[k] = __ldcg(a.u + k);
     __syncthreads();
     if (warp == 0) {
-      const double pr = sum_squares(d, lane, [&](int k) { return fma(-theta, v[k], u[k]); });
+      const double pr = sum_squares(n, lane, [&](int k) { return fma(-theta, v[k], u[k]); });
       if (lane == 0) red[0] = pr;
     } else if (warp == 1) {
-      const double pu = sum_squares(d, lane, [&](int k) { return u[k]; });
+      const double pu = sum_squares(n, lane, [&](int k) { return u[k]; });
       if (lane == 0) red[1] = pu;
     }
     __syncthreads();
     resid = sqrt(red[0]);
     const double nu = sqrt(red[1]);
     __syncthreads();
-    if (!(nu > 0.0)) {  // v is in the null space of W: only possible for W = 0
+    if (!(nu > 0.0)) {  // v is in the null space of X: only possible for W = 0
       theta = 0.0;
       resid = 0.0;
       converged = 1;
       break;
     }
-    for (int k = tid; k < d; k += kSpThreads) v[k] = u[k] / nu;
+    for (int k = tid; k < n; k += kSpThreads) v[k] = u[k] / nu;
     __syncthreads();
     if (it >= 2 && fabs(theta - theta_prev) <= 1e-13 * theta && resid <= 1e-10 * theta) {
       converged = 1;
@@ -403,7 +403,9 @@ __global__ void __launch_bounds__(kSpThreads) k_spectral(const SpectralArgs a) {
 // One warp per unit (y, 32 classes j) of the upper triangle, a lane per pair;
 // the mirrored pair squares the negated differences, the same sum. Bound by
 // the FP64 pipe: two instructions per feature and 32 pairs.
-__global__ void __launch_bounds__(kSpThreads) k_row_norms(const double* __restrict__ WdT, int C, int Cp, int d,
+// Feature k of class c is Wt[(c / 32) bs + k ks + c % 32].
+__global__ void __launch_bounds__(kSpThreads) k_row_norms(const double* __restrict__ Wt, size_t bs, size_t ks, int C,
+                                                          int Cp, int d,
                                                           float* __restrict__ Wnorm32,
                                                           double* __restrict__ pairnorm,
                                                           double* __restrict__ inv_pairnorm,
@@ -413,10 +415,11 @@ __global__ void __launch_bounds__(kSpThreads) k_row_norms(const double* __restri
   const int nb = Cp / 32;
   if (unit < nb) {
     const int c = unit * 32 + lane;
+    const double* wc = Wt + (size_t)unit * bs + lane;
     double n2 = 0.0;
 #pragma unroll 8
     for (int k = 0; k < d; ++k) {
-      const double x = WdT[(size_t)k * Cp + c];
+      const double x = wc[k * ks];
       n2 = fma(x, x, n2);
     }
     if (c < C) Wnorm32[c] = __double2float_ru(sqrt(n2) * (1.0 + 1e-15));
@@ -431,10 +434,12 @@ __global__ void __launch_bounds__(kSpThreads) k_row_norms(const double* __restri
   }
   if (jb >= nb) return;
   const int y = r, j = jb * 32 + lane;
+  const double* wy = Wt + (size_t)(y >> 5) * bs + (y & 31);
+  const double* wj = Wt + (size_t)jb * bs + lane;
   double acc = 0.0;
 #pragma unroll 8
   for (int k = 0; k < d; ++k) {
-    const double e = WdT[(size_t)k * Cp + y] - WdT[(size_t)k * Cp + j];
+    const double e = wy[k * ks] - wj[k * ks];
     acc = fma(e, e, acc);
   }
   if (j >= C || j < y) return;
@@ -487,8 +492,8 @@ int sym_tiles(int d, int R) {
 
 template <int R>
 void launch_spectral(lipcache* h, SpectralArgs a, cudaStream_t s) {
-  a.n_tiles = sym_tiles(a.d, R);
-  const int units = (a.Cp > a.dp ? a.Cp : a.dp) / 32;
+  a.n_tiles = sym_tiles(a.n, R);
+  const int units = (a.mp > a.np ? a.mp : a.np) / 32;
   int grid = a.n_tiles > units ? a.n_tiles : units;
   if (grid > h->num_sms) grid = h->num_sms;
   void* args[] = {&a};
@@ -502,45 +507,53 @@ void launch_spectral(lipcache* h, SpectralArgs a, cudaStream_t s) {
 size_t spectral_work_bytes(int d, int C) {
   const size_t Cp = (size_t)(C + 31) / 32 * 32;
   const size_t dp = (size_t)(d + 31) / 32 * 32;
-  return sizeof(double) * (2 * dp * d + dp * C + Cp * d + C + d) + 16;
+  return sizeof(double) * (2 * dp * d + dp * C + Cp * d + C + d) + 16;  // (either orientation)
 }
 
 void spectral_norm(lipcache* h, cudaStream_t s) {
   const int d = h->d, C = h->C;
+  // The transpose of a head with fewer classes than features: a squaring's
+  // chains and tiles shrink with the smaller dimension (the kernel, C = 10,
+  // d = 64: 85 us on W, 58 on W^T; C = 200, d = 256: 441 and 380). Without squarings the start
+  // vector is fixed and the iteration stays on W.
+  const bool tr = C < d && h->squarings > 0;
   SpectralArgs a;
   a.W = h->W;
-  a.C = C;
-  a.d = d;
-  a.Cp = (C + 31) / 32 * 32;
-  a.dp = (d + 31) / 32 * 32;
+  a.m = tr ? d : C;
+  a.n = tr ? C : d;
+  a.rs = tr ? 1 : d;
+  a.cs = tr ? d : 1;
+  a.mp = (a.m + 31) / 32 * 32;
+  a.np = (a.n + 31) / 32 * 32;
   a.squarings = h->squarings;
   a.max_iter = h->max_iter;
   double* p = reinterpret_cast<double*>(h->spec_work);
   a.A[0] = p;
-  a.A[1] = a.A[0] + (size_t)a.dp * d;
-  a.Wd = a.A[1] + (size_t)a.dp * d;
-  a.WdT = a.Wd + (size_t)a.dp * C;
-  a.w = a.WdT + (size_t)a.Cp * d;
-  a.u = a.w + C;
-  a.ctr = reinterpret_cast<unsigned*>(a.u + d);
+  a.A[1] = a.A[0] + (size_t)a.np * a.n;
+  a.X = a.A[1] + (size_t)a.np * a.n;
+  a.XT = a.X + (size_t)a.np * a.m;
+  a.w = a.XT + (size_t)a.mp * a.n;
+  a.u = a.w + a.m;
+  a.ctr = reinterpret_cast<unsigned*>(a.u + a.n);
   a.res = h->spec;
   LC_CUDA(cudaMemsetAsync(a.ctr, 0, sizeof(unsigned), s));
   // a barrier that expired leaves this in place: neither converged nor degenerate
   LC_CUDA(cudaMemsetAsync(h->spec, 0xff, sizeof(SpecResult), s));
   // Chains per warp: one while the tiles of one-row warps fit the SMs once
-  // (d <= 128: 80 tiles); above, two do the same products per sub-partition
-  // with half the panel scaling (d = 256: 144 tiles).
-  if (d <= 128)
+  // (n <= 160: 120 tiles); above, two do the same products per sub-partition
+  // with half the panel loads (n = 256: 144 tiles).
+  if (sym_tiles(a.n, 1) <= h->num_sms)
     launch_spectral<1>(h, a, s);
   else
     launch_spectral<2>(h, a, s);
+  const int Cp = (C + 31) / 32 * 32;
   const bool tight = h->radius_mode == LIPCACHE_RADIUS_TIGHT;
-  const int nb = a.Cp / 32;
+  const int nb = Cp / 32;
   int units = nb;
   if (tight)
     for (int jb = 0; jb < nb; ++jb) units += C < 32 * (jb + 1) ? C : 32 * (jb + 1);
   k_row_norms<<<(units + kSpWarps - 1) / kSpWarps, kSpThreads, 0, s>>>(
-      a.WdT, C, a.Cp, d, h->Wnorm32, tight ? h->pairnorm : nullptr, tight ? h->inv_pairnorm : nullptr,
+      tr ? a.X : a.XT, tr ? (size_t)32 * d : 32, tr ? 32 : (size_t)Cp, C, Cp, d, h->Wnorm32, tight ? h->pairnorm : nullptr, tight ? h->inv_pairnorm : nullptr,
       tight ? h->ipn_up32 : nullptr, tight ? h->ipn_dn32 : nullptr);
   LC_LAUNCH_CHECK("k_row_norms");
   if (tight) {

@@ -73,11 +73,12 @@ def test_sigma_vs_oracle_svd(dev, name, W):
     cache.close()
 
 
-@pytest.mark.parametrize("C,d", [(2, 1), (3, 31), (33, 32), (40, 129), (300, 127), (5, 257), (64, 640)])
+@pytest.mark.parametrize("C,d", [(2, 1), (3, 31), (33, 32), (32, 33), (40, 129), (300, 127), (161, 300),
+                                  (300, 161), (5, 257), (64, 640)])
 @pytest.mark.parametrize("squarings", [40, 0])
 def test_sigma_tile_edges(dev, C, d, squarings):
     """Shapes around the spectral kernel's tiles (32 columns, one or two rows
-    per warp, 128-step chunks) and both start vectors, against LAPACK. The
+    per warp, 128-step chunks), both orientations and both start vectors, against LAPACK. The
     oracle comparison's bound (1e-10): the iteration stops at a residual of
     1e-10 theta, whose effect on theta is of second order."""
     from paper_2608_13144_gb300.lipcache import LipCache

@@ -209,4 +209,28 @@ __device__ __forceinline__ float screen_value(float a, float scale, float tau) {
     return __fsub_rn(a, tau);
 }
 
+// Turns a row's 32 products into tau_j - value_j (value_j as screen_value's; a
+// pair passes if that is <= -kappa, rounding to nearest being symmetric) and
+// returns their minimum: two pairs per instruction, and no sign change of the
+// terms. tau: 16-byte aligned, in global memory (LDG) or shared memory.
+template <int KIND, bool LDG>
+__device__ __forceinline__ float screen_chunk(uint32_t (&v)[32], const float* __restrict__ tau, float scale) {
+  const uint64_t ns = ptx::pack_f32x2(__float_as_uint(-scale), __float_as_uint(-scale));
+  float m = INFINITY;
+#pragma unroll
+  for (int j = 0; j < 32; j += 4) {
+    const ulonglong2* p = reinterpret_cast<const ulonglong2*>(tau + j);
+    const ulonglong2 tt = LDG ? __ldg(p) : *p;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const uint64_t a = ptx::pack_f32x2(v[j + 2 * u], v[j + 2 * u + 1]), tu = u ? tt.y : tt.x;
+      const uint64_t x = KIND == kF16 ? ptx::fma_f32x2(a, ns, tu) : ptx::sub_f32x2(tu, a);
+      v[j + 2 * u] = (uint32_t)x;
+      v[j + 2 * u + 1] = (uint32_t)(x >> 32);
+      m = fminf(m, fminf(__uint_as_float(v[j + 2 * u]), __uint_as_float(v[j + 2 * u + 1])));
+    }
+  }
+  return m;
+}
+
 }  // namespace lc

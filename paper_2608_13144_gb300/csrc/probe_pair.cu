@@ -347,11 +347,15 @@ __global__ void __launch_bounds__(kThreads, 1)
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive_cluster(lead_acc_empty + 8 * buf);
           }
+          // with close keys and few features most passing chunks hold no pair
+          // that passes
+          const float least = screen_chunk<KIND, false>(v, my_tau + ch * 32, scl);
+          const bool some = ((pass >> ch) & 1u) && least <= -kap;
+          if (!__any_sync(0xffffffffu, some)) continue;
           uint32_t mask = 0;
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
-            mask |= (uint32_t)(screen_value<KIND>(__uint_as_float(v[j]), scl, my_tau[ch * 32 + j]) >= kap) << j;
-          recheck_warp(rck, (pass >> ch) & 1u ? mask : 0u, row, key0 + ch * 32, lane, ncand);
+          for (int j = 0; j < 32; ++j) mask |= (uint32_t)(__uint_as_float(v[j]) <= -kap) << j;
+          recheck_warp(rck, some ? mask : 0u, row, key0 + ch * 32, lane, ncand);
         }
         kap = kap_next;
         scl = scl_next;

@@ -147,9 +147,9 @@ __device__ void trace_scale(const double* S, int n, int lane, double* red) {
 // of two that normalises S (taken on the result, so the panels need no
 // products of their own: 1 / tr S on the panels, a division and up to 40
 // multiplications per 128 steps of a warp, took 55 us of 435 at C = 200,
-// d = 256 and 15 of 73 at C = 10, d = 64). S (K rows, blocked layout) is symmetric or is the operand
-// itself, so one panel of columns and one of rows serve, and only i <= j is
-// computed ((j, i) would add the same products in the same order). A tile is
+// d = 256 and 15 of 73 at C = 10, d = 64). S (K rows, blocked layout) is
+// symmetric or is the operand itself, so one panel of columns and one of rows
+// serve, and only i <= j is computed ((j, i) would add the same products in the same order). A tile is
 // 32 columns (lanes) by 4 R rows (R chains per warp); tiles are numbered over
 // the upper triangle.
 template <int R>

@@ -1352,7 +1352,9 @@ __global__ void __launch_bounds__(1024) k_scan(int32_t* __restrict__ cnt, int32_
                                                int32_t* __restrict__ rank, int64_t n) {
   __shared__ int64_t carry;
   const int tid = threadIdx.x;
+  ptx::launch_dependents();  // (the scatter)
   if (tid == 0) carry = 0;
+  ptx::wait_prerequisites();
   // the FP64 pass may have changed a listed row's acceptance: recount its
   // 32-row block (rows listed twice in a block write the same values)
   const int nfix = st->fix_count;
@@ -1447,6 +1449,7 @@ constexpr int kTailBlocks = 8;  // blocks of the launch that clear the rows past
 __global__ void __launch_bounds__(256) k_scatter(ScatterArgs a, int vec) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (blockIdx.x < kTailBlocks) {
+    ptx::wait_prerequisites();
     zero_tail(a.t, a.dpad, *a.size, (int)(blockIdx.x * 256 + threadIdx.x), kTailBlocks * 256);
     return;
   }
@@ -1460,6 +1463,7 @@ __global__ void __launch_bounds__(256) k_scatter(ScatterArgs a, int vec) {
       v0[u] = (row0 + u < a.n && lane < d4) ? __ldg(reinterpret_cast<const float4*>(a.H + (size_t)(row0 + u) * a.d) + lane)
                                             : make_float4(0.f, 0.f, 0.f, 0.f);
   }
+  ptx::wait_prerequisites();
   int64_t mydst = -2;  // past the end
   if (lane < kScatterRows && row0 + lane < a.n) {
     const int64_t row = row0 + lane;
@@ -1785,8 +1789,21 @@ void certify_insert(lipcache* h, const float* H, int64_t n, const int32_t* paylo
                     int64_t* out_index, float* out_radius, cudaStream_t s, const int64_t* miss_of) {
   launch_certify(h, H, n, payload, require_consistency, miss_of, s);
   const int nb = (int)((n + kRows - 1) / kRows);
-  k_scan<<<1, 1024, 0, s>>>(h->ins_bcount, h->ins_boffset, nb, h->report->total, h->stats, &h->report->size, h->ins_size0,
-                            h->ins_fix, h->ins_accept, h->ins_rank, n);
+  // The scan starts while the certify kernel's last CTAs run and the scatter's
+  // first rows load while the scan waits (29 inserts
+  // of 65,536 rows with their setup: 4,434 us without, 4,322 with).
+  cudaLaunchAttribute behind;
+  behind.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  behind.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.attrs = &behind;
+  cfg.numAttrs = 1;
+  cfg.stream = s;
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3(1024);
+  LC_CUDA(cudaLaunchKernelEx(&cfg, k_scan, h->ins_bcount, h->ins_boffset, nb, &h->report->total[0],
+                             (const DevStats*)h->stats, &h->report->size, h->ins_size0, (const int32_t*)h->ins_fix,
+                             (const uint8_t*)h->ins_accept, h->ins_rank, n));
   LC_LAUNCH_CHECK("k_scan");
   ScatterArgs sa;
   sa.H = H;
@@ -1811,7 +1828,9 @@ void certify_insert(lipcache* h, const float* H, int64_t n, const int32_t* paylo
   sa.st = h->stats;
   const int vec = (h->d % 4 == 0 && ((uintptr_t)H & 15) == 0) ? 1 : 0;
   const int64_t rows_per_block = 8 * kScatterRows;
-  k_scatter<<<(unsigned)(kTailBlocks + (n + rows_per_block - 1) / rows_per_block), 256, 0, s>>>(sa, vec);
+  cfg.gridDim = dim3((unsigned)(kTailBlocks + (n + rows_per_block - 1) / rows_per_block));
+  cfg.blockDim = dim3(256);
+  LC_CUDA(cudaLaunchKernelEx(&cfg, k_scatter, sa, vec));
   LC_LAUNCH_CHECK("k_scatter");
 }
 

@@ -804,6 +804,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     wn_s[i] = i < C ? __ldg(a.Wnorm32 + i) : 0.f;
   }
   if (warp == 1) {
+    ptx::launch_dependents();  // (the scan)
     ptx::tmem_alloc(ptx::smem_u32(tmem_slot), kTmemCols);
     ptx::tmem_relinquish();
   }

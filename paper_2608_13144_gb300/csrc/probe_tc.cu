@@ -102,7 +102,12 @@ struct TcArgs {
 
 // Pairs on their way from the epilogue warps to the recheck warp (shared
 // memory): pair number k is in slot k % kRecheckQ once seq there is k + 1.
+// Without that warp (short ranges) each epilogue warp keeps its own kWarpQ of
+// the slots and rechecks what they hold when they are full or its tiles are
+// done: one round of loads instead of one per chunk (256 queries on 2,000
+// entries, d = 64, 113 pairs: 19.4 us per chunk, 15.7 us so).
 constexpr int kRecheckQ = 64;
+constexpr int kWarpQ = kRecheckQ / kEpiWarps;
 struct RecheckQueue {
   int n;      // slots reserved
   int taken;  // pairs rechecked (their slots are free)
@@ -417,6 +422,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     int t = 0;
     bool ok = true;
     unsigned long long ncand = 0;
+    int held = 0;  // pairs in this warp's own slots
+    auto flush = [&]() {
+      __syncwarp();
+      int2 pr = make_int2(0, 0);
+      if (lane < held) pr = rq->pair[ew * kWarpQ + lane];
+      recheck_warp(rck, lane < held ? 1u : 0u, pr.x, pr.y, lane, ncand);
+      held = 0;
+      __syncwarp();
+    };
     RunCursor rc(a, cluster_id, n_clusters);
     int kt, qt0, qt1;
     while (ok && rc.next(a, rank, kt, qt0, qt1)) {
@@ -519,9 +533,15 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int cnt = __reduce_add_sync(0xffffffffu, mine);
           const int first_key = key0 + h * BN + ch * 32;
           // to the recheck warp if there are tiles to go on with and its queue
-          // has room, else here
+          // has room, or to the warp's own slots, else here
           int base = -1;
-          if (lane == 0 && a.queue) {
+          if (!a.queue) {
+            if (held + cnt > kWarpQ && held) flush();
+            if (cnt <= kWarpQ) {
+              base = held;
+              held += cnt;
+            }
+          } else if (lane == 0) {
             volatile RecheckQueue* vq = rq;
             for (int n = vq->n; n + cnt - vq->taken <= kRecheckQ;) {
               const int was = atomicCAS(&rq->n, n, n + cnt);
@@ -544,9 +564,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (lane >= o) at += x;
           }
           for (at += base - mine; mask; mask &= mask - 1, ++at) {
-            rq->pair[at % kRecheckQ] = make_int2(row, first_key + __ffs((int)mask) - 1);
-            __threadfence_block();
-            *(volatile int*)&rq->seq[at % kRecheckQ] = at + 1;
+            const int slot = a.queue ? at % kRecheckQ : ew * kWarpQ + at;
+            rq->pair[slot] = make_int2(row, first_key + __ffs((int)mask) - 1);
+            if (a.queue) {
+              __threadfence_block();
+              *(volatile int*)&rq->seq[slot] = at + 1;
+            }
           }
           __syncwarp();
         }
@@ -555,6 +578,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         scl = scl_next;
       }
     }
+    if (held) flush();
     __syncwarp();
     if (lane == 0) {
       __threadfence_block();

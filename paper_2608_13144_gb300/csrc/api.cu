@@ -179,11 +179,14 @@ void lc::harvest_timing(lipcache* h, bool all) {
 }
 
 // After a synchronised probe: E_DEVICE if a bounded wait of the kernel expired.
+static void require_probe_ok(lipcache* h) {
+  LC_REQUIRE((h->stats_host->abort_flag & lc::kProbeAborted) == 0, LIPCACHE_E_DEVICE,
+             "a bounded wait of the probe kernel expired; the batch's queries were reported as misses");
+}
 static void require_no_abort(lipcache* h, cudaStream_t s) {
   lc::fetch_report(h, s);
   LC_CUDA(cudaStreamSynchronize(s));
-  LC_REQUIRE(h->stats_host->abort_flag == 0, LIPCACHE_E_DEVICE,
-             "a bounded wait of the probe kernel expired; the batch's queries were reported as misses");
+  require_probe_ok(h);
 }
 
 LC_API const char* lipcache_last_error(void) { return g_err.c_str(); }
@@ -439,10 +442,11 @@ LC_API lipcache_status lipcache_probe_writeback(lipcache_t* h, const float* Q, i
     use_device(h);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     lc::probe(h, Q, B, out_index, out_label, out_dist, s);
-    require_no_abort(h, s);  // an aborted probe reports misses: write nothing back
+    // (an aborted probe reports misses and leaves its flag: nothing is written back)
     lc::certify_insert(h, Q, B, payload, require_consistency, out_inserted, nullptr, s, out_index);
     lc::fetch_report(h, s);
     LC_CUDA(cudaStreamSynchronize(s));
+    require_probe_ok(h);
     LC_REQUIRE(h->stats_host->abort_flag == 0, LIPCACHE_E_DEVICE, lc::kCertifyAbortMessage);
     const int64_t acc = h->report_host->total[0];
     const int64_t first = h->size;

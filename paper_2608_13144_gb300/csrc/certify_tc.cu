@@ -1595,7 +1595,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   if (threadIdx.x == 0 && *abort_s) {
     atomicAdd(&stats->errors, 1ull);
-    atomicExch(&stats->abort_flag, 1);
+    atomicOr(&stats->abort_flag, kCertifyAborted);
   }
   if (warp == 1) {
     ptx::tc_fence_after();

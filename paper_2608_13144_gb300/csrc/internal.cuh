@@ -141,12 +141,15 @@ struct SpecResult {
 struct DevStats {
   unsigned long long candidates;
   unsigned long long errors;
-  int abort_flag;  // set by a kernel whose bounded wait expired; cleared per probe
+  int abort_flag;  // kernels whose bounded wait expired; cleared per probe and certification
   int fix_count;   // rows of the current certification listed for the FP64 pass (cleared per certification)
   unsigned long long ins_pairs;      // (row, class) pairs refined by the tensor certify kernel
   unsigned long long ins_full_rows;  // row halves it refined over every class
   unsigned long long ins_fp64_rows;  // rows re-certified by the FP64 pass
 };
+
+// Bits of abort_flag.
+constexpr int kProbeAborted = 1, kCertifyAborted = 2;
 
 // What a call may have to report to the host, in one block: one copy.
 struct DevReport {

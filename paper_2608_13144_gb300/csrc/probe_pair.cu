@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // direct at this one before the cluster retires.
     if (threadIdx.x == 0) {
       atomicAdd(&a.stats->errors, 1ull);
-      atomicExch(&a.stats->abort_flag, 1);
+      atomicExch(&a.stats->abort_flag, kProbeAborted);
     }
     __nanosleep(50000);
   }

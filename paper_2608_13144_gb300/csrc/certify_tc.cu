@@ -627,53 +627,41 @@ __device__ __forceinline__ void refine_lanes(const WA& wa, uint32_t zs, int c, i
 }
 
 // The tight radius (Eq. 29) of one row on one warp, for rows the screen
-// cannot settle (several possible y^G, Mb not below 1e38, more candidates than
-// slots): every class refined with the compensated dot product by the four
-// 8-lane groups, two classes per group at a time (refine2, the error factor of
-// 8-lane groups), into the warp's result cells by class; then, lane = class,
-// y^G the largest refined logit (lowest class on ties) and Eq. 29 over every
-// other class in FP64. The row's features come from the tile in shared memory
-// (row rz). res_hi / res_lo: the warp's cells (at least 256 each), free here.
-// Returns (on every lane) whether the row was listed for the FP64 pass.
+// cannot settle (Mb not below 1e38) or with more candidates than slots: the
+// row's candidates (m0, m1: the chunks' masks of the two column halves, all
+// classes where the screen says nothing) refined with the compensated dot
+// product, a class per lane (refine_lane), into the warp's result cells by class;
+// then, lane = class, y^G the largest refined logit (lowest class on ties) and
+// Eq. 29 over every other candidate in FP64. The row's features come from the
+// tile in shared memory (row rz). res_hi / res_lo, list: the warp's cells (at
+// least 256 each), free here. Returns (on every lane) whether the row was listed
+// for the FP64 pass; np: classes refined. (Every class of such a row took about
+// 75 us of a warp with a streamed head, d = 256, C = 200, while the tile's other
+// warps waited: 307 us per 65,536 rows with 107 of them, 190 with the candidates.)
 template <class WA>
-__device__ bool tc_tight_row_warp(const CertArgs& a, int64_t row, int rz, const WA& wa, uint32_t zs,
-                                  const float* __restrict__ wn_s, const float* __restrict__ b_s, float kn, int lane,
-                                  float* res_hi, float* res_lo, uint8_t* acc_slot) {
+__device__ bool tc_tight_row_warp(const CertArgs& a, int64_t row, int rz, const WA& wa, uint32_t zs, const uint4& m0,
+                                  const uint4& m1, const float* __restrict__ wn_s, const float* __restrict__ b_s,
+                                  float kn, int lane, int* list, float* res_hi, float* res_lo, uint8_t* acc_slot,
+                                  int& np) {
   constexpr int kPer = 8;  // classes per lane (C <= 256)
-  const int d = a.d, C = a.C;
-  const int g8 = lane / kGroupTc, sub = lane % kGroupTc;
+  const int d = a.d;
   const float hn = norm_upper(kn);
-  if constexpr (!std::is_same<WA, WSm>::value) {
-    // the head's rows come from L2: a class per lane (refine_lane, the same
-    // bits) keeps 32 rows' loads in flight, two per 8-lane group eight
-    for (int c0 = 0; c0 < C; c0 += 32) {
-      const int c = c0 + lane < C ? c0 + lane : C - 1;
-      float hi, lo;
-      refine_lane(wa, zs, c, rz, b_s[c], d, hi, lo);
-      if (c0 + lane < C) {
-        res_hi[c] = hi;
-        res_lo[c] = lo;
-      }
-    }
-  } else {
-    for (int c0 = 0; c0 < C; c0 += 2 * (32 / kGroupTc)) {
-      int cp[2];
-  #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int c = c0 + 2 * g8 + u;
-        cp[u] = c < C ? c : C - 1;  // a valid class; the result is not stored
-      }
-      const int rp[2] = {rz, rz};
-      const float bp[2] = {b_s[cp[0]], b_s[cp[1]]};
-      float hi[2], lo[2];
-      refine2(wa, zs, cp, rp, bp, d, sub, hi, lo);
-      if (sub == 0)
-  #pragma unroll
-        for (int u = 0; u < 2; ++u)
-          if (c0 + 2 * g8 + u < C) {
-            res_hi[c0 + 2 * g8 + u] = hi[u];
-            res_lo[c0 + 2 * g8 + u] = lo[u];
-          }
+  const uint32_t cm[kPer] = {m0.x, m1.x, m0.y, m1.y, m0.z, m1.z, m0.w, m1.w};
+  int K = 0;
+#pragma unroll
+  for (int t = 0; t < kPer; ++t) {
+    if ((cm[t] >> lane) & 1u) list[K + __popc(cm[t] & ((1u << lane) - 1u))] = 32 * t + lane;
+    K += __popc(cm[t]);
+  }
+  np = K;
+  __syncwarp();
+  for (int i0 = 0; i0 < K; i0 += 32) {
+    const int c = list[i0 + lane < K ? i0 + lane : K - 1];
+    float hi, lo;
+    refine_lane(wa, zs, c, rz, b_s[c], d, hi, lo);
+    if (i0 + lane < K) {
+      res_hi[c] = hi;
+      res_lo[c] = lo;
     }
   }
   __syncwarp();
@@ -687,7 +675,7 @@ __device__ bool tc_tight_row_warp(const CertArgs& a, int64_t row, int rz, const 
     vh[t] = NAN;
     vl[t] = 0.f;
     ve[t] = 0.f;
-    if (c < C) {
+    if ((cm[t] >> lane) & 1u) {
       const float hi = res_hi[c], lo = res_lo[c];
       vh[t] = hi;
       vl[t] = lo;
@@ -729,7 +717,7 @@ __device__ bool tc_tight_row_warp(const CertArgs& a, int64_t row, int rz, const 
 #pragma unroll
   for (int t = 0; t < kPer; ++t) {
     const int j = lane + 32 * t;
-    if (j >= C || j == y) continue;
+    if (!((cm[t] >> lane) & 1u) || j == y) continue;
     tight_term(a, y, j, vy, ey, (double)vh[t] + (double)vl[t], (double)ve[t], rmin, smin);
   }
   rmin = warp_min_d(rmin);
@@ -743,7 +731,7 @@ __device__ bool tc_tight_row_warp(const CertArgs& a, int64_t row, int rz, const 
 // chunks stream through a ring for the MMAs, tile after tile, and the
 // refinement reads its rows from L2, four 32-byte spans ahead. It replaces FP32
 // logits on the CUDA cores with FP64 sums: 100,000 rows, d = 256, C = 200, tight
-// radius, 72.8 ms then, 0.60 ms now (floor: 30 us of HBM, 11 us of TF32).
+// radius, 72.8 ms then, 0.36 ms now (floor: 30 us of HBM, 11 us of TF32).
 // Bound by the epilogue, as the resident kernel, plus the L2 latency of the
 // head's rows.
 template <bool TIGHT, bool WSTREAM>
@@ -1310,6 +1298,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // the row's lane keeps its slots' classes (one byte each)
       int P = 0, cnt = 0;
       uint32_t cls_lo = 0, cls_hi = 0;
+      uint4 cm = make_uint4(0u, 0u, 0u, 0u);  // tight: this half's candidates, a word per chunk
       auto append = [&](uint32_t mask, int ch) {
         if (!live || fb) mask = 0;
         while (__any_sync(kFull, mask != 0)) {
@@ -1340,6 +1329,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         if constexpr (TIGHT) {
           ma = pass2_chunk_tight(va, ch, E, lo1, im1, U1, irow1, !unc);
           if (two) mbk = pass2_chunk_tight(vb, ch + 2, E, lo1, im1, U1, irow1, !unc);
+          if (ch < 4) {
+            cm.x = ma;
+            cm.y = mbk;
+          } else {
+            cm.z = ma;
+            cm.w = mbk;
+          }
         } else {
           ma = pass2_chunk(va, ch, T);
           if (two) mbk = pass2_chunk(vb, ch + 2, T);
@@ -1536,10 +1532,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         const unsigned fbm = __ballot_sync(kFull, rowfb);
         if (lane == 0) {
           n_pairs += (unsigned long long)P;
-          if (half == 0) {
-            n_full += (unsigned long long)__popc(fbm);
-            n_pairs += (unsigned long long)__popc(fbm) * (unsigned long long)C;
+          if (half == 0) n_full += (unsigned long long)__popc(fbm);
+        }
+        if (fbm != 0) {
+          // (the partner has read the first pass's exchange: its space is free)
+          if (fb) {
+            auto all = [&](int ch) { return C <= ch * 32 ? 0u : C >= ch * 32 + 32 ? 0xffffffffu : (1u << (C - ch * 32)) - 1u; };
+            cm = make_uint4(all(half), all(half + 2), all(half + 4), all(half + 6));
           }
+          reinterpret_cast<uint4*>(x1)[half * kBM + r] = cm;
         }
         if (half == 1) {
           tx.rmin[r] = rmin;
@@ -1562,9 +1563,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           if ((k & 1) == half) {
             const float knw = __shfl_sync(kFull, kn, ow);
             const int64_t frow = (int64_t)tile * kBM + rq + ow;
-            if (tc_tight_row_warp(a, frow, rq + ow, wa, zs, wn_s, bias_s, knw, lane, res_hi, res_lo,
-                                  &acc_s[rq + ow]) &&
-                fixq && lane == 0)
+            int np;
+            const uint4* cx = reinterpret_cast<const uint4*>(x1);
+            const bool fix = tc_tight_row_warp(a, frow, rq + ow, wa, zs, cx[rq + ow], cx[kBM + rq + ow], wn_s, bias_s, knw,
+                                               lane, list, res_hi, res_lo, &acc_s[rq + ow], np);
+            n_pairs += (unsigned long long)np;
+            if (fix && fixq && lane == 0)
               fixq_push(fixq, (int)frow, knw, abort_s, kWaitLimit);
             __syncwarp();
           }

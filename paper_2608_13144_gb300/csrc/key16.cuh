@@ -46,6 +46,18 @@ struct Half16Check {
   }
 };
 
+// Whether four values pass that test by their largest alone (most do: the sums
+// took 2 of the scatter's 15 us per 65,536 rows of 128 features). With m =
+// max |x_i| <= 65,504 every error is at most 2^-11 |x_i| or, below the normal
+// range, 2^-25: e2 <= 2^-22 n2 + 2^-48, and n2 >= m^2 >= 2^-20 makes the last
+// term at most 2^-28 n2, within 2^-22 (1 + 2^-6) n2. Four zeros pass. NaN does not
+// show in the maximum: a sum that is not finite fails.
+__device__ __forceinline__ bool four_fit(const float4& v) {
+  const float m = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+  const float s = (v.x + v.y) + (v.z + v.w);
+  return s == s && m <= 65504.f && (m >= 9.765625e-4f || m == 0.f);
+}
+
 // One row of the copy by one warp, from a zero-padded FP32 source of n
 // features (n <= d16; the rest is zero). Returns whether the copy serves.
 __device__ __forceinline__ bool store_key16(const float* __restrict__ src, int n, __half* __restrict__ dst, int d16,

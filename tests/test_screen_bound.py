@@ -574,3 +574,22 @@ def test_fp16_screen_error_within_half_of_c(d, kind):
     assert np.all(err <= bound * norms)
     c = 2 * (2.0 ** -9 + 2.0 ** -20 + d * 2.0 ** -22)
     assert bound + d * 2.0 ** -22 <= 0.55 * c
+
+
+@pytest.mark.parametrize("top", [2.0 ** -10, 2.0 ** -10 * (1 + 2.0 ** -23), 1e-3, 1.0, 65504.0])
+def test_four_values_pass_the_fp16_check_by_their_largest(top):
+    """The scatter takes four values whose largest lies in [2^-10, 65504] as
+    fitting without their sums: the sums' test (error at most 2^-22 (1 + 2^-7)^2
+    of the squares) then holds, whatever the other three are, with the largest
+    rounding errors of each binade and below FP16's normal range."""
+    rng = np.random.default_rng(5)
+    half_ulp = np.float32(1 + 2.0 ** -11)  # halfway between two FP16 numbers
+    below = np.concatenate([half_ulp * np.float32(2.0) ** np.arange(-30, -10), [2.0 ** -25, 3 * 2.0 ** -25, 0.0],
+                            np.float32(2.0) ** -14 * (1 + rng.random(50)), 2.0 ** -24 * (0.5 + np.arange(40))])
+    x = rng.choice(below.astype(np.float32), (20000, 4))
+    x = np.minimum(x, np.float32(top))
+    x[:, 0] = np.float32(top)
+    x[::2, 0] = np.minimum(np.float32(top) * half_ulp, np.float32(65504.0))
+    x *= rng.choice(np.float32([-1, 1]), x.shape)
+    x64, x16 = x.astype(np.float64), x.astype(np.float16).astype(np.float64)
+    assert np.all(((x64 - x16) ** 2).sum(1) <= 2.0 ** -22 * (1 + 2.0 ** -7) ** 2 * (x64 ** 2).sum(1))

@@ -7,8 +7,8 @@ certified insertion of Algorithm 1. Default workload: the scale stress case,
 a 4,000,000-entry cache of d = 128 FP32 GuardNet-like features (C = 200
 classes, Lipschitz-constrained head) probed in batches of 4,096 queries, 25%
 of them near-duplicates of cached rows. Inputs are seeded synthetic data
-(synth.py); the key table (2.06 GB) is larger than L2, so no L2 flush is
-needed between steps.
+(synth.py); the key table (2.06 GB, and the 1.02 GB FP16 copy that the screen
+reads) is larger than L2, so no L2 flush is needed between steps.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--workload NAME]
   python bench.py --impl reference ...   # FP64 CPU oracle on host cores
@@ -55,7 +55,8 @@ def parse():
     p.add_argument("--path", default="auto", choices=["auto", "tensor", "tensor_single", "tensor_pair", "exact"])
     p.add_argument("--cpu-seconds", type=float, default=15.0, help="budget of the oracle CPU baseline")
     p.add_argument("--no-cpu-baseline", action="store_true")
-    p.add_argument("--no-tf32-peak", action="store_true", help="skip the live cuBLAS TF32 peak measurement")
+    p.add_argument("--no-fp16-peak", "--no-tf32-peak", dest="no_fp16_peak", action="store_true",
+                   help="skip the live cuBLAS FP16 peak measurement")
     p.add_argument("--sustain-s", type=float, default=3.0,
                    help="seconds of back-to-back probe steps after the timed region, reported as `sustained` "
                         "with their clocks (0: skip)")
@@ -193,19 +194,22 @@ def workload_data(w: synth.Workload):
 
 
 def roofline(w: synth.Workload, N: int, B: int, kernel_ms: float, pk: dict, pk_kind: str,
-             kernel: str = "k_probe_tc") -> dict:
+             kernel: str = "k_probe_tc", fp16: bool = True) -> dict:
+    """Roofline of one probe batch. fp16: the screen reads the FP16 copy of
+    the keys with FP16 MMAs (the same dense rate as BF16); else the FP32 keys."""
     flops = 2.0 * B * N * w.d
-    bytes_ = N * (4.0 * w.d + 4.0) + 4.0 * B * w.d + 16.0 * B
-    tf32_peak = pk["bf16_tflops"] * TF32_OVER_BF16
+    bytes_ = N * ((2.0 if fp16 else 4.0) * w.d + 4.0) + 4.0 * B * w.d + 16.0 * B
+    tc_peak = pk["bf16_tflops"] * (1.0 if fp16 else TF32_OVER_BF16)
     hbm_peak = pk["hbm_gbs"]
-    t_tc = flops / (tf32_peak * 1e12)
+    t_tc = flops / (tc_peak * 1e12)
     t_hbm = bytes_ / (hbm_peak * 1e9)
     s = kernel_ms * 1e-3
     if t_tc >= t_hbm:
         ach = flops / s / 1e12
-        return {"bound": "tensor", "achieved": ach, "peak": tf32_peak, "unit": "TFLOP/s", "frac": ach / tf32_peak,
+        return {"bound": "tensor", "achieved": ach, "peak": tc_peak, "unit": "TFLOP/s", "frac": ach / tc_peak,
                 "traffic": None, "algorithmic_flops": flops, "algorithmic_bytes": bytes_,
-                "peak_source": f"{pk_kind} bf16 burst x nominal tf32/bf16 ratio {TF32_OVER_BF16:.4f}",
+                "peak_source": f"{pk_kind} bf16 burst" + (" (the dense FP16 rate is the same)" if fp16 else
+                                                          f" x nominal tf32/bf16 ratio {TF32_OVER_BF16:.4f}"),
                 "kernel": kernel, "kernel_ms": kernel_ms,
                 "hbm_frac": bytes_ / s / 1e9 / hbm_peak}
     ach = bytes_ / s / 1e9
@@ -240,21 +244,21 @@ def event_floor_ms(dev, reps: int = 50) -> float:
     return statistics.median(out)
 
 
-def measure_tf32_peak(dev, n: int = 8192, reps: int = 10, sustain_s: float = 2.0) -> dict:
-    """Dense TF32 tensor throughput of this GPU, measured in this run the way
-    the BF16 peak of MEASURED_PEAKS.json was: a cuBLAS (torch.matmul) FP32 GEMM
-    with TF32 tensor cores allowed, n^3 with n = 8192 (2 n^3 flops), best of
+def measure_fp16_peak(dev, n: int = 8192, reps: int = 10, sustain_s: float = 2.0) -> dict:
+    """Dense FP16 tensor throughput of this GPU, measured in this run the way
+    the BF16 peak of MEASURED_PEAKS.json was: a cuBLAS (torch.matmul) FP16 GEMM
+    (FP32 accumulation), n^3 with n = 8192 (2 n^3 flops), best of
     `reps` timed with CUDA events (burst), then back to back for `sustain_s`
     seconds (sustained), with nvidia-smi clocks sampled meanwhile. A
     measurement for the roofline only; the lookup never calls cuBLAS."""
     import torch
-    prev = torch.backends.cuda.matmul.allow_tf32
-    torch.backends.cuda.matmul.allow_tf32 = True
+    prev = torch.backends.cuda.matmul.allow_fp16_reduced_precision_reduction
+    torch.backends.cuda.matmul.allow_fp16_reduced_precision_reduction = False
     try:
         g = torch.Generator(device=dev).manual_seed(1)
-        a = torch.randn(n, n, device=dev, generator=g)
-        b = torch.randn(n, n, device=dev, generator=g)
-        c = torch.empty(n, n, device=dev)
+        a = torch.randn(n, n, device=dev, generator=g).half()
+        b = torch.randn(n, n, device=dev, generator=g).half()
+        c = torch.empty(n, n, device=dev, dtype=torch.float16)
         for _ in range(3):
             torch.matmul(a, b, out=c)
         torch.cuda.synchronize(dev)
@@ -282,14 +286,15 @@ def measure_tf32_peak(dev, n: int = 8192, reps: int = 10, sustain_s: float = 2.0
         clocks = clk.stop()
         del a, b, c
         return {"burst_tflops": 2.0 * n ** 3 / best / 1e12, "sustained_tflops": sustained, "clocks": clocks,
-                "how": f"torch.matmul FP32 {n}^3 with TF32 tensor cores (cuBLAS): best of {reps} (burst), "
+                "how": f"torch.matmul FP16 {n}^3 (cuBLAS): best of {reps} (burst), "
                        f"back to back for {sustain_s:.0f} s (sustained)"}
     finally:
-        torch.backends.cuda.matmul.allow_tf32 = prev
+        torch.backends.cuda.matmul.allow_fp16_reduced_precision_reduction = prev
 
 
 # main probe kernel per path: name, ncu summary, the sources its hash covers
-INSERT_KERNELS = {1: "k_certify_wt", 2: "k_certify_wres", 3: "k_certify", 4: "k_certify_tc"}
+INSERT_KERNELS = {1: "k_certify_wt", 2: "k_certify_wres", 3: "k_certify (k_certify_tc, head streamed, where it applies)",
+                  4: "k_certify_tc"}
 PROBE_KERNELS = {
     4: ("k_probe_pair", "k_probe_pair_scale.md", ("probe_pair.cu", "tc_ptx.cuh", "probe_common.cuh")),
     3: ("k_probe_tc", "k_probe_tc_scale.md", ("probe_tc.cu", "tc_ptx.cuh", "probe_common.cuh")),
@@ -513,14 +518,18 @@ def run_ours(args, dist: Dist):
     cache.close()
 
     path_id = info["last_probe_path"]
-    rf = roofline(w, N, B, kernel_ms, pk, pk_kind, PROBE_KERNELS[path_id][0])
+    fp16 = path_id in (3, 4)  # these keys fit the FP16 copy
+    rf = roofline(w, N, B, kernel_ms, pk, pk_kind, PROBE_KERNELS[path_id][0], fp16)
     tf32_derived = pk["bf16_tflops"] * TF32_OVER_BF16
-    if rf["bound"] == "tensor" and not args.no_tf32_peak:
-        # the TF32 peak measured live beside the derived one (MEASURED_PEAKS.json holds BF16 only)
-        tf = measure_tf32_peak(dev)
+    if rf["bound"] == "tensor" and not args.no_fp16_peak:
+        # the FP16 peak measured live beside the recorded BF16 one
+        tf = measure_fp16_peak(dev)
         tf["frac_of_burst"] = rf["achieved"] / tf["burst_tflops"]
         tf["frac_of_sustained"] = rf["achieved"] / tf["sustained_tflops"]
-        rf["tf32_measured"] = tf
+        rf["fp16_measured"] = tf
+    # kernels of a step: the screen's prologue, the main kernel, and a
+    # finalize kernel for batches the main kernel does not finalize itself
+    launches = (1 if path_id == 2 else 2) + (1 if B > 2048 else 0)
     if path_id in (3, 4) and w.N == synth.WORKLOADS[w.name].N:
         rf["traffic"] = recorded_traffic(w.name, path_id)
     # context for short kernels: the part of each per-kernel event interval
@@ -530,20 +539,21 @@ def run_ours(args, dist: Dist):
     line = {
         "metric": METRIC, "value": value, "unit": "queries/s", "n_gpus": dist.world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": tmax / args.steps * 1e3, "higher_is_better": True,
-        "scaling": "weak", "vs_baseline": None, "dtype": "tf32" if info["last_probe_path"] in (3, 4) else "fp32",
+        "scaling": "weak", "vs_baseline": None, "dtype": "fp16 screen, fp32 decisions" if fp16 else "fp32",
         "data": "synthetic (seeded Gaussian-mixture GuardNet features; no datasets or trained weights)",
         "config": {"workload": w.name, "N": N, "d": w.d, "C": w.C, "batch": B, "radius": "conservative",
                    "near_duplicates": w.dup_frac, "near_duplicate_noise": w.noise,
                    "probe_path": {2: "exact", 3: "tensor_single", 4: "tensor_pair"}[info["last_probe_path"]],
                    "parallelism": "single",
-                   "l2": f"inputs larger than L2 ({N * (4 * info['d_pad'] + 16) / 1e9:.2f} GB key table)"},
+                   "l2": f"inputs larger than L2 ({N * (4 * info['d_pad'] + 16) / 1e9:.2f} GB key table"
+                         + (f", {N * 2 * w.d / 1e9:.2f} GB FP16 copy read per step)" if fp16 else ")")},
         "pairs_per_s": value * N,
         "roofline": rf,
         "cpu_baseline": cpu,
         "parity": parity,
         "e2e": {"value": e2e_value, "unit": "queries/s", "h2d_bytes_per_step": B * w.d * 4,
                 "d2h_bytes_per_step": B * (8 + 4 + 4)},
-        "gpu_launches": 3 * args.steps,
+        "gpu_launches": launches * args.steps,
         "sustained": sustained,
         "clocks": clocks,
         "insert": insert_summary(w, n_acc, insert_ms, torch.cuda.get_device_properties(dev).multi_processor_count,

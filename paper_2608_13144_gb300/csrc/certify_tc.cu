@@ -1498,7 +1498,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           // refined values and their errors (u_j above the FP64 term, l_j below
           // its certified lower bound): only a candidate with l_j <= min u can
           // have either minimum, usually one per row. The same minima. (65,536 rows
-          // of d = 128, C = 200: 136 us without the bracket, 126 us with it;
+          // of d = 128, C = 200: 136 us without the bracket, 126 us with it
+          // (107 since rows with many candidates refine those only);
           // 50,000 of d = 64, C = 10: 47 and 39.5 us.)
           // (unrolled, so that the table loads of all candidates are in flight)
           const float eyf = refined_err(a.g2f8, wn_s[yg], hn, bias_s[yg]);

@@ -4,7 +4,7 @@
 // The screen, its operands (FP16 or TF32), its bound and the recheck are those
 // of probe_tc.cu; what changes is the schedule: it serves rows too long for
 // 256-key tiles of a single CTA (49,999 keys x 1,001 queries at d = 500, FP16:
-// 63 us, before on the CUDA cores 2,196 us). At the single-CTA MMA shape (M = 128 queries,
+// 51 us, before on the CUDA cores 2,192 us). At the single-CTA MMA shape (M = 128 queries,
 // N = 256 keys) the operand reads plus the query-stage writes fill the SM's
 // shared-memory bandwidth, so the epilogue's reads come out of MMA
 // throughput. A pair MMA (tcgen05.mma.cta_group::2, M = 256, N = 256) reads

@@ -209,18 +209,33 @@ __device__ __forceinline__ float screen_value(float a, float scale, float tau) {
     return __fsub_rn(a, tau);
 }
 
+// A chunk's 32 screen terms, loaded while the products leave tensor memory.
+// tau: 16-byte aligned, in global memory (LDG) or shared memory.
+struct ChunkTau {
+  ulonglong2 t[8];
+};
+template <bool LDG>
+__device__ __forceinline__ void load_chunk_tau(ChunkTau& c, const float* __restrict__ tau) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    if constexpr (LDG)
+      asm volatile("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(c.t[j].x), "=l"(c.t[j].y) : "l"(tau + 4 * j));
+    else
+      c.t[j] = *reinterpret_cast<const ulonglong2*>(tau + 4 * j);
+  }
+}
+
 // Turns a row's 32 products into tau_j - value_j (value_j as screen_value's; a
 // pair passes if that is <= -kappa, rounding to nearest being symmetric) and
 // returns their minimum: two pairs per instruction, and no sign change of the
-// terms. tau: 16-byte aligned, in global memory (LDG) or shared memory.
-template <int KIND, bool LDG>
-__device__ __forceinline__ float screen_chunk(uint32_t (&v)[32], const float* __restrict__ tau, float scale) {
+// terms.
+template <int KIND>
+__device__ __forceinline__ float screen_chunk(uint32_t (&v)[32], const ChunkTau& tau, float scale) {
   const uint64_t ns = ptx::pack_f32x2(__float_as_uint(-scale), __float_as_uint(-scale));
   float m = INFINITY;
 #pragma unroll
   for (int j = 0; j < 32; j += 4) {
-    const ulonglong2* p = reinterpret_cast<const ulonglong2*>(tau + j);
-    const ulonglong2 tt = LDG ? __ldg(p) : *p;
+    const ulonglong2 tt = tau.t[j / 4];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const uint64_t a = ptx::pack_f32x2(v[j + 2 * u], v[j + 2 * u + 1]), tu = u ? tt.y : tt.x;

@@ -341,6 +341,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           chunks &= chunks - 1;
           uint32_t v[32];
           ptx::tmem_ld32(tbase + (uint32_t)(ch * 32), v);
+          ChunkTau ct;
+          load_chunk_tau<false>(ct, my_tau + ch * 32);
           ptx::tmem_wait_ld();
           if (chunks == 0) {
             ptx::tc_fence_before();
@@ -349,7 +351,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           // with close keys and few features most passing chunks hold no pair
           // that passes
-          const float least = screen_chunk<KIND, false>(v, my_tau + ch * 32, scl);
+          const float least = screen_chunk<KIND>(v, ct, scl);
           const bool some = ((pass >> ch) & 1u) && least <= -kap;
           if (!__any_sync(0xffffffffu, some)) continue;
           uint32_t mask = 0;

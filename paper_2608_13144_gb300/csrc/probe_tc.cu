@@ -513,6 +513,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           chunks &= chunks - 1;
           uint32_t v[32];
           ptx::tmem_ld32(tbase + (uint32_t)(ch * 32), v);
+          ChunkTau ct;
+          load_chunk_tau<!kTauStaged>(ct, (kTauStaged ? my_tau : tau_g) + ch * 32);
           ptx::tmem_wait_ld();
           if (chunks == 0) {
             ptx::tc_fence_before();
@@ -521,8 +523,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           // with close keys and few features most passing chunks hold no pair
           // that passes (1.5 million keys x 1,909 queries like them, d = 24: 1005 us
-          // with 32 loads, products and comparisons for each, 662 with this)
-          const float least = screen_chunk<KIND, !kTauStaged>(v, (kTauStaged ? my_tau : tau_g) + ch * 32, scl);
+          // with 32 loads, products and comparisons for each, 619 with this)
+          const float least = screen_chunk<KIND>(v, ct, scl);
           const bool some = ((pass >> ch) & 1u) && least <= -kap;
           if (!__any_sync(0xffffffffu, some)) continue;
           uint32_t mask = 0;

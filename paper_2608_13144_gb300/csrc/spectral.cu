@@ -108,11 +108,30 @@ struct SpectralArgs {
   double* A[2];    // n x np, blocked layout (columns from n on are never read into a result)
   double* X;       // m x np, blocked layout: X in FP64, zero past n
   double* XT;      // n x mp, zero past m
-  double* w;       // m
-  double* u;       // n
+  double* w;       // segments(n) x mp: partial sums of X v
+  double* u;       // segments(m) x np: partial sums of X^T w
   unsigned* ctr;   // grid barrier, zero at launch
   SpecResult* res;
 };
+
+// The iteration's products run in segments of kSeg steps, each a chain of its
+// own on some warp of the grid, added in order afterwards: a chain's step takes
+// 64 cycles, so whole chains took 5 to 8 us a product at 128 to 256 steps (the
+// kernel at C = 200: d = 128 179 -> 162 us, d = 256 380 -> 356 us).
+constexpr int kSeg = 32;
+__host__ __device__ constexpr int segments(int n) { return (n + kSeg - 1) / kSeg; }
+__device__ __forceinline__ double add_segments(const double* p, int stride, int n) {
+  double s = 0.0;
+  for (int g0 = 0; g0 < n; g0 += 8) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = g0 + u < n ? __ldcg(p + (size_t)(g0 + u) * stride) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (g0 + u < n) s += v[u];
+  }
+  return s;
+}
 
 // Element (k, j) of a matrix with K rows in column blocks of 32: a block's
 // rows are contiguous (a panel of 32 columns is one stream; rows of a
@@ -334,31 +353,30 @@ __global__ void __launch_bounds__(kSpThreads) k_spectral(const SpectralArgs a) {
   for (int k = tid; k < n; k += kSpThreads) v[k] /= nv;
   __syncthreads();
 
-  const int mu = mp / 32, nu32 = a.np / 32;  // 32-lane units of the two products
+  const int mu = mp / 32, nu32 = a.np / 32;  // 32-lane units of the two products, times their segments
+  const int sv = segments(n), sw = segments(m);
   double theta = 0.0, theta_prev = -1.0, resid = INFINITY;
   int it = 0, converged = 0;
   for (it = 1; it <= a.max_iter; ++it) {
-    for (int g = blockIdx.x + gridDim.x * warp; g < mu; g += gridDim.x * kSpWarps) {
-      const int r = g * 32 + lane;
-      const double acc = chain16(a.XT + r, mp, v, n);
-      if (r < m) a.w[r] = acc;
+    for (int g = blockIdx.x + gridDim.x * warp; g < mu * sv; g += gridDim.x * kSpWarps) {
+      const int r = g % mu * 32 + lane, k0 = g / mu * kSeg;
+      a.w[(size_t)(g / mu) * mp + r] = chain16(a.XT + (size_t)k0 * mp + r, mp, v + k0, n - k0 < kSeg ? n - k0 : kSeg);
     }
     if (!sync_grid()) return;
-    for (int r = tid; r < m; r += kSpThreads) w[r] = __ldcg(a.w + r);
+    for (int r = tid; r < m; r += kSpThreads) w[r] = add_segments(a.w + r, mp, sv);
     __syncthreads();
     if (warp == kSpWarps - 1) {
       const double p = sum_squares(m, lane, [&](int r) { return w[r]; });
       if (lane == 0) red[0] = p;
     } else {
-      for (int g = blockIdx.x + gridDim.x * warp; g < nu32; g += gridDim.x * (kSpWarps - 1)) {
-        const int k = g * 32 + lane;
-        const double acc = chain16(a.X + blk(0, k, m), 32, w, m);
-        if (k < n) a.u[k] = acc;
+      for (int g = blockIdx.x + gridDim.x * warp; g < nu32 * sw; g += gridDim.x * (kSpWarps - 1)) {
+        const int k = g % nu32 * 32 + lane, r0 = g / nu32 * kSeg;
+        a.u[(size_t)(g / nu32) * a.np + k] = chain16(a.X + blk(r0, k, m), 32, w + r0, m - r0 < kSeg ? m - r0 : kSeg);
       }
     }
     if (!sync_grid()) return;
     theta = red[0];
-    for (int k = tid; k < n; k += kSpThreads) u[k] = __ldcg(a.u + k);
+    for (int k = tid; k < n; k += kSpThreads) u[k] = add_segments(a.u + k, a.np, sw);
     __syncthreads();
     if (warp == 0) {
       const double pr = sum_squares(n, lane, [&](int k) { return fma(-theta, v[k], u[k]); });
@@ -507,14 +525,15 @@ void launch_spectral(lipcache* h, SpectralArgs a, cudaStream_t s) {
 size_t spectral_work_bytes(int d, int C) {
   const size_t Cp = (size_t)(C + 31) / 32 * 32;
   const size_t dp = (size_t)(d + 31) / 32 * 32;
-  return sizeof(double) * (2 * dp * d + dp * C + Cp * d + C + d) + 16;  // (either orientation)
+  return sizeof(double) * (2 * dp * d + dp * C + Cp * d + segments(d) * Cp + segments(C) * dp) + 16;  // (either orientation)
 }
 
 void spectral_norm(lipcache* h, cudaStream_t s) {
   const int d = h->d, C = h->C;
   // The transpose of a head with fewer classes than features: a squaring's
   // chains and tiles shrink with the smaller dimension (the kernel, C = 10,
-  // d = 64: 85 us on W, 58 on W^T; C = 200, d = 256: 441 and 380). Without squarings the start
+  // d = 64: 85 us on W, 58 on W^T; C = 200, d = 256: 441 and 380; both with whole
+  // chains in the iteration). Without squarings the start
   // vector is fixed and the iteration stays on W.
   const bool tr = C < d && h->squarings > 0;
   SpectralArgs a;
@@ -533,8 +552,8 @@ void spectral_norm(lipcache* h, cudaStream_t s) {
   a.X = a.A[1] + (size_t)a.np * a.n;
   a.XT = a.X + (size_t)a.np * a.m;
   a.w = a.XT + (size_t)a.mp * a.n;
-  a.u = a.w + a.m;
-  a.ctr = reinterpret_cast<unsigned*>(a.u + a.n);
+  a.u = a.w + (size_t)segments(a.n) * a.mp;
+  a.ctr = reinterpret_cast<unsigned*>(a.u + (size_t)segments(a.m) * a.np);
   a.res = h->spec;
   LC_CUDA(cudaMemsetAsync(a.ctr, 0, sizeof(unsigned), s));
   // a barrier that expired leaves this in place: neither converged nor degenerate

@@ -151,6 +151,15 @@ static __device__ __noinline__ void recheck_warp(const Recheck& a, uint32_t mask
   }
 }
 
+// The screen constant of rows that are no query (those that fill the last query
+// tile up). An entry's screen term is -inf where its radius overflows (an
+// empirical policy's, a head whose rows coincide or nearly vanish), which beats
+// any constant that can be compared; every comparison with a NaN fails, so such
+// a row passes neither the chunk test nor a pair's. The recheck reads the
+// caller's own rows, which end with the last query, and the words of the
+// rows past it stay empty.
+__device__ __forceinline__ float no_query_kappa() { return __int_as_float(0x7fffffff); }
+
 // Operand kinds of the tensor screen. Both stream 128-byte rows (one swizzle
 // row) per chunk and advance 32 bytes per MMA. kF16 reads the table's FP16
 // copy: the same 11-bit significand as TF32, rounded to nearest instead of

@@ -214,3 +214,56 @@ def test_batches_in_a_row(dev, d, n, nq):
                 assert np.array_equal(x[:k].view(np.uint8), y.view(np.uint8)), (path, k)
     c.close()
     fresh.close()
+
+
+@pytest.mark.parametrize("kind", ["fp16", "tf32"])
+@pytest.mark.parametrize("radius", ["global", "coinciding"])
+@pytest.mark.parametrize("B", [129, 257, 640])
+def test_overflowing_radius_ragged_batch(dev, kind, radius, B):
+    """Entries whose radius overflows have a screen term of -inf, which every
+    query passes; the rows that fill the last query tile up must not: the
+    screen rechecks no more than B x size pairs, and a larger exact batch
+    afterwards finds no hit of theirs. The queries are the first rows of a
+    larger buffer."""
+    from paper_2608_13144_gb300.lipcache import LipCache
+    n, d, C = 700, 48, 4
+    rng = np.random.default_rng(B)
+    s = np.float32(1.0 if kind == "fp16" else 1e5)  # 1e5: no FP16 copy of the keys serves
+    rows = torch.from_numpy(rng.standard_normal((n, d)).astype(np.float32) * s).to(dev)
+    buf = torch.from_numpy(rng.standard_normal((2048, d)).astype(np.float32) * s).to(dev)
+    far = torch.from_numpy(rng.standard_normal((1024, d)).astype(np.float32) * s * np.float32(3)).to(dev)
+    W = (rng.standard_normal((C, d)) / d).astype(np.float32) / s
+    b = np.zeros(C, np.float32)
+    if radius == "coinciding":  # every row the same: no class can take over, r* = +inf
+        W[:] = W[0]
+        b = np.arange(C, dtype=np.float32)
+
+    def cache():
+        c = LipCache(d, C, n, "tight", device=dev)
+        c.set_head(torch.from_numpy(W).to(dev), torch.from_numpy(b).to(dev))
+        c.insert(rows)
+        c.set_probe_path("exact")
+        return c
+
+    c, fresh = cache(), cache()
+    ref_far = [t.cpu().numpy() for t in fresh.probe(far)]
+    if radius == "global":
+        c.set_radius_policy("global", 1e30)
+    ref = [t.cpu().numpy() for t in c.probe(buf[:B])]
+    assert (ref[0] >= 0).all()
+    for path in ("tensor", "tensor_single", "tensor_pair"):
+        if radius == "global":
+            c.set_radius_policy("global", 1e30)
+        c.set_probe_path(path)
+        c.reset_stats()
+        got = [t.cpu().numpy() for t in c.probe(buf[:B])]
+        for x, y in zip(ref, got):
+            assert np.array_equal(x, y), path
+        assert c.info()["candidates"] == B * c.size  # (every pair of a query passes, no other)
+        if radius == "global":
+            c.set_radius_policy("certified")
+        c.set_probe_path("exact")
+        for x, y in zip(ref_far, [t.cpu().numpy() for t in c.probe(far)]):
+            assert np.array_equal(x, y), path
+    c.close()
+    fresh.close()

@@ -23,6 +23,11 @@
  *    4-byte alignment. Indices are int64 in cache insertion order.
  *  - A cache handle is not thread-safe: calls on one handle must be
  *    serialised by the caller. Distinct handles are independent.
+ *  - The calls on one handle share its scratch memory, so their work must not
+ *    overlap on the GPU either: order streams that use one handle with an
+ *    event (or synchronise). The results of overlapping probes are undefined;
+ *    later calls are not affected. lipcache_probe_noalloc has scratch of its
+ *    own: see there.
  *  - Inputs are not validated element by element: a NaN logit margin fails
  *    r > 0 (the row is rejected); a NaN query fails the strict hit test
  *    (it misses and falls back to MainNet).
@@ -420,7 +425,8 @@ lipcache_status lipcache_probe_host(lipcache_t* h, const float* Q_host, int64_t 
  * scratch lives in one fixed array compiled into the library
  * (LIPCACHE_NOALLOC_SCRATCH_BYTES per device, held by every GPU that loads
  * the library until the process exits, with 4 bytes for each of the most rows
- * it can serve beside it) and nothing is allocated.
+ * it can serve beside it) and nothing is allocated. It may overlap on the GPU
+ * with lipcache_probe, also of the same handle.
  * Limit: ceil(B/128)*128 * (4*d_pad + 12) bytes, plus alignment, must fit the
  * array (e.g. 4,096 queries at d <= 256); larger batches get E_INVALID with
  * the sizes in the message. The first call on a device resolves the array's

@@ -230,6 +230,7 @@ LC_API lipcache_status lipcache_create(int32_t d, int32_t C, int64_t capacity, i
       c.take(h->table.label, rows);
       c.take(h->table.yG, rows);
       c.take(h->report, 1);
+      c.take(h->done, lipcache::kDoneSlots + 1);
       c.take(h->ins_size0, 1);
       c.take(h->spec, 1);
       c.take(h->W, (size_t)C * d);
@@ -247,7 +248,8 @@ LC_API lipcache_status lipcache_create(int32_t d, int32_t C, int64_t capacity, i
     });
     LC_CUDA(cudaMemset(h->table.tau, 0x7f, sizeof(float) * rows));
     LC_CUDA(cudaMemset(h->table.rr, 0, sizeof(float) * rows));
-    LC_CUDA(cudaMemset(h->report, 0, sizeof(lc::DevReport)));
+    LC_CUDA(cudaMemset(h->report, 0, (size_t)((unsigned char*)(h->done + lipcache::kDoneSlots + 1) -
+                                              (unsigned char*)h->report)));
     static_assert(sizeof(lc::DevReport) + sizeof(lc::SpecResult) + 64 <= kPinBlock, "one block holds all three");
     h->host_arena = pin_take();
     std::memset(h->host_arena, 0, kPinBlock);

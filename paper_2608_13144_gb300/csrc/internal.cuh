@@ -156,8 +156,6 @@ struct DevReport {
   int64_t total[4];  // rows appended by the last insert; consistency counts
   int64_t size;      // table size
   int64_t unfit;     // entries whose FP16 copy does not serve the screen
-  unsigned done_ctas;  // finished CTAs of a probe kernel that finalizes itself (0 between probes)
-  unsigned pad;
   DevStats stats;
 };
 
@@ -254,6 +252,14 @@ struct lipcache {
   int32_t* ins_bcount = nullptr;
   int32_t* ins_boffset = nullptr;
   lc::DevReport* report = nullptr;       // device
+  // Counters of finished CTAs, for the probe kernels that finalize themselves:
+  // each is 0 but while its launch runs. Launches take them in turn, so that
+  // probes which overlap on the GPU (streams that nothing orders) leave every
+  // counter at 0 behind them; a probe captured into a graph, which may be
+  // replayed beside any other, takes the last one and clears it itself.
+  static constexpr unsigned kDoneSlots = 64;
+  unsigned* done = nullptr;              // device, kDoneSlots + 1
+  unsigned done_next = 0;
   lc::DevReport* report_host = nullptr;  // pinned; report_host->unfit is settled with `size`
   // The table size also lives on the device: k_scan takes an insert's base
   // index from it and advances it, so inserts chain on their stream without
@@ -269,8 +275,10 @@ struct lipcache {
   float* qpad = nullptr;
   float* kappa = nullptr;
   float* qscale = nullptr;  // power-of-two scale of each FP16 query
-  unsigned long long* best = nullptr;  // every word is empty (all ones) between probes ...
-  bool best_clean = false;             // ... unless this is false
+  // Every word is empty (all ones) between probes, unless best_clean is false:
+  // the probe that fills words empties them, after the last of its CTAs.
+  unsigned long long* best = nullptr;
+  bool best_clean = false;
   // host-buffer probe staging
   int64_t hq_cap = 0;
   float* hq = nullptr;
@@ -394,6 +402,7 @@ struct ProbeBuffers {
   float* kappa;
   float* scale;
   unsigned long long* best;
+  unsigned* done;  // the counter of finished CTAs
 };
 // probe_tc.cu: the tensor probe; `path` is LIPCACHE_PROBE_TENSOR (kernel
 // chosen by shape), _TENSOR_SINGLE or _TENSOR_PAIR. Returns the kernel that
@@ -408,7 +417,7 @@ void launch_probe_pair(lipcache* h, int64_t B, bool f16, const ProbeBuffers& b, 
 // probe.cu / probe_tc.cu: the probe on caller-provided scratch memory
 void probe_external_scratch(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* out_label,
                             float* out_dist, float* qpad, float* kappa, float* qscale, unsigned long long* best,
-                            cudaStream_t s);
+                            unsigned* done, cudaStream_t s);
 // api.cu: run fn(ctx) with the C ABI's error handling (status + message)
 lipcache_status run_guarded(void (*fn)(void*), void* ctx);
 // api.cu: harvest completed timing events (blocking on the oldest if `all`

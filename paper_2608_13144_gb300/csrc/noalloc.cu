@@ -27,17 +27,21 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[LIPCACHE_NOALLO
 // of the array above
 constexpr int64_t kMaxRows = LIPCACHE_NOALLOC_SCRATCH_BYTES / (4 * 32 + 12);
 static __device__ float g_noalloc_scale[kMaxRows];
+// and the counter of finished CTAs (a probe of the same handle on its own
+// scratch may run beside this one)
+static __device__ unsigned g_noalloc_done;
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 void* g_scratch_addr[kMaxDevices] = {};
 void* g_scale_addr[kMaxDevices] = {};
+void* g_done_addr[kMaxDevices] = {};
 
-// Device address of g_noalloc_scratch on the current device. In host code the
+// Device addresses of these variables on the current device. In host code the
 // symbol's name only stands for the variable; its device address comes from
 // cudaGetSymbolAddress, resolved once per device (on the first call of that
 // device) and cached.
-void* scratch_address(int device, void*& scale) {
+void* scratch_address(int device, void*& scale, void*& done) {
   LC_REQUIRE(device >= 0 && device < kMaxDevices, LIPCACHE_E_INVALID, "device ordinal out of range");
   std::lock_guard<std::mutex> lock(g_mu);
   if (!g_scratch_addr[device]) {
@@ -46,10 +50,14 @@ void* scratch_address(int device, void*& scale) {
     LC_REQUIRE(p != nullptr, LIPCACHE_E_CUDA, "cudaGetSymbolAddress returned NULL for the scratch array");
     void* q = nullptr;
     LC_CUDA(cudaGetSymbolAddress(&q, g_noalloc_scale));
+    void* r = nullptr;
+    LC_CUDA(cudaGetSymbolAddress(&r, g_noalloc_done));
     g_scale_addr[device] = q;
+    g_done_addr[device] = r;
     g_scratch_addr[device] = p;
   }
   scale = g_scale_addr[device];
+  done = g_done_addr[device];
   return g_scratch_addr[device];
 }
 
@@ -108,12 +116,12 @@ LC_API lipcache_status lipcache_probe_noalloc(lipcache_t* h, const float* Q, int
                      "asynchronous inserts are pending: settle them (lipcache_size) before capturing a probe");
           lc::settle_size(c.h);
         }
-        void* scale = nullptr;
-        unsigned char* base = static_cast<unsigned char*>(scratch_address(c.h->device, scale));
+        void *scale = nullptr, *done = nullptr;
+        unsigned char* base = static_cast<unsigned char*>(scratch_address(c.h->device, scale, done));
         lc::probe_external_scratch(c.h, c.Q, c.B, c.oi, c.ol, c.od, reinterpret_cast<float*>(base + L.qpad),
                                    reinterpret_cast<float*>(base + L.kappa), static_cast<float*>(scale),
                                    reinterpret_cast<unsigned long long*>(base + L.best),
-                                   reinterpret_cast<cudaStream_t>(c.s));
+                                   static_cast<unsigned*>(done), reinterpret_cast<cudaStream_t>(c.s));
       },
       &ctx);
 }

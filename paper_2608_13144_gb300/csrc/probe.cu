@@ -41,10 +41,13 @@ constexpr unsigned kFull = 0xffffffffu;
 __global__ void __launch_bounds__(256) k_prologue(const float* __restrict__ Q, int64_t B, int d, int dpad,
                                                   int64_t Bpad, float* __restrict__ qpad, float* __restrict__ kappa,
                                                   unsigned long long* __restrict__ best, double one_minus_c,
-                                                  DevStats* __restrict__ st) {
+                                                  unsigned* __restrict__ done, DevStats* __restrict__ st) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   ptx::launch_dependents();
-  if (blockIdx.x == 0 && threadIdx.x == 0) st->abort_flag = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    st->abort_flag = 0;
+    *done = 0u;
+  }
   const int64_t row = (int64_t)blockIdx.x * 8 + warp;
   if (row >= Bpad) return;
   float part = 0.f;
@@ -73,11 +76,15 @@ __global__ void __launch_bounds__(256) k_prologue(const float* __restrict__ Q, i
 __global__ void __launch_bounds__(256) k_prologue16(const float* __restrict__ Q, int64_t B, int d, int d16,
                                                     int64_t Bpad, __half* __restrict__ q16, float* __restrict__ kappa,
                                                     float* __restrict__ qscale, unsigned long long* __restrict__ best,
-                                                    double one_minus_c, DevStats* __restrict__ st) {
+                                                    double one_minus_c, unsigned* __restrict__ done,
+                                                    DevStats* __restrict__ st) {
   constexpr int kMaxChunk = 8;  // d <= 512
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   ptx::launch_dependents();
-  if (blockIdx.x == 0 && threadIdx.x == 0) st->abort_flag = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    st->abort_flag = 0;
+    *done = 0u;
+  }
   const int64_t row = (int64_t)blockIdx.x * 8 + warp;
   if (row >= Bpad) return;
   const float* src = Q + (size_t)row * d;
@@ -222,7 +229,19 @@ __global__ void k_finalize(ProbeOut out) {
   if (q < out.B) finalize_query(out, q, out.abort && *out.abort != 0);
 }
 
-void ensure_probe_scratch(lipcache* h, int64_t Bpad, cudaStream_t s) {
+// Empties the reduction words and clears the counter.
+__global__ void k_clear(unsigned long long* __restrict__ best, int64_t B, unsigned* __restrict__ done) {
+  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < B) best[q] = ~0ull;
+  if (q == 0) *done = 0u;
+}
+
+void clear_words(unsigned long long* best, int64_t n, unsigned* done, cudaStream_t s) {
+  k_clear<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(best, n, done);
+  LC_LAUNCH_CHECK("k_clear");
+}
+
+void ensure_probe_scratch(lipcache* h, int64_t Bpad) {
   if (Bpad <= h->q_cap) return;
   int64_t cap = h->q_cap ? h->q_cap : 1024;
   while (cap < Bpad) cap *= 2;
@@ -233,9 +252,7 @@ void ensure_probe_scratch(lipcache* h, int64_t Bpad, cudaStream_t s) {
     c.take(h->qscale, (size_t)cap);
     c.take(h->best, (size_t)cap);
   });
-  h->best_clean = false;
-  LC_CUDA(cudaMemsetAsync(h->best, 0xff, sizeof(unsigned long long) * (size_t)cap, s));
-  h->best_clean = true;
+  h->best_clean = false;  // (the next probe empties them, on its stream)
   h->q_cap = cap;
 }
 
@@ -244,8 +261,7 @@ void ensure_probe_scratch(lipcache* h, int64_t Bpad, cudaStream_t s) {
 bool tensor_path_supported(int dpad) { return dpad <= 256; }
 
 void reserve_probe(lipcache* h, int64_t max_batch) {
-  ensure_probe_scratch(h, (max_batch + 127) / 128 * 128, nullptr);
-  LC_CUDA(cudaStreamSynchronize(nullptr));  // (later probes may run on any stream)
+  ensure_probe_scratch(h, (max_batch + 127) / 128 * 128);
 }
 
 // The small kernels around the tensor probe prefer the same shared-memory
@@ -264,7 +280,7 @@ void set_probe_carveout(lipcache* h) {
 
 namespace {
 // The launch sequence of a probe on the given buffers. `clean`: every
-// reduction word is empty.
+// reduction word is empty and the counter is 0.
 void probe_on(lipcache* h, int64_t B, const ProbeBuffers& b, bool clean, int64_t* out_index, int32_t* out_label,
               float* out_dist, bool timing, cudaStream_t s) {
   const int64_t Bpad = (B + 127) / 128 * 128;
@@ -278,19 +294,19 @@ void probe_on(lipcache* h, int64_t B, const ProbeBuffers& b, bool clean, int64_t
   ProbeOut out{b.best, B, h->table.label, out_index, out_label, out_dist, &h->stats->abort_flag, nullptr};
   // the main kernel finalizes small batches itself (the exact one also only
   // where its CTAs, which count themselves, are few)
-  if (h->size > 0 && B <= kFusedQueries && (!exact || ex * ey <= 4096)) out.done = &h->report->done_ctas;
+  if (h->size > 0 && B <= kFusedQueries && (!exact || ex * ey <= 4096)) out.done = b.done;
   if (exact || h->size == 0) {
-    if (!clean) LC_CUDA(cudaMemsetAsync(b.best, 0xff, sizeof(unsigned long long) * (size_t)B, s));
+    if (!clean) clear_words(b.best, B, b.done, s);
     if (h->size == 0) LC_CUDA(cudaMemsetAsync(&h->stats->abort_flag, 0, sizeof(int), s));
   } else {
     const unsigned pgrid = (unsigned)((Bpad + 7) / 8);
     if (f16) {
       k_prologue16<<<pgrid, 256, 0, s>>>(b.Q, B, h->d, h->table.d16, Bpad, static_cast<__half*>(b.q), b.kappa, b.scale,
-                                         b.best, 1.0 - h->c_scr, h->stats);
+                                         b.best, 1.0 - h->c_scr, b.done, h->stats);
       LC_LAUNCH_CHECK("k_prologue16");
     } else {
       k_prologue<<<pgrid, 256, 0, s>>>(b.Q, B, h->d, h->dpad, Bpad, static_cast<float*>(b.q), b.kappa, b.best,
-                                       1.0 - h->c_scr, h->stats);
+                                       1.0 - h->c_scr, b.done, h->stats);
       LC_LAUNCH_CHECK("k_prologue");
     }
   }
@@ -330,23 +346,36 @@ void probe_on(lipcache* h, int64_t B, const ProbeBuffers& b, bool clean, int64_t
 
 void probe(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* out_label, float* out_dist,
            cudaStream_t s) {
-  ensure_probe_scratch(h, (B + 127) / 128 * 128, s);
+  ensure_probe_scratch(h, (B + 127) / 128 * 128);
+  // A captured probe runs whenever its graph is replayed, so it assumes nothing
+  // of the words and the counter. (A stream that cannot be asked: as captured.)
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    cap = cudaStreamCaptureStatusActive;
+  }
+  ProbeBuffers b{Q, h->qpad, h->kappa, h->qscale, h->best, h->done + lipcache::kDoneSlots};
+  if (cap != cudaStreamCaptureStatusNone) {
+    probe_on(h, B, b, false, out_index, out_label, out_dist, true, s);
+    return;
+  }
+  b.done = h->done + h->done_next++ % lipcache::kDoneSlots;
+  if (!h->best_clean) clear_words(h->best, h->q_cap, b.done, s);
   // (the finalizing kernel empties the words it reads; a call that throws on
   // the way leaves them in doubt)
-  const bool clean = h->best_clean;
   h->best_clean = false;
-  probe_on(h, B, ProbeBuffers{Q, h->qpad, h->kappa, h->qscale, h->best}, clean, out_index, out_label, out_dist, true, s);
+  probe_on(h, B, b, true, out_index, out_label, out_dist, true, s);
   h->best_clean = true;
 }
 
 // The same launch sequence as probe(), on scratch memory the caller
 // provides (qpad: Bpad x d_pad floats, kappa and qscale: Bpad floats, best:
-// Bpad words, Bpad = B rounded up to 128; the FP16 form of the queries,
-// d16 <= 2 d_pad halves per row, takes qpad's place). Allocates nothing.
+// Bpad words, Bpad = B rounded up to 128; done: one word; the FP16 form of the
+// queries, d16 <= 2 d_pad halves per row, takes qpad's place). Allocates nothing.
 void probe_external_scratch(lipcache* h, const float* Q, int64_t B, int64_t* out_index, int32_t* out_label,
                             float* out_dist, float* qpad, float* kappa, float* qscale, unsigned long long* best,
-                            cudaStream_t s) {
-  probe_on(h, B, ProbeBuffers{Q, qpad, kappa, qscale, best}, false, out_index, out_label, out_dist, false, s);
+                            unsigned* done, cudaStream_t s) {
+  probe_on(h, B, ProbeBuffers{Q, qpad, kappa, qscale, best, done}, false, out_index, out_label, out_dist, false, s);
 }
 
 }  // namespace lc

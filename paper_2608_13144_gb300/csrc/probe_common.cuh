@@ -30,7 +30,7 @@ struct ProbeOut {
   int32_t* out_label;  // nullable
   float* dist;         // nullable
   const int* abort;    // nullable: non-zero turns the batch into misses
-  unsigned* done;      // zero between launches; null: k_finalize follows
+  unsigned* done;      // zero at the launch and left so; null: k_finalize follows
 };
 
 // Unpack query q's word, and leave it empty for the next batch.

@@ -266,7 +266,9 @@ lipcache_status lipcache_probe(lipcache_t* h, const float* Q, int64_t B, int64_t
  * on capacity: E_FULL, before any work, if size + min(n, budget_total)
  * exceeds it (K-center: min(n, C x budget_per_class)). Errors: those of
  * lipcache_insert and lipcache_probe; E_STATE under an empirical radius
- * policy; E_INVALID for an unknown strategy or budgets it does not take.
+ * policy; E_INVALID for an unknown strategy or budgets it does not take;
+ * E_DEVICE if a bounded wait of a probe kernel expired (what the chunks before
+ * it kept stays in the cache; n_selected is 0).
  */
 lipcache_status lipcache_insert_select(lipcache_t* h, const float* H, int64_t n, const int32_t* payload,
                                        int32_t require_consistency, int32_t strategy, int64_t budget_total,
@@ -380,8 +382,8 @@ lipcache_status lipcache_read_head(lipcache_t* h, float* W_host, float* b_host, 
  * arrives on: the bounded wait (~2^31 cycles, about a second) expires, the
  * kernel takes its abort path (no trap, no hang), the batch's queries come
  * back as misses, lipcache_info.device_errors counts the aborted CTAs, and
- * the synchronous entry points (lipcache_probe_host, _probe_writeback)
- * return LIPCACHE_E_DEVICE. The exact kernel has no waits and is unaffected.
+ * the synchronous entry points (lipcache_probe_host, _probe_writeback,
+ * _insert_select) return LIPCACHE_E_DEVICE. The exact kernel has no waits and is unaffected.
  * flags = 0 restores normal operation. Errors: E_INVALID (unknown bits).
  */
 #define LIPCACHE_DEBUG_STALL_PROBE 1

@@ -279,6 +279,7 @@ struct ResolveArgs {
   int32_t* class_cnt;      // per class, kept in this call
   SelState* st;
   int32_t* list;           // kept members in order
+  const DevStats* stats;   // abort_flag set: the chunk's probe gave up, `hit` says nothing
   int kc, C, budget_pc;
   long long budget_total;
 };
@@ -291,7 +292,7 @@ struct ResolveArgs {
 // in batches: the undecided members before the first one that another
 // undecided member covers are independent, so each is kept unless its class or
 // the call runs out of budget before it (ranks by ballot); what they cover
-// drops out. Labels, hits and class counts are in shared memory. Bound by the
+// drops out. A chunk whose probe gave up keeps nothing. Labels, hits and class counts are in shared memory. Bound by the
 // chain of groups, ~1,200 cycles each on a pool where a third of the members
 // are near-duplicates; one warp walking the members took 160 ns for each
 // (4,096 members: 80 us, before 665 us).
@@ -305,6 +306,7 @@ __global__ void __launch_bounds__(1024) k_sel_resolve(ResolveArgs a) {
   __shared__ int32_t cnt_s[LIPCACHE_MAX_CLASSES];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int groups = (a.kc + 31) / 32;
+  const bool aborted = a.stats->abort_flag != 0;
   auto load_row = [&](int g, uint32_t (&w)[kPer]) {
     const int j = 32 * g + warp;
 #pragma unroll
@@ -320,7 +322,7 @@ __global__ void __launch_bounds__(1024) k_sel_resolve(ResolveArgs a) {
   for (int j = tid; j < kSelChunk; j += 1024) {
     const bool in = j < a.kc;
     const int32_t lab = in ? a.label[a.rows[j]] : -1;
-    free_s[j] = in && a.hit[j] < 0 ? 1 : 0;
+    free_s[j] = in && a.hit[j] < 0 && !aborted ? 1 : 0;
     lab_s[j] = (int16_t)(a.budget_pc > 0 && lab >= 0 && lab < a.C ? lab : -1);
   }
   int nk = 0;
@@ -681,6 +683,7 @@ int64_t select_insert(lipcache* h, const float* H, int64_t n, const int32_t* pay
     ra.class_cnt = x.class_cnt;
     ra.st = st;
     ra.list = x.list;
+    ra.stats = h->stats;
     ra.kc = kc;
     ra.C = h->C;
     ra.budget_pc = budget_per_class;
@@ -707,9 +710,14 @@ int64_t select_insert(lipcache* h, const float* H, int64_t n, const int32_t* pay
     k_sel_scatter<<<(unsigned)(kTailBlocks + (kc + 7) / 8), 256, 0, s>>>(sa);
     LC_LAUNCH_CHECK("k_sel_scatter");
     pick();  // the next chunk's members, so that one wait serves both
-    fetch_report(h, s);  // (the next chunk's probe: whether the FP16 copies still serve)
+    fetch_report(h, s);  // (the next chunk's probe: whether the FP16 copies still serve; an aborted one)
     LC_CUDA(cudaStreamSynchronize(s));
     h->size += hs->n_list;
+    if (h->stats_host->abort_flag) {
+      store_size_dev(h, s);  // the chunks before this one stay
+      LC_CUDA(cudaStreamSynchronize(s));
+      throw Error(LIPCACHE_E_DEVICE, "a bounded wait of the probe kernel expired: the selection stopped");
+    }
   }
   store_size_dev(h, s);  // the table grew from the host
   return hs->kept;

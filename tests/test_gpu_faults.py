@@ -110,3 +110,37 @@ def test_certify_stall_aborts_cleanly(dev):
     check_insert(idx.cpu().numpy(), rad.cpu().numpy(), n, ref, (W, b, rows, 1.0))
     assert c.size == n
     c.close()
+
+
+def test_stalled_probe_stops_a_selection(dev):
+    """A selection whose chunk's probe gives up does not take the misses it
+    reports for uncovered candidates: it appends nothing of that chunk and
+    returns E_DEVICE; the cache goes on."""
+    from paper_2608_13144_gb300._lib import LipCacheError
+    from paper_2608_13144_gb300.lipcache import LipCache
+    w = synth.WORKLOADS["tiny"]
+    W, b = synth.head(w)
+    rows = torch.from_numpy(synth.cache_rows(w)).to(dev)
+    n = rows.shape[0]
+
+    def cache():
+        c = LipCache(w.d, w.C, 3 * n, device=dev)
+        c.set_head(torch.from_numpy(W).to(dev), torch.from_numpy(b).to(dev))
+        c.insert(rows[: n // 2])
+        c.set_probe_path("tensor")
+        return c
+
+    c, fresh = cache(), cache()
+    size = c.size
+    want = fresh.insert_select(rows)
+    c.set_debug(STALL)
+    with pytest.raises(LipCacheError) as e:
+        c.insert_select(rows)
+    assert e.value.status == 8 and c.size == size and c.info()["device_errors"] > 0
+    c.set_debug(0)
+    got = c.insert_select(rows)
+    for x, y in zip(want, got):
+        assert torch.equal(x, y) if torch.is_tensor(x) else x == y
+    assert want[2] < n  # the first half is covered by itself
+    c.close()
+    fresh.close()

@@ -20,6 +20,8 @@
 // main kernel (exact: every pair on CUDA cores; tensor: tcgen05 screen +
 // recheck, probe_tc.cu), which unpacks small batches itself, and else
 // k_finalize.
+#include <algorithm>
+
 #include "internal.cuh"
 #include "probe_common.cuh"
 
@@ -328,9 +330,16 @@ void probe_on(lipcache* h, int64_t B, const ProbeBuffers& b, bool clean, int64_t
       h->last_grid = (int)(ex * ey);
       h->last_cluster = 1;
       const int qvec = h->d % 4 == 0 && ((uintptr_t)b.Q & 15) == 0;
-      k_probe_exact<<<dim3((unsigned)ex, (unsigned)ey), 256, 0, s>>>(b.Q, B, h->d, qvec, h->table.keys, h->probe_rr(),
-                                                                     h->size, h->dpad, b.best, out, h->stats);
-      LC_LAUNCH_CHECK("k_probe_exact");
+      // (a grid has at most 65,535 rows of CTAs: batches above 4,194,240 take two
+      // launches; they are not finalized by the kernel)
+      constexpr int64_t kMaxRows = 65535;
+      for (int64_t y0 = 0; y0 < ey; y0 += kMaxRows) {
+        const int64_t q0 = y0 * kEQ, n = std::min(B - q0, kMaxRows * kEQ);
+        const dim3 grid((unsigned)ex, (unsigned)((n + kEQ - 1) / kEQ));
+        k_probe_exact<<<grid, 256, 0, s>>>(b.Q + (size_t)q0 * h->d, n, h->d, qvec, h->table.keys, h->probe_rr(),
+                                           h->size, h->dpad, b.best + q0, out, h->stats);
+        LC_LAUNCH_CHECK("k_probe_exact");
+      }
     }
     if (slot >= 0) {
       LC_CUDA(cudaEventRecord(h->tev1[slot], s));

@@ -267,3 +267,24 @@ def test_overflowing_radius_ragged_batch(dev, kind, radius, B):
             assert np.array_equal(x, y), path
     c.close()
     fresh.close()
+
+
+@pytest.mark.parametrize("B", [65535 * 64, 65535 * 64 + 1, 1 << 22])
+def test_largest_exact_batches(dev, B):
+    """The exact kernel on batches around the most query tiles a grid has rows
+    for, up to the largest batch a probe takes."""
+    rng = np.random.default_rng(5)
+    rows = rng.standard_normal((70, 4)).astype(np.float32)
+    c = make(dev, 4, 3, rows)
+    c.insert(torch.from_numpy(rows).to(dev))
+    c.set_probe_path("exact")
+    R = torch.from_numpy(rows).to(dev)
+    Q = R[torch.arange(B, device=dev) % 70]
+    Q[1::2] += 1e3  # (misses)
+    out = c.probe(Q)
+    small = c.probe(Q[:140])
+    for x, y in zip(small, out):
+        want = x.repeat((B + 139) // 140)[:B]
+        assert torch.equal(want, y)
+    assert (small[0][::2] >= 0).any() and (small[0][1::2] == -1).all()
+    c.close()

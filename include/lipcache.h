@@ -149,8 +149,10 @@ typedef struct lipcache_info {
  * Create an empty cache for d-dimensional GuardNet features and a C-class
  * head (Sec. 3.1 notation: z in R^d, W in R^{C x d}). Allocates the key table
  * for `capacity` entries on the current CUDA device: 4 d_pad + 24 bytes per
- * entry and, for d <= 512 and where the memory allows it, an FP16 copy of the
- * keys (2 d bytes, d rounded up to 64) that the tensor screen reads.
+ * entry and, for d <= 512, an FP16 copy of the keys (2 d bytes, d rounded up to
+ * 64) that the tensor screen reads, unless it would take more than a quarter of
+ * the memory then free (the screen then reads the keys in TF32; for d > 256 the
+ * exact kernel takes the probes).
  *   d           1 .. LIPCACHE_MAX_DIM
  *   C           2 .. LIPCACHE_MAX_CLASSES
  *   capacity    1 .. LIPCACHE_MAX_CAPACITY

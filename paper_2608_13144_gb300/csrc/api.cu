@@ -258,15 +258,15 @@ LC_API lipcache_status lipcache_create(int32_t d, int32_t C, int64_t capacity, i
     h->sel_host = h->host_arena + kPinBlock - 64;
     h->stats = &h->report->stats;
     h->stats_host = &h->report_host->stats;
-    // The FP16 copy of the keys (d <= 512), last and only where it leaves room
-    // for scratch: a table without one is screened in TF32.
+    // The FP16 copy of the keys (d <= 512), last and only where it takes no more
+    // than a quarter of the memory then free, so that scratch and other caches
+    // find room: a table without one is screened in TF32. (Asking costs 4 us.)
     if (d <= 512) {
       h->table.d16 = (d + 63) / 64 * 64;
       const size_t bytes = sizeof(__half) * rows * (size_t)h->table.d16;
-      constexpr size_t kGiB = size_t(1) << 30;
       size_t avail = 0, all = 0;
-      if (bytes > 4 * kGiB) LC_CUDA(cudaMemGetInfo(&avail, &all));
-      if ((bytes > 4 * kGiB && avail < bytes + 8 * kGiB) || cudaMalloc(&h->table.keys16, bytes) != cudaSuccess) {
+      LC_CUDA(cudaMemGetInfo(&avail, &all));
+      if (bytes > avail / 4 || cudaMalloc(&h->table.keys16, bytes) != cudaSuccess) {
         cudaGetLastError();
         h->table.keys16 = nullptr;
       }

@@ -147,3 +147,30 @@ def test_noalloc_beside_probe(path):
         torch.cuda.synchronize()
         _same(g, ref, 200)
     c.close()
+
+
+def test_half_copy_leaves_memory():
+    """The FP16 copy of the keys is only taken where it leaves three quarters of
+    the free memory: a table of two fifths of the memory has none, a small one
+    has. (Memory is reserved here, not written.)"""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2608_13144_gb300.lipcache import LipCache
+    dev = torch.device("cuda", 0)
+    LipCache(32, 4, 256, device=dev).close()  # the library's own memory
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+
+    def taken(capacity):
+        before = torch.cuda.mem_get_info(dev)[0]
+        c = LipCache(32, 4, capacity, device=dev)
+        after = torch.cuda.mem_get_info(dev)[0]
+        c.close()
+        return before - after
+
+    per = 4 * 32 + 24  # bytes per entry, and 2 * 64 with the copy
+    free = torch.cuda.mem_get_info(dev)[0]
+    big = int(0.4 * free / per)
+    assert taken(big) < per * big + (1 << 28)
+    small = 1 << 20
+    assert taken(small) >= (per + 128) * small

@@ -460,7 +460,7 @@ def run_ours(args, dist: Dist):
     dist.barrier()
     step_s = e0.elapsed_time(e1) * 1e-3
     clocks = clk.stop()
-    info = cache.info()
+    info, screen = cache.info(), cache.screen_info()
     cache.enable_timing(False)
     kernel_ms = info["kernel_ms_total"] / max(1, info["kernel_launches"])
     hits = sum(int((o[0] >= 0).sum()) for o in outs[: min(nb, args.steps)])
@@ -518,7 +518,7 @@ def run_ours(args, dist: Dist):
     cache.close()
 
     path_id = info["last_probe_path"]
-    fp16 = path_id in (3, 4)  # these keys fit the FP16 copy
+    fp16 = path_id in (3, 4) and screen["fp16"]
     rf = roofline(w, N, B, kernel_ms, pk, pk_kind, PROBE_KERNELS[path_id][0], fp16)
     tf32_derived = pk["bf16_tflops"] * TF32_OVER_BF16
     if rf["bound"] == "tensor" and not args.no_fp16_peak:

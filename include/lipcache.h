@@ -145,6 +145,14 @@ typedef struct lipcache_info {
                                    pin to 5e-6 relative */
 } lipcache_info;
 
+/* The key table's FP16 copy (lipcache_get_screen_info). */
+typedef struct lipcache_screen_info {
+  int64_t unfit;      /* entries whose FP16 copy does not serve the screen (overflow, the subnormal range);
+                         0 without a copy */
+  int32_t fp16_copy;  /* 1: the table has an FP16 copy of its keys */
+  int32_t fp16;       /* 1: tensor probes screen in FP16 (a copy, and every entry fits); 0: in TF32 */
+} lipcache_screen_info;
+
 /*
  * Create an empty cache for d-dimensional GuardNet features and a C-class
  * head (Sec. 3.1 notation: z in R^d, W in R^{C x d}). Allocates the key table
@@ -479,6 +487,11 @@ lipcache_status lipcache_enable_timing(lipcache_t* h, int32_t on);
  * timings (introspection; no counterpart in the paper). Synchronises the
  * device work of this handle. */
 lipcache_status lipcache_get_info(lipcache_t* h, lipcache_info* info);
+
+/* Fill *info (host): which operands the tensor probe's screen reads, and why
+ * (introspection; no counterpart in the paper). Settles asynchronous inserts
+ * first (synchronises their stream). Errors: E_INVALID, E_CUDA. */
+lipcache_status lipcache_get_screen_info(lipcache_t* h, lipcache_screen_info* info);
 
 /* Zero the candidate / device-error counters and the kernel-time sum
  * (instrumentation; no counterpart in the paper). */

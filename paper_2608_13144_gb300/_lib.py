@@ -23,7 +23,8 @@ EXPORTS = ["lipcache_create", "lipcache_set_head", "lipcache_insert", "lipcache_
            "lipcache_probe_noalloc", "lipcache_probe_writeback", "lipcache_consistency",
            "lipcache_set_radius_policy", "lipcache_insert_select", "lipcache_set_debug", "lipcache_read_entries", "lipcache_read_head",
            "lipcache_set_probe_path", "lipcache_set_radius_scale", "lipcache_set_spectral_options",
-           "lipcache_reserve", "lipcache_enable_timing", "lipcache_get_info", "lipcache_reset_stats",
+           "lipcache_reserve", "lipcache_enable_timing", "lipcache_get_info",
+           "lipcache_get_screen_info", "lipcache_reset_stats",
            "lipcache_size", "lipcache_destroy", "lipcache_last_error"]
 
 
@@ -39,6 +40,10 @@ class Info(C.Structure):
                 ("policy_param", C.c_double), ("insert_kernel_ms_total", C.c_double),
                 ("insert_kernel_launches", C.c_int64), ("insert_refined_pairs", C.c_int64),
                 ("insert_full_rows", C.c_int64), ("insert_fp64_rows", C.c_int64)]
+
+
+class ScreenInfo(C.Structure):
+    _fields_ = [("unfit", C.c_int64), ("fp16_copy", C.c_int32), ("fp16", C.c_int32)]
 
 
 class LipCacheError(RuntimeError):
@@ -79,6 +84,7 @@ def load(path: str = LIB_PATH):
         "lipcache_reserve": ([vp, i64], C.c_int),
         "lipcache_enable_timing": ([vp, i32], C.c_int),
         "lipcache_get_info": ([vp, C.POINTER(Info)], C.c_int),
+        "lipcache_get_screen_info": ([vp, C.POINTER(ScreenInfo)], C.c_int),
         "lipcache_reset_stats": ([vp], C.c_int),
         "lipcache_size": ([vp], i64),
         "lipcache_destroy": ([vp], None),

@@ -661,6 +661,17 @@ LC_API lipcache_status lipcache_reset_stats(lipcache_t* h) {
   });
 }
 
+LC_API lipcache_status lipcache_get_screen_info(lipcache_t* h, lipcache_screen_info* info) {
+  return guarded([&] {
+    check_handle(h);
+    LC_REQUIRE(info != nullptr, LIPCACHE_E_INVALID, "info is NULL");
+    sync_size(h);
+    info->unfit = h->report_host->unfit;
+    info->fp16_copy = h->table.keys16 != nullptr ? 1 : 0;
+    info->fp16 = h->f16_screen() ? 1 : 0;
+  });
+}
+
 LC_API lipcache_status lipcache_get_info(lipcache_t* h, lipcache_info* info) {
   return guarded([&] {
     check_handle(h);

@@ -12,7 +12,7 @@ import numpy as np
 import torch
 
 from . import _lib
-from ._lib import Info, check
+from ._lib import Info, ScreenInfo, check
 
 RADIUS_MODES = {"conservative": _lib.RADIUS_CONSERVATIVE, "tight": _lib.RADIUS_TIGHT}
 PROBE_PATHS = {"auto": _lib.PROBE_AUTO, "tensor": _lib.PROBE_TENSOR, "exact": _lib.PROBE_EXACT,
@@ -293,6 +293,14 @@ class LipCache:
         inf = Info()
         check(self.L.lipcache_get_info(self._h, C.byref(inf)))
         return {name: getattr(inf, name) for name, _ in Info._fields_}
+
+    def screen_info(self) -> dict:
+        """What the tensor probe's screen reads: fp16 (bool), fp16_copy (the
+        table has an FP16 copy of its keys) and unfit (entries it does not
+        serve; one is enough for the screen to read the keys in TF32)."""
+        inf = ScreenInfo()
+        check(self.L.lipcache_get_screen_info(self._h, C.byref(inf)))
+        return {"fp16": bool(inf.fp16), "fp16_copy": bool(inf.fp16_copy), "unfit": int(inf.unfit)}
 
     @property
     def size(self) -> int:

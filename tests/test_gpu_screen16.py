@@ -149,23 +149,68 @@ def test_rows_past_the_end(dev, how, n):
     c.close()
 
 
-@pytest.mark.parametrize("what", ["large", "small", "mixed"])
+@pytest.mark.parametrize("what", ["large", "small"])
 def test_unfit_tables(dev, what):
-    """Entries FP16 does not hold (overflow, the subnormal range): the table is
-    screened in TF32, with the same results; a fitting cache beside it is not
-    affected."""
+    """Tables FP16 does not hold (overflow, the subnormal range) are screened in
+    TF32, with the same results."""
     rng = np.random.default_rng(3)
     rows, Q = data(rng, 2000, 64, 300)
-    if what == "large":
-        rows, Q = rows * np.float32(1e5), Q * np.float32(1e5)
-    elif what == "small":
-        rows, Q = rows * np.float32(1e-6), Q * np.float32(1e-6)
-    c = make(dev, 64, 5, rows, capacity=2001)
+    s = np.float32(1e5 if what == "large" else 1e-6)
+    rows, Q = rows * s, Q * s
+    c = make(dev, 64, 5, rows)
+    assert c.screen_info() == {"fp16": True, "fp16_copy": True, "unfit": 0}
     c.insert(torch.from_numpy(rows).to(dev))
-    if what == "mixed":
-        c.insert(torch.full((1, 64), 7e4, device=dev))
-        c.insert(torch.from_numpy(rows[:0]).to(dev))
+    inf = c.screen_info()
+    assert inf["fp16_copy"] and not inf["fp16"] and inf["unfit"] > c.size // 2
     same_as_exact(c, torch.from_numpy(Q).to(dev), ["tensor", "tensor_pair"])
+    c.close()
+
+
+@pytest.mark.parametrize("what", ["large", "small"])
+@pytest.mark.parametrize("grow", ["insert", "unaligned", "scalar", "async", "select", "kcenter", "writeback"])
+def test_unfit_entries_counted(dev, grow, what):
+    """Every path that appends entries counts those whose FP16 copy does not
+    serve: 3 among 500 whose copies do send the whole table to the TF32 screen,
+    and queries next to them hit them. (The features of the small ones round to
+    zero in FP16: an FP16 screen would lose their hits.) A table without such an
+    entry stays in FP16."""
+    d = 65 if grow == "scalar" else 64  # d % 4 != 0: features moved one by one
+    rng = np.random.default_rng(11)
+    rows, Q = data(rng, 500, d, 200)
+    s = np.float32(1e5 if what == "large" else 1e-8)
+    odd = rng.standard_normal((3, d)).astype(np.float32) * s
+    near = odd[np.arange(30) % 3] + s * np.float32(1e-3) * rng.standard_normal((30, d)).astype(np.float32)
+
+    def grown(rows):
+        c = make(dev, d, 6, rows, capacity=1200)
+        R = torch.from_numpy(rows).to(dev)
+        if grow == "unaligned":
+            buf = torch.zeros(rows.size + 1, device=dev)
+            buf[1:] = R.reshape(-1)
+            c.insert(buf[1:].view(rows.shape))
+        elif grow == "async":
+            for k in range(0, len(rows), 100):
+                c.insert(R[k:k + 100], wait=False)
+        elif grow in ("select", "kcenter"):
+            c.insert_select(R, strategy="kcenter" if grow == "kcenter" else "radius_dedup",
+                            budget_per_class=400 if grow == "kcenter" else 0)
+        elif grow == "writeback":
+            c.probe_writeback(R)
+        else:
+            c.insert(R)
+        return c
+
+    at = np.array([7, 250, 502])
+    mixed = np.insert(rows, at - np.arange(3), odd, axis=0)
+    assert np.array_equal(mixed[at], odd)
+    c = grown(mixed)
+    assert c.screen_info() == {"fp16": False, "fp16_copy": True, "unfit": 3}
+    ref = same_as_exact(c, torch.from_numpy(np.concatenate([near, Q])).to(dev), ["tensor", "tensor_pair"])
+    keys = c.entries()["keys"]
+    assert (ref[0][:30] >= 0).all() and np.array_equal(keys[ref[0][:30]], odd[np.arange(30) % 3])
+    c.close()
+    c = grown(rows)
+    assert c.screen_info() == {"fp16": True, "fp16_copy": True, "unfit": 0}
     c.close()
 
 

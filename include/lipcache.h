@@ -84,6 +84,9 @@ typedef enum lipcache_status {
 #define LIPCACHE_INSERT_TILE64 2
 #define LIPCACHE_INSERT_STREAMED 3
 #define LIPCACHE_INSERT_TENSOR 4
+/* Bits of lipcache_insert_kernels: 1 << one of these, STREAMED being the
+ * CUDA-core kernel there, and this one for TENSOR with a streamed head. */
+#define LIPCACHE_INSERT_BIT_TENSOR_STREAMED 32
 
 /* Radius policies of the probe (lipcache_set_radius_policy). */
 #define LIPCACHE_POLICY_CERTIFIED 0  /* per-entry certified radius (Eq. 21 or Eq. 29) */
@@ -364,7 +367,8 @@ lipcache_status lipcache_set_radius_policy(lipcache_t* h, int32_t policy, double
  * Read back cache entries [first, first + n) (insertion order): the triples
  * (z_i, y~_i, r_i) of the cache (Sec. 3.1), with y^G of each key, e.g. to
  * inspect a cache or to persist it: re-inserting the returned keys with their
- * labels as payload into a cache with the same head rebuilds the same entries.
+ * labels as payload into a cache with the same head rebuilds the same entries
+ * (see lipcache_read_head for the radii).
  *   keys_host    n x d FP32 (host), nullable
  *   radius_host  n FP32 (host), nullable: the reported radius r of each entry
  *   label_host   n int32 (host), nullable: payload
@@ -379,7 +383,10 @@ lipcache_status lipcache_read_entries(lipcache_t* h, int64_t first, int64_t n, f
  * classification head (Eq. 5), back to the host (with
  * lipcache_read_entries, what a checkpoint needs: a cache is restored by
  * set_head and re-inserting the entries' keys with their labels as payload,
- * which re-certifies them to the same radii).
+ * which re-certifies them: to the same radii, bit for bit, where the kernels
+ * that lipcache_insert_kernels names give the same bits on both sides, else
+ * to radii within 1e-5 relative, each being within 5e-6 of the exact one. Which
+ * kernel takes an insert depends on d, C and the rows' alignment).
  *   W_host  C x d FP32 row-major (host), nullable
  *   b_host  C FP32 (host), nullable
  * Synchronises `stream`. Errors: E_STATE (no head), E_CUDA.
@@ -492,6 +499,12 @@ lipcache_status lipcache_get_info(lipcache_t* h, lipcache_info* info);
  * (introspection; no counterpart in the paper). Settles asynchronous inserts
  * first (synchronises their stream). Errors: E_INVALID, E_CUDA. */
 lipcache_status lipcache_get_screen_info(lipcache_t* h, lipcache_screen_info* info);
+
+/* The certify kernels that rows passed to the table so far went through, a bit
+ * each (1 << LIPCACHE_INSERT_*, LIPCACHE_INSERT_BIT_TENSOR_STREAMED; 0 for
+ * NULL): what a checkpoint needs to know whether its radii come back bit for
+ * bit (introspection; no counterpart in the paper). */
+int64_t lipcache_insert_kernels(const lipcache_t* h);
 
 /* Zero the candidate / device-error counters and the kernel-time sum
  * (instrumentation; no counterpart in the paper). */

@@ -15,6 +15,7 @@ OK, E_INVALID, E_STATE, E_DEGENERATE_HEAD, E_FULL, E_NOT_CONVERGED, E_CUDA, E_NO
 STATUS_NAMES = {0: "OK", 1: "E_INVALID", 2: "E_STATE", 3: "E_DEGENERATE_HEAD", 4: "E_FULL", 5: "E_NOT_CONVERGED",
                 6: "E_CUDA", 7: "E_NOMEM", 8: "E_DEVICE"}
 RADIUS_CONSERVATIVE, RADIUS_TIGHT = 0, 1
+INSERT_STREAMED_BIT = 1 << 3  # 1 << LIPCACHE_INSERT_STREAMED
 NOALLOC_SCRATCH_BYTES = 4259840  # LIPCACHE_NOALLOC_SCRATCH_BYTES
 PROBE_AUTO, PROBE_TENSOR, PROBE_EXACT, PROBE_TENSOR_SINGLE, PROBE_TENSOR_PAIR = 0, 1, 2, 3, 4
 
@@ -24,7 +25,7 @@ EXPORTS = ["lipcache_create", "lipcache_set_head", "lipcache_insert", "lipcache_
            "lipcache_set_radius_policy", "lipcache_insert_select", "lipcache_set_debug", "lipcache_read_entries", "lipcache_read_head",
            "lipcache_set_probe_path", "lipcache_set_radius_scale", "lipcache_set_spectral_options",
            "lipcache_reserve", "lipcache_enable_timing", "lipcache_get_info",
-           "lipcache_get_screen_info", "lipcache_reset_stats",
+           "lipcache_get_screen_info", "lipcache_insert_kernels", "lipcache_reset_stats",
            "lipcache_size", "lipcache_destroy", "lipcache_last_error"]
 
 
@@ -85,6 +86,7 @@ def load(path: str = LIB_PATH):
         "lipcache_enable_timing": ([vp, i32], C.c_int),
         "lipcache_get_info": ([vp, C.POINTER(Info)], C.c_int),
         "lipcache_get_screen_info": ([vp, C.POINTER(ScreenInfo)], C.c_int),
+        "lipcache_insert_kernels": ([vp], i64),
         "lipcache_reset_stats": ([vp], C.c_int),
         "lipcache_size": ([vp], i64),
         "lipcache_destroy": ([vp], None),

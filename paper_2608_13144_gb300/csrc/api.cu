@@ -661,6 +661,8 @@ LC_API lipcache_status lipcache_reset_stats(lipcache_t* h) {
   });
 }
 
+LC_API int64_t lipcache_insert_kernels(const lipcache_t* h) { return h ? h->insert_kernels : 0; }
+
 LC_API lipcache_status lipcache_get_screen_info(lipcache_t* h, lipcache_screen_info* info) {
   return guarded([&] {
     check_handle(h);

@@ -1737,6 +1737,7 @@ void launch_certify(lipcache* h, const float* H, int64_t n, const int32_t* paylo
     bool head_streamed = false;
     fixed_in_kernel = certify_tc_launch(h, a, s, head_streamed);
     h->last_insert_kernel = head_streamed ? LIPCACHE_INSERT_STREAMED : LIPCACHE_INSERT_TENSOR;
+    h->last_insert_bit = head_streamed ? LIPCACHE_INSERT_BIT_TENSOR_STREAMED : 1 << LIPCACHE_INSERT_TENSOR;
   } else if ((!a.tight || h->ipn_up32) && vec16 && ncg > 0 && L.total <= 227 * 1024 &&
              !(h->debug_flags & LIPCACHE_DEBUG_INSERT_TILE64)) {
     const int64_t nb32 = (n + 31) / 32;
@@ -1763,6 +1764,7 @@ void launch_certify(lipcache* h, const float* H, int64_t n, const int32_t* paylo
     kern<<<grid, kThreads, L.total, s>>>(a, L, h->wt_prep, nb32);
     LC_LAUNCH_CHECK("k_certify_wt");
     h->last_insert_kernel = LIPCACHE_INSERT_WIDE_TILE;
+    h->last_insert_bit = 1 << LIPCACHE_INSERT_WIDE_TILE;
   } else if (h->C <= 256 && smem_wres <= 220 * 1024) {
     const int n_tiles = (int)((n + kWTile - 1) / kWTile);
     const int grid = n_tiles < h->num_sms ? n_tiles : h->num_sms;
@@ -1772,6 +1774,7 @@ void launch_certify(lipcache* h, const float* H, int64_t n, const int32_t* paylo
     k_certify_wres<<<grid, kThreads, smem_wres, s>>>(a, Cp, h->dpad, n_tiles, vec);
     LC_LAUNCH_CHECK("k_certify_wres");
     h->last_insert_kernel = LIPCACHE_INSERT_TILE64;
+    h->last_insert_bit = 1 << LIPCACHE_INSERT_TILE64;
   } else {
     const size_t smem = certify_smem_bytes(h->d, h->C);
     LC_CUDA(cudaFuncSetAttribute(k_certify, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1779,6 +1782,7 @@ void launch_certify(lipcache* h, const float* H, int64_t n, const int32_t* paylo
     k_certify<<<nb, kThreads, smem, s>>>(a);
     LC_LAUNCH_CHECK("k_certify");
     h->last_insert_kernel = LIPCACHE_INSERT_STREAMED;
+    h->last_insert_bit = 1 << LIPCACHE_INSERT_STREAMED;
   }
   // the FP64 pass over the rows the kernel listed (a few per 100,000; none
   // from the kernels that refine in FP64 already), unless the kernel ran it
@@ -1800,6 +1804,7 @@ void launch_certify(lipcache* h, const float* H, int64_t n, const int32_t* paylo
 void certify_insert(lipcache* h, const float* H, int64_t n, const int32_t* payload, int require_consistency,
                     int64_t* out_index, float* out_radius, cudaStream_t s, const int64_t* miss_of) {
   launch_certify(h, H, n, payload, require_consistency, miss_of, s);
+  h->insert_kernels |= h->last_insert_bit;
   const int nb = (int)((n + kRows - 1) / kRows);
   // The scan starts while the certify kernel's last CTAs run and the scatter's
   // first rows load while the scan waits (29 inserts
@@ -1873,6 +1878,7 @@ void require_certify_ok(lipcache* h, cudaStream_t s) {
 void certify_rows(lipcache* h, const float* H, int64_t n, const int32_t* payload, int require_consistency,
                   cudaStream_t s) {
   launch_certify(h, H, n, payload, require_consistency, nullptr, s);
+  h->insert_kernels |= h->last_insert_bit;
 }
 
 void consistency_check(lipcache* h, const float* Q, int64_t B, const int64_t* hit_index, int8_t* out,

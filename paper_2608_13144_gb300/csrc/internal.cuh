@@ -321,6 +321,8 @@ struct lipcache {
   bool probe_carveout_set = false;     // the prologue / finalize kernels' carveout preference
   int debug_flags = 0;     // LIPCACHE_DEBUG_* test hooks
   int last_insert_kernel = 0;  // LIPCACHE_INSERT_*
+  int last_insert_bit = 0;     // its bit of lipcache_insert_kernels
+  int64_t insert_kernels = 0;  // kernels that certified the rows passed to the table so far
   float* wt_prep = nullptr;    // the head in the wide-tile certify kernel's shared-memory layout
   size_t wt_prep_cap = 0;      // bytes allocated
   int wt_prep_ncg = 0;         // classes per thread it was laid out for (0: stale)

@@ -229,7 +229,8 @@ class LipCache:
     def save(self, path: str):
         """Checkpoint: the configuration, the head and the entries' keys and
         labels (numpy .npz). LipCache.load re-certifies the keys under the
-        head, which gives the same radii; radii are stored only to check it."""
+        head; the radii and the kernels that gave them are stored only to
+        check it."""
         inf = self.info()
         W, b = self.head()
         e = self.entries()
@@ -239,7 +240,8 @@ class LipCache:
         np.savez(path, d=self.d, C=self.C, capacity=inf["capacity"], radius_mode=mode,
                  radius_scale=inf["radius_scale"], probe_path=path_name, radius_policy=policy,
                  policy_param=inf["policy_param"], sigma=inf["sigma"], W=W, b=b, keys=e["keys"],
-                 label=e["label"], radius=e["radius"])
+                 label=e["label"], radius=e["radius"],
+                 insert_kernels=self.insert_kernels())
 
     @classmethod
     def load(cls, path: str, device: int | torch.device | None = None, batch: int = 65536) -> "LipCache":
@@ -247,9 +249,10 @@ class LipCache:
         the keys with their labels as payload (Algorithm 1 again), restore
         the probe path and radius policy. Raises if sigma differs from the
         saved one by more than 1e-12 (its iteration's accuracy) or a radius
-        by more than 4 units in its last place (which
-        certify kernel takes a batch depends on its size and alignment, and
-        their refinements round differently in the last place)."""
+        from the saved one: by a bit where both come from the same sigma and
+        from certify kernels that give the same bits, else (rows inserted
+        from buffers of another alignment, a file that does not name its
+        kernels) by more than the kernels' bound."""
         z = np.load(path if str(path).endswith(".npz") else str(path) + ".npz")
         c = cls(int(z["d"]), int(z["C"]), int(z["capacity"]), str(z["radius_mode"]), device=device)
         c.set_radius_scale(float(z["radius_scale"]))
@@ -262,13 +265,31 @@ class LipCache:
                                  torch.from_numpy(label[s:s + batch]).to(c.device))
             if n != len(keys[s:s + batch]):
                 raise ValueError("a saved entry was not re-certified")
-        ulps = np.abs(c.entries()["radius"].view(np.int32).astype(np.int64) - z["radius"].view(np.int32))
-        if ulps.max(initial=0) > 4:
+        radius, saved = c.entries()["radius"], z["radius"]
+        same = radius.view(np.uint32) == saved.view(np.uint32)
+        if not ("insert_kernels" in z.files and sigma == float(z["sigma"]) and
+                c._same_bits(int(z["insert_kernels"]), c.insert_kernels())):
+            # each kernel's radius is within 5e-6 of the exact one, and rounded once
+            with np.errstate(invalid="ignore"):
+                same |= np.abs(radius - saved) <= np.float32(1.02e-5) * saved
+        if not same.all():
             raise ValueError("re-certified radii differ from the saved ones")
         c.set_probe_path(str(z["probe_path"]))
         if str(z["radius_policy"]) != "certified":
             c.set_radius_policy(str(z["radius_policy"]), float(z["policy_param"]))
         return c
+
+    def insert_kernels(self) -> int:
+        """The certify kernels the inserted rows went through, a bit each."""
+        return int(self.L.lipcache_insert_kernels(self._h))
+
+    def _same_bits(self, a: int, b: int) -> bool:
+        """Whether the kernels of the two masks certify to the same bits: a
+        single kernel and itself; for the conservative radius, all but the
+        CUDA-core kernel that streams the head."""
+        if self.info()["radius_mode"] == _lib.RADIUS_CONSERVATIVE and not (a | b) & _lib.INSERT_STREAMED_BIT:
+            return True
+        return a == b and a & (a - 1) == 0
 
     def set_debug(self, flags: int):
         """Failure-detection test hooks (LIPCACHE_DEBUG_*; 0 = off)."""

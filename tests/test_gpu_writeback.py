@@ -325,3 +325,53 @@ def test_checkpoint_roundtrip(dev, tmp_path, mode, policy):
         np.testing.assert_array_equal(x.cpu().numpy(), y.cpu().numpy())
     cache.close()
     again.close()
+
+
+@pytest.mark.parametrize("mode", ["conservative", "tight"])
+@pytest.mark.parametrize("d,C,aligned", [(64, 10, True), (64, 10, False), (256, 200, True), (256, 200, False),
+                                         (66, 10, True)])
+def test_checkpoint_radii_checked(dev, tmp_path, mode, d, C, aligned):
+    """Radii that the same kernels certify have to come back bit for bit; those
+    of other kernels (rows that were not 16-byte aligned), or of a file that
+    does not name them, within the kernels' bound. A file whose radii or sigma
+    are further off is refused."""
+    from paper_2608_13144_gb300.lipcache import LipCache
+    rng = np.random.default_rng(d + C)
+    n = 3000
+    rows = rng.standard_normal((n, d)).astype(np.float32)
+    buf = torch.zeros(n * d + 4, device=dev)
+    H = buf[0 if aligned else 1:][:n * d].view(n, d)
+    H.copy_(T(rows, dev))
+    c = LipCache(d, C, n, mode, device=dev)
+    c.set_head(T((rng.standard_normal((C, d)) / 8).astype(np.float32), dev), T(np.zeros(C, np.float32), dev))
+    c.insert(H)
+    path = str(tmp_path / "cache.npz")
+    c.save(path)
+    z = dict(np.load(path))
+    kernels = int(z["insert_kernels"])
+    assert kernels and kernels & (kernels - 1) == 0
+    again = LipCache.load(path, device=dev)
+    exact = again._same_bits(kernels, again.insert_kernels())
+    assert exact or not aligned
+    assert not exact or np.array_equal(again.entries()["radius"], z["radius"])
+    again.close()
+    c.close()
+
+    def load(**change):
+        np.savez(path, **{k: v for k, v in {**z, **change}.items() if v is not None})
+        LipCache.load(path, device=dev).close()
+
+    r = z["radius"]
+    bit, off = r.copy(), r.copy()
+    bit[7] = np.nextafter(bit[7], np.float32(np.inf))
+    off[7] *= np.float32(1 + 3e-5)
+    if exact:
+        with pytest.raises(ValueError):
+            load(radius=bit)
+    else:
+        load(radius=bit)
+    load(radius=bit, insert_kernels=None)
+    load(sigma=z["sigma"] * (1 + 5e-13), radius=bit)
+    for bad in (dict(radius=off), dict(radius=off, insert_kernels=None), dict(sigma=z["sigma"] * (1 + 1e-11))):
+        with pytest.raises(ValueError):
+            load(**bad)

@@ -611,7 +611,7 @@ def insert_summary(w, n_acc, insert_ms, sms, clocks, kernel=None, tf32_peak=None
                                                 "frac": achieved / tf32_peak,
                                                 "peak_kind": "measured bf16 burst x nominal tf32/bf16 ratio"},
                                "alu_equiv": {"peak": alu_peak, "frac": achieved / alu_peak, "peak_kind": alu_kind},
-                               "refined_pairs_per_row": pairs / w.N, "rows_refined_over_all_classes": full_rows}
+                               "refined_pairs_per_row": pairs / w.N, "rows_off_the_usual_path": full_rows}
         else:
             out["roofline"] = {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "TFLOP/s",
                                "frac": achieved / alu_peak, "peak_kind": alu_kind}

@@ -308,7 +308,7 @@ lipcache_status lipcache_insert_select(lipcache_t* h, const float* H, int64_t n,
  * probed or written and E_FULL is returned (the number of misses is not known
  * in advance). Errors: those of lipcache_probe and lipcache_insert;
  * E_DEVICE if a bounded wait of the probe kernel expired (the probe outputs
- * then report misses and nothing is written back).
+ * then report misses, out_inserted is -1 and nothing is written back).
  */
 lipcache_status lipcache_probe_writeback(lipcache_t* h, const float* Q, int64_t B, const int32_t* payload,
                                          int32_t require_consistency, int64_t* out_index, int32_t* out_label,
@@ -445,7 +445,8 @@ lipcache_status lipcache_probe_host(lipcache_t* h, const float* Q_host, int64_t 
  * (LIPCACHE_NOALLOC_SCRATCH_BYTES per device, held by every GPU that loads
  * the library until the process exits, with 4 bytes for each of the most rows
  * it can serve beside it) and nothing is allocated. It may overlap on the GPU
- * with lipcache_probe, also of the same handle.
+ * with lipcache_probe, also of the same handle (they share only the flag of an
+ * expired wait, which either may then miss: device_errors counts it).
  * Limit: ceil(B/128)*128 * (4*d_pad + 12) bytes, plus alignment, must fit the
  * array (e.g. 4,096 queries at d <= 256); larger batches get E_INVALID with
  * the sizes in the message. The first call on a device resolves the array's

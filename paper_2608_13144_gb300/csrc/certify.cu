@@ -14,8 +14,8 @@
 // E_c = gamma_{d+2} (||W_c|| ||z|| + |b_c|), keeps every class whose FP32
 // interval can reach the true top two, and recomputes those classes with a
 // compensated FP32 dot product (Dot2, Ogita, Rump and Oishi 2005) kept as an
-// unevaluated pair hi + lo, accurate to 2 gamma_{d+40}^2 (||W_c|| ||z|| +
-// |b_c|). The true top-1 and runner-up are always among them, so m is the
+// unevaluated pair hi + lo, accurate to G (||W_c|| ||z|| + |b_c|) with the G of
+// dot2_factor. The true top-1 and runner-up are always among them, so m is the
 // margin of the full logit vector to ~1e-10 relative of the logit scale.
 // FP64 runs at a small fraction of the FP32 rate on this GPU, so only the
 // per-row margin and radius use it. For the tight radius the wide-tile kernel
@@ -30,7 +30,8 @@
 // acceptance threshold rr <= r_safe^2 (1 - eps_rc) on the canonical FP32
 // squared distance, and the screen term tau.
 //
-// Three kernels compute the FP32 logits. When d % 4 == 0 and the head fits
+// The tensor kernel (certify_tc.cu) takes what its limits allow; for the rest
+// three kernels here compute the FP32 logits. When d % 4 == 0 and the head fits
 // in shared memory, persistent CTAs keep W^T resident and take 128-row chunks
 // with 8 x NCG register tiles and the interval pass in registers
 // (k_certify_wt, both radii); with d % 4 != 0, 64-row tiles with the logits in

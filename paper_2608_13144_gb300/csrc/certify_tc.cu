@@ -32,14 +32,17 @@
 // valid for every possible y^G (its logit above lo_1, since it is at least
 // s_y1; r* below a bound from y1's row) picks the candidates, and y^G is the
 // largest refined one.
-// Each half reduces Eq. 29 over its own candidates in FP64; rows with more
-// candidates than slots take a one-warp path over every class.
+// Each half reduces Eq. 29 over its own candidates in FP64; a row with more
+// candidates than slots has them refined on one warp, a class per lane (every
+// class where the screen says nothing).
 //
 // Schedule. Persistent CTAs, one per SM, 384 threads:
-//   warp 0     TMA producer: W (resident, 128-byte swizzle, rows past C zero
-//              filled), then each tile's 128 rows (one 16 KB box per 32-feature
-//              chunk, features past d zero filled) into one of nzb buffers,
-//              and the CTA's next tile into L2;
+//   warp 0     TMA producer: W (128-byte swizzle, rows past C zero filled),
+//              once where it stays resident beside a tile's features, else in
+//              32-feature chunks through a ring for every tile (WSTREAM, below);
+//              each tile's 128 rows (one 16 KB box per 32-feature chunk,
+//              features past d zero filled) into one of nzb buffers, and the
+//              CTA's next tile into L2;
 //   warp 1     TMEM allocation; one thread issues the MMAs of a tile into one
 //              of two accumulators (columns 0 / 256);
 //   warps 2-9  epilogue, two warps per TMEM lane quarter (32 rows), each
@@ -48,9 +51,9 @@
 //              in shared memory and the top two s~ of its columns (with their
 //              classes for the tight radius), exchanged with the partner warp
 //              through a named barrier; then the candidates of its columns
-//              into the warp's pair list. The four groups of 8 lanes refine
-//              the list eight pairs at a time (two per group) into cells by
-//              (row, slot), from which each row's lane takes its own results.
+//              into the warp's pair list. The lanes refine the list a pair
+//              each (a short last round two or four lanes a pair) into cells
+//              by (row, slot), from which each row's lane takes its own results.
 //              Conservative radius: a row with more than kMaxCandTc candidates
 //              in a half, or whose Mb is not below 1e38, has every class of
 //              that half refined; the partners' running selections are merged
@@ -58,8 +61,9 @@
 //              above; such rows take the one-warp path. Rows the finals list
 //              for the FP64 pass go into a queue in shared memory;
 //   warp 10    the FP64 pass (fix_row_warp) over the queued rows, with the
-//              head read in place, while the epilogue goes on with later
-//              tiles (when its queue and scratch fit in shared memory; else
+//              head read in place (a streamed head from global memory), while
+//              the epilogue goes on with later tiles (when its queue and
+//              scratch fit in shared memory; else
 //              the rows stay listed for the stand-alone pass);
 //   warp 11    idle.
 // Every mbarrier wait is bounded; a role that gives up raises the CTA's abort

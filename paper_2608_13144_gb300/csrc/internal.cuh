@@ -76,14 +76,16 @@ constexpr double kU64 = 1.1102230246251565e-16;   // 2^-53
 inline double gamma32(int n) { return n * kU32 / (1.0 - n * kU32); }
 inline double gamma64(int n) { return n * kU64 / (1.0 - n * kU64); }
 
-// Relative error bound of the canonical FP32 squared distance (probe_common.cuh): every term e_j^2 passes one subtraction rounding (which
+// Relative error bound of the canonical FP32 squared distance
+// (probe_common.cuh): every term e_j^2 passes one subtraction rounding (which
 // at most doubles in the square), at most 32 roundings inside its 32-wide
 // chunk and at most d_pad/32 - 1 roundings while the chunk sums are added, so
 // |S~ - S| <= gamma_{d_pad/32 + 33} S (all terms are non-negative). A small
 // slack covers the FP64 arithmetic that forms the threshold.
 inline double eps_recheck(int dpad) { return gamma32(dpad / 32 + 33) * (1.0 + 1.0 / 1024); }
 
-// Relative slack of the tensor-core screen. With TF32 operands (10 explicit
+// Relative slack of the tensor-core screen (of FP16 operands: key16.cuh, half
+// of what this allows). With TF32 operands (10 explicit
 // mantissa bits, error <= 2^-10 relative whether truncated or rounded) a
 // product is within (2^-9 + 2^-20)|q_j k_j|; FP32-or-better accumulation of
 // d_pad products adds at most d_pad 2^-22 sum|q_j k_j|. The sum |q_j k_j| is
@@ -144,7 +146,7 @@ struct DevStats {
   int abort_flag;  // kernels whose bounded wait expired; cleared per probe and certification
   int fix_count;   // rows of the current certification listed for the FP64 pass (cleared per certification)
   unsigned long long ins_pairs;      // (row, class) pairs refined by the tensor certify kernel
-  unsigned long long ins_full_rows;  // row halves it refined over every class
+  unsigned long long ins_full_rows;  // rows (conservative radius: row halves) off its usual path
   unsigned long long ins_fp64_rows;  // rows re-certified by the FP64 pass
 };
 
@@ -230,7 +232,7 @@ struct lipcache {
   lc::SpecResult* spec = nullptr;        // device
   lc::SpecResult* spec_host = nullptr;   // pinned
 
-  unsigned char* arena = nullptr;       // the table (but its FP16 copy), the head's arrays above, the report, ins_size0
+  unsigned char* arena = nullptr;       // the table (but its FP16 copy), the head's arrays above, the report, the counters, ins_size0
   unsigned char* ins_arena = nullptr;   // insert scratch
   unsigned char* q_arena = nullptr;     // probe scratch
   unsigned char* h_arena = nullptr;     // host-buffer probe staging

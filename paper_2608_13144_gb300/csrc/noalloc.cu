@@ -10,10 +10,11 @@
 // The array is a file-scope __device__ variable: every GPU that loads the
 // library holds LIPCACHE_NOALLOC_SCRATCH_BYTES of it until the process exits.
 // All calls on a device share it and each call overwrites what it needs
-// (padded queries, per-query screen constants, and the reduction words,
-// which the prologue kernel resets to their empty value), so calls whose
-// work overlaps on the GPU (different streams, handles or threads on the
-// same device) race on it and must be serialised by the caller.
+// (the queries as the screen reads them, per-query screen constants, and the
+// reduction words, which a kernel of the call first resets to their empty
+// value), so calls whose work overlaps on the GPU (different streams, handles
+// or threads on the same device) race on it and must be serialised by the
+// caller. lipcache_probe shares none of it.
 #include <mutex>
 
 #include "internal.cuh"

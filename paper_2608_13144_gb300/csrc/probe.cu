@@ -18,8 +18,8 @@
 // Kernels: k_prologue / k_prologue16 (pads or rounds the queries, per-query
 // screen constant, clears the reduction words; not for the exact kernel), the
 // main kernel (exact: every pair on CUDA cores; tensor: tcgen05 screen +
-// recheck, probe_tc.cu), which unpacks small batches itself, and else
-// k_finalize.
+// recheck, probe_tc.cu and probe_pair.cu), which unpacks small batches itself,
+// and else k_finalize. k_clear empties the words where nothing before did.
 #include <algorithm>
 
 #include "internal.cuh"

@@ -21,7 +21,7 @@
 // counted on the pair leader's barriers (.cta_group::2).
 // Per CTA (320 threads):
 //   warp 0     TMA producer (both CTAs): the CTA's key half (one barrier pair
-//              per 32-float chunk) and its query quarter of every stage;
+//              per 128-byte chunk) and its query quarter of every stage;
 //   warp 1     allocates the pair's TMEM (both CTAs); in the leader, one
 //              thread issues the pair MMAs into one of two accumulators and
 //              releases query stages (all four CTAs), key chunks and

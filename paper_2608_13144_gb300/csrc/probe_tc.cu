@@ -1,6 +1,6 @@
-// Tensor-core probe: screen every (query, key) pair with a TF32 tcgen05
-// contraction, recheck the few candidates with the exact canonical FP32
-// distance (Sec. 3.4, Algorithm 2, Eqs. 13-15; cost model Eq. 16).
+// Tensor-core probe: screen every (query, key) pair with a tcgen05 contraction
+// in FP16 (or TF32, below), recheck the few candidates with the exact canonical
+// FP32 distance (Sec. 3.4, Algorithm 2, Eqs. 13-15; cost model Eq. 16).
 //
 // Operands. The screen reads the table's FP16 copy and FP16 queries scaled per
 // row by a power of two (key16.cuh): the same 11-bit significand as TF32, at
@@ -21,7 +21,8 @@
 //     a > (1 - c) |q|^2 / 2 + ((1 - c) |k|^2 - R_k) / 2 = kappa_q + tau_k,
 // with kappa_q (per query, k_prologue) rounded down and tau_k (per key,
 // stored at insertion) rounded down. The epilogue keeps a pair iff
-// fl(a - tau_k) >= kappa_q, which therefore never drops an acceptable pair.
+// fl(a - tau_k) >= kappa_q, which therefore never drops an acceptable pair. Rows
+// that fill the last query tile up have a NaN for kappa and pass nothing.
 // It first tests each 32-key chunk with fl(max a - min tau) >= kappa_q, which no
 // chunk holding a kept pair fails; the maximum comes with the TMEM load
 // (tcgen05.ld.red), and only a passing chunk's products are looked at.
@@ -662,7 +663,8 @@ void launch_nh(lipcache* h, int64_t B, const ProbeBuffers& b, const ProbeOut& ou
   a.stats = h->stats;
   // With one to three tiles per cluster the recheck warp's turn would only come
   // at the end: 256 x 50,000 at d = 64 13.4 us without it, 15.0 with; 1,024 x
-  // 50,000 at d = 128 (ten tiles) 22.1 without, 20.7 with.
+  // 50,000 at d = 128 (ten tiles) 22.1 without, 20.7 with. The line lies between
+  // these two; nothing in between was measured.
   a.queue = n_pairs * a.nq >= 6 * (int64_t)max_clusters ? 1 : 0;
   a.debug_stall = (h->debug_flags & LIPCACHE_DEBUG_STALL_PROBE) ? 1 : 0;
   const Layout<BN> L{NH * a.nch, a.nst, a.tau_staged};

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(256) k_prologue(const float* __restrict__ Q, i
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(kFull, part, o);
   if (lane == 0) {
-    kappa[row] = row < B ? __double2float_rd(one_minus_c * (double)part * 0.5) : no_query_kappa();
+    kappa[row] = __double2float_rd(one_minus_c * (double)part * 0.5);  // (not read from B on)
     best[row] = ~0ull;
   }
 }
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256) k_prologue16(const float* __restrict__ Q,
       *reinterpret_cast<__half2*>(q16 + (size_t)row * d16 + 64 * i + 2 * lane) =
           __floats2half2_rn(x[i][0] * down, x[i][1] * down);
   if (lane == 0) {
-    kappa[row] = row < B ? __fsub_rd(__double2float_rd(one_minus_c * (double)part * 0.5), 1e-29f) : no_query_kappa();
+    kappa[row] = __fsub_rd(__double2float_rd(one_minus_c * (double)part * 0.5), 1e-29f);  // (not read from B on)
     qscale[row] = __int_as_float((127 + e) << 23);
     best[row] = ~0ull;
   }

@@ -153,14 +153,17 @@ static __device__ __noinline__ void recheck_warp(const Recheck& a, uint32_t mask
   }
 }
 
-// The screen constant of rows that are no query (those that fill the last query
-// tile up). An entry's screen term is -inf where its radius overflows (an
-// empirical policy's, a head whose rows coincide or nearly vanish), which beats
-// any constant that can be compared; every comparison with a NaN fails, so such
-// a row passes neither the chunk test nor a pair's. The recheck reads the
-// caller's own rows, which end with the last query, and the words of the
-// rows past it stay empty.
-__device__ __forceinline__ float no_query_kappa() { return __int_as_float(0x7fffffff); }
+// The screen constant of a row of a query tile: kappa, or a NaN for the rows from
+// B on that fill the last tile up. An entry's screen term is -inf where its
+// radius overflows (an empirical policy's, a head whose rows coincide or nearly
+// vanish), which beats any constant that can be compared; every comparison with
+// a NaN fails, so such a row passes neither the chunk test nor a pair's. The
+// recheck reads the caller's own rows, which end with the last query, and the
+// words of the rows past it stay empty. (Decided here by the launch's own B:
+// scratch holds another batch's constants where calls overlap.)
+__device__ __forceinline__ float row_kappa(const float* __restrict__ kappa, int64_t row, int64_t B) {
+  return row < B ? __ldg(kappa + row) : __int_as_float(0x7fffffff);
+}
 
 // Operand kinds of the tensor screen. Both stream 128-byte rows (one swizzle
 // row) per chunk and advance 32 bytes per MMA. kF16 reads the table's FP16

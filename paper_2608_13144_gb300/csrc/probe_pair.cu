@@ -291,13 +291,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       const int row_off = (int)pos * kHM + quarter * 32 + lane;
       int64_t row = (int64_t)qt0 * kBM + row_off;
-      float kap = row < a.bpad ? __ldg(a.kappa + row) : no_query_kappa();
+      float kap = row_kappa(a.kappa, row, a.out.B);
       float scl = KIND == kF16 && row < a.bpad ? __ldg(a.qscale + row) : 1.f;
       for (int qt = qt0; qt < qt1; ++qt, ++t) {
         const int buf = t & 1;
         row = (int64_t)qt * kBM + row_off;
         const int64_t row_next = row + kBM;
-        const float kap_next = (qt + 1 < qt1 && row_next < a.bpad) ? __ldg(a.kappa + row_next) : no_query_kappa();
+        const float kap_next = qt + 1 < qt1 ? row_kappa(a.kappa, row_next, a.out.B) : 0.f;
         const float scl_next = (KIND == kF16 && qt + 1 < qt1 && row_next < a.bpad) ? __ldg(a.qscale + row_next) : 1.f;
         ok = ptx::mbar_wait(acc_full + 8 * buf, (uint32_t)((t >> 1) & 1), abort_s, kWaitLimit);
         ok = __all_sync(0xffffffffu, ok);  // warp-uniform before the aligned TMEM loads

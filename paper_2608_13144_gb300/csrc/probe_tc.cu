@@ -21,8 +21,8 @@
 //     a > (1 - c) |q|^2 / 2 + ((1 - c) |k|^2 - R_k) / 2 = kappa_q + tau_k,
 // with kappa_q (per query, k_prologue) rounded down and tau_k (per key,
 // stored at insertion) rounded down. The epilogue keeps a pair iff
-// fl(a - tau_k) >= kappa_q, which therefore never drops an acceptable pair. Rows
-// that fill the last query tile up have a NaN for kappa and pass nothing.
+// fl(a - tau_k) >= kappa_q, which therefore never drops an acceptable pair. The
+// rows that fill the last query tile up get a NaN for kappa and pass nothing.
 // It first tests each 32-key chunk with fl(max a - min tau) >= kappa_q, which no
 // chunk holding a kept pair fails; the maximum comes with the TMEM load
 // (tcgen05.ld.red), and only a passing chunk's products are looked at.
@@ -460,12 +460,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
           tmin[h][ch] = m;
         }
-      float kap = __ldg(a.kappa + qt0 * kBM + quarter * 32 + lane);
+      float kap = row_kappa(a.kappa, qt0 * kBM + quarter * 32 + lane, a.out.B);
       float scl = KIND == kF16 ? __ldg(a.qscale + qt0 * kBM + quarter * 32 + lane) : 1.f;
       for (int qt = qt0; qt < qt1 && ok; ++qt) {
         const int row = qt * kBM + quarter * 32 + lane;
         // next tile's screen constant, fetched while this accumulator is produced
-        const float kap_next = (qt + 1 < qt1) ? __ldg(a.kappa + row + kBM) : 0.f;
+        const float kap_next = (qt + 1 < qt1) ? row_kappa(a.kappa, row + kBM, a.out.B) : 0.f;
         const float scl_next = (KIND == kF16 && qt + 1 < qt1) ? __ldg(a.qscale + row + kBM) : 1.f;
 #pragma unroll
         for (int h = 0; h < NH; ++h, ++t) {
